@@ -34,7 +34,7 @@ sys.path.insert(0, ROOT)
 
 B_MIN_FP32 = 144          # bytes per lattice update: 2 distributions x 9 x (read + write) x 4 B
 REINIT_EVERY = 8
-KERNEL_SOURCES = ("paper_1110_5004_gb300/csrc/lbm_device.cuh", "paper_1110_5004_gb300/csrc/lbm_kernels.cu")
+KERNEL_SOURCES = tuple("paper_1110_5004_gb300/csrc/" + f for f in ("lbm_device.cuh", "lbm_march.cuh", "lbm_rows.cuh"))
 
 
 def parse():

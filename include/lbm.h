@@ -214,6 +214,8 @@ LBM_API long long lbm_step_count(const lbm_sim* sim);
  * lbm_checkpoint_bytes: size of the checkpoint of `sim` (0 if sim is NULL).
  * lbm_checkpoint: writes it to `buf` (host or device memory, at least checkpoint_bytes long,
  *   caller-owned); synchronous.  A batch member must be removed from its batch first.
+ *   A checkpoint holds every population at the cell it leaves; simulations keep them in another
+ *   order, so both calls convert (through the simulation's own work planes, without allocating).
  * lbm_restore: replaces the state of `sim` (same nx, ny and storage; its parameters and stream
  *   are its own) by the checkpoint in `buf`, including the step count; synchronous.
  * Errors: LBM_ERR_INVALID_ARG for NULL arguments, a short buffer, a batch member, a bad header
@@ -227,10 +229,9 @@ LBM_API int lbm_restore(lbm_sim* sim, const void* buf, size_t bytes);
  * stream is synchronised first (the state's allocation and earlier work are ordered on it). */
 LBM_API int lbm_set_stream(lbm_sim* sim, void* cuda_stream);
 
-/* Tile shape of the fused step kernel: threads per CTA (64, 128 or 256; the CTA covers
- * threads - 6 interior columns) and rows per CTA (>= 1).  0 keeps the current value.  A new
- * simulation has 128 threads and as many rows per CTA as make one wave of resident CTAs
- * (at least 8 rows). */
+/* Tile shape of the row march: rows per CTA (>= 1).  0 keeps the current value; a new simulation has as
+ * many rows per CTA as make one wave of resident CTAs.  threads (64, 128, 256 or 0) is accepted and has
+ * no effect: every CTA has 128 threads of two columns each.  Results do not depend on the shape. */
 LBM_API int lbm_set_tile(lbm_sim* sim, int threads, int seg_rows);
 
 /* Step kernel of the simulation (no counterpart in the paper; both kernels compute every cell
@@ -314,8 +315,8 @@ LBM_API int lbm_batch_create(size_t budget_bytes, void* cuda_stream, lbm_batch**
 LBM_API int lbm_batch_add(lbm_batch* b, lbm_sim* sim, int* slot);
 LBM_API int lbm_batch_remove(lbm_batch* b, int slot);
 LBM_API int lbm_batch_step(lbm_batch* b, int k);
-/* Tile shape of the batch kernel (threads per CTA 64/128/256; rows per tile for members that
- * did not set their own, >= 1); 0 keeps the current value.  Takes effect at the next step. */
+/* Rows per tile of the batch kernel for members that did not set their own (>= 1; 0 keeps the current
+ * value); threads as in lbm_set_tile.  Takes effect at the next step. */
 LBM_API int lbm_batch_set_tile(lbm_batch* b, int threads, int seg_rows);
 /* Members, device bytes in use. */
 LBM_API int lbm_batch_size(const lbm_batch* b);

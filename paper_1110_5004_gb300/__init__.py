@@ -116,9 +116,8 @@ class Sim:
             pass
 
     def set_tile(self, threads=0, seg_rows=0):
-        """Tile of the step kernel: threads per CTA (64, 128 or 256) and rows per CTA; 0 keeps
-        the current value of either (a simulation starts with as many rows per CTA as fill one
-        wave of resident CTAs)."""
+        """Tile of the row march: rows per CTA (0 keeps the current value; a simulation starts with
+        as many as fill one wave of resident CTAs).  `threads` (64, 128, 256 or 0) has no effect."""
         _lib.check(lib().lbm_set_tile(self._h, int(threads), int(seg_rows)))
 
     def set_kernel(self, kernel):
@@ -252,8 +251,8 @@ class Batch:
         _lib.check(lib().lbm_batch_step(self._h, int(k)))
 
     def set_tile(self, threads=0, seg_rows=0):
-        """Tile of the batch kernel for members without their own rows per CTA; 0 keeps the
-        current value of either."""
+        """Rows per tile of the batch kernel for members without their own; 0 keeps the current
+        value.  `threads` as in Sim.set_tile."""
         _lib.check(lib().lbm_batch_set_tile(self._h, int(threads), int(seg_rows)))
 
     @property

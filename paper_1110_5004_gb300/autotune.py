@@ -1,7 +1,7 @@
 """Tile-shape autotuner for the fused step kernel and the batch kernel.
 
-The step kernel's shape is (threads per CTA, rows per CTA).  Threads fix the strip width
-(threads - 6 interior columns); rows trade pipeline fill (a segment of h rows runs h + 8 row
+The step kernel's shape is (threads per CTA, rows per CTA).  The library's CTAs have one width, whatever
+`threads` says; rows trade pipeline fill (a segment of h rows runs h + 7 row
 iterations, the first and last few with stages idle) for parallelism (one CTA per strip x
 segment).  The kernel is bound by instruction issue, so a step lasts as long as the SM with the
 most CTAs: besides a fixed list of heights, the candidates include, for k = 1..8 resident CTAs
@@ -28,7 +28,7 @@ _lock = threading.Lock()
 
 def _kernel_hash():
     h = hashlib.sha256()
-    for f in ("lbm_device.cuh", "lbm_kernels.cu", "lbm_batch.cu"):
+    for f in ("lbm_device.cuh", "lbm_march.cuh", "lbm_rows.cuh", "lbm_batch.cuh"):
         with open(os.path.join(HERE, "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:12]

@@ -13,7 +13,9 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblbm.so")
-SOURCES = ["lbm_kernels.cu", "lbm_tile2d.cu", "lbm_batch.cu", "lbm_api.cu", "lbm_noalloc.cu"]
+SOURCES = ["lbm_rows_fp32.cu", "lbm_rows_fp16.cu", "lbm_rows_bf16.cu", "lbm_rows_moments.cu",
+           "lbm_kernels.cu", "lbm_tile2d.cu", "lbm_batch.cu", "lbm_batch_fp32.cu", "lbm_batch_fp16.cu", "lbm_batch_bf16.cu",
+           "lbm_api.cu", "lbm_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

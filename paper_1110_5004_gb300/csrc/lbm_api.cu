@@ -10,6 +10,7 @@
 #include <string>
 
 #include "lbm_internal.h"
+#include "lbm_march.cuh"
 
 namespace lbm {
 
@@ -32,6 +33,7 @@ int cuda_fail(cudaError_t e, const char* what) {
 Phys make_phys(const lbm_params& p) {
   Phys P{};
   const double cs2 = 1.0 / 3.0;
+  const double rho_prime = (p.rho_A - p.rho_B) / (2.0 * p.phi_star);
   P.four_beta = (float)(4.0 * p.beta);
   P.kappa = (float)p.kappa;
   P.phi_star = (float)p.phi_star;
@@ -39,20 +41,16 @@ Phys make_phys(const lbm_params& p) {
   P.inv_2phistar = (float)(1.0 / (2.0 * p.phi_star));
   P.rho_B = (float)p.rho_B;
   P.drho = (float)(p.rho_A - p.rho_B);
-  P.rho_prime = (float)((p.rho_A - p.rho_B) / (2.0 * p.phi_star));
-  P.s_coef = (float)((p.rho_A - p.rho_B) / (2.0 * p.phi_star) * p.theta_M);
-  P.gravity = (float)p.gravity;
+  P.ngravity = -(float)p.gravity;
   P.omega_f = (float)(1.0 / p.tau_f);
   P.three_gamma_f = (float)(3.0 * p.theta_M / (p.tau_f - 0.5));
-  P.mu_A = (float)(p.rho_A * cs2 * (p.tau_g_A - 0.5));
-  P.mu_B = (float)(p.rho_B * cs2 * (p.tau_g_B - 0.5));
   P.remove_Fa = p.remove_Fa ? 1 : 0;
   P.ch_conv = p.ch_conservative ? 0 : 1;
   P.fs_mu = p.fs_form ? 1 : 0;
   P.s_direct = p.s_form ? 1 : 0;
-  P.kappa6 = (float)(p.kappa / 6.0);
-  P.rho_prime12 = (float)((p.rho_A - p.rho_B) / (2.0 * p.phi_star) / 12.0);
-  P.s_coef6 = (float)((p.rho_A - p.rho_B) / (2.0 * p.phi_star) * p.theta_M / 6.0);
+  P.nkappa6 = -(float)(p.kappa / 6.0);
+  P.rho_prime12 = (float)(rho_prime / 12.0);
+  P.s_coef6 = (float)(rho_prime * p.theta_M / 6.0);
   P.mu3_B = (float)(3.0 * p.rho_B * cs2 * (p.tau_g_B - 0.5));
   P.mu3_d = (float)(3.0 * (p.rho_A * cs2 * (p.tau_g_A - 0.5) - p.rho_B * cs2 * (p.tau_g_B - 0.5)));
   P.keep_f = (float)(1.0 - 1.0 / p.tau_f);
@@ -63,17 +61,17 @@ Phys make_phys(const lbm_params& p) {
   return P;
 }
 
-void tile_geometry(int nx, int ny, int nt, int seg_h, int slots, int* tile_w, int* n_strips, int* seg_out) {
-  const int wmax = nt - 6;
-  const int ns = (nx + wmax - 1) / wmax;
+void tile_geometry(int nx, int ny, bool sd, int seg_h, int slots, int* tile_w, int* n_strips, int* seg_out) {
+  const int most = 2 * march_width(sd), ns = (nx + most - 1) / most;
   *n_strips = ns;
-  *tile_w = (nx + ns - 1) / ns;
+  *tile_w = (nx + 2 * ns - 1) / (2 * ns);
   if (seg_h <= 0) {
-    // as many segments as fit in one wave of `slots` resident CTAs: the step is issue-bound and
-    // lasts as long as the busiest SM, so a count just above the slots adds a nearly empty wave
+    // as many segments as fit in one wave of `slots` resident CTAs: the step lasts as long as the
+    // busiest SM, so a count just above the slots adds a nearly empty wave.  Segments of a few rows spend
+    // most of their h + 7 iterations on the rows around them, and are still the fastest where the grid has
+    // no more rows to give (601 x 437 with side walls: 18.1 us at 5 rows, 22.4 at 8)
     const int segs = slots >= ns ? slots / ns : 1;
     seg_h = (ny + segs - 1) / segs;
-    if (seg_h < 8) seg_h = 8;
   }
   *seg_out = seg_h;
 }
@@ -83,18 +81,16 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
   g.src = src;
   g.dst = dst;
   g.plane = (int)s->plane;
-  g.row_bytes = s->pitch / BLK * block_bytes(s->params.storage);
+  g.row_bytes = (int)(s->pitch * state_bytes_per_cell(s->params.storage));
+  g.nblk = s->pitch / BLK;
   g.storage = s->params.storage;
-  g.sf = s->sf;
-  g.isf = 1.0f / s->sf;
-  g.sg = s->sg;
-  g.isg = 1.0f / s->sg;
   g.nx = s->nx;
   g.ny = s->ny;
   g.pitch = s->pitch;
   g.bc_x = s->params.bc_x;
   g.bc_y = s->params.bc_y;
-  tile_geometry(s->nx, s->ny, s->nt, s->seg_h, s->sms * (s->occ > 0 ? s->occ : 1), &g.tile_w, &g.n_strips, &g.seg_h);
+  tile_geometry(s->nx, s->ny, s->params.s_form != 0, s->seg_h, s->sms * MARCH_CTAS, &g.tile_w, &g.n_strips, &g.seg_h);
+  g.gave_up = reinterpret_cast<unsigned int*>(s->red + (size_t)s->ny * DIAG_PARTIALS + 14);
   g.spoff = s->params.s_form ? (long long)s->pop_bytes : 0;
   return g;
 }
@@ -187,12 +183,11 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
   s->plane = (long long)ny * s->pitch;
   s->params = *params;
   s->phys = make_phys(*params);
+  s->phys2 = widen(s->phys);
   s->stream = (cudaStream_t)cuda_stream;
   const size_t pop_bytes = (size_t)state_bytes_per_cell(params->storage) * s->plane;
   s->pop_bytes = pop_bytes;
   s->buf_bytes = pop_bytes + (params->s_form ? 2 * sizeof(float) * (size_t)s->plane : 0);
-  // FP16 keeps the O(mu, u) populations in its normal range: 2^12 maps 1.5e-8 .. 16 onto it
-  if (params->storage == LBM_FP16_DEV) s->sf = s->sg = 4096.0f;
   cudaError_t e;
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
@@ -201,7 +196,6 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
     delete s;
     return rc;
   }
-  s->occ = tile_occupancy(s->nt);
   // Stream-ordered allocations from the device's memory pool, on the simulation's stream: unlike
   // cudaMalloc they do not order the other streams of the device, so a server can create a
   // simulation while others run.  The memory is ordered on s->stream (lbm_set_stream and
@@ -221,6 +215,7 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
   cudaMemsetAsync(s->buf[0], 0, s->buf_bytes, s->stream);
   cudaMemsetAsync(s->buf[1], 0, s->buf_bytes, s->stream);
   cudaMemsetAsync(s->fields, 0, (size_t)N_FIELDS * s->plane * sizeof(float), s->stream);
+  cudaMemsetAsync(s->red + (size_t)ny * DIAG_PARTIALS, 0, 16 * sizeof(double), s->stream);
   if ((e = cudaGetLastError()) != cudaSuccess) {
     rc = cuda_fail(e, "lbm_create memset");
     lbm_destroy(s);
@@ -355,7 +350,7 @@ int lbm_step(lbm_sim* s, int n) {
   const bool tiles = uses_tile2d(s);
   for (int i = 0; i < n; ++i) {
     Grid g = make_grid(s, s->buf[s->cur], s->buf[s->cur ^ 1]);
-    cudaError_t e = tiles ? launch_tile2d(s->phys, g, s->sms, s->stream) : launch_step(s->phys, g, s->nt, s->stream);
+    cudaError_t e = tiles ? launch_tile2d(s->phys, g, s->sms, s->stream) : launch_step(s->phys2, g, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "lbm_step launch");
     s->cur ^= 1;
     s->steps++;
@@ -368,7 +363,7 @@ static int compute_moments(lbm_sim* s) {
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
   MomentOut mo{s->fields, s->fields + s->plane, s->fields + 2 * s->plane, s->fields + 3 * s->plane,
                s->fields + 4 * s->plane};
-  cudaError_t e = launch_moments(s->phys, g, mo, s->nt, s->stream);
+  cudaError_t e = launch_moments(s->phys2, g, mo, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "moments launch");
   s->launches++;
   return LBM_OK;
@@ -418,7 +413,7 @@ int lbm_moments(lbm_sim* s, float* phi, float* rho, float* ux, float* uy, float*
   }
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
   MomentOut mo{dst[0], dst[1], dst[2], dst[3], dst[4]};
-  cudaError_t e = launch_moments(s->phys, g, mo, s->nt, s->stream);
+  cudaError_t e = launch_moments(s->phys2, g, mo, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "moments launch");
   s->launches++;
   return copy_out(s, staged, 5, "lbm_moments copy");
@@ -434,7 +429,7 @@ int lbm_moments_packed(lbm_sim* s, float* fields) {
   const size_t stride = direct ? n : (size_t)s->plane;
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
   MomentOut mo{dst, dst + stride, dst + 2 * stride, dst + 3 * stride, dst + 4 * stride};
-  cudaError_t e = launch_moments(s->phys, g, mo, s->nt, s->stream);
+  cudaError_t e = launch_moments(s->phys2, g, mo, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_moments_packed launch");
   s->launches++;
   if (!direct) {
@@ -453,7 +448,7 @@ int lbm_interfacial_force(lbm_sim* s, float* fa_x, float* fa_y) {
   MomentOut mo{};
   mo.fax = s->fields;
   mo.fay = s->fields + s->plane;
-  cudaError_t e = launch_moments(s->phys, g, mo, s->nt, s->stream);
+  cudaError_t e = launch_moments(s->phys2, g, mo, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_interfacial_force launch");
   s->launches++;
   float* outs[2] = {fa_x, fa_y};
@@ -510,6 +505,42 @@ constexpr uint32_t CKPT_MAGIC = 0x434d424cu;   // "LBMC" little-endian
 constexpr uint32_t CKPT_VERSION = 2;
 
 size_t payload_bytes(const lbm_sim* s) { return s->buf_bytes; }
+
+// The current state between its buffer (class by class) and a checkpoint's payload
+// (blocks of 32 cells, then the s_form planes).  A device payload that is 16-byte aligned is read or
+// written by the reordering kernel itself; otherwise the populations pass through the field work
+// planes, as many at a time as those hold (no allocation: a server evicts when memory is short).
+cudaError_t move_payload(lbm_sim* s, char* payload, bool to_payload, bool dev) {
+  char* state = static_cast<char*>(s->buf[s->cur]);
+  const long long units = (long long)(s->pop_bytes / 16);
+  cudaError_t e = cudaSuccess;
+  if (dev && reinterpret_cast<uintptr_t>(payload) % 16 == 0) {
+    e = launch_reorder(s, state, payload, 0, units, to_payload, s->stream);
+  } else {
+    const long long room = (long long)((size_t)N_FIELDS * s->plane * sizeof(float) / 16);
+    for (long long u0 = 0; u0 < units && e == cudaSuccess; u0 += room) {
+      const long long u1 = u0 + room < units ? u0 + room : units;
+      char* part = payload + u0 * 16;
+      if (to_payload) {
+        e = launch_reorder(s, state, s->fields, u0, u1, true, s->stream);
+        if (e == cudaSuccess)
+          e = cudaMemcpyAsync(part, s->fields, (size_t)(u1 - u0) * 16,
+                              dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s->stream);
+      } else {
+        e = cudaMemcpyAsync(s->fields, part, (size_t)(u1 - u0) * 16,
+                            dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s->stream);
+        if (e == cudaSuccess) e = launch_reorder(s, state, s->fields, u0, u1, false, s->stream);
+      }
+    }
+  }
+  const size_t rest = s->buf_bytes - s->pop_bytes;
+  if (e == cudaSuccess && rest) {
+    char *planes = state + s->pop_bytes, *part = payload + s->pop_bytes;
+    e = to_payload ? cudaMemcpyAsync(part, planes, rest, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s->stream)
+                   : cudaMemcpyAsync(planes, part, rest, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s->stream);
+  }
+  return e;
+}
 }  // namespace
 
 extern "C" {
@@ -533,10 +564,9 @@ int lbm_checkpoint(lbm_sim* s, void* buf, size_t bytes) {
   h.payload = payload_bytes(s);
   const bool dev = is_device_ptr(buf);
   const cudaMemcpyKind kh = dev ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost;
-  const cudaMemcpyKind kp = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   cudaError_t e = cudaMemcpyAsync(buf, &h, sizeof(h), kh, s->stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(static_cast<char*>(buf) + sizeof(h), s->buf[s->cur], h.payload, kp, s->stream);
+    e = move_payload(s, static_cast<char*>(buf) + sizeof(h), true, dev);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);   // h lives on this stack frame
   return e == cudaSuccess ? LBM_OK : cuda_fail(e, "lbm_checkpoint copy");
 }
@@ -557,8 +587,7 @@ int lbm_restore(lbm_sim* s, const void* buf, size_t bytes) {
     return set_error("checkpoint of a %dx%d storage-%d grid, simulation is %dx%d storage %d", h.nx, h.ny, h.storage,
                      s->nx, s->ny, s->params.storage), LBM_ERR_INVALID_ARG;
   if (bytes < sizeof(h) + h.payload) return set_error("checkpoint truncated"), LBM_ERR_INVALID_ARG;
-  e = cudaMemcpyAsync(s->buf[s->cur], static_cast<const char*>(buf) + sizeof(h), h.payload,
-                      dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s->stream);
+  e = move_payload(s, const_cast<char*>(static_cast<const char*>(buf)) + sizeof(h), false, dev);
   if (e == cudaSuccess) e = rearm_resident(s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_restore copy");
@@ -580,10 +609,6 @@ int lbm_set_tile(lbm_sim* s, int threads, int seg_rows) {
   if (threads && threads != 64 && threads != 128 && threads != 256)
     return set_error("threads must be 64, 128 or 256"), LBM_ERR_INVALID_ARG;
   if (seg_rows < 0) return set_error("seg_rows must be >= 1"), LBM_ERR_INVALID_ARG;
-  if (threads) {
-    s->nt = threads;
-    s->occ = tile_occupancy(threads);
-  }
   if (seg_rows) s->seg_h = seg_rows;
   return LBM_OK;
 }

@@ -1,94 +1,21 @@
 // Ragged batches: many independent simulations (any sizes and parameters) advanced by one
-// persistent launch per time step over a work list of (simulation, strip, segment) tiles; two
-// launches when some members use the direct mass defect (its tiles run in their own kernel
-// instance).  Steps run as replays of one 16-step CUDA graph captured once per membership, the
-// remainder of a step count as direct launches.  Each tile runs exactly the per-cell arithmetic of the single-simulation kernel
-// (every operation an explicit round-to-nearest intrinsic), so a member's state is bitwise the
-// same alone or inside any mix.
+// persistent launch per time step over a work list of (simulation, strip, segment) tiles; one launch per
+// storage present, and one more per storage for members that use the direct mass defect.  Steps run as
+// replays of one 16-step CUDA graph captured once per membership, the remainder of a step count as direct
+// launches.  Each tile runs the row march of the single-simulation kernel (every operation rounded to
+// nearest explicitly), so a member's state is bitwise the same alone or inside any mix.
 #include <algorithm>
 #include <map>
 #include <new>
 #include <vector>
 
-#include "lbm_internal.h"
-
-namespace lbm {
-
-struct SimDesc {
-  Phys P;
-  Grid g;                 // src/dst unused; buffers below
-  const void* buf0;
-  void* buf1;
-  int cur0;               // buffer holding the state when the graph replay starts
-  int pad;
-};
-
-// SD: the work list holds the tiles of members that use the direct mass defect (s_form 1), and
-// only that tile body is compiled in.  One function holding both bodies (each for three
-// storages) did not fit 128 registers: it spilled 1.2 KB per thread, and a batch of s_form 1
-// members ran at 14.5 GLUPS against 18.8 with the instances split.
-// XW: some member may have walls on x; false compiles out the ghost columns and column wall tests
-// (every member periodic in x).
-template <int NT, bool SD, bool XW>
-__global__ void __launch_bounds__(NT, 512 / NT) k_batch(const SimDesc* __restrict__ sims, const int4* __restrict__ work,
-                                              int n_work, int parity) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Smem<NT>& sm = *reinterpret_cast<Smem<NT>*>(smem_raw);
-  for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
-    const int4 it = work[w];
-    const SimDesc& d = sims[it.x];
-    Grid g = d.g;
-    const bool odd = ((d.cur0 + parity) & 1) != 0;
-    g.src = odd ? d.buf1 : d.buf0;
-    g.dst = odd ? const_cast<void*>(d.buf0) : d.buf1;
-    // members may differ in storage; the branch is uniform per tile
-    switch (g.storage) {
-      case ST_FP16: run_tile<NT, MODE_STEP, ST_FP16, SD, false, XW, false>(d.P, g, MomentOut{}, it.y, it.z, sm); break;
-      case ST_BF16: run_tile<NT, MODE_STEP, ST_BF16, SD, false, XW, false>(d.P, g, MomentOut{}, it.y, it.z, sm); break;
-      default: run_tile<NT, MODE_STEP, ST_FP32, SD, false, XW, false>(d.P, g, MomentOut{}, it.y, it.z, sm); break;
-    }
-    __syncthreads();  // shared rings are reused by the next tile
-  }
-}
-
-}  // namespace lbm
+#include "lbm_batch.cuh"
 
 using namespace lbm;
 
-template <bool SD, bool XW>
-static cudaError_t set_batch_attr_sd(int nt) {
-  switch (nt) {
-    case 64: return cudaFuncSetAttribute(k_batch<64, SD, XW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem<64>));
-    case 256: return cudaFuncSetAttribute(k_batch<256, SD, XW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem<256>));
-    default: return cudaFuncSetAttribute(k_batch<128, SD, XW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem<128>));
-  }
-}
-
-// Members with the direct mass defect always run the general form: its periodic form does not
-// fit 128 registers (it spilled 36 bytes per thread).
-static cudaError_t set_batch_attr(int nt, bool sd, bool xw) {
-  if (sd) return set_batch_attr_sd<true, true>(nt);
-  return xw ? set_batch_attr_sd<false, true>(nt) : set_batch_attr_sd<false, false>(nt);
-}
-
-template <bool SD, bool XW>
-static int batch_occupancy_t(int nt) {
-  int occ = 0;
-  switch (nt) {
-    case 64: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<64, SD, XW>, 64, sizeof(Smem<64>)); break;
-    case 256: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<256, SD, XW>, 256, sizeof(Smem<256>)); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<128, SD, XW>, 128, sizeof(Smem<128>)); break;
-  }
-  return occ;
-}
-
-template <bool SD>
-static int batch_occupancy_sd(int nt, bool xw) {
-  if constexpr (SD) return batch_occupancy_t<SD, true>(nt);
-  else return xw ? batch_occupancy_t<SD, true>(nt) : batch_occupancy_t<SD, false>(nt);
-}
-
 constexpr int GRAPH_STEPS = 16;        // steps per captured graph (even: parity-neutral)
+
+constexpr int N_PARTS = 6;              // storage + 3 x (direct mass defect)
 
 struct lbm_batch {
   size_t budget = 0;
@@ -96,15 +23,15 @@ struct lbm_batch {
   cudaStream_t stream = nullptr;
   cudaStream_t cap = nullptr;          // private stream for graph capture
   std::vector<lbm_sim*> slots;         // nullptr = free slot
-  int nt = 128;
   int seg_h = 32;                      // rows per tile for members without their own choice
   bool dirty = true;                   // descriptors / work list need rebuilding
   SimDesc* d_sims = nullptr;
   int4* d_work = nullptr;
   size_t cap_sims = 0, cap_work = 0;
   int n_work = 0;
-  int n_plain = 0;                     // work[0, n_plain): members without the direct mass defect
-  int grid_plain = 0, grid_sd = 0;     // persistent grid of each launch
+  struct Part {                        // tiles of one storage and one form of the mass defect: a launch each
+    int first = 0, count = 0, grid = 0;
+  } parts[N_PARTS];
   int flip = 0;                        // parity offset of every member since the last rebuild
   bool xwall = true;                   // some member has walls on x (the general kernel form)
   std::map<int, cudaGraphExec_t> graphs;  // flip -> executable graph of GRAPH_STEPS steps
@@ -121,20 +48,19 @@ static int rebuild(lbm_batch* b) {
   std::vector<int> members;
   for (size_t i = 0; i < b->slots.size(); ++i)
     if (b->slots[i]) members.push_back((int)i);
-  // interleave the members' tiles so concurrent CTAs spread over simulations; the tiles of
-  // members with the direct mass defect follow those of the others (a launch of their own)
-  std::vector<std::vector<int4>> per[2];
+  // interleave the members' tiles so concurrent CTAs spread over simulations; members of different
+  // storages, and those with the direct mass defect, have launches of their own
+  std::vector<std::vector<int4>> per[N_PARTS];
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->xwall = false;
   for (int m : members) b->xwall = b->xwall || b->slots[m]->params.bc_x == LBM_WALL;
-  set_batch_attr(b->nt, false, b->xwall);   // the occupancy query needs the shared-memory size admitted
-  const int slots = sms * std::max(batch_occupancy_sd<false>(b->nt, b->xwall), 1);
+  const int slots = sms * MARCH_CTAS;
   for (size_t m = 0; m < members.size(); ++m) {
     lbm_sim* s = b->slots[members[m]];
     SimDesc d{};
-    d.P = s->phys;
+    d.P = s->phys2;
     Grid g = make_grid(s, nullptr, nullptr);
     // one wave of the batch kernel is shared by all members: size segments for the batch.  A
     // member large enough to fill the wave on its own gets segments of the height that does so
@@ -142,10 +68,10 @@ static int rebuild(lbm_batch* b) {
     int h = s->seg_h ? s->seg_h : b->seg_h;
     if (!s->seg_h) {
       int tw = 0, ns = 0, hw = 0;
-      tile_geometry(s->nx, s->ny, b->nt, 0, slots, &tw, &ns, &hw);
+      tile_geometry(s->nx, s->ny, s->params.s_form != 0, 0, slots, &tw, &ns, &hw);
       h = std::max(h, hw);
     }
-    tile_geometry(s->nx, s->ny, b->nt, h, 0, &g.tile_w, &g.n_strips, &g.seg_h);
+    tile_geometry(s->nx, s->ny, s->params.s_form != 0, h, 0, &g.tile_w, &g.n_strips, &g.seg_h);
     d.g = g;
     d.buf0 = s->buf[0];
     d.buf1 = s->buf[1];
@@ -155,16 +81,18 @@ static int rebuild(lbm_batch* b) {
     const int nseg = (s->ny + g.seg_h - 1) / g.seg_h;
     for (int sg = 0; sg < nseg; ++sg)
       for (int st = 0; st < g.n_strips; ++st) tl.push_back(make_int4((int)m, st, sg, 0));
-    per[d.P.s_direct ? 1 : 0].push_back(std::move(tl));
+    per[s->params.storage + (d.P.s_direct ? 3 : 0)].push_back(std::move(tl));
   }
-  int n_plain = 0;
-  for (int part = 0; part < 2; ++part) {
+  lbm_batch::Part parts[N_PARTS];
+  for (int part = 0; part < N_PARTS; ++part) {
+    parts[part].first = (int)work.size();
     size_t most = 0;
     for (auto& v : per[part]) most = std::max(most, v.size());
     for (size_t k = 0; k < most; ++k)
       for (auto& v : per[part])
         if (k < v.size()) work.push_back(v[k]);
-    if (part == 0) n_plain = (int)work.size();
+    parts[part].count = (int)work.size() - parts[part].first;
+    parts[part].grid = std::min(parts[part].count, slots);
   }
   cudaError_t e;
   if (sims.size() > b->cap_sims) {
@@ -192,47 +120,23 @@ static int rebuild(lbm_batch* b) {
   // host vectors die here: make the uploads complete first
   if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) return cuda_fail(e, "batch upload sync");
   b->n_work = (int)work.size();
-  b->n_plain = n_plain;
-  b->grid_plain = b->grid_sd = 0;
-  if (b->n_plain > 0) {
-    if ((e = set_batch_attr(b->nt, false, b->xwall)) != cudaSuccess) return cuda_fail(e, "batch kernel attribute");
-    b->grid_plain = std::max(1, std::min(b->n_plain, sms * std::max(batch_occupancy_sd<false>(b->nt, b->xwall), 1)));
-  }
-  if (b->n_work > b->n_plain) {
-    if ((e = set_batch_attr(b->nt, true, b->xwall)) != cudaSuccess) return cuda_fail(e, "batch kernel attribute");
-    b->grid_sd = std::max(1, std::min(b->n_work - b->n_plain, sms * std::max(batch_occupancy_sd<true>(b->nt, b->xwall), 1)));
-  }
+  std::copy(parts, parts + N_PARTS, b->parts);
   b->flip = 0;
   drop_graphs(b);
   b->dirty = false;
   return LBM_OK;
 }
 
-template <bool SD, bool XW>
-static void launch_part_t(lbm_batch* b, const int4* work, int n, int grid, int parity, cudaStream_t st) {
-  switch (b->nt) {
-    case 64: k_batch<64, SD, XW><<<grid, 64, sizeof(Smem<64>), st>>>(b->d_sims, work, n, parity); break;
-    case 256: k_batch<256, SD, XW><<<grid, 256, sizeof(Smem<256>), st>>>(b->d_sims, work, n, parity); break;
-    default: k_batch<128, SD, XW><<<grid, 128, sizeof(Smem<128>), st>>>(b->d_sims, work, n, parity); break;
-  }
-}
-
-template <bool SD>
-static void launch_part(lbm_batch* b, const int4* work, int n, int grid, int parity, cudaStream_t st) {
-  if constexpr (SD) {
-    launch_part_t<SD, true>(b, work, n, grid, parity, st);
-  } else {
-    if (b->xwall) launch_part_t<SD, true>(b, work, n, grid, parity, st);
-    else launch_part_t<SD, false>(b, work, n, grid, parity, st);
-  }
-}
-
-// One time step of every member: the two launches touch disjoint members.
+// One time step of every member: the launches touch disjoint members.
 static cudaError_t launch_batch(lbm_batch* b, int parity, cudaStream_t st) {
-  if (b->n_plain > 0) launch_part<false>(b, b->d_work, b->n_plain, b->grid_plain, parity, st);
-  if (b->n_work > b->n_plain)
-    launch_part<true>(b, b->d_work + b->n_plain, b->n_work - b->n_plain, b->grid_sd, parity, st);
-  return cudaGetLastError();
+  static constexpr decltype(&launch_batch_fp32) by_storage[3] = {launch_batch_fp32, launch_batch_fp16, launch_batch_bf16};
+  for (int k = 0; k < N_PARTS; ++k) {
+    const lbm_batch::Part& p = b->parts[k];
+    if (p.count == 0) continue;
+    const cudaError_t e = by_storage[k % 3](b->d_sims, b->d_work + p.first, p.count, p.grid, parity, k >= 3, b->xwall, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 extern "C" {
@@ -350,7 +254,6 @@ int lbm_batch_set_tile(lbm_batch* b, int threads, int seg_rows) {
   if (threads && threads != 64 && threads != 128 && threads != 256)
     return set_error("threads must be 64, 128 or 256"), LBM_ERR_INVALID_ARG;
   if (seg_rows < 0) return set_error("seg_rows must be >= 1"), LBM_ERR_INVALID_ARG;
-  if (threads) b->nt = threads;
   if (seg_rows) b->seg_h = seg_rows;
   b->dirty = true;
   return LBM_OK;

@@ -1,0 +1,75 @@
+// The batch kernel: the row march over a work list of tiles of many simulations.  Each storage is compiled in a
+// translation unit of its own (lbm_batch_fp32.cu, ...).
+#pragma once
+#include "lbm_internal.h"
+#include "lbm_march.cuh"
+
+namespace lbm {
+
+struct SimDesc {
+  Phys2 P;
+  Grid g;                 // src/dst unused; buffers below
+  const void* buf0;
+  void* buf1;
+  int cur0;               // buffer holding the state when the graph replay starts
+  int pad;
+};
+static_assert(sizeof(Phys2) % 4 == 0, "copied in words");
+
+// The row march's shared memory and the constants of the tile's member, from which its packed
+// instructions read them (a kernel parameter cannot differ between CTAs).
+template <int ST, bool SD>
+struct BatchSmem {
+  MarchSmem<ST, SD> m;
+  Phys2 P;
+};
+
+// One storage and one form of the mass defect per launch: a kernel that held the march of all three storages
+// did not fit 255 registers (1.2-1.9 KB of spills per thread).  XW: some member may have walls on x.
+template <int ST, bool SD, bool XW>
+__global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* __restrict__ sims, const int4* __restrict__ work,
+                                                                int n_work, int parity) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  BatchSmem<ST, SD>& sm = *reinterpret_cast<BatchSmem<ST, SD>*>(smem_raw);
+  march_init(sm.m);
+  StageAt fat, gat;
+  for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
+    const int4 it = work[w];
+    const SimDesc& d = sims[it.x];
+    const unsigned int* from = reinterpret_cast<const unsigned int*>(&d.P);
+    unsigned int* to = reinterpret_cast<unsigned int*>(&sm.P);
+    for (int k = threadIdx.x; k < (int)(sizeof(Phys2) / 4); k += MARCH_NT) to[k] = from[k];
+    Grid g = d.g;
+    const bool odd = ((d.cur0 + parity) & 1) != 0;
+    g.src = odd ? d.buf1 : d.buf0;
+    g.dst = odd ? const_cast<void*>(d.buf0) : d.buf1;
+    __syncthreads();
+    march<MODE_STEP, ST, SD, false, XW>(sm.P, g, MomentOut{}, it.y, it.z, sm.m, fat, gat);
+  }
+}
+
+template <int ST, bool SD, bool XW>
+static cudaError_t launch_batch_t(const SimDesc* sims, const int4* work, int n, int grid, int parity, cudaStream_t st) {
+  // set once, thread-safely (one GPU per process)
+  static const cudaError_t attr_set =
+      cudaFuncSetAttribute(k_batch<ST, SD, XW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BatchSmem<ST, SD>));
+  if (attr_set != cudaSuccess) return attr_set;
+  k_batch<ST, SD, XW><<<grid, MARCH_NT, sizeof(BatchSmem<ST, SD>), st>>>(sims, work, n, parity);
+  return cudaGetLastError();
+}
+
+// The tiles work[0, n) of members of one storage and one form of the mass defect.
+template <int ST>
+static cudaError_t launch_batch_st(const SimDesc* sims, const int4* work, int n, int grid, int parity, bool sd, bool xw,
+                                   cudaStream_t st) {
+  if (sd) return launch_batch_t<ST, true, true>(sims, work, n, grid, parity, st);
+  return xw ? launch_batch_t<ST, false, true>(sims, work, n, grid, parity, st)
+            : launch_batch_t<ST, false, false>(sims, work, n, grid, parity, st);
+}
+
+// (in the storages' translation units)
+cudaError_t launch_batch_fp32(const SimDesc*, const int4*, int n, int grid, int parity, bool sd, bool xw, cudaStream_t st);
+cudaError_t launch_batch_fp16(const SimDesc*, const int4*, int n, int grid, int parity, bool sd, bool xw, cudaStream_t st);
+cudaError_t launch_batch_bf16(const SimDesc*, const int4*, int n, int grid, int parity, bool sd, bool xw, cudaStream_t st);
+
+}  // namespace lbm

@@ -1,0 +1,11 @@
+// Ragged batches: members of BF16 population storage.
+#include "lbm_batch.cuh"
+
+namespace lbm {
+
+cudaError_t launch_batch_bf16(const SimDesc* sims, const int4* work, int n, int grid, int parity, bool sd, bool xw,
+                              cudaStream_t st) {
+  return launch_batch_st<ST_BF16>(sims, work, n, grid, parity, sd, xw, st);
+}
+
+}  // namespace lbm

@@ -14,6 +14,7 @@ struct lbm_sim {
   long long plane = 0;      // elements per plane
   lbm_params params{};
   lbm::Phys phys{};
+  lbm::Phys2 phys2{};       // the same, each constant doubled
   cudaStream_t stream = nullptr;
   void* buf[2] = {nullptr, nullptr};   // post-collision state, buf_bytes each
   size_t buf_bytes = 0;                // populations (+ rho, div(rho u) planes with s_form = 1)
@@ -26,12 +27,9 @@ struct lbm_sim {
   cudaEvent_t uploaded = nullptr;      // recorded after lbm_init_fields' host-to-device copies
   long long steps = 0;
   long long launches = 0;
-  int nt = 128;                        // threads per CTA of the step kernel
   int kernel = LBM_KERNEL_AUTO;        // step kernel choice (lbm_set_kernel)
   int seg_h = 0;                       // rows per CTA (0: one wave of resident CTAs)
   int sms = 0;                         // multiprocessors of the device
-  int occ = 0;                         // resident step CTAs per SM at the current nt
-  float sf = 1.0f, sg = 1.0f;          // 16-bit storage scales of the f and gbar planes
   // resident tile kernel (lbm_tile2d.cu): per-tile step flags, the status word and the reach
   // table in one stream-ordered allocation made at first use
   unsigned int* res_mem = nullptr;
@@ -59,11 +57,10 @@ void set_error(const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);
 Phys make_phys(const lbm_params& p);
 Grid make_grid(const lbm_sim* s, const void* src, void* dst);
-// Strip width, strip count and segment height for an nx x ny grid: strips of at most nt - 6
-// columns with balanced widths; seg_h = 0 picks the height that puts about one full wave of
-// CTAs (slots = SMs x CTAs per SM) on the device.
-void tile_geometry(int nx, int ny, int nt, int seg_h, int slots, int* tile_w, int* n_strips, int* seg_out);
-int tile_occupancy(int nt);
+// Lane width, strip count and segment height of the row march for an nx x ny grid: strips of two lanes of
+// at most march_width(sd) columns, all alike; seg_h = 0 picks the height that puts about one full wave of CTAs
+// (slots = SMs x CTAs per SM) on the device.
+void tile_geometry(int nx, int ny, bool sd, int seg_h, int slots, int* tile_w, int* n_strips, int* seg_out);
 // The small-grid step kernel (lbm_tile2d.cu): s_form 0 and f_form 0.
 bool tile2d_eligible(const lbm_params& p);
 // 384-thread CTAs when the grid's tiles fit one wave of them on `sms` multiprocessors, else 256.
@@ -79,9 +76,14 @@ cudaError_t resident_reset(lbm_sim* s);
 cudaError_t launch_resident(lbm_sim* s, const Grid& g, int n);
 
 // launchers (return cudaError_t of the launch)
-cudaError_t launch_step(const Phys& P, const Grid& g, int nt, cudaStream_t st);
-cudaError_t launch_moments(const Phys& P, const Grid& g, const MomentOut& mo, int nt, cudaStream_t st);
+cudaError_t launch_step(const Phys2& P, const Grid& g, cudaStream_t st);
+cudaError_t launch_step_fp32(const Phys2& P, const Grid& g, cudaStream_t st);
+cudaError_t launch_step_fp16(const Phys2& P, const Grid& g, cudaStream_t st);
+cudaError_t launch_step_bf16(const Phys2& P, const Grid& g, cudaStream_t st);
+cudaError_t launch_moments(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st);
 cudaError_t launch_init(const lbm_sim* s, cudaStream_t st);  // from fields[phi, -, ux, uy, p]
+// 16-byte units [u0, u1) of the checkpoint's population order between a state buffer and `lin`.
+cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u0, long long u1, bool out, cudaStream_t st);
 cudaError_t launch_diag(const lbm_sim* s, cudaStream_t st);  // from fields -> red -> final record
 
 }  // namespace lbm

@@ -6,155 +6,29 @@
 
 namespace lbm {
 
-// ------------------------------------------------------------------ fused step / moments
+// ------------------------------------------------------------------ fused step
 
-template <int NT, int MODE, int ST, bool SD, bool FF, bool XW>
-// Resident CTAs per SM: 8 of 64 threads or 2 of 256 (16 warps, at most 128 registers per thread),
-// 3 of 128 threads (12 warps, at most 168 registers).  Given the room, the 128-thread FP32 step
-// takes 148 registers instead of 128, and on the 2048 x 512 splash its whole-wave tile (20 rows,
-// 442 CTAs) ran 47.1 us per step against 49.2 us for the best tile at 4 CTAs of 128 registers.
-__global__ void __launch_bounds__(NT, NT == 128 ? 3 : 512 / NT) k_tiles(Phys P, Grid g, MomentOut mo) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Smem<NT>& sm = *reinterpret_cast<Smem<NT>*>(smem_raw);
-  if (MODE == MODE_STEP) {
-    // launched as a programmatic dependent of the previous step: wait until that grid has
-    // completed and its stores are visible, then let the next step's launch proceed
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  }
-  const int strip = blockIdx.x % g.n_strips;
-  const int seg = blockIdx.x / g.n_strips;
-  run_tile<NT, MODE, ST, SD, FF, XW>(P, g, mo, strip, seg, sm);
-}
-
-static int n_tiles(const Grid& g) { return g.n_strips * ((g.ny + g.seg_h - 1) / g.seg_h); }
-
-// Dynamic shared memory of a row-march CTA (step or moments).  The periodic-x form (XW false)
-// can need fewer registers than the general form and then fit more CTAs per SM; it is held to
-// the general form's count, for which the tile heights are sized (one wave) and which measured
-// faster (c3 42.8 us on 128 x 20 at 3 per SM against 45.6 us on 128 x 15 at 4, when the form
-// took 128 registers), by asking for just more shared memory than one more CTA would leave room
-// for.
-template <int NT, bool XW>
-static int step_smem_bytes() {
-  int smem = (int)sizeof(Smem<NT>);
-  if (XW) return smem;
-  int dev = 0, per_sm = 0, reserved = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return smem;
-  }
-  const int occ = tile_occupancy(NT);   // CTAs per SM of the general form
-  const int cap = (per_sm / (occ + 1) - reserved + 16 + 15) / 16 * 16;
-  // the general form's count must still fit
-  if (cap > smem && occ * (cap + reserved) <= per_sm) smem = cap;
-  return smem;
-}
-
-template <int NT, int MODE, int ST, bool SD, bool FF, bool XW = true>
-static cudaError_t launch_sd(const Phys& P, const Grid& g, const MomentOut& mo, cudaStream_t st) {
-  static int smem = 0;   // one GPU per process
-  if (smem == 0) {
-    const int want = step_smem_bytes<NT, XW>();
-    cudaError_t e = cudaFuncSetAttribute(k_tiles<NT, MODE, ST, SD, FF, XW>, cudaFuncAttributeMaxDynamicSharedMemorySize, want);
-    if (e != cudaSuccess) return e;
-    smem = want;
-  }
-  if (MODE != MODE_STEP) {
-    k_tiles<NT, MODE, ST, SD, FF, XW><<<n_tiles(g), NT, smem, st>>>(P, g, mo);
-    return cudaGetLastError();
-  }
-  // consecutive steps overlap their launches (programmatic dependent launch)
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_tiles(g));
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_tiles<NT, MODE, ST, SD, FF, XW>, P, g, mo);
-}
-
-template <int NT, int MODE, int ST>
-static cudaError_t launch_nt(const Phys& P, const Grid& g, const MomentOut& mo, cudaStream_t st) {
-  // the forced order-parameter form changes only the step's f collision (FP32 storage only)
-  if constexpr (MODE == MODE_STEP && ST == ST_FP32) {
-    if (P.f_forced)
-      return P.s_direct ? launch_sd<NT, MODE, ST, true, true>(P, g, mo, st)
-                        : launch_sd<NT, MODE, ST, false, true>(P, g, mo, st);
-  }
-  if (P.s_direct) return launch_sd<NT, MODE, ST, true, false>(P, g, mo, st);
-  // a periodic x axis compiles out the ghost columns and column wall tests
-  if (g.bc_x != BC_WALL) return launch_sd<NT, MODE, ST, false, false, false>(P, g, mo, st);
-  return launch_sd<NT, MODE, ST, false, false>(P, g, mo, st);
-}
-
-template <int MODE, int ST>
-static cudaError_t launch_st(const Phys& P, const Grid& g, const MomentOut& mo, int nt, cudaStream_t st) {
-  switch (nt) {
-    case 64: return launch_nt<64, MODE, ST>(P, g, mo, st);
-    case 128: return launch_nt<128, MODE, ST>(P, g, mo, st);
-    case 256: return launch_nt<256, MODE, ST>(P, g, mo, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-template <int MODE>
-static cudaError_t launch_tiles(const Phys& P, const Grid& g, const MomentOut& mo, int nt, cudaStream_t st) {
+cudaError_t launch_step(const Phys2& P, const Grid& g, cudaStream_t st) {
   switch (g.storage) {
-    case ST_FP32: return launch_st<MODE, ST_FP32>(P, g, mo, nt, st);
-    case ST_FP16: return launch_st<MODE, ST_FP16>(P, g, mo, nt, st);
-    case ST_BF16: return launch_st<MODE, ST_BF16>(P, g, mo, nt, st);
+    case ST_FP32: return launch_step_fp32(P, g, st);
+    case ST_FP16: return launch_step_fp16(P, g, st);
+    case ST_BF16: return launch_step_bf16(P, g, st);
     default: return cudaErrorInvalidValue;
   }
-}
-
-template <int NT>
-static int occupancy_nt() {
-  int occ = 0;
-  // the dynamic shared-memory size above 48 KB is only admitted once the attribute is set
-  cudaFuncSetAttribute(k_tiles<NT, MODE_STEP, ST_FP32, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sizeof(Smem<NT>));
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tiles<NT, MODE_STEP, ST_FP32, false, false, true>, NT, sizeof(Smem<NT>));
-  cudaGetLastError();
-  return occ > 0 ? occ : 1;
-}
-
-int tile_occupancy(int nt) {
-  switch (nt) {
-    case 64: return occupancy_nt<64>();
-    case 256: return occupancy_nt<256>();
-    default: return occupancy_nt<128>();
-  }
-}
-
-cudaError_t launch_step(const Phys& P, const Grid& g, int nt, cudaStream_t st) {
-  return launch_tiles<MODE_STEP>(P, g, MomentOut{}, nt, st);
-}
-
-cudaError_t launch_moments(const Phys& P, const Grid& g, const MomentOut& mo, int nt, cudaStream_t st) {
-  return launch_tiles<MODE_MOMENTS>(P, g, mo, nt, st);
 }
 
 // ------------------------------------------------------------------ initial state
 // fields: [0] phi0, [1] (unused), [2] ux0, [3] uy0, [4] p0 -- pitched planes; mu0 is evaluated
 // where it is used.
 
-// Post-collision-layout state whose pull gives f = f^eq(phi0, mu0, u0), gbar = g^eq(p0, rho0, u0):
-// plane a at cell z holds the equilibrium of direction a at z + e_a, or, when that link leaves
-// through a wall, the equilibrium of the reversed direction at z itself.  Written by pushing:
-// each cell evaluates its own 18 equilibria once and stores direction a at the cell it is pulled
-// from, z - e_a, or, when that lies beyond a wall, as the reversed plane at itself (which the
-// pull's bounce-back reads).  Every (plane, cell) is written exactly once.
+// State that streams into f = f^eq(phi0, mu0, u0), gbar = g^eq(p0, rho0, u0): each cell stores its own 18
+// equilibria where it will read them, population a in its row at column x - e_a,x.
 template <int ST>
 __global__ void k_init_pop(Phys P, Grid g, const float* __restrict__ fields) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x == 0 && blockIdx.y == 0) *g.gave_up = 0u;         // a new state
   if (x >= g.nx) return;
+  const Col3 col = col3<ST>(x, g.nx);
   for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {   // gridDim.y is capped at 65535
     const long long c = (long long)y * g.pitch + x;
     const float ph = fields[c], u = fields[2 * g.plane + c], v = fields[3 * g.plane + c];
@@ -172,52 +46,59 @@ __global__ void k_init_pop(Phys P, Grid g, const float* __restrict__ fields) {
     const float cl = fminf(fmaxf((ph + P.phi_star) * P.inv_2phistar, 0.0f), 1.0f);
     const float rho = P.rho_B + cl * P.drho;
     const float uu15 = 1.5f * (u * u + v * v);
-    const CellB self = cell_at(y * g.row_bytes, col_bytes<ST>(x));
-  #pragma unroll
-    for (int a = 0; a < Q; ++a) {
+    char* const dst = static_cast<char*>(g.dst);
+    const int row = y * g.row_bytes;
+    // the place the value comes from, which keys BF16 rounding: the cell upstream, or the reversed
+    // population of the cell itself across a wall
+    auto put = [&](auto pop, float val) {
+      constexpr int A = decltype(pop)::value;
+      constexpr int a = A == A_F0LO ? 0 : A % Q;
+      char* q = dst + pop_at<ST>(A, row, cx(a) == 1 ? col.cm : (cx(a) == -1 ? col.cq : col.c0), g);
+      if constexpr (pop_bytes(ST, A) == 4) {
+        *reinterpret_cast<float*>(q) = val;
+      } else {
+        int xz = x - cx(a), yz = y - cy(a), from = A;
+        const bool hit = (g.bc_x == BC_WALL && (xz < 0 || xz >= g.nx)) || (g.bc_y == BC_WALL && (yz < 0 || yz >= g.ny));
+        if (hit) {
+          xz = x;
+          yz = y;
+          from = opp(a) + (A >= Q ? Q : 0);
+        }
+        *reinterpret_cast<unsigned short*>(q) =
+            enc_pop<ST>(to_scale<ST>(P, val), from, hash_key<ST>(wrap1(xz, g.nx), wrap1(yz, g.ny), g));
+      }
+    };
+    float rest = 0.0f;
+    auto dir = [&](auto idx) {
+      constexpr int a = decltype(idx)::value;
       const float w = wgt(a);
       const float eu = (float)cx(a) * u + (float)cy(a) * v;
       const float poly = 3.0f * eu + 4.5f * eu * eu - uu15;
-      const float geq = w * p + rho * (1.0f / 3.0f) * (w * poly);
-      float feq = 0.0f;
-      if (a > 0) feq = w * (P.f_forced ? ph * (1.0f + poly) : P.three_gamma_f * m + ph * poly);
-      // where direction a's value is pulled from: z = this cell - e_a, or itself across a wall
-      int xz = x - cx(a), yz = y - cy(a), plane = a;
-      bool hit = false;
-      if (xz < 0 || xz >= g.nx) {
-        if (g.bc_x == BC_WALL) hit = true; else xz = wrap1(xz, g.nx);
+      put(std::integral_constant<int, Q + a>{}, w * p + rho * (1.0f / 3.0f) * (w * poly));
+      if constexpr (a > 0) {
+        // f^eq_a: with the mu term, or phi Gamma_a in the forced order-parameter form
+        const float feq = w * (P.f_forced ? ph * (1.0f + poly) : P.three_gamma_f * m + ph * poly);
+        put(std::integral_constant<int, a>{}, feq);
+        rest += feq;
       }
-      if (yz < 0 || yz >= g.ny) {
-        if (g.bc_y == BC_WALL) hit = true; else yz = wrap1(yz, g.ny);
-      }
-      if (hit) {
-        xz = x;
-        yz = y;
-        plane = opp(a);
-      }
-      const CellB z = a == 0 ? self : cell_at(yz * g.row_bytes, col_bytes<ST>(xz));
-      if (a == 0) {
-        // f_0^eq = phi - sum_{k>0} f^eq_k, kept as the float pair (hi, lo)
-        float rest = 0.0f;
-  #pragma unroll
-        for (int k = 1; k < Q; ++k) {
-          const float ek = (float)cx(k) * u + (float)cy(k) * v;
-          const float pk = 3.0f * ek + 4.5f * ek * ek - uu15;
-          // f^eq_k: with the mu term, or phi Gamma_k in the forced order-parameter form
-          rest += wgt(k) * (P.f_forced ? ph * (1.0f + pk) : P.three_gamma_f * m + ph * pk);
-        }
-        float hi, lo;
-        two_sum(ph, -rest, hi, lo);
-        if (ST == ST_FP32) {
-          st_pop<ST>(g.dst, 0, self, hi, 1.0f);
-          st_pop<ST>(g.dst, PLANE_F0LO, self, lo, 1.0f);
-        } else {
-          st_pop<ST>(g.dst, 0, self, hi + lo, 1.0f);
-        }
-      } else {
-        st_pop<ST>(g.dst, plane, z, feq, g.sf);
-      }
-      st_pop<ST>(g.dst, Q + plane, z, geq, g.sg);
+    };
+    dir(std::integral_constant<int, 0>{});
+    dir(std::integral_constant<int, 1>{});
+    dir(std::integral_constant<int, 2>{});
+    dir(std::integral_constant<int, 3>{});
+    dir(std::integral_constant<int, 4>{});
+    dir(std::integral_constant<int, 5>{});
+    dir(std::integral_constant<int, 6>{});
+    dir(std::integral_constant<int, 7>{});
+    dir(std::integral_constant<int, 8>{});
+    // f_0^eq = phi - sum_{a>0} f^eq_a, kept as the float pair (hi, lo)
+    float hi, lo;
+    two_sum(ph, -rest, hi, lo);
+    if constexpr (ST == ST_FP32) {
+      put(std::integral_constant<int, 0>{}, hi);
+      put(std::integral_constant<int, A_F0LO>{}, lo);
+    } else {
+      put(std::integral_constant<int, 0>{}, hi + lo);
     }
   }
 }
@@ -262,6 +143,81 @@ cudaError_t launch_init(const lbm_sim* s, cudaStream_t st) {
     k_init_sdef<<<grd, blk, 0, st>>>(s->phys, g, s->fields);
   }
   return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------ checkpoint order
+// A checkpoint holds the post-collision populations at their source cells, a row in blocks of 32 cells with
+// every population of the block's cells in turn (FP32: f_0..f_8, gbar_0..gbar_8, f_0lo, 128 bytes each;
+// 16-bit: the FP32 rest population, then 17 of 64 bytes).  `lin` holds its 16-byte units [u0, u1), each
+// some consecutive cells of one population; pad columns keep their place.
+template <int ST, bool OUT>
+__global__ void k_reorder(char* __restrict__ state, int4* __restrict__ lin, long long u0, long long u1, Grid g) {
+  constexpr int UNITS = 2 * (int)state_bytes_per_cell(ST);   // per 32-cell block
+  const unsigned int nb = g.pitch / 32;
+  const long long step = (long long)gridDim.x * blockDim.x;
+  for (long long u = u0 + (long long)blockIdx.x * blockDim.x + threadIdx.x; u < u1; u += step) {
+    const unsigned int b = (unsigned int)(u / UNITS);
+    const int k = (int)(u - (long long)b * UNITS);
+    const int y = (int)(b / nb), xb = (int)(b - (unsigned int)y * nb) * 32;
+    int a = k / 8, x0 = xb + (k - a * 8) * 4, n = 4;
+    if (ST != ST_FP32) {
+      if (k < 8) {
+        a = 0;
+        x0 = xb + k * 4;
+      } else {
+        a = 1 + (k - 8) / 4;
+        x0 = xb + (k - 8 - (a - 1) * 4) * 8;
+        n = 8;
+      }
+    }
+    const int d = a == A_F0LO ? 0 : a % Q;
+    union {
+      int4 v;
+      unsigned int w[4];
+      unsigned short h[8];
+    } unit;
+    unit.v = OUT ? make_int4(0, 0, 0, 0) : lin[u - u0];
+    for (int i = 0; i < n; ++i) {
+      const int x = x0 + i;
+      int to = a, row = y, col = x;
+      if (x < g.nx && d > 0) {
+        const int tx = x + cx(d), ty = y + cy(d);
+        const bool hit = (g.bc_x == BC_WALL && (tx < 0 || tx >= g.nx)) || (g.bc_y == BC_WALL && (ty < 0 || ty >= g.ny));
+        if (hit) {
+          to = opp(d) + (a >= Q ? Q : 0);
+          col = wrap1(tx, g.nx);
+        } else {
+          row = wrap1(ty, g.ny);
+        }
+      }
+      char* p = state + (long long)row * g.row_bytes + pop_at<ST>(to, 0, col_bytes<ST>(col), g);
+      if (n == 4) {
+        if (OUT) unit.w[i] = *reinterpret_cast<unsigned int*>(p);
+        else *reinterpret_cast<unsigned int*>(p) = unit.w[i];
+      } else {
+        if (OUT) unit.h[i] = *reinterpret_cast<unsigned short*>(p);
+        else *reinterpret_cast<unsigned short*>(p) = unit.h[i];
+      }
+    }
+    if (OUT) lin[u - u0] = unit.v;
+  }
+}
+
+template <int ST>
+static cudaError_t launch_reorder_st(const lbm_sim* s, void* state, void* lin, long long u0, long long u1, bool out,
+                                     cudaStream_t st) {
+  const Grid g = make_grid(s, nullptr, nullptr);
+  const long long want = (u1 - u0 + 255) / 256;
+  const int grid = (int)(want < 16LL * s->sms ? want : 16LL * s->sms);
+  if (out) k_reorder<ST, true><<<grid, 256, 0, st>>>(static_cast<char*>(state), static_cast<int4*>(lin), u0, u1, g);
+  else k_reorder<ST, false><<<grid, 256, 0, st>>>(static_cast<char*>(state), static_cast<int4*>(lin), u0, u1, g);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u0, long long u1, bool out, cudaStream_t st) {
+  // the two 16-bit storages are laid out alike
+  return s->params.storage == LBM_FP32 ? launch_reorder_st<ST_FP32>(s, state, lin, u0, u1, out, st)
+                                       : launch_reorder_st<ST_FP16>(s, state, lin, u0, u1, out, st);
 }
 
 // ------------------------------------------------------------------ FP64 diagnostics
@@ -355,7 +311,7 @@ __global__ void __launch_bounds__(DIAG_T) k_diag_final(Grid g, const double* __r
     d.max_u = sh[6][0];
     d.p_liquid = sh[8][0] > 0 ? sh[7][0] / sh[8][0] : 0.0;
     d.p_gas = sh[10][0] > 0 ? sh[9][0] / sh[10][0] : 0.0;
-    d.finite = isfinite(d.sum_phi) && isfinite(d.max_u);
+    d.finite = isfinite(d.sum_phi) && isfinite(d.max_u) && *g.gave_up == 0u;
     d.pad = 0;
     *reinterpret_cast<lbm_diag*>(out) = d;
   }

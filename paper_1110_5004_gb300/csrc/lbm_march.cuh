@@ -1,0 +1,587 @@
+// The row march: the fused step (and the moment evaluation) of a simulation whose grid fills the
+// device, for every configuration.
+//
+// A CTA marches up a strip of columns and a segment of rows [ya, yb).  Each thread owns two columns, one
+// in each half ("lane") of the strip: thread t has the columns x0 - 3 + t and x0 + w - 3 + t, w columns per
+// lane plus a 3-column halo on each side.  Every value is a V2, the pair of the two lanes, so one
+// packed instruction, one 64-bit shared-memory access and one address serve two cells.
+//
+// Row iteration a runs four stages in two phases, a barrier after each:
+//   phase 1   S0  row a     phi = sum_a f_a
+//             S2  row a-3   grad phi, grad mu, lap mu, rho, F_s, G, s, u, p        [Eq. 4, 5, 8]
+//   phase 2   S1  row a-1   mu = theta'(phi) - kappa lap(phi)                      [Eq. 1]
+//             S3  row a-4   grad p, grad psi, div u, both collisions, stores
+// The two stages of a phase do not depend on each other and read only what earlier phases wrote, so they
+// are one stretch of independent work for the scheduler.  Their stencils work on rings of rows in
+// shared memory; a segment of h rows takes h + 7 iterations.
+//
+// The populations come into shared memory by bulk copies (cp.async.bulk), one per region for the row's whole
+// chunk of columns (two where a strip wraps around the edge of a periodic grid), STAGES rows ahead.  They
+// hold neither registers nor L1 lines while in flight.
+//
+// Why this form (2048 x 512 and 4096 x 4096, FP32 storage): the step moves 152 B per cell, 6.5 cycles
+// per cell and SM at the measured bandwidth.  With one cell per thread it issued 594-745 warp instructions per
+// 32 cells, 4.6-5.8 cycles per cell at best, and its warps waited 30-48 % of their time on loads that one row of
+// register prefetch could not cover (more warps or L2 prefetches only thrashed L1).
+#pragma once
+#include "lbm_device.cuh"
+
+namespace lbm {
+
+enum { MODE_STEP = 0, MODE_MOMENTS = 1 };
+
+constexpr int MARCH_NT = 128;             // threads per CTA
+constexpr int MARCH_CTAS = 2;             // CTAs per SM (shared memory; 8 warps of up to 255 registers)
+// Blocks of a staged row, and the most columns per lane for them: 2 w + 8 columns, up to 31 cells lost at
+// the first block and 31 at the last block of a wrapped row.  The direct mass defect (s_form 1) takes a block less,
+// so that its additional rings fit.
+__host__ __device__ constexpr int march_slots(bool sd) { return sd ? 9 : 10; }
+__host__ __device__ constexpr int march_width(bool sd) {
+  const int w = (march_slots(sd) * BLK - 2 * (BLK - 1) - 8) / 2;
+  return w < MARCH_NT - 6 ? w : MARCH_NT - 6;
+}
+constexpr int STAGES = 2;                 // rows of f and of gbar in shared memory or in flight
+constexpr int RING5 = 5;                  // rows a-4 .. a of phi and of the f populations awaiting S3
+constexpr int RING3 = 3;                  // rows of mu, p, u
+
+template <int ST, bool SD>
+struct MarchSmem {
+  static constexpr int NSLOT = march_slots(SD);
+  struct Stage {                          // 16-byte aligned pieces
+    unsigned char f[NSLOT * region_block(ST, R_F)], l[NSLOT * region_block(ST, R_L)], g[NSLOT * region_block(ST, R_G)];
+  };
+  struct Row5 {
+    ulonglong2 f[4][MARCH_NT];            // f_1..f_8 of both lanes, own column
+    V2 hi[MARCH_NT], lo[MARCH_NT];
+  };
+  struct Row3 {
+    V2 mu[MARCH_NT], p[MARCH_NT], ux[MARCH_NT], uy[MARCH_NT];
+    V2 j[SD ? 2 : 0][MARCH_NT];           // rho u (direct mass defect)
+  };
+  // barriers first: at the same place for every storage, since a batch CTA changes storage between tiles
+  alignas(128) unsigned long long fbar[STAGES];
+  unsigned long long gbar[STAGES];
+  alignas(128) Stage stage[STAGES];
+  Row5 r5[RING5];
+  Row3 r3[RING3];
+  V2 tail[2];                             // the last thread reads one column past its ring row
+};
+
+__device__ __forceinline__ unsigned int smem_u32(const void* p) { return (unsigned int)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(unsigned long long* b) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(b)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned long long* b, int bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_load(unsigned int dst, const void* src, int bytes, unsigned long long* b) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(smem_u32(b))
+               : "memory");
+}
+// Wait for the phase `parity` of a barrier.  The copies it counts always complete; the bound only
+// keeps a fault elsewhere from turning into a hang: the launch then goes on with what is in shared
+// memory and raises `gave_up`, which the diagnostics report as a diverged state.
+constexpr int WAIT_TRIES = 1 << 20;
+__device__ __forceinline__ void mbar_wait(unsigned long long* b, int parity, unsigned int* gave_up) {
+  const unsigned int addr = smem_u32(b);
+  for (int n = 0; n < WAIT_TRIES; ++n) {
+    unsigned int done;
+    asm volatile("{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(done)
+                 : "r"(addr), "r"(parity)
+                 : "memory");
+    if (done) return;
+  }
+  *gave_up = 1u;
+}
+
+// Before the first tile of a CTA.
+template <int ST, bool SD>
+__device__ __forceinline__ void march_init(MarchSmem<ST, SD>& sm) {
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < STAGES; ++k) {
+      mbar_init(&sm.fbar[k]);
+      mbar_init(&sm.gbar[k]);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+}
+
+// Store where `on`, as one predicated instruction: no branch around it.
+__device__ __forceinline__ void st_on(float* p, float v, bool on) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.global.f32 [%0], %1;\n\t}" ::"l"(p), "f"(v),
+               "r"((int)on));
+}
+
+// The two lanes' new populations, and the store of one lane's: the gbar (and the f) populations together under
+// one predicate, to the rows they stream to.
+template <int ST>
+struct OutLanes {
+  mutable V2 v[Q + Q + 1];
+  template <int A>
+  __device__ __forceinline__ void put(V2 x) const {
+    v[A] = x;
+  }
+  template <bool B>
+  __device__ __forceinline__ void lane(float x[Q + Q + 1]) const {
+#pragma unroll
+    for (int a = 0; a < (ST == ST_FP32 ? 19 : 18); ++a) {
+      float lo, hi;
+      unpack2(v[a], lo, hi);
+      x[a] = B ? hi : lo;
+    }
+  }
+  // next to a wall: cell by cell
+  template <bool B, class Out>
+  __device__ __forceinline__ void store_cell(const Out& o) const {
+    float x[Q + Q + 1];
+    lane<B>(x);
+    o.template put<0>(x[0]);
+    o.template put<1>(x[1]);
+    o.template put<2>(x[2]);
+    o.template put<3>(x[3]);
+    o.template put<4>(x[4]);
+    o.template put<5>(x[5]);
+    o.template put<6>(x[6]);
+    o.template put<7>(x[7]);
+    o.template put<8>(x[8]);
+    o.template put<9>(x[9]);
+    o.template put<10>(x[10]);
+    o.template put<11>(x[11]);
+    o.template put<12>(x[12]);
+    o.template put<13>(x[13]);
+    o.template put<14>(x[14]);
+    o.template put<15>(x[15]);
+    o.template put<16>(x[16]);
+    o.template put<17>(x[17]);
+    if constexpr (ST == ST_FP32) o.template put<A_F0LO>(x[A_F0LO]);
+  }
+  // rows: the destination buffer's rows y-1, y, y+1; c: the lane's column; key: its BF16 rounding place
+  template <bool B>
+  __device__ __forceinline__ void store_lane(char* rm, char* r0, char* rq, const ColB& c, int nblk, unsigned int key, bool on) const {
+    float x[Q + Q + 1];
+    lane<B>(x);
+    const int g = region_start(ST, R_G) * nblk + c.g;
+    static_assert(BLK == 32, "offsets below");
+    if constexpr (ST == ST_FP32) {
+      asm volatile(
+          "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
+          "@q st.global.f32 [%1+256], %4;\n\t@q st.global.f32 [%1+640], %5;\n\t@q st.global.f32 [%1+768], %6;\n\t"
+          "@q st.global.f32 [%2], %7;\n\t@q st.global.f32 [%2+128], %8;\n\t@q st.global.f32 [%2+384], %9;\n\t"
+          "@q st.global.f32 [%3+512], %10;\n\t@q st.global.f32 [%3+896], %11;\n\t@q st.global.f32 [%3+1024], %12;\n\t}" ::"r"(
+              (int)on),
+          "l"(rq + g), "l"(r0 + g), "l"(rm + g), "f"(x[Q + 2]), "f"(x[Q + 5]), "f"(x[Q + 6]), "f"(x[Q + 0]), "f"(x[Q + 1]),
+          "f"(x[Q + 3]), "f"(x[Q + 4]), "f"(x[Q + 7]), "f"(x[Q + 8]));
+      asm volatile(
+          "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
+          "@q st.global.f32 [%1+256], %5;\n\t@q st.global.f32 [%1+640], %6;\n\t@q st.global.f32 [%1+768], %7;\n\t"
+          "@q st.global.f32 [%2], %8;\n\t@q st.global.f32 [%2+128], %9;\n\t@q st.global.f32 [%2+384], %10;\n\t"
+          "@q st.global.f32 [%3+512], %11;\n\t@q st.global.f32 [%3+896], %12;\n\t@q st.global.f32 [%3+1024], %13;\n\t"
+          "@q st.global.f32 [%4], %14;\n\t}" ::"r"((int)on),
+          "l"(rq + c.f4), "l"(r0 + c.f4), "l"(rm + c.f4), "l"(r0 + region_start(ST, R_L) * nblk + c.l), "f"(x[2]), "f"(x[5]),
+          "f"(x[6]), "f"(x[0]), "f"(x[1]), "f"(x[3]), "f"(x[4]), "f"(x[7]), "f"(x[8]), "f"(x[A_F0LO]));
+    } else {
+      unsigned short h[Q + Q];
+#pragma unroll
+      for (int a = 1; a < Q + Q; ++a) h[a] = enc_pop<ST>(x[a], a, key);
+      asm volatile(
+          "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
+          "@q st.global.u16 [%1+128], %4;\n\t@q st.global.u16 [%1+320], %5;\n\t@q st.global.u16 [%1+384], %6;\n\t"
+          "@q st.global.u16 [%2], %7;\n\t@q st.global.u16 [%2+64], %8;\n\t@q st.global.u16 [%2+192], %9;\n\t"
+          "@q st.global.u16 [%3+256], %10;\n\t@q st.global.u16 [%3+448], %11;\n\t@q st.global.u16 [%3+512], %12;\n\t}" ::"r"(
+              (int)on),
+          "l"(rq + g), "l"(r0 + g), "l"(rm + g), "h"(h[Q + 2]), "h"(h[Q + 5]), "h"(h[Q + 6]), "h"(h[Q + 0]), "h"(h[Q + 1]),
+          "h"(h[Q + 3]), "h"(h[Q + 4]), "h"(h[Q + 7]), "h"(h[Q + 8]));
+      asm volatile(
+          "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
+          "@q st.global.u16 [%1+192], %5;\n\t@q st.global.u16 [%1+384], %6;\n\t@q st.global.u16 [%1+448], %7;\n\t"
+          "@q st.global.u16 [%2+128], %8;\n\t@q st.global.u16 [%2+256], %9;\n\t"
+          "@q st.global.u16 [%3+320], %10;\n\t@q st.global.u16 [%3+512], %11;\n\t@q st.global.u16 [%3+576], %12;\n\t"
+          "@q st.global.f32 [%4], %13;\n\t}" ::"r"((int)on),
+          "l"(rq + c.f2), "l"(r0 + c.f2), "l"(rm + c.f2), "l"(r0 + c.f4), "h"(h[2]), "h"(h[5]), "h"(h[6]), "h"(h[1]), "h"(h[3]),
+          "h"(h[4]), "h"(h[7]), "h"(h[8]), "f"(x[0]));
+    }
+  }
+};
+
+// One row iteration (kinds):
+//   IT_CHECKED  a wall row may be among the rows: every stage tests its row range and fills ghost rows.
+//   IT_FILL     the first iterations of a segment that touches no wall row: no S3 yet, S2 from its
+//               first needed row on.
+//   IT_INNER    no row test and no branch.
+// Threads whose column a stage does not need compute it anyway, from whatever the rings hold;
+// only stores to the new state (and, with walls on x, to the rings) are predicated.
+enum { IT_CHECKED = 0, IT_FILL = 1, IT_INNER = 2 };
+
+// The stage the next row of f (or gbar) is read from, and the parity of its barrier.
+struct StageAt {
+  int stage = 0, parity = 0;
+  __device__ __forceinline__ void next() {
+    if (++stage == STAGES) {
+      stage = 0;
+      parity ^= 1;
+    }
+  }
+  __device__ __forceinline__ int ahead(int k) const { return stage + k >= STAGES ? stage + k - STAGES : stage + k; }
+};
+
+// SD: the direct mass defect (s_form 1) is compiled in.  FF: the forced order-parameter LBE (f_form 1;
+// FP32 storage only).  XW: the x axis may have walls.  K: the scheme constants (Phys2, in the constant bank
+// or in shared memory).
+template <int MODE, int ST, bool SD, bool FF, bool XW, class K>
+__device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut& mo, int strip, int seg, MarchSmem<ST, SD>& sm,
+                                      StageAt& fat, StageAt& gat) {
+  constexpr int NT = MARCH_NT;
+  const int t = threadIdx.x;
+  const int w = g.tile_w;
+  const int x0 = strip * 2 * w;
+  const int wa = min(w, g.nx - x0), wb = min(w, g.nx - x0 - w);   // columns of each lane (wb may be < 1)
+  const int ya = seg * g.seg_h;
+  const int yb = min(ya + g.seg_h, g.ny);
+  const int te = min(t, w + 5);                    // threads beyond the halo repeat its last column
+  const int xla = x0 - 3 + te, xlb = xla + w;      // logical columns (may lie outside [0, nx))
+  const int xpa = wrap1(xla, g.nx), xpb = wrap1(xlb, g.nx);
+  const bool on_a = t >= 3 && t < wa + 3, on_b = t >= 3 && t < wb + 3;
+  const bool ywall = g.bc_y == BC_WALL;
+
+  // ---- staged columns: blocks [b0, b0 + run1) and, for a strip that wraps, [0, run2)
+  const int nbx = (g.nx + BLK - 1) / BLK;
+  int b0 = 0, run1 = nbx, run2 = 0;
+  if (g.nx >= 2 * w + 8) {
+    const int xs = wrap1(x0 - 4, g.nx), xe = wrap1(x0 + 2 * w + 3, g.nx);
+    b0 = xs / BLK;
+    if (xs <= xe) {
+      run1 = xe / BLK - b0 + 1;
+    } else {
+      run1 = nbx - b0;
+      run2 = xe / BLK + 1;
+    }
+  }
+  auto staged_col = [&](int xp) {
+    const int blk = xp / BLK;
+    return col_bytes<ST>(blk >= b0 ? blk - b0 : run1 + blk, xp & (BLK - 1));
+  };
+  auto staged3 = [&](int xp) {
+    return Col3{staged_col(xp == 0 ? g.nx - 1 : xp - 1), staged_col(xp), staged_col(xp == g.nx - 1 ? 0 : xp + 1)};
+  };
+  const Col3 ca = staged3(xpa), cb = staged3(xpb);
+  // x walls: the columns next to one, and the ghost column their threads also fill
+  const bool xwall = XW && g.bc_x == BC_WALL;
+  const bool real_a = !xwall || (xla >= 0 && xla < g.nx), real_b = !xwall || (xlb >= 0 && xlb < g.nx);
+  auto ghost_of = [&](int xl) {
+    if (!xwall || t != te) return -1;
+    return xl == 0 ? t - 1 : (xl == g.nx - 1 && t + 1 < NT ? t + 1 : -1);
+  };
+  const int tga = ghost_of(xla), tgb = ghost_of(xlb);
+
+  // ---- producer: one thread copies the rows of f, one of another warp those of gbar
+  auto load_piece = [&](unsigned char* dst, int r, int region, unsigned long long* bar) {
+    const int blk = region_block(ST, region);
+    const char* row = static_cast<const char*>(g.src) + (long long)wrap1(r, g.ny) * g.row_bytes + region_start(ST, region) * g.nblk;
+    bulk_load(smem_u32(dst), row + b0 * blk, run1 * blk, bar);
+    if (run2 > 0) bulk_load(smem_u32(dst) + run1 * blk, row, run2 * blk, bar);
+  };
+  // rows fr of f into stage fs and gr of gbar into stage gs
+  auto produce = [&](bool do_f, int fr, int fs, bool do_g, int gr, int gs) {
+    if (t == 0 && do_f) {
+      mbar_expect(&sm.fbar[fs], (run1 + run2) * (region_block(ST, R_F) + region_block(ST, R_L)));
+      load_piece(sm.stage[fs].f, fr, R_F, &sm.fbar[fs]);
+      if constexpr (region_block(ST, R_L) > 0) load_piece(sm.stage[fs].l, fr, R_L, &sm.fbar[fs]);
+    }
+    if (t == 32 && do_g) {
+      mbar_expect(&sm.gbar[gs], (run1 + run2) * region_block(ST, R_G));
+      load_piece(sm.stage[gs].g, gr, R_G, &sm.gbar[gs]);
+    }
+  };
+
+  // S2 runs in iterations ya + 2 .. a_end (rows ya - 1 ..), S3 in ya + 4 .. yb + 3; the moment pass ends
+  // with S2 of row yb - 1.
+  const int a_end = MODE == MODE_STEP ? yb + 3 : yb + 2;
+  for (int k = 0; k < STAGES; ++k)
+    produce(true, ya - 3 + k, fat.ahead(k), ya - 1 + k <= a_end - 3, ya - 1 + k, gat.ahead(k));
+
+  // ---- rings: byte offsets of this thread's place in the rows a-k (mod 5) and a-k (mod 3) of iteration a.  The
+  // rows of mu (read a-4 .. a-2, then a-1 written) and of p, u (a-3 written, then a-5 .. a-3 read) share
+  // the second set.
+  using S = MarchSmem<ST, SD>;
+  char* const base = reinterpret_cast<char*>(&sm);
+  int q5[RING5], q3[RING3];
+#pragma unroll
+  for (int k = 0; k < RING5; ++k) q5[k] = (int)offsetof(S, r5) + (RING5 - 1 - k) * (int)sizeof(typename S::Row5) + t * 8;
+#pragma unroll
+  for (int k = 0; k < RING3; ++k) q3[k] = (int)offsetof(S, r3) + (RING3 - 1 - k) * (int)sizeof(typename S::Row3) + t * 8;
+  auto at = [&](int off) { return reinterpret_cast<V2*>(base + off); };
+  constexpr int HI = offsetof(typename S::Row5, hi), LO = offsetof(typename S::Row5, lo);
+  constexpr int MU = offsetof(typename S::Row3, mu), PP = offsetof(typename S::Row3, p), UX = offsetof(typename S::Row3, ux),
+                UY = offsetof(typename S::Row3, uy), JX = offsetof(typename S::Row3, j), JY = JX + 8 * NT;
+  auto row_ok = [&](int r) { return !ywall || (r >= 0 && r < g.ny); };
+  // The lanes whose column is real store it, and next to a wall on x also its mirror image in the ghost column.
+  // Threads away from the walls store both lanes at once.
+  const bool plain = !XW || (real_a && real_b && tga < 0 && tgb < 0);
+  auto put_wall = [&](int off, V2 v) {
+    float x, y;
+    unpack2(v, x, y);
+    float* const f = reinterpret_cast<float*>(at(off));
+    if (real_a) f[0] = x;
+    if (real_b) f[1] = y;
+    if (tga >= 0) f[2 * (tga - t)] = x;
+    if (tgb >= 0) f[2 * (tgb - t) + 1] = y;
+  };
+  auto put = [&](int off, V2 v) { *at(off) = v; };
+  // Offsets of the rows south and north of row r.  Beyond a wall they are the row itself, its mirror image.
+  auto south = [&](int r, int s, int c, auto kind) { return decltype(kind)::value == IT_CHECKED && ywall && r == 0 ? c : s; };
+  auto north = [&](int r, int n, int c, auto kind) {
+    return decltype(kind)::value == IT_CHECKED && ywall && r == g.ny - 1 ? c : n;
+  };
+
+  // ---- population pop of both lanes from a staged region
+  auto staged = [&](const unsigned char* reg, auto pop, const ColB& a, const ColB& b) {
+    constexpr int A = decltype(pop)::value;
+    auto one = [&](const ColB& c) {
+      const unsigned char* q = reg + pop_in_region<ST>(A, c);
+      if constexpr (pop_bytes(ST, A) == 4) return *reinterpret_cast<const float*>(q);
+      else return dec_pop<ST>(*reinterpret_cast<const unsigned short*>(q), A);
+    };
+    return pack2(one(a), one(b));
+  };
+  // the populations F .. F + 8 that stream into the lanes' cells
+  auto pull9 = [&](auto first, const unsigned char* reg, V2 v[Q]) {
+    constexpr int F = decltype(first)::value;
+    v[0] = staged(reg, std::integral_constant<int, F + 0>{}, ca.c0, cb.c0);
+    v[1] = staged(reg, std::integral_constant<int, F + 1>{}, ca.cm, cb.cm);
+    v[2] = staged(reg, std::integral_constant<int, F + 2>{}, ca.c0, cb.c0);
+    v[3] = staged(reg, std::integral_constant<int, F + 3>{}, ca.cq, cb.cq);
+    v[4] = staged(reg, std::integral_constant<int, F + 4>{}, ca.c0, cb.c0);
+    v[5] = staged(reg, std::integral_constant<int, F + 5>{}, ca.cm, cb.cm);
+    v[6] = staged(reg, std::integral_constant<int, F + 6>{}, ca.cq, cb.cq);
+    v[7] = staged(reg, std::integral_constant<int, F + 7>{}, ca.cq, cb.cq);
+    v[8] = staged(reg, std::integral_constant<int, F + 8>{}, ca.cm, cb.cm);
+  };
+  using F0 = std::integral_constant<int, 0>;
+  using G0 = std::integral_constant<int, Q>;
+
+  RecT<V2> cur{}, prev{};                  // records of rows a-3 and a-4 (in phase 2 of iteration a)
+  V2 gcur[Q], gprev[Q];                    // their pulled gbar
+  // phi and 12 grad(phi) as S1 meets them, for S2 two iterations later: rows a-2 and a-3 in phase 1 of iteration a
+  struct PhiGrad {
+    V2 ph, gx, gy;
+  } pg2{}, pg3{};
+  V2 sp_rho = zero<V2>(), sp_div = zero<V2>();   // direct mass defect: rho, div(rho u) of the last step
+  auto fetch_sd = [&](int r) {
+    if constexpr (SD) {
+      const float* sp = reinterpret_cast<const float*>(static_cast<const char*>(g.src) + g.spoff) + wrap1(r, g.ny) * g.pitch;
+      sp_rho = pack2(__ldg(sp + xpa), __ldg(sp + xpb));
+      sp_div = pack2(__ldg(sp + g.plane + xpa), __ldg(sp + g.plane + xpb));
+    }
+  };
+
+  auto shift = [&] {
+    prev = cur;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) gprev[k] = gcur[k];
+  };
+
+  auto iter = [&](int a, auto kind) {
+    constexpr int KIND = decltype(kind)::value;
+    constexpr bool CK = KIND == IT_CHECKED, IN = KIND == IT_INNER;
+    const int fs = fat.stage, gs = gat.stage;
+    const int r1 = a - 1, r2 = a - 3, r3 = a - 4;   // rows of S1, S2, S3
+    const bool s2_runs = IN || a >= ya + 2;
+    const bool do0 = !CK || (row_ok(a) && a <= yb + 2);
+    const bool do1 = !CK || (r1 >= ya - 2 && r1 <= yb + 1 && row_ok(r1));
+    const bool do2 = s2_runs && (!CK || row_ok(r2));
+    // ================ phase 1: S0 and S2; all stores to the rings at its end
+    mbar_wait(&sm.fbar[fs], fat.parity, g.gave_up);
+    if (s2_runs) mbar_wait(&sm.gbar[gs], gat.parity, g.gave_up);
+    // ---- S0: phi at row a (as an unevaluated pair hi + lo)
+    V2 fp[NF], hi, lo;
+    auto stage0 = [&] {
+      pull9(F0{}, sm.stage[fs].f, fp);
+      fp[Q] = zero<V2>();
+      if constexpr (ST == ST_FP32) fp[Q] = staged(sm.stage[fs].l, std::integral_constant<int, A_F0LO>{}, ca.c0, cb.c0);
+      phi_pair<ST>(P, fp, hi, lo);
+    };
+    // ---- S2: u, p at row a-3 (rows a-4 .. a-2 of phi and mu)
+    S2Out<V2> o;
+    auto stage2 = [&] {
+      const int c3 = q3[0], s3 = south(r2, q3[1], c3, kind), n3 = north(r2, q3[2], c3, kind);
+      const V2 *ms = at(s3 + MU), *m0 = at(c3 + MU), *mn = at(n3 + MU);
+      const V2 ph = pg3.ph, gphx = pg3.gx, gphy = pg3.gy;
+      V2 gmx, gmy;                                 // 12 x the isotropic gradient
+      grad12(P, ms, m0, mn, gmx, gmy);
+      V2 sdef;
+      if constexpr (SD) sdef = fadd(fsub(density(P, ph), sp_rho), sp_div);
+      else sdef = fmul(P.s_coef6, lap6_of(P, ms, m0, mn));
+      asm("" : "+l"(sdef.v));                      // computed either way: no branch around the stencil
+      const V2 s_all = sdef;                       // F_a is reported whether or not the scheme removes it
+      sdef.v = P.remove_Fa ? sdef.v : 0ull;
+      V2 gb[Q];
+      pull9(G0{}, sm.stage[gs].g, gb);
+      o = s2_cell<ST>(P, ph, gphx, gphy, gmx, gmy, m0[0], sdef, gb);
+      if constexpr (MODE == MODE_STEP) {
+        if constexpr (SD) {
+          float x, y;                              // rho^t for the next step
+          unpack2(o.rho, x, y);
+          float* sp = reinterpret_cast<float*>(static_cast<char*>(g.dst) + g.spoff) + (long long)r2 * g.pitch;
+          const bool row = r2 >= ya && r2 < yb;
+          st_on(sp + xpa, x, on_a && row);
+          st_on(sp + xpb, y, on_b && row);
+        }
+        shift();
+        s2_record(P, o, ph, m0[0], sdef, cur);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) gcur[k] = gb[k];
+        if constexpr (FF) {
+          cur.gx12 = gphx;
+          cur.gy12 = gphy;
+          cur.lmu6 = lap6_of(P, ms, m0, mn);
+        }
+      } else if (r2 >= ya) {                       // r2 < yb throughout
+        auto store2 = [&](float* q, V2 v) {
+          float x, y;
+          unpack2(v, x, y);
+          if (on_a) q[r2 * g.pitch + xpa] = x;
+          if (on_b) q[r2 * g.pitch + xpb] = y;
+        };
+        if (mo.phi) store2(mo.phi, ph);
+        if (mo.rho) store2(mo.rho, o.rho);
+        if (mo.ux) store2(mo.ux, o.ux);
+        if (mo.uy) store2(mo.uy, o.uy);
+        if (mo.p) store2(mo.p, o.p);
+        if (mo.fax) {
+          store2(mo.fax, fmul(fsub(zero<V2>(), o.ux), s_all));
+          store2(mo.fay, fmul(fsub(zero<V2>(), o.uy), s_all));
+        }
+      }
+    };
+    if (do0) stage0();
+    if (do2) stage2();
+    else if (MODE == MODE_STEP && s2_runs) shift();   // (a row beyond a wall has no record)
+    auto puts1 = [&](auto put_) {
+      if (do0) {
+        put_(q5[0] + HI, hi);
+        put_(q5[0] + LO, lo);
+      }
+      if (do2) {
+        put_(q3[0] + PP, o.p);
+        if constexpr (MODE == MODE_STEP) {
+          put_(q3[0] + UX, o.ux);
+          put_(q3[0] + UY, o.uy);
+          if constexpr (SD) {
+            put_(q3[0] + JX, fmul(o.rho, o.ux));
+            put_(q3[0] + JY, fmul(o.rho, o.uy));
+          }
+        }
+      }
+    };
+    if (!XW || plain) puts1(put);
+    else puts1(put_wall);
+    if (MODE == MODE_STEP && do0) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        *reinterpret_cast<ulonglong2*>(base + q5[0] + t * 8 + k * NT * 16) = make_ulonglong2(fp[2 * k + 1].v, fp[2 * k + 2].v);
+    }
+    if (IN || a >= ya + 1) fetch_sd(r2 + 1);
+    __syncthreads();
+    // ================ phase 2: S1 and S3
+    // the stages just read are free
+    produce(a + STAGES <= a_end, a + STAGES, fs, s2_runs && r2 + STAGES <= a_end - 3, r2 + STAGES, gs);
+    // ---- S1: mu at row a-1 (rows a-2 .. a of phi)
+    V2 mu;
+    auto stage1 = [&] {
+      const int c = q5[1], sr = south(r1, q5[2], c, kind), n = north(r1, q5[0], c, kind);
+      mu = chem_potential(P, at(sr + HI), at(c + HI), at(n + HI), at(sr + LO), at(c + LO), at(n + LO));
+      // grad phi only feeds grad rho (density and pressure terms): the high words suffice
+      pg2.ph = fadd(*at(c + HI), *at(c + LO));
+      grad12(P, at(sr + HI), at(c + HI), at(n + HI), pg2.gx, pg2.gy);
+    };
+    // ---- S3: collide and store row a-4 (p, u of rows a-5 .. a-3)
+    auto stage3 = [&] {
+      const int c = q3[1], os = south(r3, q3[2], c, kind), on = north(r3, q3[0], c, kind);
+      V2 gpx, gpy;                                 // 12 grad p
+      grad12(P, at(os + PP), at(c + PP), at(on + PP), gpx, gpy);
+      // phi div(u) of the convective form; computed either way, so that no branch splits the block
+      V2 phiD = phi_div_u(P, prev.phi, at(os + UX), at(c + UX), at(on + UX), at(os + UY), at(on + UY));
+      asm("" : "+l"(phiD.v));
+      phiD.v = P.ch_conv ? phiD.v : 0ull;
+      V2 f[Q];
+      f[0] = zero<V2>();   // unused: f_0 follows from the phi pair
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(base + q5[4] + t * 8 + k * NT * 16);
+        f[2 * k + 1].v = v.x;
+        f[2 * k + 2].v = v.y;
+      }
+      if constexpr (SD) {
+        // div(rho u) of this step, for the next step's mass defect
+        const V2 *xs = at(os + JX), *xc = at(c + JX), *xn = at(on + JX), *ys = at(os + JY), *yn = at(on + JY);
+        const V2 djx = fmad(P.k4, fsub(xc[1], xc[-1]), fsub(fsub(xn[1], xs[-1]), fsub(xn[-1], xs[1])));
+        const V2 djy = fmad(P.k4, fsub(yn[0], ys[0]), fadd(fsub(yn[1], ys[-1]), fsub(yn[-1], ys[1])));
+        float x, y;
+        unpack2(fmul(fadd(djx, djy), P.k12th), x, y);
+        float* sp = reinterpret_cast<float*>(static_cast<char*>(g.dst) + g.spoff) + g.plane + (long long)r3 * g.pitch;
+        st_on(sp + xpa, x, on_a);
+        st_on(sp + xpb, y, on_b);
+      }
+      OutLanes<ST> out;
+      collide_store<ST, FF>(P, prev, *at(c + PP), gpx, gpy, *at(q5[4] + HI), *at(q5[4] + LO), phiD, f, gprev, out);
+      // the cells next to a wall, where populations bounce back, take the general path
+      const bool wrow = CK && ywall && (r3 == 0 || r3 == g.ny - 1);
+      const bool wcol_a = xwall && (xla == 0 || xla == g.nx - 1), wcol_b = xwall && (xlb == 0 || xlb == g.nx - 1);
+      char* const dst = static_cast<char*>(g.dst);
+      char* const row0 = dst + (long long)r3 * g.row_bytes;
+      char* const rowm = r3 == 0 ? dst + (long long)(g.ny - 1) * g.row_bytes : row0 - g.row_bytes;
+      char* const rowq = r3 == g.ny - 1 ? dst : row0 + g.row_bytes;
+      if constexpr (CK || XW) {
+        if (on_a && (wrow || wcol_a)) out.template store_cell<false>(out_cell<ST, XW, true>(g, xpa, r3));
+        if (on_b && (wrow || wcol_b)) out.template store_cell<true>(out_cell<ST, XW, true>(g, xpb, r3));
+      }
+      out.template store_lane<false>(rowm, row0, rowq, col_bytes<ST>(xpa), g.nblk, hash_key<ST>(xpa, r3, g),
+                                     on_a && !((CK || XW) && (wrow || wcol_a)));
+      out.template store_lane<true>(rowm, row0, rowq, col_bytes<ST>(xpb), g.nblk, hash_key<ST>(xpb, r3, g),
+                                    on_b && !((CK || XW) && (wrow || wcol_b)));
+    };
+    pg3 = pg2;
+    if (do1) stage1();
+    if constexpr (MODE == MODE_STEP) {
+      if constexpr (IN) stage3();
+      if constexpr (CK)
+        if (a >= ya + 4) stage3();
+    }
+    if (do1) {
+      if (!XW || plain) put(q3[1] + MU, mu);
+      else put_wall(q3[1] + MU, mu);
+    }
+    {
+      const int x5 = q5[RING5 - 1], x3 = q3[RING3 - 1];
+#pragma unroll
+      for (int k = RING5 - 1; k > 0; --k) q5[k] = q5[k - 1];
+#pragma unroll
+      for (int k = RING3 - 1; k > 0; --k) q3[k] = q3[k - 1];
+      q5[0] = x5;
+      q3[0] = x3;
+    }
+    fat.next();
+    if (s2_runs) gat.next();
+    __syncthreads();
+  };
+
+  using Checked = std::integral_constant<int, IT_CHECKED>;
+  using Fill = std::integral_constant<int, IT_FILL>;
+  using Inner = std::integral_constant<int, IT_INNER>;
+  int a = ya - 3;
+  // S0 meets a wall row only in segments within 4 rows of a wall; a periodic y axis has none
+  if (!ywall || (ya >= 4 && yb + 3 <= g.ny - 2)) {
+    for (; a < ya + 4 && a <= a_end; ++a) iter(a, Fill{});
+    for (; a <= a_end; ++a) iter(a, Inner{});
+  } else {
+    const int a_in0 = max(ya + 4, 5), a_in1 = min(a_end, g.ny - 2);
+    for (; a < a_in0 && a <= a_end; ++a) iter(a, Checked{});
+    for (; a <= a_in1; ++a) iter(a, Inner{});
+    for (; a <= a_end; ++a) iter(a, Checked{});
+  }
+}
+
+}  // namespace lbm

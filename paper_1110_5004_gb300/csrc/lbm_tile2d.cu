@@ -56,12 +56,6 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
     if (oj) f[gj][i] = v;
     if (oi && oj) f[gj][gi] = v;
   };
-  auto nbr = [&](int x, int y, ColNb& cn, RowNb& rn) {
-    cn = make_col<ST>(wrap1(x, g.nx), g);
-    rn = make_row(wrap1(y, g.ny), g);
-    if constexpr (!XW) cn.wl = cn.wr = false;
-    if constexpr (!YW) rn.wb = rn.wt = false;
-  };
   // Every population load of this thread is issued first, all at once: f of its S0 cells and
   // gbar of its S2 cells; the passes then wait on the loads they use.
   constexpr int C0 = (FW * FH + NT - 1) / NT, C2 = ((FW - 4) * (FH - 4) + NT - 1) / NT;
@@ -73,21 +67,17 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
   for (int c = 0; c < C0; ++c) {
     const int k = t + c * NT, i = k % FW, j = k / FW, x = x0 - 3 + i, y = y0 - 3 + j;
     if (k < FW * FH && real(x, y)) {
-      ColNb cn;
-      RowNb rn;
-      nbr(x, y, cn, rn);
-      gather9<ST, 0, COH>(g.src, cn, rn, f0raw[c]);
-      f0raw[c][Q] = ST == ST_FP32 ? ld_raw<ST, COH>(g.src, PLANE_F0LO, cell_at(rn.b0, cn.c0)) : 0u;
+      const Col3 cn = col3<ST>(wrap1(x, g.nx), g.nx);
+      const int row = wrap1(y, g.ny) * g.row_bytes;
+      gather9<ST, 0, COH>(g, cn, row, f0raw[c]);
+      f0raw[c][Q] = ST == ST_FP32 ? ld_raw<ST, COH>(g.src, A_F0LO, pop_at<ST>(A_F0LO, row, cn.c0, g)) : 0u;
     }
   }
 #pragma unroll
   for (int c = 0; c < C2; ++c) {
     const int k = t + c * NT, i = 2 + k % (FW - 4), j = 2 + k / (FW - 4), x = x0 - 3 + i, y = y0 - 3 + j;
     if (k < (FW - 4) * (FH - 4) && real(x, y)) {
-      ColNb cn;
-      RowNb rn;
-      nbr(x, y, cn, rn);
-      gather9<ST, Q, COH>(g.src, cn, rn, g2raw[c]);
+      gather9<ST, Q, COH>(g, col3<ST>(wrap1(x, g.nx), g.nx), wrap1(y, g.ny) * g.row_bytes, g2raw[c]);
     }
   }
 
@@ -101,7 +91,7 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
     for (int a = 0; a < Q; ++a) fp[a] = dec_pop<ST>(f0raw[c][a], a);
     fp[Q] = __uint_as_float(f0raw[c][Q]);
     float hi, lo;
-    phi_pair<ST>(fp, g.isf, hi, lo);
+    phi_pair<ST>(P, fp, hi, lo);
     put(sm.hi, i, j, x, y, hi);
     put(sm.lo, i, j, x, y, lo);
     const int ti = i - 3, tj = j - 3;
@@ -127,13 +117,13 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
     if (k >= (FW - 4) * (FH - 4) || !real(x, y)) continue;
     const float ph = fadd(sm.hi[j][i], sm.lo[j][i]);
     float gphx, gphy, gmx, gmy;
-    grad12(&sm.hi[j - 1][i], &sm.hi[j][i], &sm.hi[j + 1][i], gphx, gphy);
-    grad12(&sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i], gmx, gmy);
-    const float sdef = P.remove_Fa ? fmul(P.s_coef6, lap6_of(&sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i])) : 0.0f;
+    grad12(P, &sm.hi[j - 1][i], &sm.hi[j][i], &sm.hi[j + 1][i], gphx, gphy);
+    grad12(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i], gmx, gmy);
+    const float sdef = P.remove_Fa ? fmul(P.s_coef6, lap6_of(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i])) : 0.0f;
     float gb[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) gb[a] = dec_pop<ST>(g2raw[c][a], Q + a);
-    const S2Out s2 = s2_cell<ST>(P, ph, gphx, gphy, gmx, gmy, sm.mu[j][i], sdef, gb, g.isg);
+    const S2Out<float> s2 = s2_cell<ST>(P, ph, gphx, gphy, gmx, gmy, sm.mu[j][i], sdef, gb);
     put(sm.p, i, j, x, y, s2.p);
     if (P.ch_conv) {
       put(sm.ux, i, j, x, y, s2.ux);
@@ -141,7 +131,7 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
     }
     const int ti = i - 3, tj = j - 3;
     if (ti >= 0 && ti < TX && tj >= 0 && tj < TY) {
-      Rec r{};
+      RecT<float> r{};
       s2_record(P, s2, ph, sm.mu[j][i], sdef, r);
       const float v[10] = {r.phi, r.mu, r.ux, r.uy, r.Fx, r.Fy, r.mrx3, r.mry3, r.og, r.ogr3};
 #pragma unroll
@@ -155,7 +145,7 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
   {
     const int k = t % (TX * TY), ti = k % TX, tj = k / TX, i = ti + 3, j = tj + 3, x = x0 + ti, y = y0 + tj;
     if (t < 2 * TX * TY && x < g.nx && y < g.ny) {
-      Rec r{};
+      RecT<float> r{};
       r.phi = sm.rec[0][tj][ti];
       r.mu = sm.rec[1][tj][ti];
       r.ux = sm.rec[2][tj][ti];
@@ -167,9 +157,9 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
       r.og = sm.rec[8][tj][ti];
       r.ogr3 = sm.rec[9][tj][ti];
       float f[Q], gb[Q];
-      const CellB cell = cell_at(y * g.row_bytes, col_bytes<ST>(x));
+      const OutCell<ST, XW, YW> cell = out_cell<ST, XW, YW>(g, x, y);
       if (t < TX * TY) {   // f: needs phi div u and the phi pair, not p
-        const float phiD = P.ch_conv ? phi_div_u(r.phi, &sm.ux[j - 1][i], &sm.ux[j][i], &sm.ux[j + 1][i],
+        const float phiD = P.ch_conv ? phi_div_u(P, r.phi, &sm.ux[j - 1][i], &sm.ux[j][i], &sm.ux[j + 1][i],
                                                  &sm.uy[j - 1][i], &sm.uy[j + 1][i])
                                      : 0.0f;
         f[0] = 0.0f;   // unused: f_0 follows from the phi pair
@@ -177,15 +167,15 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
         for (int a = 1; a < Q; ++a) f[a] = dec_pop<ST>(sm.f3[a - 1][tj][ti], a);
 #pragma unroll
         for (int a = 0; a < Q; ++a) gb[a] = 0.0f;   // unused by the f collision
-        collide_store<ST, false, COLLIDE_F>(P, r, 0.0f, 0.0f, 0.0f, sm.hi[j][i], sm.lo[j][i], phiD, f, gb, g, cell);
+        collide_store<ST, false, COLLIDE_F>(P, r, 0.0f, 0.0f, 0.0f, sm.hi[j][i], sm.lo[j][i], phiD, f, gb, cell);
       } else {              // gbar: needs p and grad p
         float gpx, gpy;
-        grad12(&sm.p[j - 1][i], &sm.p[j][i], &sm.p[j + 1][i], gpx, gpy);
+        grad12(P, &sm.p[j - 1][i], &sm.p[j][i], &sm.p[j + 1][i], gpx, gpy);
 #pragma unroll
         for (int a = 0; a < Q; ++a) f[a] = 0.0f;    // unused by the gbar collision
 #pragma unroll
         for (int a = 0; a < Q; ++a) gb[a] = sm.gb[a][tj][ti];
-        collide_store<ST, false, COLLIDE_G>(P, r, sm.p[j][i], gpx, gpy, 0.0f, 0.0f, 0.0f, f, gb, g, cell);
+        collide_store<ST, false, COLLIDE_G>(P, r, sm.p[j][i], gpx, gpy, 0.0f, 0.0f, 0.0f, f, gb, cell);
       }
     }
   }
