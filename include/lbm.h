@@ -286,7 +286,7 @@ LBM_API const char* lbm_last_error(void);
  *                   the current device or in managed memory (anything else: LBM_ERR_INVALID_ARG);
  *   ny <= 8192 (larger grids: LBM_ERR_INVALID_ARG with a message), nx >= 1, phi_star > 0;
  *   step            copied into out->step;
- *   cuda_stream     stream the two reduction kernels run on (NULL: legacy default stream);
+ *   cuda_stream     stream the reduction runs on (NULL: legacy default stream);
  *   out             host or device lbm_diag; a host record is filled before return (the stream
  *                   is synchronised) and LBM_ERR_DIVERGED is returned if the fields are not
  *                   finite; a device record is written asynchronously.  Synchronising is not

@@ -90,7 +90,7 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
   g.bc_x = s->params.bc_x;
   g.bc_y = s->params.bc_y;
   tile_geometry(s->nx, s->ny, s->params.s_form != 0, s->seg_h, s->sms * MARCH_CTAS, &g.tile_w, &g.n_strips, &g.seg_h);
-  g.gave_up = reinterpret_cast<unsigned int*>(s->red + (size_t)s->ny * DIAG_PARTIALS + 14);
+  g.gave_up = gave_up(s);
   g.spoff = s->params.s_form ? (long long)s->pop_bytes : 0;
   return g;
 }
@@ -350,7 +350,7 @@ int lbm_step(lbm_sim* s, int n) {
   const bool tiles = uses_tile2d(s);
   for (int i = 0; i < n; ++i) {
     Grid g = make_grid(s, s->buf[s->cur], s->buf[s->cur ^ 1]);
-    cudaError_t e = tiles ? launch_tile2d(s->phys, g, s->sms, s->stream) : launch_step(s->phys2, g, s->stream);
+    cudaError_t e = tiles ? launch_tile2d(s->phys, g, nullptr, s->sms, s->stream) : launch_step(s->phys2, g, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "lbm_step launch");
     s->cur ^= 1;
     s->steps++;
@@ -359,11 +359,19 @@ int lbm_step(lbm_sim* s, int n) {
   return LBM_OK;
 }
 
+// The moment pass of the current state.  Small grids take the tile kernel's three passes, whose
+// latency is that of one tile, instead of a march over rows.
+static cudaError_t moments_of(const lbm_sim* s, const Grid& g, const MomentOut& mo) {
+  if (s->params.s_form == 0 && (long long)s->nx * s->ny <= SMALL_GRID_MOMENTS)
+    return launch_tile2d(s->phys, g, &mo, s->sms, s->stream);
+  return launch_moments(s->phys2, g, mo, s->stream);
+}
+
 static int compute_moments(lbm_sim* s) {
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
   MomentOut mo{s->fields, s->fields + s->plane, s->fields + 2 * s->plane, s->fields + 3 * s->plane,
                s->fields + 4 * s->plane};
-  cudaError_t e = launch_moments(s->phys2, g, mo, s->stream);
+  cudaError_t e = moments_of(s, g, mo);
   if (e != cudaSuccess) return cuda_fail(e, "moments launch");
   s->launches++;
   return LBM_OK;
@@ -413,7 +421,7 @@ int lbm_moments(lbm_sim* s, float* phi, float* rho, float* ux, float* uy, float*
   }
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
   MomentOut mo{dst[0], dst[1], dst[2], dst[3], dst[4]};
-  cudaError_t e = launch_moments(s->phys2, g, mo, s->stream);
+  cudaError_t e = moments_of(s, g, mo);
   if (e != cudaSuccess) return cuda_fail(e, "moments launch");
   s->launches++;
   return copy_out(s, staged, 5, "lbm_moments copy");
@@ -429,7 +437,7 @@ int lbm_moments_packed(lbm_sim* s, float* fields) {
   const size_t stride = direct ? n : (size_t)s->plane;
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
   MomentOut mo{dst, dst + stride, dst + 2 * stride, dst + 3 * stride, dst + 4 * stride};
-  cudaError_t e = launch_moments(s->phys2, g, mo, s->stream);
+  cudaError_t e = moments_of(s, g, mo);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_moments_packed launch");
   s->launches++;
   if (!direct) {
@@ -448,7 +456,7 @@ int lbm_interfacial_force(lbm_sim* s, float* fa_x, float* fa_y) {
   MomentOut mo{};
   mo.fax = s->fields;
   mo.fay = s->fields + s->plane;
-  cudaError_t e = launch_moments(s->phys2, g, mo, s->stream);
+  cudaError_t e = moments_of(s, g, mo);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_interfacial_force launch");
   s->launches++;
   float* outs[2] = {fa_x, fa_y};
@@ -462,7 +470,7 @@ int lbm_diagnostics(lbm_sim* s, lbm_diag* out) {
   if (rc) return rc;
   cudaError_t e = launch_diag(s, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "diagnostics launch");
-  s->launches += 2;
+  s->launches++;
   e = cudaMemcpyAsync(&s->h_diag, s->red + (long long)s->ny * DIAG_PARTIALS, sizeof(lbm_diag),
                       cudaMemcpyDeviceToHost, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "diagnostics copy");

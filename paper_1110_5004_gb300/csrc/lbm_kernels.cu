@@ -2,6 +2,7 @@
 // FP64 diagnostics, with their launchers.
 #include <math.h>
 
+#include "lbm_diag.cuh"
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -221,109 +222,14 @@ cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u
 }
 
 // ------------------------------------------------------------------ FP64 diagnostics
-// Stage 1: one block per row, fixed per-thread stride and fixed tree -> 12 partials per row.
-// Stage 2: one block folds the rows in a fixed order.  Results are bitwise reproducible.
-
-constexpr int DIAG_T = 256;
-
-__device__ __forceinline__ void tree_sum(double* sh, int t) {
-  for (int s = DIAG_T / 2; s > 0; s >>= 1) {
-    if (t < s) sh[t] += sh[t + s];
-    __syncthreads();
-  }
-}
-__device__ __forceinline__ void tree_max(double* sh, int t) {
-  for (int s = DIAG_T / 2; s > 0; s >>= 1) {
-    if (t < s) {
-      const double a = sh[t], b = sh[t + s];
-      sh[t] = (a >= b || a != a) ? a : b;   // NaN propagates
-    }
-    __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(DIAG_T) k_diag_rows(Phys P, Grid g, const float* __restrict__ fields,
-                                                      double* __restrict__ part) {
-  __shared__ double sh[DIAG_PARTIALS][DIAG_T];
-  const int y = blockIdx.x, t = threadIdx.x;
-  const float* phi = fields + (long long)y * g.pitch;
-  const float* ux = fields + 2 * g.plane + (long long)y * g.pitch;
-  const float* uy = fields + 3 * g.plane + (long long)y * g.pitch;
-  const float* pp = fields + 4 * g.plane + (long long)y * g.pitch;
-  double acc[DIAG_PARTIALS] = {0};
-  const double phs = P.phi_star;
-  for (int x = t; x < g.nx; x += DIAG_T) {
-    const double ph = phi[x], u = ux[x], v = uy[x], p = pp[x];
-    double c = (ph + phs) / (2.0 * phs);
-    c = c < 0.0 ? 0.0 : (c > 1.0 ? 1.0 : c);
-    acc[0] += ph;
-    acc[1] += c;
-    acc[2] += c * x;
-    acc[3] += c * y;
-    acc[4] += c * u;
-    acc[5] += c * v;
-    const double um = sqrt(u * u + v * v);
-    if (!(um <= acc[6])) acc[6] = um;
-    if (ph > 0.9 * phs) { acc[7] += p; acc[8] += 1.0; }
-    if (ph < -0.9 * phs) { acc[9] += p; acc[10] += 1.0; }
-  }
-  for (int k = 0; k < 11; ++k) sh[k][t] = acc[k];
-  __syncthreads();
-  for (int k = 0; k < 11; ++k) {
-    if (k == 6) tree_max(sh[k], t); else tree_sum(sh[k], t);
-  }
-  if (t < 11) part[(long long)y * DIAG_PARTIALS + t] = sh[t][0];
-  if (t == 11) part[(long long)y * DIAG_PARTIALS + 11] = 0.0;
-}
-
-__global__ void __launch_bounds__(DIAG_T) k_diag_final(Grid g, const double* __restrict__ part,
-                                                       double* __restrict__ out, long long step) {
-  __shared__ double sh[DIAG_PARTIALS][DIAG_T];
-  const int t = threadIdx.x;
-  double acc[DIAG_PARTIALS] = {0};
-  for (int y = t; y < g.ny; y += DIAG_T) {
-    const double* r = part + (long long)y * DIAG_PARTIALS;
-    for (int k = 0; k < 11; ++k) {
-      if (k == 6) {
-        if (!(r[6] <= acc[6])) acc[6] = r[6];
-      } else {
-        acc[k] += r[k];
-      }
-    }
-    if (!(r[1] <= acc[11])) acc[11] = r[1];   // widest liquid chord
-  }
-  for (int k = 0; k < DIAG_PARTIALS; ++k) sh[k][t] = acc[k];
-  __syncthreads();
-  for (int k = 0; k < DIAG_PARTIALS; ++k) {
-    if (k == 6 || k == 11) tree_max(sh[k], t); else tree_sum(sh[k], t);
-  }
-  if (t == 0) {
-    lbm_diag d;
-    d.step = step;
-    d.sum_phi = sh[0][0];
-    d.liquid_area = sh[1][0];
-    const double sc = sh[1][0];
-    d.centroid_x = sc > 0 ? sh[2][0] / sc : 0.0;
-    d.centroid_y = sc > 0 ? sh[3][0] / sc : 0.0;
-    d.vel_x = sc > 0 ? sh[4][0] / sc : 0.0;
-    d.vel_y = sc > 0 ? sh[5][0] / sc : 0.0;
-    d.spread_radius = 0.5 * sh[11][0];
-    d.max_u = sh[6][0];
-    d.p_liquid = sh[8][0] > 0 ? sh[7][0] / sh[8][0] : 0.0;
-    d.p_gas = sh[10][0] > 0 ? sh[9][0] / sh[10][0] : 0.0;
-    d.finite = isfinite(d.sum_phi) && isfinite(d.max_u) && *g.gave_up == 0u;
-    d.pad = 0;
-    *reinterpret_cast<lbm_diag*>(out) = d;
-  }
-}
 
 cudaError_t launch_diag(const lbm_sim* s, cudaStream_t st) {
-  Grid g = make_grid(s, nullptr, nullptr);
-  k_diag_rows<<<s->ny, DIAG_T, 0, st>>>(s->phys, g, s->fields, s->red);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_diag_final<<<1, DIAG_T, 0, st>>>(g, s->red, s->red + (long long)s->ny * DIAG_PARTIALS, s->steps);
-  return cudaGetLastError();
+  const float* f = s->fields;
+  double* record = s->red + (long long)s->ny * DIAG_PARTIALS;
+  DiagIn d = diag_in(f, f + 2 * s->plane, f + 3 * s->plane, f + 4 * s->plane, s->nx, s->ny, s->pitch, s->phys.phi_star, s->red,
+                     record, diag_done(s), s->steps);
+  d.gave_up = gave_up(s);
+  return launch_diag_rows(d, st);
 }
 
 }  // namespace lbm

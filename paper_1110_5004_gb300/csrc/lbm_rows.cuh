@@ -13,12 +13,10 @@ __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_march(const __grid_con
   extern __shared__ __align__(128) unsigned char smem_raw[];
   MarchSmem<ST, SD>& sm = *reinterpret_cast<MarchSmem<ST, SD>*>(smem_raw);
   march_init(sm);
-  if (MODE == MODE_STEP) {
-    // launched as a programmatic dependent of the previous step: wait until that grid has
-    // completed and its stores are visible, then let the next step's launch proceed
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  }
+  // launched as a programmatic dependent of the previous step: wait until that grid has
+  // completed and its stores are visible, then let the next launch proceed
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   StageAt fat, gat;
   march<MODE, ST, SD, FF, XW>(P, g, mo, blockIdx.x % g.n_strips, blockIdx.x / g.n_strips, sm, fat, gat);
 }
@@ -39,7 +37,7 @@ static cudaError_t launch_march(const Phys2& P, const Grid& g, const MomentOut& 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // consecutive steps overlap their launches
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = MODE == MODE_STEP ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_march<MODE, ST, SD, FF, XW>, P, g, mo);
 }
 

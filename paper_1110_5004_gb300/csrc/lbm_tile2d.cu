@@ -34,8 +34,10 @@ struct Smem2D {
 // population loads through L2 only, for a launch in which other CTAs write the state it reads.
 // XW, YW: walls possible on x, on y; false (a periodic axis) compiles out that axis's wall tests
 // and ghost writes.
-template <int ST, int TX, int TY, int NT, bool COH, bool XW = true, bool YW = true>
-__device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int tiles_x, int tile, Smem2D<TX, TY>& sm) {
+// MOM: only the macroscopic fields, written to `mo` by S2 (which ends the tile).
+template <int ST, int TX, int TY, int NT, bool COH, bool XW = true, bool YW = true, bool MOM = false>
+__device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int tiles_x, int tile, Smem2D<TX, TY>& sm,
+                                            const MomentOut& mo = MomentOut{}) {
   using S = Smem2D<TX, TY>;
   constexpr int FW = S::FW, FH = S::FH;
   const int t = threadIdx.x;
@@ -95,7 +97,7 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
     put(sm.hi, i, j, x, y, hi);
     put(sm.lo, i, j, x, y, lo);
     const int ti = i - 3, tj = j - 3;
-    if (ti >= 0 && ti < TX && tj >= 0 && tj < TY) {
+    if (!MOM && ti >= 0 && ti < TX && tj >= 0 && tj < TY) {
 #pragma unroll
       for (int a = 1; a < Q; ++a) sm.f3[a - 1][tj][ti] = f0raw[c][a];
     }
@@ -115,15 +117,32 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
   for (int c = 0; c < C2; ++c) {
     const int k = t + c * NT, i = 2 + k % (FW - 4), j = 2 + k / (FW - 4), x = x0 - 3 + i, y = y0 - 3 + j;
     if (k >= (FW - 4) * (FH - 4) || !real(x, y)) continue;
+    if (MOM && (i < 3 || i >= TX + 3 || j < 3 || j >= TY + 3 || x >= g.nx || y >= g.ny)) continue;
     const float ph = fadd(sm.hi[j][i], sm.lo[j][i]);
     float gphx, gphy, gmx, gmy;
     grad12(P, &sm.hi[j - 1][i], &sm.hi[j][i], &sm.hi[j + 1][i], gphx, gphy);
     grad12(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i], gmx, gmy);
-    const float sdef = P.remove_Fa ? fmul(P.s_coef6, lap6_of(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i])) : 0.0f;
+    const float s_all = P.remove_Fa || (MOM && mo.fax)
+                            ? fmul(P.s_coef6, lap6_of(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i]))
+                            : 0.0f;
+    const float sdef = P.remove_Fa ? s_all : 0.0f;
     float gb[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) gb[a] = dec_pop<ST>(g2raw[c][a], Q + a);
     const S2Out<float> s2 = s2_cell<ST>(P, ph, gphx, gphy, gmx, gmy, sm.mu[j][i], sdef, gb);
+    if constexpr (MOM) {
+      const int o = y * g.pitch + x;
+      if (mo.phi) mo.phi[o] = ph;
+      if (mo.rho) mo.rho[o] = s2.rho;
+      if (mo.ux) mo.ux[o] = s2.ux;
+      if (mo.uy) mo.uy[o] = s2.uy;
+      if (mo.p) mo.p[o] = s2.p;
+      if (mo.fax) {
+        mo.fax[o] = fmul(-s2.ux, s_all);
+        mo.fay[o] = fmul(-s2.uy, s_all);
+      }
+      continue;
+    }
     put(sm.p, i, j, x, y, s2.p);
     if (P.ch_conv) {
       put(sm.ux, i, j, x, y, s2.ux);
@@ -140,6 +159,7 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
       for (int a = 0; a < Q; ++a) sm.gb[a][tj][ti] = gb[a];
     }
   }
+  if constexpr (MOM) return;
   __syncthreads();
   // ---- S3: collide and store the tile's own cells
   {
@@ -192,6 +212,15 @@ __global__ void __launch_bounds__(NT) k_tile2d(Phys P, Grid g, int tiles_x) {
   tile2d_step<ST, TX, TY, NT, false, XW, YW>(P, g, tiles_x, blockIdx.x, *reinterpret_cast<Smem2D<TX, TY>*>(smem_raw));
 }
 
+// The macroscopic fields of a small grid: S0, S1 and S2 of the same tiles.
+template <int ST, int TX, int TY, int NT, bool XW, bool YW>
+__global__ void __launch_bounds__(NT) k_tile2d_moments(Phys P, Grid g, int tiles_x, MomentOut mo) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  tile2d_step<ST, TX, TY, NT, false, XW, YW, true>(P, g, tiles_x, blockIdx.x, *reinterpret_cast<Smem2D<TX, TY>*>(smem_raw), mo);
+}
+
 // Shared memory to ask for so that at most `cap` CTAs fit on an SM (at least `need`): a grid of
 // few tiles then spreads evenly over the SMs instead of piling several CTAs onto some while
 // others idle.  0 when the device attributes cannot be read.
@@ -219,19 +248,22 @@ static int smem_for_cap(int need, int cap) {
   return want;
 }
 
+// mo: null for a step, else the moment pass.
 template <int ST, int TX, int TY, int NT, bool XW, bool YW>
-static cudaError_t launch_tile2d_shape(const Phys& P, const Grid& g, int sms, cudaStream_t st) {
+static cudaError_t launch_tile2d_shape(const Phys& P, const Grid& g, const MomentOut* mo, int sms, cudaStream_t st) {
   using S = Smem2D<TX, TY>;
-  static bool attr_set = false;   // one GPU per process
-  if (!attr_set) {
+  // set once, thread-safely (one GPU per process)
+  static const cudaError_t attr_set = [] {
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_tile2d<ST, TX, TY, NT, XW, YW>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_tile2d_moments<ST, TX, TY, NT, XW, YW>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    return e;
+  }();
+  if (attr_set != cudaSuccess) return attr_set;
   const int tx = (g.nx + TX - 1) / TX, ty = (g.ny + TY - 1) / TY;
   const int tiles = tx * ty, cap = (tiles + sms - 1) / sms;   // CTAs per SM for one even wave
   cudaLaunchConfig_t cfg = {};
@@ -244,6 +276,7 @@ static cudaError_t launch_tile2d_shape(const Phys& P, const Grid& g, int sms, cu
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (mo) return cudaLaunchKernelEx(&cfg, k_tile2d_moments<ST, TX, TY, NT, XW, YW>, P, g, tx, *mo);
   return cudaLaunchKernelEx(&cfg, k_tile2d<ST, TX, TY, NT, XW, YW>, P, g, tx);
 }
 
@@ -251,10 +284,10 @@ constexpr int T2D_TX = 16, T2D_TY = 8, T2D_NT = 256, T2D_NT_WAVE = 384;
 
 // The wall forms: both axes periodic, walls on y only (the paper's experiments), or general.
 template <int ST, int NT>
-static cudaError_t launch_tile2d_bc(const Phys& P, const Grid& g, int sms, cudaStream_t st) {
-  if (g.bc_x != BC_WALL && g.bc_y != BC_WALL) return launch_tile2d_shape<ST, T2D_TX, T2D_TY, NT, false, false>(P, g, sms, st);
-  if (g.bc_x != BC_WALL) return launch_tile2d_shape<ST, T2D_TX, T2D_TY, NT, false, true>(P, g, sms, st);
-  return launch_tile2d_shape<ST, T2D_TX, T2D_TY, NT, true, true>(P, g, sms, st);
+static cudaError_t launch_tile2d_bc(const Phys& P, const Grid& g, const MomentOut* mo, int sms, cudaStream_t st) {
+  if (g.bc_x != BC_WALL && g.bc_y != BC_WALL) return launch_tile2d_shape<ST, T2D_TX, T2D_TY, NT, false, false>(P, g, mo, sms, st);
+  if (g.bc_x != BC_WALL) return launch_tile2d_shape<ST, T2D_TX, T2D_TY, NT, false, true>(P, g, mo, sms, st);
+  return launch_tile2d_shape<ST, T2D_TX, T2D_TY, NT, true, true>(P, g, mo, sms, st);
 }
 
 // 16 x 8 cells per CTA.  256 threads: every frame cell of S0 in two rounds, one for S1 and S2,
@@ -267,18 +300,18 @@ static cudaError_t launch_tile2d_bc(const Phys& P, const Grid& g, int sms, cudaS
 // CTAs share an SM (smem_for_cap).
 
 template <int ST>
-static cudaError_t launch_tile2d_st(const Phys& P, const Grid& g, int sms, cudaStream_t st) {
-  static int slots = -1;   // CTAs of the 384-thread form resident at once (one GPU per process)
-  if (slots < 0) {
-    int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &occ, k_tile2d<ST, T2D_TX, T2D_TY, T2D_NT_WAVE, true, true>, T2D_NT_WAVE, sizeof(Smem2D<T2D_TX, T2D_TY>));
-    if (e != cudaSuccess) return e;
-    slots = occ * sms;
-  }
+static cudaError_t launch_tile2d_st(const Phys& P, const Grid& g, const MomentOut* mo, int sms, cudaStream_t st) {
+  // CTAs of the 384-thread form resident per SM (one GPU per process; thread-safe)
+  static const int occ = [] {
+    int n = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tile2d<ST, T2D_TX, T2D_TY, T2D_NT_WAVE, true, true>, T2D_NT_WAVE,
+                                                         sizeof(Smem2D<T2D_TX, T2D_TY>)) == cudaSuccess ? n : -1;
+  }();
+  if (occ < 0) return cudaErrorInvalidConfiguration;
+  const int slots = occ * sms;
   const long long tiles = (long long)((g.nx + T2D_TX - 1) / T2D_TX) * ((g.ny + T2D_TY - 1) / T2D_TY);
-  if (tiles <= slots) return launch_tile2d_bc<ST, T2D_NT_WAVE>(P, g, sms, st);
-  return launch_tile2d_bc<ST, T2D_NT>(P, g, sms, st);
+  if (tiles <= slots) return launch_tile2d_bc<ST, T2D_NT_WAVE>(P, g, mo, sms, st);
+  return launch_tile2d_bc<ST, T2D_NT>(P, g, mo, sms, st);
 }
 
 // ---- Resident form: one launch advances n steps.  Every CTA stays on the device and steps its
@@ -495,11 +528,11 @@ cudaError_t launch_resident(lbm_sim* s, const Grid& g, int n) {
   return e;
 }
 
-cudaError_t launch_tile2d(const Phys& P, const Grid& g, int sms, cudaStream_t st) {
+cudaError_t launch_tile2d(const Phys& P, const Grid& g, const MomentOut* mo, int sms, cudaStream_t st) {
   switch (g.storage) {
-    case ST_FP16: return launch_tile2d_st<ST_FP16>(P, g, sms, st);
-    case ST_BF16: return launch_tile2d_st<ST_BF16>(P, g, sms, st);
-    default: return launch_tile2d_st<ST_FP32>(P, g, sms, st);
+    case ST_FP16: return launch_tile2d_st<ST_FP16>(P, g, mo, sms, st);
+    case ST_BF16: return launch_tile2d_st<ST_BF16>(P, g, mo, sms, st);
+    default: return launch_tile2d_st<ST_FP32>(P, g, mo, sms, st);
   }
 }
 
