@@ -196,16 +196,15 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
     delete s;
     return rc;
   }
+  const size_t field_bytes = (size_t)N_FIELDS * s->plane * sizeof(float);
+  const size_t red_bytes = ((size_t)ny * DIAG_PARTIALS + 16) * sizeof(double);
   // Stream-ordered allocations from the device's memory pool, on the simulation's stream: unlike
   // cudaMalloc they do not order the other streams of the device, so a server can create a
   // simulation while others run.  The memory is ordered on s->stream (lbm_set_stream and
   // lbm_batch_add synchronise it before other streams use the state).
   if ((e = cudaMallocAsync(&s->buf[0], s->buf_bytes, s->stream)) != cudaSuccess ||
       (e = cudaMallocAsync(&s->buf[1], s->buf_bytes, s->stream)) != cudaSuccess ||
-      (e = cudaMallocAsync(reinterpret_cast<void**>(&s->fields), (size_t)N_FIELDS * s->plane * sizeof(float),
-                           s->stream)) != cudaSuccess ||
-      (e = cudaMallocAsync(reinterpret_cast<void**>(&s->red), ((size_t)ny * DIAG_PARTIALS + 16) * sizeof(double),
-                           s->stream)) != cudaSuccess ||
+      (e = cudaMallocAsync(reinterpret_cast<void**>(&s->fields), field_bytes + red_bytes, s->stream)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&s->uploaded, cudaEventDisableTiming)) != cudaSuccess) {
     rc = cuda_fail(e, "lbm_create allocation");
     lbm_destroy(s);
@@ -214,8 +213,8 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
   // zero the pad columns once so no uninitialised memory is ever read back
   cudaMemsetAsync(s->buf[0], 0, s->buf_bytes, s->stream);
   cudaMemsetAsync(s->buf[1], 0, s->buf_bytes, s->stream);
-  cudaMemsetAsync(s->fields, 0, (size_t)N_FIELDS * s->plane * sizeof(float), s->stream);
-  cudaMemsetAsync(s->red + (size_t)ny * DIAG_PARTIALS, 0, 16 * sizeof(double), s->stream);
+  s->red = reinterpret_cast<double*>(s->fields + (size_t)N_FIELDS * s->plane);   // behind the work planes
+  cudaMemsetAsync(s->fields, 0, field_bytes + red_bytes, s->stream);
   if ((e = cudaGetLastError()) != cudaSuccess) {
     rc = cuda_fail(e, "lbm_create memset");
     lbm_destroy(s);
@@ -487,8 +486,7 @@ int lbm_destroy(lbm_sim* s) {
   if (!s) return LBM_OK;
   if (s->stream || s->buf[0]) cudaStreamSynchronize(s->stream);
   // back to the pool, ordered on the stream: no device-wide synchronisation
-  for (void* p : {s->buf[0], s->buf[1], static_cast<void*>(s->fields), static_cast<void*>(s->red),
-                  static_cast<void*>(s->res_mem)})
+  for (void* p : {s->buf[0], s->buf[1], static_cast<void*>(s->fields), static_cast<void*>(s->res_mem)})
     if (p) cudaFreeAsync(p, s->stream);
   if (s->uploaded) cudaEventDestroy(s->uploaded);
   delete s;

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* _
     g.src = odd ? d.buf1 : d.buf0;
     g.dst = odd ? const_cast<void*>(d.buf0) : d.buf1;
     __syncthreads();
-    march<MODE_STEP, ST, SD, false, XW>(sm.P, g, MomentOut{}, it.y, it.z, sm.m, fat, gat);
+    march<MODE_STEP, ST, SD, false, XW, false>(sm.P, g, MomentOut{}, it.y, it.z, sm.m, fat, gat);
   }
 }
 

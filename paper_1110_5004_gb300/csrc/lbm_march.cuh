@@ -230,7 +230,8 @@ struct StageAt {
 // SD: the direct mass defect (s_form 1) is compiled in.  FF: the forced order-parameter LBE (f_form 1;
 // FP32 storage only).  XW: the x axis may have walls.  K: the scheme constants (Phys2, in the constant bank
 // or in shared memory).
-template <int MODE, int ST, bool SD, bool FF, bool XW, class K>
+// PDL: the launch is a programmatic dependent of the previous one and waits for it here, once its addresses are formed.
+template <int MODE, int ST, bool SD, bool FF, bool XW, bool PDL, class K>
 __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut& mo, int strip, int seg, MarchSmem<ST, SD>& sm,
                                       StageAt& fat, StageAt& gat) {
   constexpr int NT = MARCH_NT;
@@ -299,6 +300,11 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
   // S2 runs in iterations ya + 2 .. a_end (rows ya - 1 ..), S3 in ya + 4 .. yb + 3; the moment pass ends
   // with S2 of row yb - 1.
   const int a_end = MODE == MODE_STEP ? yb + 3 : yb + 2;
+  if constexpr (PDL) {
+    // until the previous grid has completed and its stores are visible; then let the next launch proceed
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   for (int k = 0; k < STAGES; ++k)
     produce(true, ya - 3 + k, fat.ahead(k), ya - 1 + k <= a_end - 3, ya - 1 + k, gat.ahead(k));
 

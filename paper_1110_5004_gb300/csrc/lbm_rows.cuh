@@ -13,12 +13,8 @@ __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_march(const __grid_con
   extern __shared__ __align__(128) unsigned char smem_raw[];
   MarchSmem<ST, SD>& sm = *reinterpret_cast<MarchSmem<ST, SD>*>(smem_raw);
   march_init(sm);
-  // launched as a programmatic dependent of the previous step: wait until that grid has
-  // completed and its stores are visible, then let the next launch proceed
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   StageAt fat, gat;
-  march<MODE, ST, SD, FF, XW>(P, g, mo, blockIdx.x % g.n_strips, blockIdx.x / g.n_strips, sm, fat, gat);
+  march<MODE, ST, SD, FF, XW, true>(P, g, mo, blockIdx.x % g.n_strips, blockIdx.x / g.n_strips, sm, fat, gat);
 }
 
 template <int MODE, int ST, bool SD, bool FF, bool XW>

@@ -65,21 +65,44 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
   // to thread k + TX * TY, so the longest stage runs at half the chain.
   static_assert(NT >= 2 * TX * TY, "S3 needs two threads per tile cell");
   unsigned int f0raw[C0][NF], g2raw[C2][Q];
+  // The addresses of these loads are formed before the launch waits for the previous step, while that is still
+  // running: the step of a 128 x 128 grid, whose length is the latency of one tile, 3.12 -> 2.49 us.
+  Col3 fcol[C0], gcol[C2];
+  int frow[C0], grow[C2];
+#pragma unroll
+  for (int c = 0; c < C0; ++c) {
+    const int k = t + c * NT, i = k % FW, j = k / FW;
+    fcol[c] = col3<ST>(wrap1(x0 - 3 + i, g.nx), g.nx);
+    frow[c] = wrap1(y0 - 3 + j, g.ny) * g.row_bytes;
+    asm volatile("" ::"r"(fcol[c].cm.f4), "r"(fcol[c].c0.f4), "r"(fcol[c].cq.f4), "r"(fcol[c].c0.l), "r"(frow[c]));
+  }
+#pragma unroll
+  for (int c = 0; c < C2; ++c) {
+    const int k = t + c * NT, i = 2 + k % (FW - 4), j = 2 + k / (FW - 4);
+    gcol[c] = col3<ST>(wrap1(x0 - 3 + i, g.nx), g.nx);
+    grow[c] = wrap1(y0 - 3 + j, g.ny) * g.row_bytes;
+    asm volatile("" ::"r"(gcol[c].cm.g), "r"(gcol[c].c0.g), "r"(gcol[c].cq.g), "r"(grow[c]));
+  }
+  if constexpr (!COH) {
+    // Launched as a programmatic dependent of the previous step: wait until that grid has
+    // completed and its stores are visible, then let the next step's grid be scheduled, so that
+    // its launch overlaps this one instead of following it.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
 #pragma unroll
   for (int c = 0; c < C0; ++c) {
     const int k = t + c * NT, i = k % FW, j = k / FW, x = x0 - 3 + i, y = y0 - 3 + j;
     if (k < FW * FH && real(x, y)) {
-      const Col3 cn = col3<ST>(wrap1(x, g.nx), g.nx);
-      const int row = wrap1(y, g.ny) * g.row_bytes;
-      gather9<ST, 0, COH>(g, cn, row, f0raw[c]);
-      f0raw[c][Q] = ST == ST_FP32 ? ld_raw<ST, COH>(g.src, A_F0LO, pop_at<ST>(A_F0LO, row, cn.c0, g)) : 0u;
+      gather9<ST, 0, COH>(g, fcol[c], frow[c], f0raw[c]);
+      f0raw[c][Q] = ST == ST_FP32 ? ld_raw<ST, COH>(g.src, A_F0LO, pop_at<ST>(A_F0LO, frow[c], fcol[c].c0, g)) : 0u;
     }
   }
 #pragma unroll
   for (int c = 0; c < C2; ++c) {
     const int k = t + c * NT, i = 2 + k % (FW - 4), j = 2 + k / (FW - 4), x = x0 - 3 + i, y = y0 - 3 + j;
     if (k < (FW - 4) * (FH - 4) && real(x, y)) {
-      gather9<ST, Q, COH>(g, col3<ST>(wrap1(x, g.nx), g.nx), wrap1(y, g.ny) * g.row_bytes, g2raw[c]);
+      gather9<ST, Q, COH>(g, gcol[c], grow[c], g2raw[c]);
     }
   }
 
@@ -204,20 +227,193 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
 template <int ST, int TX, int TY, int NT, bool XW, bool YW>
 __global__ void __launch_bounds__(NT) k_tile2d(Phys P, Grid g, int tiles_x) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // Launched as a programmatic dependent of the previous step: wait until that grid has
-  // completed and its stores are visible, then let the next step's grid be scheduled, so that
-  // its launch overlaps this one instead of following it.
+  tile2d_step<ST, TX, TY, NT, false, XW, YW>(P, g, tiles_x, blockIdx.x, *reinterpret_cast<Smem2D<TX, TY>*>(smem_raw));
+}
+
+// ---- Two tiles per CTA, side by side in x, each value the pair of the two tiles' cells (V2): the same four passes
+// with packed arithmetic and one shared-memory access for both.  For a periodic x axis.
+template <int TX, int TY>
+struct SmemPair {
+  static constexpr int FW = TX + 6, FH = TY + 6;
+  V2 hi[FH][FW], lo[FH][FW], mu[FH][FW], p[FH][FW], ux[FH][FW], uy[FH][FW];
+  V2 rec[10][TY][TX];
+  V2 gb[Q][TY][TX];
+  V2 f3[Q - 1][TY][TX];
+};
+
+template <int ST, bool YW>
+struct OutPair {
+  OutCell<ST, false, YW> a, b;
+  bool on_a, on_b;
+  template <int A>
+  __device__ __forceinline__ void put(V2 v) const {
+    float x, y;
+    unpack2(v, x, y);
+    if (on_a) a.template put<A>(x);
+    if (on_b) b.template put<A>(y);
+  }
+};
+
+template <int ST, int TX, int TY, int NT, int CTAS, bool YW>
+__global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant__ Phys2 P, const __grid_constant__ Grid g, int pairs_x) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  using S = SmemPair<TX, TY>;
+  S& sm = *reinterpret_cast<S*>(smem_raw);
+  constexpr int FW = S::FW, FH = S::FH;
+  const int t = threadIdx.x;
+  const int x0 = (blockIdx.x % pairs_x) * 2 * TX, y0 = (blockIdx.x / pairs_x) * TY;
+  const bool ywall = YW && g.bc_y == BC_WALL;
+  // the grid is at least a tile and its halo wide and high: one period is enough to wrap
+  auto near = [](int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); };
+  auto real = [&](int y) { return !ywall || (y >= 0 && y < g.ny); };
+  // store at (i, j) and, for a cell next to a wall, at its mirror image beyond it
+  auto put = [&](V2 (*f)[FW], int i, int j, int y, V2 v) {
+    f[j][i] = v;
+    const int gj = ywall ? (y == 0 ? j - 1 : (y == g.ny - 1 ? j + 1 : -1)) : -1;
+    if (gj >= 0 && gj < FH) f[gj][i] = v;
+  };
+  constexpr int C0 = (FW * FH + NT - 1) / NT, C2 = ((FW - 4) * (FH - 4) + NT - 1) / NT;
+  static_assert(NT >= 2 * TX * TY, "S3 needs two threads per pair of cells");
+  Col3 fa[C0], fb[C0], ga[C2], gbc[C2];
+  int frow[C0], grow[C2];
+#pragma unroll
+  for (int c = 0; c < C0; ++c) {
+    const int k = t + c * NT, i = k % FW, j = k / FW;
+    fa[c] = col3<ST>(near(x0 - 3 + i, g.nx), g.nx);
+    fb[c] = col3<ST>(near(x0 - 3 + i + TX, g.nx), g.nx);
+    frow[c] = near(y0 - 3 + j, g.ny) * g.row_bytes;
+  }
+#pragma unroll
+  for (int c = 0; c < C2; ++c) {
+    const int k = t + c * NT, i = 2 + k % (FW - 4), j = 2 + k / (FW - 4);
+    ga[c] = col3<ST>(near(x0 - 3 + i, g.nx), g.nx);
+    gbc[c] = col3<ST>(near(x0 - 3 + i + TX, g.nx), g.nx);
+    grow[c] = near(y0 - 3 + j, g.ny) * g.row_bytes;
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  tile2d_step<ST, TX, TY, NT, false, XW, YW>(P, g, tiles_x, blockIdx.x, *reinterpret_cast<Smem2D<TX, TY>*>(smem_raw));
+  unsigned int fr[C0][2][NF], gr[C2][2][Q];
+#pragma unroll
+  for (int c = 0; c < C0; ++c) {
+    const int k = t + c * NT, j = k / FW;
+    if (k < FW * FH && real(y0 - 3 + j)) {
+      gather9<ST, 0>(g, fa[c], frow[c], fr[c][0]);
+      gather9<ST, 0>(g, fb[c], frow[c], fr[c][1]);
+      fr[c][0][Q] = ST == ST_FP32 ? ld_raw<ST>(g.src, A_F0LO, pop_at<ST>(A_F0LO, frow[c], fa[c].c0, g)) : 0u;
+      fr[c][1][Q] = ST == ST_FP32 ? ld_raw<ST>(g.src, A_F0LO, pop_at<ST>(A_F0LO, frow[c], fb[c].c0, g)) : 0u;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < C2; ++c) {
+    const int k = t + c * NT, j = 2 + k / (FW - 4);
+    if (k < (FW - 4) * (FH - 4) && real(y0 - 3 + j)) {
+      gather9<ST, Q>(g, ga[c], grow[c], gr[c][0]);
+      gather9<ST, Q>(g, gbc[c], grow[c], gr[c][1]);
+    }
+  }
+  // ---- S0
+#pragma unroll
+  for (int c = 0; c < C0; ++c) {
+    const int k = t + c * NT, i = k % FW, j = k / FW, y = y0 - 3 + j;
+    if (k >= FW * FH || !real(y)) continue;
+    V2 fp[NF], hi, lo;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) fp[a] = pack2(dec_pop<ST>(fr[c][0][a], a), dec_pop<ST>(fr[c][1][a], a));
+    fp[Q] = pack2(__uint_as_float(fr[c][0][Q]), __uint_as_float(fr[c][1][Q]));
+    phi_pair<ST>(P, fp, hi, lo);
+    put(sm.hi, i, j, y, hi);
+    put(sm.lo, i, j, y, lo);
+    const int ti = i - 3, tj = j - 3;
+    if (ti >= 0 && ti < TX && tj >= 0 && tj < TY) {
+#pragma unroll
+      for (int a = 1; a < Q; ++a) sm.f3[a - 1][tj][ti] = fp[a];
+    }
+  }
+  __syncthreads();
+  // ---- S1
+  for (int k = t; k < (FW - 2) * (FH - 2); k += NT) {
+    const int i = 1 + k % (FW - 2), j = 1 + k / (FW - 2), y = y0 - 3 + j;
+    if (!real(y)) continue;
+    put(sm.mu, i, j, y,
+        chem_potential(P, &sm.hi[j - 1][i], &sm.hi[j][i], &sm.hi[j + 1][i], &sm.lo[j - 1][i], &sm.lo[j][i], &sm.lo[j + 1][i]));
+  }
+  __syncthreads();
+  // ---- S2
+#pragma unroll
+  for (int c = 0; c < C2; ++c) {
+    const int k = t + c * NT, i = 2 + k % (FW - 4), j = 2 + k / (FW - 4), y = y0 - 3 + j;
+    if (k >= (FW - 4) * (FH - 4) || !real(y)) continue;
+    const V2 ph = fadd(sm.hi[j][i], sm.lo[j][i]);
+    V2 gphx, gphy, gmx, gmy;
+    grad12(P, &sm.hi[j - 1][i], &sm.hi[j][i], &sm.hi[j + 1][i], gphx, gphy);
+    grad12(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i], gmx, gmy);
+    const V2 sdef = P.remove_Fa ? fmul(P.s_coef6, lap6_of(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i])) : zero<V2>();
+    V2 gv[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) gv[a] = pack2(dec_pop<ST>(gr[c][0][a], Q + a), dec_pop<ST>(gr[c][1][a], Q + a));
+    const S2Out<V2> s2 = s2_cell<ST>(P, ph, gphx, gphy, gmx, gmy, sm.mu[j][i], sdef, gv);
+    put(sm.p, i, j, y, s2.p);
+    if (P.ch_conv) {
+      put(sm.ux, i, j, y, s2.ux);
+      put(sm.uy, i, j, y, s2.uy);
+    }
+    const int ti = i - 3, tj = j - 3;
+    if (ti >= 0 && ti < TX && tj >= 0 && tj < TY) {
+      RecT<V2> r{};
+      s2_record(P, s2, ph, sm.mu[j][i], sdef, r);
+      const V2 v[10] = {r.phi, r.mu, r.ux, r.uy, r.Fx, r.Fy, r.mrx3, r.mry3, r.og, r.ogr3};
+#pragma unroll
+      for (int q = 0; q < 10; ++q) sm.rec[q][tj][ti] = v[q];
+#pragma unroll
+      for (int a = 0; a < Q; ++a) sm.gb[a][tj][ti] = gv[a];
+    }
+  }
+  __syncthreads();
+  // ---- S3: the f and the gbar collision of a pair of cells by two threads
+  {
+    const int k = t % (TX * TY), ti = k % TX, tj = k / TX, i = ti + 3, j = tj + 3, xa = x0 + ti, xb = xa + TX, y = y0 + tj;
+    if (t < 2 * TX * TY && xa < g.nx && y < g.ny) {
+      RecT<V2> r{};
+      r.phi = sm.rec[0][tj][ti];
+      r.mu = sm.rec[1][tj][ti];
+      r.ux = sm.rec[2][tj][ti];
+      r.uy = sm.rec[3][tj][ti];
+      r.Fx = sm.rec[4][tj][ti];
+      r.Fy = sm.rec[5][tj][ti];
+      r.mrx3 = sm.rec[6][tj][ti];
+      r.mry3 = sm.rec[7][tj][ti];
+      r.og = sm.rec[8][tj][ti];
+      r.ogr3 = sm.rec[9][tj][ti];
+      const OutPair<ST, YW> out{out_cell<ST, false, YW>(g, xa, y), out_cell<ST, false, YW>(g, xb < g.nx ? xb : xa, y), true, xb < g.nx};
+      const V2 z = zero<V2>();
+      V2 f[Q], gv[Q];
+      if (t < TX * TY) {
+        const V2 phiD = P.ch_conv ? phi_div_u(P, r.phi, &sm.ux[j - 1][i], &sm.ux[j][i], &sm.ux[j + 1][i], &sm.uy[j - 1][i],
+                                              &sm.uy[j + 1][i])
+                                  : z;
+        f[0] = z;
+#pragma unroll
+        for (int a = 1; a < Q; ++a) f[a] = sm.f3[a - 1][tj][ti];
+#pragma unroll
+        for (int a = 0; a < Q; ++a) gv[a] = z;
+        collide_store<ST, false, COLLIDE_F>(P, r, z, z, z, sm.hi[j][i], sm.lo[j][i], phiD, f, gv, out);
+      } else {
+        V2 gpx, gpy;
+        grad12(P, &sm.p[j - 1][i], &sm.p[j][i], &sm.p[j + 1][i], gpx, gpy);
+#pragma unroll
+        for (int a = 0; a < Q; ++a) f[a] = z;
+#pragma unroll
+        for (int a = 0; a < Q; ++a) gv[a] = sm.gb[a][tj][ti];
+        collide_store<ST, false, COLLIDE_G>(P, r, sm.p[j][i], gpx, gpy, z, z, z, f, gv, out);
+      }
+    }
+  }
 }
 
 // The macroscopic fields of a small grid: S0, S1 and S2 of the same tiles.
 template <int ST, int TX, int TY, int NT, bool XW, bool YW>
 __global__ void __launch_bounds__(NT) k_tile2d_moments(Phys P, Grid g, int tiles_x, MomentOut mo) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   tile2d_step<ST, TX, TY, NT, false, XW, YW, true>(P, g, tiles_x, blockIdx.x, *reinterpret_cast<Smem2D<TX, TY>*>(smem_raw), mo);
 }
 
@@ -290,6 +486,26 @@ static cudaError_t launch_tile2d_bc(const Phys& P, const Grid& g, const MomentOu
   return launch_tile2d_shape<ST, T2D_TX, T2D_TY, NT, true, true>(P, g, mo, sms, st);
 }
 
+template <int ST, int NT, int CTAS, bool YW>
+static cudaError_t launch_tile2d_pair_t(const Phys2& P, const Grid& g, cudaStream_t st) {
+  using S = SmemPair<T2D_TX, T2D_TY>;
+  static const cudaError_t attr_set =
+      cudaFuncSetAttribute(k_tile2d_pair<ST, T2D_TX, T2D_TY, NT, CTAS, YW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(S));
+  if (attr_set != cudaSuccess) return attr_set;
+  const int px = (g.nx + 2 * T2D_TX - 1) / (2 * T2D_TX), ty = (g.ny + T2D_TY - 1) / T2D_TY;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(px * ty);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = sizeof(S);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_tile2d_pair<ST, T2D_TX, T2D_TY, NT, CTAS, YW>, P, g, px);
+}
+
 // 16 x 8 cells per CTA.  256 threads: every frame cell of S0 in two rounds, one for S1 and S2,
 // and the collisions split between the f and gbar threads.  Measured against 16 x 8 / 128
 // threads, 16 x 4 / 256, 8 x 8 / 64, 128 and 256, 16 x 16 / 256, 32 x 4 / 256 and 32 x 8 / 256
@@ -310,6 +526,19 @@ static cudaError_t launch_tile2d_st(const Phys& P, const Grid& g, const MomentOu
   if (occ < 0) return cudaErrorInvalidConfiguration;
   const int slots = occ * sms;
   const long long tiles = (long long)((g.nx + T2D_TX - 1) / T2D_TX) * ((g.ny + T2D_TY - 1) / T2D_TY);
+  // Beyond one wave of single tiles, and where x is periodic, two tiles per CTA: 320 threads and 2 CTAs per SM while
+  // the pairs fit one such wave, else 256 threads and 3 CTAs.  Single tiles -> pairs, us per step: 256^2 (256 pairs)
+  // 5.27 -> 4.91, 150 x 450 (285) 5.54 -> 5.08, 320^2 (400) 7.87 -> 6.65, 384^2 (576) 9.58 -> 9.04, 256 x 1024 (1024)
+  // 15.5 -> 13.9.  A little over one wave of 3 per SM (512 pairs: 256 x 512 8.70 -> 8.94) they stay single.
+  const long long pairs = (long long)((g.nx + 2 * T2D_TX - 1) / (2 * T2D_TX)) * ((g.ny + T2D_TY - 1) / T2D_TY);
+  const bool tail = pairs > 3LL * sms && 2 * pairs <= 7LL * sms;
+  if (!mo && tiles > slots && !tail && g.bc_x != BC_WALL && g.nx >= 2 * T2D_TX + 6 && g.ny >= T2D_TY + 6) {
+    const Phys2 P2 = widen(P);
+    const bool yw = g.bc_y == BC_WALL;
+    if (pairs <= 2LL * sms)
+      return yw ? launch_tile2d_pair_t<ST, 320, 2, true>(P2, g, st) : launch_tile2d_pair_t<ST, 320, 2, false>(P2, g, st);
+    return yw ? launch_tile2d_pair_t<ST, 256, 3, true>(P2, g, st) : launch_tile2d_pair_t<ST, 256, 3, false>(P2, g, st);
+  }
   if (tiles <= slots) return launch_tile2d_bc<ST, T2D_NT_WAVE>(P, g, mo, sms, st);
   return launch_tile2d_bc<ST, T2D_NT>(P, g, mo, sms, st);
 }
