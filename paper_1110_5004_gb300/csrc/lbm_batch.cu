@@ -5,6 +5,7 @@
 // launches.  Each tile runs the row march of the single-simulation kernel (every operation rounded to
 // nearest explicitly), so a member's state is bitwise the same alone or inside any mix.
 #include <algorithm>
+#include <array>
 #include <map>
 #include <new>
 #include <vector>
@@ -23,7 +24,7 @@ struct lbm_batch {
   cudaStream_t stream = nullptr;
   cudaStream_t cap = nullptr;          // private stream for graph capture
   std::vector<lbm_sim*> slots;         // nullptr = free slot
-  int seg_h = 32;                      // rows per tile for members without their own choice
+  int seg_h = 0;                       // rows per tile for members without their own choice (0: chosen here)
   bool dirty = true;                   // descriptors / work list need rebuilding
   SimDesc* d_sims = nullptr;
   int4* d_work = nullptr;
@@ -57,19 +58,44 @@ static int rebuild(lbm_batch* b) {
   b->xwall = false;
   for (int m : members) b->xwall = b->xwall || b->slots[m]->params.bc_x == LBM_WALL;
   const int slots = sms * MARCH_CTAS;
+  auto part_of = [](const lbm_sim* s) { return s->params.storage + (s->params.s_form ? 3 : 0); };
+  // Rows per tile.  A launch takes as many rounds as its tiles fill of the device's slots, and a round as many row
+  // iterations as its tiles have: the height that makes rounds x (h + 7) least, heights evened out within each member
+  // (48 members of the c4 mix: 2 full rounds instead of 3.5, taken as 4, at a fixed 32 rows).
+  int rows[N_PARTS];
+  for (int part = 0; part < N_PARTS; ++part) {
+    std::vector<std::array<int, 3>> shape;   // strips, rows, own rows per tile
+    for (int m : members) {
+      const lbm_sim* s = b->slots[m];
+      if (part_of(s) != part) continue;
+      int tw, ns, hh;
+      tile_geometry(s->nx, s->ny, s->params.s_form != 0, 1, 0, &tw, &ns, &hh);
+      shape.push_back({ns, s->ny, s->seg_h ? s->seg_h : b->seg_h});
+    }
+    long long best = -1;
+    rows[part] = 32;
+    for (int h = 4; h <= 512 && !shape.empty(); h += h < 64 ? 1 : h / 16) {
+      long long tiles = 0;
+      for (const auto& q : shape) {
+        const int hh = q[2] ? q[2] : h;
+        tiles += (long long)q[0] * ((q[1] + hh - 1) / hh);
+      }
+      const long long cost = (tiles + slots - 1) / slots * (h + 7);
+      if (best < 0 || cost < best) {
+        best = cost;
+        rows[part] = h;
+      }
+    }
+  }
   for (size_t m = 0; m < members.size(); ++m) {
     lbm_sim* s = b->slots[members[m]];
     SimDesc d{};
     d.P = s->phys2;
     Grid g = make_grid(s, nullptr, nullptr);
-    // one wave of the batch kernel is shared by all members: size segments for the batch.  A
-    // member large enough to fill the wave on its own gets segments of the height that does so
-    // (as a simulation stepped alone): fewer, taller tiles cut its pipeline-fill rows.
     int h = s->seg_h ? s->seg_h : b->seg_h;
-    if (!s->seg_h) {
-      int tw = 0, ns = 0, hw = 0;
-      tile_geometry(s->nx, s->ny, s->params.s_form != 0, 0, slots, &tw, &ns, &hw);
-      h = std::max(h, hw);
+    if (!h) {
+      const int segs = (s->ny + rows[part_of(s)] - 1) / rows[part_of(s)];
+      h = (s->ny + segs - 1) / segs;
     }
     tile_geometry(s->nx, s->ny, s->params.s_form != 0, h, 0, &g.tile_w, &g.n_strips, &g.seg_h);
     d.g = g;
@@ -81,7 +107,7 @@ static int rebuild(lbm_batch* b) {
     const int nseg = (s->ny + g.seg_h - 1) / g.seg_h;
     for (int sg = 0; sg < nseg; ++sg)
       for (int st = 0; st < g.n_strips; ++st) tl.push_back(make_int4((int)m, st, sg, 0));
-    per[s->params.storage + (d.P.s_direct ? 3 : 0)].push_back(std::move(tl));
+    per[part_of(s)].push_back(std::move(tl));
   }
   lbm_batch::Part parts[N_PARTS];
   for (int part = 0; part < N_PARTS; ++part) {

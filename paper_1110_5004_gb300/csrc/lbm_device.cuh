@@ -363,15 +363,16 @@ __device__ __forceinline__ V from_scale(const K& P, V v) {
 // keeps it within 0.05 %; the f populations round to nearest (rounding them stochastically as well
 // gained nothing, and rounding only them left the 3.6 %).
 // The offset is a hash of the value's own bits and its place, so every kernel rounds a
-// given value at a given place alike and runs stay deterministic.  NaN and infinity keep
-// round-to-nearest, so a diverged state stays non-finite.
+// given value at a given place alike and runs stay deterministic.  NaN and infinity stay NaN and infinity, so a
+// diverged state stays non-finite.
 __device__ __forceinline__ unsigned short bf16_stochastic(float v, unsigned int where) {
   const unsigned int bits = __float_as_uint(v);
   // the high half of a product with an odd constant depends on every bit of the other factor
   const unsigned int offset = ((bits ^ where) * 0x9e3779b1u) >> 16;
-  const unsigned int rounded = (bits + offset) >> 16;
-  const bool special = (bits & 0x7f800000u) == 0x7f800000u;
-  return special ? __bfloat16_as_ushort(__float2bfloat16_rn(v)) : static_cast<unsigned short>(rounded);
+  // the magnitude saturates at the largest NaN, so that no carry reaches the sign; infinities and the NaN that
+  // arithmetic produces (all bits set) stay what they are
+  const unsigned int mag = min((bits & 0x7fffffffu) + offset, 0x7fffffffu);
+  return static_cast<unsigned short>((mag | (bits & 0x80000000u)) >> 16);
 }
 // 16-bit encoding of population a (already in storage scale).
 template <int ST>
