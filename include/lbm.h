@@ -159,7 +159,8 @@ LBM_API int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stre
 
 /* Set the state at t = 0 from phi0, ux0, uy0, p0 (nx*ny float32 each, host or device; ux0,
  * uy0 and p0 may be NULL for zero): f = f^eq(phi0, mu0, u0), gbar = g^eq(p0, rho0, u0).
- * Asynchronous for device inputs; host inputs are copied before return, and the initialisation
+ * Asynchronous for device inputs, which the kernel reads in place (they must stay as they are until it has
+ * run on the stream); host inputs are copied before return, and the initialisation
  * kernels stay queued on the simulation's stream behind those copies. */
 LBM_API int lbm_init_fields(lbm_sim* sim, const float* phi0, const float* ux0, const float* uy0,
                     const float* p0);
@@ -168,8 +169,8 @@ LBM_API int lbm_init_fields(lbm_sim* sim, const float* phi0, const float* ux0, c
 LBM_API int lbm_step(lbm_sim* sim, int n);
 
 /* Macroscopic fields of the current state (phi, rho, ux, uy, p; any pointer may be NULL),
- * row-major nx*ny float32 each, host or device.  Synchronises the stream.  When nx is a multiple
- * of 32, device outputs are written by the moment kernel itself; the others are copied from the
+ * row-major nx*ny float32 each, host or device.  Synchronises the stream.  Outputs that are all in memory of
+ * the simulation's device are written by the moment kernel itself; else they are copied from the
  * simulation's work planes. */
 LBM_API int lbm_moments(lbm_sim* sim, float* phi, float* rho, float* ux, float* uy, float* p);
 

@@ -240,28 +240,48 @@ static cudaError_t rearm_resident(lbm_sim* s) {
   return resident_reset(s);
 }
 
-static int upload_field(lbm_sim* s, int k, const float* src) {
-  float* dst = s->fields + (long long)k * s->plane;
-  cudaError_t e;
-  if (!src) {
-    e = cudaMemsetAsync(dst, 0, (size_t)s->plane * sizeof(float), s->stream);
-  } else {
-    const cudaMemcpyKind kind = is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    e = copy_field(s, dst, (size_t)s->pitch * sizeof(float), src, (size_t)s->nx * sizeof(float), kind);
+// Device memory that this simulation's kernels can address as floats: on the current device or managed, and aligned.
+static bool addressable(const void* p) {
+  cudaPointerAttributes a;
+  int dev = 0;
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(float) != 0) return false;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
   }
-  return e == cudaSuccess ? LBM_OK : cuda_fail(e, "lbm_init_fields upload");
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+}
+
+// Initial field k (0 phi0, 1 ux0, 2 uy0, 3 p0): read in place by the initialisation kernel where it can address the
+// memory (copying device fields into work planes first took a third of its traffic), else through its work plane.
+static int take_field(lbm_sim* s, int k, const float* src, InitIn* in, bool* host) {
+  in->f[k] = src;
+  in->pitch[k] = s->nx;
+  if (!src || addressable(src)) return LBM_OK;
+  const int plane = k == 0 ? 0 : k + 1;
+  float* dst = s->fields + (long long)plane * s->plane;
+  const bool dev = is_device_ptr(src);
+  const cudaError_t e = copy_field(s, dst, (size_t)s->pitch * sizeof(float), src, (size_t)s->nx * sizeof(float),
+                                   dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return cuda_fail(e, "lbm_init_fields upload");
+  in->f[k] = dst;
+  in->pitch[k] = s->pitch;
+  *host = *host || !dev;
+  return LBM_OK;
 }
 
 int lbm_init_fields(lbm_sim* s, const float* phi0, const float* ux0, const float* uy0, const float* p0) {
   Range range_("lbm_init_fields");
   if (!s || !phi0) return set_error("sim and phi0 are required"), LBM_ERR_INVALID_ARG;
   int rc;
-  if ((rc = upload_field(s, 0, phi0)) || (rc = upload_field(s, 2, ux0)) || (rc = upload_field(s, 3, uy0)) ||
-      (rc = upload_field(s, 4, p0)))
+  InitIn in{};
+  bool host_input = false;
+  if ((rc = take_field(s, 0, phi0, &in, &host_input)) || (rc = take_field(s, 1, ux0, &in, &host_input)) ||
+      (rc = take_field(s, 2, uy0, &in, &host_input)) || (rc = take_field(s, 3, p0, &in, &host_input)))
     return rc;
-  cudaError_t e = cudaEventRecord(s->uploaded, s->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "lbm_init_fields record");
-  e = launch_init(s, s->stream);
+  cudaError_t e = cudaSuccess;
+  if (host_input && (e = cudaEventRecord(s->uploaded, s->stream)) != cudaSuccess) return cuda_fail(e, "lbm_init_fields record");
+  e = launch_init(s, in, s->stream);
   if (e == cudaSuccess) e = rearm_resident(s);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_init_fields launch");
   s->launches += s->params.s_form ? 2 : 1;
@@ -269,8 +289,6 @@ int lbm_init_fields(lbm_sim* s, const float* phi0, const float* ux0, const float
   // host inputs must be consumed before return (pageable copies already are; pinned ones not):
   // wait for the copies only, so the initialisation kernels overlap the caller's next launches.
   // Any one host input is enough to wait: phi0 may be on the device while ux0 is pinned.
-  bool host_input = false;
-  for (const float* in : {phi0, ux0, uy0, p0}) host_input = host_input || (in && !is_device_ptr(in));
   if (host_input && (e = cudaEventSynchronize(s->uploaded)) != cudaSuccess)
     return cuda_fail(e, "lbm_init_fields sync");
   return LBM_OK;
@@ -294,16 +312,28 @@ static cudaError_t copy_planes(const lbm_sim* s, int k0, int nplanes, float* pac
 int lbm_init_fields_packed(lbm_sim* s, const float* fields) {
   Range range_("lbm_init_fields_packed");
   if (!s || !fields) return set_error("sim and fields are required"), LBM_ERR_INVALID_ARG;
-  const bool host = !is_device_ptr(fields);
-  const cudaMemcpyKind kind = host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   const size_t n = (size_t)s->nx * s->ny;
-  float* in = const_cast<float*>(fields);   // read only: copied into the work planes
-  // phi0 -> work plane 0; ux0, uy0, p0 -> work planes 2, 3, 4 (consecutive)
-  cudaError_t e = copy_planes(s, 0, 1, in, true, kind);
-  if (e == cudaSuccess) e = copy_planes(s, 2, 3, in + n, true, kind);
-  if (e == cudaSuccess) e = cudaEventRecord(s->uploaded, s->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "lbm_init_fields_packed upload");
-  e = launch_init(s, s->stream);
+  InitIn in{};
+  bool host = false;
+  cudaError_t e = cudaSuccess;
+  if (addressable(fields)) {
+    for (int k = 0; k < 4; ++k) {
+      in.f[k] = fields + k * n;
+      in.pitch[k] = s->nx;
+    }
+  } else {
+    host = !is_device_ptr(fields);
+    const cudaMemcpyKind kind = host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+    // one copy into consecutive work planes
+    e = copy_planes(s, 0, 4, const_cast<float*>(fields), true, kind);   // (read only)
+    if (e == cudaSuccess && host) e = cudaEventRecord(s->uploaded, s->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "lbm_init_fields_packed upload");
+    for (int k = 0; k < 4; ++k) {
+      in.f[k] = s->fields + (long long)k * s->plane;
+      in.pitch[k] = s->pitch;
+    }
+  }
+  e = launch_init(s, in, s->stream);
   if (e == cudaSuccess) e = rearm_resident(s);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_init_fields_packed launch");
   s->launches += s->params.s_form ? 2 : 1;
@@ -369,7 +399,7 @@ static cudaError_t moments_of(const lbm_sim* s, const Grid& g, const MomentOut& 
 static int compute_moments(lbm_sim* s) {
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
   MomentOut mo{s->fields, s->fields + s->plane, s->fields + 2 * s->plane, s->fields + 3 * s->plane,
-               s->fields + 4 * s->plane};
+               s->fields + 4 * s->plane, nullptr, nullptr, s->pitch};
   cudaError_t e = moments_of(s, g, mo);
   if (e != cudaSuccess) return cuda_fail(e, "moments launch");
   s->launches++;
@@ -390,36 +420,32 @@ static int copy_out(lbm_sim* s, float* const* outs, int n, const char* what) {
   return e == cudaSuccess ? LBM_OK : cuda_fail(e, what);
 }
 
-// The address at which the moment pass writes an nx*ny output directly, or null: device memory
-// whose rows have the work planes' pitch (nx a multiple of 32), which saves a device-to-device
-// copy.  Page-locked host memory is also addressable by the kernel, but its 4-byte stores across
-// NVLink-C2C ran slower than the bulk copy (c3 end to end: 11.76 against 12.1 GLUPS), so host
+// Outputs of the moment pass.  Where it can address all of a call's outputs it writes them in place; otherwise all go
+// through the work planes and are copied.  Page-locked host memory is also addressable by the kernel, but its 4-byte
+// stores across NVLink-C2C ran slower than the bulk copy (c3 end to end: 11.76 against 12.1 GLUPS), so host
 // outputs are always copied.
-static float* direct_target(const lbm_sim* s, float* out) {
-  if (!out || s->pitch != s->nx) return nullptr;
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, out) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  const bool device = a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
-  return device ? static_cast<float*>(a.devicePointer) : nullptr;
+static bool all_direct(float* const* outs, int n) {
+  for (int k = 0; k < n; ++k)
+    if (outs[k] && !addressable(outs[k])) return false;
+  return true;
 }
 
 int lbm_moments(lbm_sim* s, float* phi, float* rho, float* ux, float* uy, float* p) {
   Range range_("lbm_moments");
   if (!s) return set_error("sim is NULL"), LBM_ERR_INVALID_ARG;
-  // outputs the kernel can address are written by it; the others go through the work planes
   float* outs[5] = {phi, rho, ux, uy, p};
   float* dst[5];
-  float* staged[5];
+  // in place: all outputs, or, where the work planes have the same pitch, those that can be
+  const bool direct = all_direct(outs, 5);
+  float* staged[5] = {};
   for (int k = 0; k < 5; ++k) {
-    float* d = direct_target(s, outs[k]);
-    dst[k] = d ? d : (outs[k] ? s->fields + (long long)k * s->plane : nullptr);
-    staged[k] = d ? nullptr : outs[k];
+    dst[k] = outs[k];
+    if (!outs[k] || direct || (s->pitch == s->nx && addressable(outs[k]))) continue;
+    dst[k] = s->fields + (long long)k * s->plane;
+    staged[k] = outs[k];
   }
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
-  MomentOut mo{dst[0], dst[1], dst[2], dst[3], dst[4]};
+  MomentOut mo{dst[0], dst[1], dst[2], dst[3], dst[4], nullptr, nullptr, direct ? s->nx : s->pitch};
   cudaError_t e = moments_of(s, g, mo);
   if (e != cudaSuccess) return cuda_fail(e, "moments launch");
   s->launches++;
@@ -429,13 +455,11 @@ int lbm_moments(lbm_sim* s, float* phi, float* rho, float* ux, float* uy, float*
 int lbm_moments_packed(lbm_sim* s, float* fields) {
   Range range_("lbm_moments_packed");
   if (!s || !fields) return set_error("sim and fields are required"), LBM_ERR_INVALID_ARG;
-  const size_t n = (size_t)s->nx * s->ny;
-  // a device block with rows of the work pitch is written by the moment pass itself
-  float* direct = direct_target(s, fields);
-  float* dst = direct ? direct : s->fields;
-  const size_t stride = direct ? n : (size_t)s->plane;
+  const bool direct = addressable(fields);
+  float* dst = direct ? fields : s->fields;
+  const size_t stride = direct ? (size_t)s->nx * s->ny : (size_t)s->plane;
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
-  MomentOut mo{dst, dst + stride, dst + 2 * stride, dst + 3 * stride, dst + 4 * stride};
+  MomentOut mo{dst, dst + stride, dst + 2 * stride, dst + 3 * stride, dst + 4 * stride, nullptr, nullptr, direct ? s->nx : s->pitch};
   cudaError_t e = moments_of(s, g, mo);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_moments_packed launch");
   s->launches++;
@@ -452,14 +476,16 @@ int lbm_interfacial_force(lbm_sim* s, float* fa_x, float* fa_y) {
   Range range_("lbm_interfacial_force");
   if (!s) return set_error("sim is NULL"), LBM_ERR_INVALID_ARG;
   Grid g = make_grid(s, s->buf[s->cur], nullptr);
+  float* outs[2] = {fa_x, fa_y};
   MomentOut mo{};
-  mo.fax = s->fields;
-  mo.fay = s->fields + s->plane;
+  const bool direct = fa_x && fa_y && all_direct(outs, 2);   // the kernel writes both components
+  mo.fax = direct ? fa_x : s->fields;
+  mo.fay = direct ? fa_y : s->fields + s->plane;
+  mo.pitch = direct ? s->nx : s->pitch;
   cudaError_t e = moments_of(s, g, mo);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_interfacial_force launch");
   s->launches++;
-  float* outs[2] = {fa_x, fa_y};
-  return copy_out(s, outs, 2, "lbm_interfacial_force copy");
+  return copy_out(s, outs, direct ? 0 : 2, "lbm_interfacial_force copy");
 }
 
 int lbm_diagnostics(lbm_sim* s, lbm_diag* out) {

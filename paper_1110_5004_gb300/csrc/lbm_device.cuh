@@ -245,12 +245,19 @@ struct Grid {
   long long spoff;      // s_form 1: byte offset of the [rho, div(rho u)] planes in src/dst (else 0)
 };
 
-// Output planes of the moment pass (row-major with `pitch`); each may be null.  fax, fay: the
+// Outputs of the moment pass (row-major); each may be null.  fax, fay: the
 // additional interfacial force F_a = -u s of Eq. 12 (s by the simulation's s_form), evaluated
 // whichever scheme runs.
 struct MomentOut {
   float *phi, *rho, *ux, *uy, *p;
   float *fax, *fay;
+  int pitch;            // elements per row of every output
+};
+
+// Initial fields phi0, ux0, uy0, p0: rows of `pitch` elements; null for zero.
+struct InitIn {
+  const float* f[4];
+  int pitch[4];
 };
 
 __host__ __device__ __forceinline__ int wrap(int i, int n) {

@@ -89,7 +89,7 @@ cudaError_t launch_step_fp32(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_step_fp16(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_step_bf16(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_moments(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st);
-cudaError_t launch_init(const lbm_sim* s, cudaStream_t st);  // from fields[phi, -, ux, uy, p]
+cudaError_t launch_init(const lbm_sim* s, const InitIn& in, cudaStream_t st);
 // 16-byte units [u0, u1) of the checkpoint's population order between a state buffer and `lin`.
 cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u0, long long u1, bool out, cudaStream_t st);
 cudaError_t launch_diag(const lbm_sim* s, cudaStream_t st);  // from fields -> red -> final record

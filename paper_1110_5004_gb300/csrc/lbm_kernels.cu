@@ -19,30 +19,27 @@ cudaError_t launch_step(const Phys2& P, const Grid& g, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------------ initial state
-// fields: [0] phi0, [1] (unused), [2] ux0, [3] uy0, [4] p0 -- pitched planes; mu0 is evaluated
-// where it is used.
-
 // State that streams into f = f^eq(phi0, mu0, u0), gbar = g^eq(p0, rho0, u0): each cell stores its own 18
 // equilibria where it will read them, population a in its row at column x - e_a,x.
 template <int ST>
-__global__ void k_init_pop(Phys P, Grid g, const float* __restrict__ fields) {
+__global__ void k_init_pop(Phys P, Grid g, InitIn in) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x == 0 && blockIdx.y == 0) *g.gave_up = 0u;         // a new state
   if (x >= g.nx) return;
   const Col3 col = col3<ST>(x, g.nx);
+  // neighbours: beyond a wall the mirrored row or column (zero gradient)
+  const int xm = x > 0 ? x - 1 : (g.bc_x == BC_WALL ? 0 : g.nx - 1);
+  const int xq = x < g.nx - 1 ? x + 1 : (g.bc_x == BC_WALL ? x : 0);
   for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {   // gridDim.y is capped at 65535
-    const long long c = (long long)y * g.pitch + x;
-    const float ph = fields[c], u = fields[2 * g.plane + c], v = fields[3 * g.plane + c];
-    const float p = fields[4 * g.plane + c];
-    // mu0 = theta'(phi0) - kappa lap(phi0) (Eq. 1); beyond a wall phi is mirrored (zero gradient)
-    auto at = [&](int dx, int dy) {
-      int xx = x + dx, yy = y + dy;
-      xx = g.bc_x == BC_WALL ? mirror(xx, g.nx) : wrap1(xx, g.nx);
-      yy = g.bc_y == BC_WALL ? mirror(yy, g.ny) : wrap1(yy, g.ny);
-      return fields[(long long)yy * g.pitch + xx];
-    };
-    const float lap = (4.0f * (at(1, 0) + at(0, 1) + at(-1, 0) + at(0, -1)) +
-                       (at(1, 1) + at(-1, 1) + at(-1, -1) + at(1, -1)) - 20.0f * ph) * (1.0f / 6.0f);
+    const int ym = y > 0 ? y - 1 : (g.bc_y == BC_WALL ? 0 : g.ny - 1);
+    const int yq = y < g.ny - 1 ? y + 1 : (g.bc_y == BC_WALL ? y : 0);
+    auto at = [&](int k) { return in.f[k] ? in.f[k][(long long)y * in.pitch[k] + x] : 0.0f; };
+    const float *fs = in.f[0] + (long long)ym * in.pitch[0], *fc = in.f[0] + (long long)y * in.pitch[0],
+                *fn = in.f[0] + (long long)yq * in.pitch[0];
+    const float ph = fc[x], u = at(1), v = at(2), p = at(3);
+    // mu0 = theta'(phi0) - kappa lap(phi0) (Eq. 1)
+    const float lap =
+        (4.0f * (fc[xq] + fn[x] + fc[xm] + fs[x]) + (fn[xq] + fn[xm] + fs[xm] + fs[xq]) - 20.0f * ph) * (1.0f / 6.0f);
     const float m = P.four_beta * ph * (ph * ph - P.phi_star2) - P.kappa * lap;
     const float cl = fminf(fmaxf((ph + P.phi_star) * P.inv_2phistar, 0.0f), 1.0f);
     const float rho = P.rho_B + cl * P.drho;
@@ -105,43 +102,42 @@ __global__ void k_init_pop(Phys P, Grid g, const float* __restrict__ fields) {
 }
 
 // s_form 1: rho and div(rho u) of the initial fields, which stand for the step before the first.
-__global__ void k_init_sdef(Phys P, Grid g, const float* __restrict__ fields) {
+__global__ void k_init_sdef(Phys P, Grid g, InitIn in) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= g.nx) return;
+  const int xm = x > 0 ? x - 1 : (g.bc_x == BC_WALL ? 0 : g.nx - 1);
+  const int xq = x < g.nx - 1 ? x + 1 : (g.bc_x == BC_WALL ? x : 0);
   for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {   // gridDim.y is capped at 65535
-    const float* phi = fields;
-    const float* ux = fields + 2 * g.plane;
-    const float* uy = fields + 3 * g.plane;
-    auto idx = [&](int dx, int dy) {
-      int xx = x + dx, yy = y + dy;
-      xx = g.bc_x == BC_WALL ? mirror(xx, g.nx) : wrap1(xx, g.nx);
-      yy = g.bc_y == BC_WALL ? mirror(yy, g.ny) : wrap1(yy, g.ny);
-      return (long long)yy * g.pitch + xx;
+    const int ym = y > 0 ? y - 1 : (g.bc_y == BC_WALL ? 0 : g.ny - 1);
+    const int yq = y < g.ny - 1 ? y + 1 : (g.bc_y == BC_WALL ? y : 0);
+    auto at = [&](int k, int dx, int dy) {
+      const int xx = dx < 0 ? xm : (dx > 0 ? xq : x), yy = dy < 0 ? ym : (dy > 0 ? yq : y);
+      return in.f[k] ? in.f[k][(long long)yy * in.pitch[k] + xx] : 0.0f;
     };
-    auto rho = [&](long long i) { return fmad(__saturatef(fmad(phi[i], P.inv_2phistar, 0.5f)), P.drho, P.rho_B); };
-    auto jx = [&](int dx, int dy) { const long long i = idx(dx, dy); return fmul(rho(i), ux[i]); };
-    auto jy = [&](int dx, int dy) { const long long i = idx(dx, dy); return fmul(rho(i), uy[i]); };
+    auto rho = [&](int dx, int dy) { return fmad(__saturatef(fmad(at(0, dx, dy), P.inv_2phistar, 0.5f)), P.drho, P.rho_B); };
+    auto jx = [&](int dx, int dy) { return fmul(rho(dx, dy), at(1, dx, dy)); };
+    auto jy = [&](int dx, int dy) { return fmul(rho(dx, dy), at(2, dx, dy)); };
     const float djx = fmad(4.0f, fsub(jx(1, 0), jx(-1, 0)), fsub(fsub(jx(1, 1), jx(-1, -1)), fsub(jx(-1, 1), jx(1, -1))));
     const float djy = fmad(4.0f, fsub(jy(0, 1), jy(0, -1)), fadd(fsub(jy(1, 1), jy(-1, -1)), fsub(jy(-1, 1), jy(1, -1))));
     float* sp = reinterpret_cast<float*>(static_cast<char*>(g.dst) + g.spoff);
     const long long c = (long long)y * g.pitch + x;
-    sp[c] = rho(c);
+    sp[c] = rho(0, 0);
     sp[g.plane + c] = fmul(fadd(djx, djy), 1.0f / 12.0f);
   }
 }
 
-cudaError_t launch_init(const lbm_sim* s, cudaStream_t st) {
+cudaError_t launch_init(const lbm_sim* s, const InitIn& in, cudaStream_t st) {
   Grid g = make_grid(s, nullptr, s->buf[s->cur]);
   dim3 blk(128), grd((s->nx + 127) / 128, s->ny < 65535 ? s->ny : 65535);
   switch (g.storage) {
-    case ST_FP16: k_init_pop<ST_FP16><<<grd, blk, 0, st>>>(s->phys, g, s->fields); break;
-    case ST_BF16: k_init_pop<ST_BF16><<<grd, blk, 0, st>>>(s->phys, g, s->fields); break;
-    default: k_init_pop<ST_FP32><<<grd, blk, 0, st>>>(s->phys, g, s->fields); break;
+    case ST_FP16: k_init_pop<ST_FP16><<<grd, blk, 0, st>>>(s->phys, g, in); break;
+    case ST_BF16: k_init_pop<ST_BF16><<<grd, blk, 0, st>>>(s->phys, g, in); break;
+    default: k_init_pop<ST_FP32><<<grd, blk, 0, st>>>(s->phys, g, in); break;
   }
   if (s->params.s_form) {
     cudaError_t e2 = cudaGetLastError();
     if (e2 != cudaSuccess) return e2;
-    k_init_sdef<<<grd, blk, 0, st>>>(s->phys, g, s->fields);
+    k_init_sdef<<<grd, blk, 0, st>>>(s->phys, g, in);
   }
   return cudaGetLastError();
 }

@@ -448,8 +448,8 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
         auto store2 = [&](float* q, V2 v) {
           float x, y;
           unpack2(v, x, y);
-          if (on_a) q[r2 * g.pitch + xpa] = x;
-          if (on_b) q[r2 * g.pitch + xpb] = y;
+          if (on_a) q[r2 * mo.pitch + xpa] = x;
+          if (on_b) q[r2 * mo.pitch + xpb] = y;
         };
         if (mo.phi) store2(mo.phi, ph);
         if (mo.rho) store2(mo.rho, o.rho);

@@ -154,7 +154,7 @@ __device__ __forceinline__ void tile2d_step(const Phys& P, const Grid& g, int ti
     for (int a = 0; a < Q; ++a) gb[a] = dec_pop<ST>(g2raw[c][a], Q + a);
     const S2Out<float> s2 = s2_cell<ST>(P, ph, gphx, gphy, gmx, gmy, sm.mu[j][i], sdef, gb);
     if constexpr (MOM) {
-      const int o = y * g.pitch + x;
+      const int o = y * mo.pitch + x;
       if (mo.phi) mo.phi[o] = ph;
       if (mo.rho) mo.rho[o] = s2.rho;
       if (mo.ux) mo.ux[o] = s2.ux;
