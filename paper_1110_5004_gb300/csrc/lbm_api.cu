@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <initializer_list>
+#include <mutex>
 #include <new>
 #include <string>
 
@@ -140,6 +141,40 @@ static int check_params(int nx, int ny, const lbm_params* p) {
   return LBM_OK;
 }
 
+// Page-locked diagnostics records, so that the kernel writes a simulation's record to the host and no copy follows.
+// One block for the process, allocated with the first simulation (allocating page-locked memory orders the
+// streams of the device, so it is not done again); a simulation that finds no free slot copies its record.
+namespace {
+class RecordPool {
+ public:
+  lbm_diag* take() {
+    std::lock_guard<std::mutex> lock(mu_);
+    if (!tried_) {
+      tried_ = true;
+      void* p = nullptr;
+      if (cudaHostAlloc(&p, SLOTS * sizeof(lbm_diag), cudaHostAllocPortable) == cudaSuccess) {
+        for (int k = SLOTS - 1; k >= 0; --k) free_[n_++] = static_cast<lbm_diag*>(p) + k;
+      } else {
+        cudaGetLastError();
+      }
+    }
+    return n_ > 0 ? free_[--n_] : nullptr;
+  }
+  void give(lbm_diag* d) {
+    std::lock_guard<std::mutex> lock(mu_);
+    free_[n_++] = d;
+  }
+
+ private:
+  static constexpr int SLOTS = 512;
+  std::mutex mu_;
+  bool tried_ = false;
+  int n_ = 0;
+  lbm_diag* free_[SLOTS];
+};
+RecordPool g_records;
+}  // namespace
+
 }  // namespace lbm
 
 using namespace lbm;
@@ -220,6 +255,7 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
     lbm_destroy(s);
     return rc;
   }
+  s->slot = g_records.take();
   *out = s;
   return LBM_OK;
 }
@@ -496,11 +532,13 @@ int lbm_diagnostics(lbm_sim* s, lbm_diag* out) {
   cudaError_t e = launch_diag(s, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "diagnostics launch");
   s->launches++;
-  e = cudaMemcpyAsync(&s->h_diag, s->red + (long long)s->ny * DIAG_PARTIALS, sizeof(lbm_diag),
-                      cudaMemcpyDeviceToHost, s->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "diagnostics copy");
+  if (!s->slot) {
+    e = cudaMemcpyAsync(&s->h_diag, s->red + (long long)s->ny * DIAG_PARTIALS, sizeof(lbm_diag), cudaMemcpyDeviceToHost,
+                        s->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "diagnostics copy");
+  }
   if ((rc = read_resident_status(s, true)) != LBM_OK) return rc;
-  *out = s->h_diag;
+  *out = s->slot ? *s->slot : s->h_diag;
   if (!out->finite) {
     set_error("simulation diverged (non-finite state) at step %lld", out->step);
     return LBM_ERR_DIVERGED;
@@ -515,6 +553,7 @@ int lbm_destroy(lbm_sim* s) {
   for (void* p : {s->buf[0], s->buf[1], static_cast<void*>(s->fields), static_cast<void*>(s->res_mem)})
     if (p) cudaFreeAsync(p, s->stream);
   if (s->uploaded) cudaEventDestroy(s->uploaded);
+  if (s->slot) g_records.give(s->slot);
   delete s;
   return LBM_OK;
 }

@@ -22,8 +22,8 @@ struct lbm_sim {
   int cur = 0;                         // buffer holding the current state
   float* fields = nullptr;             // 6 planes: phi, rho, ux, uy, p, mu (moments and init)
   double* red = nullptr;               // reduction scratch: ny rows x 12 partials + final record
-  lbm_diag h_diag{};                   // host copy of the final record (pageable: allocating
-                                       // page-locked memory would order the streams of the device)
+  lbm_diag h_diag{};                   // host copy of the final record, for a simulation without a slot
+  lbm_diag* slot = nullptr;            // page-locked record the diagnostics kernel writes itself
   cudaEvent_t uploaded = nullptr;      // recorded after lbm_init_fields' host-to-device copies
   long long steps = 0;
   long long launches = 0;
@@ -52,7 +52,7 @@ struct Range {
 
 constexpr int N_FIELDS = 6;
 constexpr int DIAG_PARTIALS = 12;
-// Words in the spare doubles behind the diagnostics record: raised by a wait that ran out; rows of a
+// Words in the spare doubles behind the diagnostics record: raised by a wait that ran out; blocks of a
 // diagnostics launch that have finished.
 inline unsigned int* gave_up(const lbm_sim* s) { return reinterpret_cast<unsigned int*>(s->red + (size_t)s->ny * DIAG_PARTIALS + 14); }
 inline unsigned int* diag_done(const lbm_sim* s) { return gave_up(s) + 1; }

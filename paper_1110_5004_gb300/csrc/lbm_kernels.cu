@@ -221,7 +221,7 @@ cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u
 
 cudaError_t launch_diag(const lbm_sim* s, cudaStream_t st) {
   const float* f = s->fields;
-  double* record = s->red + (long long)s->ny * DIAG_PARTIALS;
+  double* record = s->slot ? reinterpret_cast<double*>(s->slot) : s->red + (long long)s->ny * DIAG_PARTIALS;
   DiagIn d = diag_in(f, f + 2 * s->plane, f + 3 * s->plane, f + 4 * s->plane, s->nx, s->ny, s->pitch, s->phys.phi_star, s->red,
                      record, diag_done(s), s->steps);
   d.gave_up = gave_up(s);

@@ -95,10 +95,10 @@ extern "C" int lbm_diagnostics_fields_noalloc(const float* phi, const float* ux,
   int rc = noalloc_scratch(&scratch);
   if (rc) return rc;
   double* record = scratch + (long long)NOALLOC_MAX_ROWS * DIAG_PARTIALS;
-  // the count of finished rows is cleared by each call: an earlier one may have been cut short
+  // the count of finished blocks is cleared by each call: an earlier one may have been cut short
   unsigned int* done = reinterpret_cast<unsigned int*>(record + 15);
   if ((e = cudaMemsetAsync(done, 0, sizeof(unsigned int), st)) != cudaSuccess)
-    return cuda_fail(e, "lbm_diagnostics_fields_noalloc: row count");
+    return cuda_fail(e, "lbm_diagnostics_fields_noalloc: block count");
   e = launch_diag_rows(diag_in(phi, ux, uy, p, nx, ny, nx, phi_star, scratch, record, done, step), st);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_diagnostics_fields_noalloc: kernel");
   e = cudaMemcpyAsync(out, record, sizeof(lbm_diag), host_out ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st);
