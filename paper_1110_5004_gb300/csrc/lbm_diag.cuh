@@ -123,10 +123,8 @@ static __global__ void __launch_bounds__(DIAG_T) k_diag(const __grid_constant__ 
         cv = fma(c, v, cv);
         if (!(__fmaf_ru(uf, uf, __fmul_ru(vf, vf)) <= u2_low)) {
           const double q = fma(u, u, v * v);
-          if (!(q <= u2)) {
-            u2 = q;
-            u2_low = __double2float_rd(q);
-          }
+          u2 = diag_max(u2, q);
+          u2_low = __double2float_rd(u2);   // NaN from here on, once there is one
         }
         if (phf > d.liq) {
           pl += p;
@@ -170,7 +168,7 @@ static __global__ void __launch_bounds__(DIAG_T) k_diag(const __grid_constant__ 
     for (int r = 0; r < rows; ++r) {
       c += chord[r];
       cy = fma(chord[r], (double)(y0 + r), cy);
-      if (!(chord[r] <= wide)) wide = chord[r];
+      wide = diag_max(wide, chord[r]);
     }
     for (int k = 0; k < DIAG_T / 32; ++k) {
       nl += count[0][k];
@@ -200,8 +198,7 @@ static __global__ void __launch_bounds__(DIAG_T) k_diag(const __grid_constant__ 
     double s = 0.0;
     for (unsigned int b = lane; b < gridDim.x; b += 32) {
       const double v = __ldcg(d.part + (long long)b * DIAG_PARTIALS + k);
-      if (!max) s += v;
-      else if (!(v <= s)) s = v;
+      s = max ? diag_max(s, v) : s + v;
     }
 #pragma unroll
     for (int h = 16; h > 0; h >>= 1) {

@@ -6,7 +6,7 @@
 
 namespace lbm {
 
-// Two CTAs of 96 threads per SM: shared memory (113 KB each in FP32 storage) and up to 255 registers.
+// Two CTAs of 128 threads per SM: shared memory (113 KB each in FP32 storage) and up to 255 registers.
 template <int MODE, int ST, bool SD, bool FF, bool XW>
 __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_march(const __grid_constant__ Phys2 P, const __grid_constant__ Grid g,
                                                        const __grid_constant__ MomentOut mo) {
