@@ -372,14 +372,25 @@ __device__ __forceinline__ V from_scale(const K& P, V v) {
 // The offset is a hash of the value's own bits and its place, so every kernel rounds a
 // given value at a given place alike and runs stay deterministic.  NaN and infinity stay NaN and infinity, so a
 // diverged state stays non-finite.
-__device__ __forceinline__ unsigned short bf16_stochastic(float v, unsigned int where) {
-  const unsigned int bits = __float_as_uint(v);
+// The conversion adds the high and the low half of its third operand to the 16 bits that it drops of the first and the
+// second value: what an integer addition to the value's bits gives, with four instructions fewer per value (4096^2: 391 ->
+// 371 us a step; 2048 x 512: 35.5 -> 34.2).
+__device__ __forceinline__ unsigned int bf16_hash(float v, unsigned int where) {
   // the high half of a product with an odd constant depends on every bit of the other factor
-  const unsigned int offset = ((bits ^ where) * 0x9e3779b1u) >> 16;
-  // the magnitude saturates at the largest NaN, so that no carry reaches the sign; infinities and the NaN that
-  // arithmetic produces (all bits set) stay what they are
-  const unsigned int mag = min((bits & 0x7fffffffu) + offset, 0x7fffffffu);
-  return static_cast<unsigned short>((mag | (bits & 0x80000000u)) >> 16);
+  return (__float_as_uint(v) ^ where) * 0x9e3779b1u;
+}
+// The bits of lo and hi (at their places) in the low and the high half.
+__device__ __forceinline__ unsigned int bf16_stochastic2(float lo, unsigned int at_lo, float hi, unsigned int at_hi) {
+  unsigned int d;
+  asm("cvt.rs.bf16x2.f32 %0, %1, %2, %3;"
+      : "=r"(d)
+      : "f"(hi), "f"(lo), "r"(__byte_perm(bf16_hash(lo, at_lo), bf16_hash(hi, at_hi), 0x7632)));
+  return d;
+}
+__device__ __forceinline__ unsigned short bf16_stochastic(float v, unsigned int where) {
+  unsigned int d;
+  asm("cvt.rs.bf16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v), "f"(0.0f), "r"(bf16_hash(v, where)));
+  return static_cast<unsigned short>(d >> 16);
 }
 // 16-bit encoding of population a (already in storage scale).
 template <int ST>

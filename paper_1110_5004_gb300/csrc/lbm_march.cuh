@@ -185,7 +185,16 @@ struct OutLanes {
     } else {
       unsigned short h[Q + Q];
 #pragma unroll
-      for (int a = 1; a < Q + Q; ++a) h[a] = enc_pop<ST>(x[a], a, key);
+      for (int a = 1; a < (ST == ST_BF16 ? Q : Q + Q); ++a) h[a] = enc_pop<ST>(x[a], a, key);
+      if constexpr (ST == ST_BF16) {               // gbar: two per conversion
+#pragma unroll
+        for (int a = Q; a < Q + Q - 1; a += 2) {
+          const unsigned int d = bf16_stochastic2(x[a], key + pop_key(a), x[a + 1], key + pop_key(a + 1));
+          h[a] = static_cast<unsigned short>(d);
+          h[a + 1] = static_cast<unsigned short>(d >> 16);
+        }
+        h[Q + Q - 1] = enc_pop<ST>(x[Q + Q - 1], Q + Q - 1, key);
+      }
       asm volatile(
           "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
           "@q st.global.u16 [%1+128], %4;\n\t@q st.global.u16 [%1+320], %5;\n\t@q st.global.u16 [%1+384], %6;\n\t"
