@@ -68,9 +68,9 @@ static int rebuild(lbm_batch* b) {
     for (int m : members) {
       const lbm_sim* s = b->slots[m];
       if (part_of(s) != part) continue;
-      int tw, ns, hh;
-      tile_geometry(s->nx, s->ny, s->params.s_form != 0, 1, 0, &tw, &ns, &hh);
-      shape.push_back({ns, s->ny, s->seg_h ? s->seg_h : b->seg_h});
+      Grid g{};
+      tile_geometry(s->nx, s->ny, s->params.s_form != 0, false, 1, 0, &g);
+      shape.push_back({g.n_strips, s->ny, s->seg_h ? s->seg_h : b->seg_h});
     }
     long long best = -1;
     rows[part] = 32;
@@ -97,14 +97,14 @@ static int rebuild(lbm_batch* b) {
       const int segs = (s->ny + rows[part_of(s)] - 1) / rows[part_of(s)];
       h = (s->ny + segs - 1) / segs;
     }
-    tile_geometry(s->nx, s->ny, s->params.s_form != 0, h, 0, &g.tile_w, &g.n_strips, &g.seg_h);
+    tile_geometry(s->nx, s->ny, s->params.s_form != 0, false, h, 0, &g);
     d.g = g;
     d.buf0 = s->buf[0];
     d.buf1 = s->buf[1];
     d.cur0 = s->cur;
     sims.push_back(d);
     std::vector<int4> tl;
-    const int nseg = (s->ny + g.seg_h - 1) / g.seg_h;
+    const int nseg = march_segs(g);
     for (int sg = 0; sg < nseg; ++sg)
       for (int st = 0; st < g.n_strips; ++st) tl.push_back(make_int4((int)m, st, sg, 0));
     per[part_of(s)].push_back(std::move(tl));

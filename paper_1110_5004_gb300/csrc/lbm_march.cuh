@@ -248,8 +248,8 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
   const int w = g.tile_w;
   const int x0 = strip * 2 * w;
   const int wa = min(w, g.nx - x0), wb = min(w, g.nx - x0 - w);   // columns of each lane (wb may be < 1)
-  const int ya = seg * g.seg_h;
-  const int yb = min(ya + g.seg_h, g.ny);
+  int ya, yb;
+  seg_rows(g, seg, &ya, &yb);
   const int te = min(t, w + 5);                    // threads beyond the halo repeat its last column
   const int xla = x0 - 3 + te, xlb = xla + w;      // logical columns (may lie outside [0, nx))
   const int xpa = wrap1(xla, g.nx), xpb = wrap1(xlb, g.nx);
