@@ -158,30 +158,51 @@ struct OutLanes {
     o.template put<17>(x[17]);
     if constexpr (ST == ST_FP32) o.template put<A_F0LO>(x[A_F0LO]);
   }
-  // rows: the destination buffer's rows y-1, y, y+1; c: the lane's column; key: its BF16 rounding place
-  template <bool B>
-  __device__ __forceinline__ void store_lane(char* rm, char* r0, char* rq, const ColB& c, int nblk, unsigned int key, bool on) const {
+  // rows: the destination buffer's rows y-1, y, y+1; c: the lane's column; key: its BF16 rounding place.  XW: the column
+  // may lie at the left (wl) or the right (wr) wall; the populations that would cross it go back reversed, to the
+  // column xw beyond the wall (wrapped), row y.
+  template <bool B, bool XW>
+  __device__ __forceinline__ void store_lane(char* rm, char* r0, char* rq, const ColB& c, int nblk, unsigned int key, bool on, bool wl,
+                                             bool wr, int xw) const {
     float x[Q + Q + 1];
     lane<B>(x);
+    if constexpr (XW) {
+      if (on && (wl || wr)) {
+        const ColB cw = col_bytes<ST>(xw);
+        auto back = [&](auto pop) {   // population A of the right wall, its mirror image of the left
+          constexpr int A = decltype(pop)::value, M = opp(A % Q) + (A >= Q ? Q : 0);
+          char* const q = r0 + region_start(ST, region_of(A)) * nblk + (wr ? pop_in_region<ST>(M, cw) : pop_in_region<ST>(A, cw));
+          if constexpr (ST == ST_FP32) *reinterpret_cast<float*>(q) = wr ? x[A] : x[M];
+          else *reinterpret_cast<unsigned short*>(q) = wr ? enc_pop<ST>(x[A], A, key) : enc_pop<ST>(x[M], M, key);
+        };
+        back(std::integral_constant<int, 1>{});
+        back(std::integral_constant<int, 5>{});
+        back(std::integral_constant<int, 8>{});
+        back(std::integral_constant<int, Q + 1>{});
+        back(std::integral_constant<int, Q + 5>{});
+        back(std::integral_constant<int, Q + 8>{});
+      }
+    }
+    const int right = on && !(XW && wr), left = on && !(XW && wl);
     const int g = region_start(ST, R_G) * nblk + c.g;
     static_assert(BLK == 32, "offsets below");
     if constexpr (ST == ST_FP32) {
       asm volatile(
-          "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
-          "@q st.global.f32 [%1+256], %4;\n\t@q st.global.f32 [%1+640], %5;\n\t@q st.global.f32 [%1+768], %6;\n\t"
-          "@q st.global.f32 [%2], %7;\n\t@q st.global.f32 [%2+128], %8;\n\t@q st.global.f32 [%2+384], %9;\n\t"
-          "@q st.global.f32 [%3+512], %10;\n\t@q st.global.f32 [%3+896], %11;\n\t@q st.global.f32 [%3+1024], %12;\n\t}" ::"r"(
+          "{\n\t.reg .pred q, r, l;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %13, 0;\n\tsetp.ne.s32 l, %14, 0;\n\t"
+          "@q st.global.f32 [%1+256], %4;\n\t@r st.global.f32 [%1+640], %5;\n\t@l st.global.f32 [%1+768], %6;\n\t"
+          "@q st.global.f32 [%2], %7;\n\t@r st.global.f32 [%2+128], %8;\n\t@l st.global.f32 [%2+384], %9;\n\t"
+          "@q st.global.f32 [%3+512], %10;\n\t@l st.global.f32 [%3+896], %11;\n\t@r st.global.f32 [%3+1024], %12;\n\t}" ::"r"(
               (int)on),
           "l"(rq + g), "l"(r0 + g), "l"(rm + g), "f"(x[Q + 2]), "f"(x[Q + 5]), "f"(x[Q + 6]), "f"(x[Q + 0]), "f"(x[Q + 1]),
-          "f"(x[Q + 3]), "f"(x[Q + 4]), "f"(x[Q + 7]), "f"(x[Q + 8]));
+          "f"(x[Q + 3]), "f"(x[Q + 4]), "f"(x[Q + 7]), "f"(x[Q + 8]), "r"(right), "r"(left));
       asm volatile(
-          "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
-          "@q st.global.f32 [%1+256], %5;\n\t@q st.global.f32 [%1+640], %6;\n\t@q st.global.f32 [%1+768], %7;\n\t"
-          "@q st.global.f32 [%2], %8;\n\t@q st.global.f32 [%2+128], %9;\n\t@q st.global.f32 [%2+384], %10;\n\t"
-          "@q st.global.f32 [%3+512], %11;\n\t@q st.global.f32 [%3+896], %12;\n\t@q st.global.f32 [%3+1024], %13;\n\t"
+          "{\n\t.reg .pred q, r, l;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %15, 0;\n\tsetp.ne.s32 l, %16, 0;\n\t"
+          "@q st.global.f32 [%1+256], %5;\n\t@r st.global.f32 [%1+640], %6;\n\t@l st.global.f32 [%1+768], %7;\n\t"
+          "@q st.global.f32 [%2], %8;\n\t@r st.global.f32 [%2+128], %9;\n\t@l st.global.f32 [%2+384], %10;\n\t"
+          "@q st.global.f32 [%3+512], %11;\n\t@l st.global.f32 [%3+896], %12;\n\t@r st.global.f32 [%3+1024], %13;\n\t"
           "@q st.global.f32 [%4], %14;\n\t}" ::"r"((int)on),
           "l"(rq + c.f4), "l"(r0 + c.f4), "l"(rm + c.f4), "l"(r0 + region_start(ST, R_L) * nblk + c.l), "f"(x[2]), "f"(x[5]),
-          "f"(x[6]), "f"(x[0]), "f"(x[1]), "f"(x[3]), "f"(x[4]), "f"(x[7]), "f"(x[8]), "f"(x[A_F0LO]));
+          "f"(x[6]), "f"(x[0]), "f"(x[1]), "f"(x[3]), "f"(x[4]), "f"(x[7]), "f"(x[8]), "f"(x[A_F0LO]), "r"(right), "r"(left));
     } else {
       unsigned short h[Q + Q];
 #pragma unroll
@@ -196,21 +217,21 @@ struct OutLanes {
         h[Q + Q - 1] = enc_pop<ST>(x[Q + Q - 1], Q + Q - 1, key);
       }
       asm volatile(
-          "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
-          "@q st.global.u16 [%1+128], %4;\n\t@q st.global.u16 [%1+320], %5;\n\t@q st.global.u16 [%1+384], %6;\n\t"
-          "@q st.global.u16 [%2], %7;\n\t@q st.global.u16 [%2+64], %8;\n\t@q st.global.u16 [%2+192], %9;\n\t"
-          "@q st.global.u16 [%3+256], %10;\n\t@q st.global.u16 [%3+448], %11;\n\t@q st.global.u16 [%3+512], %12;\n\t}" ::"r"(
+          "{\n\t.reg .pred q, r, l;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %13, 0;\n\tsetp.ne.s32 l, %14, 0;\n\t"
+          "@q st.global.u16 [%1+128], %4;\n\t@r st.global.u16 [%1+320], %5;\n\t@l st.global.u16 [%1+384], %6;\n\t"
+          "@q st.global.u16 [%2], %7;\n\t@r st.global.u16 [%2+64], %8;\n\t@l st.global.u16 [%2+192], %9;\n\t"
+          "@q st.global.u16 [%3+256], %10;\n\t@l st.global.u16 [%3+448], %11;\n\t@r st.global.u16 [%3+512], %12;\n\t}" ::"r"(
               (int)on),
           "l"(rq + g), "l"(r0 + g), "l"(rm + g), "h"(h[Q + 2]), "h"(h[Q + 5]), "h"(h[Q + 6]), "h"(h[Q + 0]), "h"(h[Q + 1]),
-          "h"(h[Q + 3]), "h"(h[Q + 4]), "h"(h[Q + 7]), "h"(h[Q + 8]));
+          "h"(h[Q + 3]), "h"(h[Q + 4]), "h"(h[Q + 7]), "h"(h[Q + 8]), "r"(right), "r"(left));
       asm volatile(
-          "{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %0, 0;\n\t"
-          "@q st.global.u16 [%1+192], %5;\n\t@q st.global.u16 [%1+384], %6;\n\t@q st.global.u16 [%1+448], %7;\n\t"
-          "@q st.global.u16 [%2+128], %8;\n\t@q st.global.u16 [%2+256], %9;\n\t"
-          "@q st.global.u16 [%3+320], %10;\n\t@q st.global.u16 [%3+512], %11;\n\t@q st.global.u16 [%3+576], %12;\n\t"
+          "{\n\t.reg .pred q, r, l;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %14, 0;\n\tsetp.ne.s32 l, %15, 0;\n\t"
+          "@q st.global.u16 [%1+192], %5;\n\t@r st.global.u16 [%1+384], %6;\n\t@l st.global.u16 [%1+448], %7;\n\t"
+          "@r st.global.u16 [%2+128], %8;\n\t@l st.global.u16 [%2+256], %9;\n\t"
+          "@q st.global.u16 [%3+320], %10;\n\t@l st.global.u16 [%3+512], %11;\n\t@r st.global.u16 [%3+576], %12;\n\t"
           "@q st.global.f32 [%4], %13;\n\t}" ::"r"((int)on),
           "l"(rq + c.f2), "l"(r0 + c.f2), "l"(rm + c.f2), "l"(r0 + c.f4), "h"(h[2]), "h"(h[5]), "h"(h[6]), "h"(h[1]), "h"(h[3]),
-          "h"(h[4]), "h"(h[7]), "h"(h[8]), "f"(x[0]));
+          "h"(h[4]), "h"(h[7]), "h"(h[8]), "f"(x[0]), "r"(right), "r"(left));
     }
   }
 };
@@ -542,21 +563,21 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
       }
       OutLanes<ST> out;
       collide_store<ST, FF>(P, prev, *at(c + PP), gpx, gpy, *at(q5[4] + HI), *at(q5[4] + LO), phiD, f, gprev, out);
-      // the cells next to a wall, where populations bounce back, take the general path
+      // a row next to a wall, where populations bounce back, takes the general path
       const bool wrow = CK && ywall && (r3 == 0 || r3 == g.ny - 1);
-      const bool wcol_a = xwall && (xla == 0 || xla == g.nx - 1), wcol_b = xwall && (xlb == 0 || xlb == g.nx - 1);
       char* const dst = static_cast<char*>(g.dst);
       char* const row0 = dst + (long long)r3 * g.row_bytes;
       char* const rowm = r3 == 0 ? dst + (long long)(g.ny - 1) * g.row_bytes : row0 - g.row_bytes;
       char* const rowq = r3 == g.ny - 1 ? dst : row0 + g.row_bytes;
-      if constexpr (CK || XW) {
-        if (on_a && (wrow || wcol_a)) out.template store_cell<false>(out_cell<ST, XW, true>(g, xpa, r3));
-        if (on_b && (wrow || wcol_b)) out.template store_cell<true>(out_cell<ST, XW, true>(g, xpb, r3));
+      if constexpr (CK) {
+        if (on_a && wrow) out.template store_cell<false>(out_cell<ST, XW, true>(g, xpa, r3));
+        if (on_b && wrow) out.template store_cell<true>(out_cell<ST, XW, true>(g, xpb, r3));
       }
-      out.template store_lane<false>(rowm, row0, rowq, col_bytes<ST>(xpa), g.nblk, hash_key<ST>(xpa, r3, g),
-                                     on_a && !((CK || XW) && (wrow || wcol_a)));
-      out.template store_lane<true>(rowm, row0, rowq, col_bytes<ST>(xpb), g.nblk, hash_key<ST>(xpb, r3, g),
-                                    on_b && !((CK || XW) && (wrow || wcol_b)));
+      const bool wr_a = xwall && xla == g.nx - 1, wr_b = xwall && xlb == g.nx - 1;
+      out.template store_lane<false, XW>(rowm, row0, rowq, col_bytes<ST>(xpa), g.nblk, hash_key<ST>(xpa, r3, g), on_a && !wrow,
+                                         xwall && xla == 0, wr_a, wr_a ? 0 : g.nx - 1);
+      out.template store_lane<true, XW>(rowm, row0, rowq, col_bytes<ST>(xpb), g.nblk, hash_key<ST>(xpb, r3, g), on_b && !wrow,
+                                        xwall && xlb == 0, wr_b, wr_b ? 0 : g.nx - 1);
     };
     pg3 = pg2;
     if (do1) stage1();
