@@ -499,7 +499,7 @@ def run_ours(args):
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": tr, "peak_kind": peak_kind,
                 "bytes_per_lu_algorithmic": b_min, "bytes_per_lu_design": 152 if storage == 0 else 76,
-                "kernel": "k_tiles<MODE_STEP> (fused gather/moments/mu/forcing/collide/store)"}
+                "kernel": "k_march<MODE_STEP> (fused gather/moments/mu/forcing/collide/store)"}
 
     # end to end through the C ABI with pinned host buffers: upload the initial fields, advance
     # REINIT_EVERY steps, read the five moment fields back

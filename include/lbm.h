@@ -206,8 +206,8 @@ LBM_API long long lbm_step_count(const lbm_sim* sim);
 /* Checkpoint / resume (no counterpart in the paper: it lets a server evict a simulation's
  * device state to host memory and resume it later bitwise).  A checkpoint is a 64-byte header
  * (magic "LBMC", version 2, nx, ny, row pitch, storage, step count, payload size) followed by
- * the raw population buffer of the current state; it holds no parameters.  Version 2 is the
- * blocked population layout: each row is pitch / 32 blocks of 32 cells, a block holding every
+ * the populations of the current state; it holds no parameters.  Version 2 is a blocked
+ * layout: each row is pitch / 32 blocks of 32 cells, a block holding every
  * population plane of its cells in turn (FP32: f_0..f_8, gbar_0..gbar_8, f_0lo, 128 B each;
  * 16-bit: the FP32 rest plane, then 17 planes of 64 B); with s_form = 1 two FP32 planes
  * [rho, div(rho u)] of ny rows x pitch follow the populations.  Version 1 checkpoints (plain
@@ -231,7 +231,8 @@ LBM_API int lbm_restore(lbm_sim* sim, const void* buf, size_t bytes);
 LBM_API int lbm_set_stream(lbm_sim* sim, void* cuda_stream);
 
 /* Tile shape of the row march: rows per CTA (>= 1).  0 keeps the current value; a new simulation has as
- * many rows per CTA as make one wave of resident CTAs.  threads (64, 128, 256 or 0) is accepted and has
+ * many rows per CTA as make one wave of resident CTAs (fewer in the CTAs at walls on y, where the wave has
+ * CTAs to spare).  threads (64, 128, 256 or 0) is accepted and has
  * no effect: every CTA has 128 threads of two columns each.  Results do not depend on the shape. */
 LBM_API int lbm_set_tile(lbm_sim* sim, int threads, int seg_rows);
 
@@ -280,7 +281,7 @@ LBM_API const char* lbm_last_error(void);
  * The paper has no counterpart: this entry point exists for callers that cannot call
  * cudaMalloc -- a host application that owns the whole device-memory budget (for example a
  * server whose pools have reserved it), or a loop that must not take the device-wide
- * synchronisation of a fresh allocation.  It allocates nothing: the per-row partial sums live
+ * synchronisation of a fresh allocation.  It allocates nothing: the partial sums live
  * in one fixed file-scope device array of the library (8192 rows x 12 doubles plus the result,
  * 768 KB, held by every GPU that loads the library until the process exits).
  *   phi, ux, uy, p  row-major nx*ny float32 each (caller-owned, read only), in device memory of
@@ -304,7 +305,8 @@ LBM_API int lbm_diagnostics_fields_noalloc(const float* phi, const float* ux, co
 
 /* ------------------------------------------------------------------ ragged batches
  * A batch advances many independent simulations (different sizes and parameters) with one
- * launch per time step over a work list of tiles from all of them.  Simulations stay owned by
+ * launch per time step over a work list of tiles from all of them (one for each storage and form of the
+ * mass defect among them).  Simulations stay owned by
  * the caller; the batch references them.  budget_bytes caps the summed lbm_device_bytes of
  * its members (0 = no cap).  lbm_batch_step(k) advances every member by k steps (replays of one
  * 16-step CUDA graph captured per membership, the rest launched directly); members keep stepping

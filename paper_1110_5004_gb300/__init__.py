@@ -219,7 +219,7 @@ class Sim:
 
 
 class Batch:
-    """Ragged batch: member simulations advance together, one persistent launch per step."""
+    """Ragged batch: member simulations advance together, one persistent launch per step (and storage)."""
 
     def __init__(self, budget_bytes=0, stream=None):
         h = ctypes.c_void_p()

@@ -3,8 +3,7 @@
 The step kernel's shape is (threads per CTA, rows per CTA).  The library's CTAs have one width, whatever
 `threads` says; rows trade pipeline fill (a segment of h rows runs h + 7 row
 iterations, the first and last few with stages idle) for parallelism (one CTA per strip x
-segment).  The kernel is bound by instruction issue, so a step lasts as long as the SM with the
-most CTAs: besides a fixed list of heights, the candidates include, for k = 1..8 resident CTAs
+segment).  A step lasts as long as the SM with the most CTAs: besides a fixed list of heights, the candidates include, for k = 1..8 resident CTAs
 per SM, the shortest height whose CTA count still fits k x SMs (one row less can add a nearly
 empty wave).  The best pair depends on the grid, the storage and the device, so it is
 measured: each candidate runs about a millisecond of steps timed with CUDA events on the

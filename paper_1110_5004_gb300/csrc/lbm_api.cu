@@ -68,23 +68,22 @@ void tile_geometry(int nx, int ny, bool sd, bool ywall, int seg_h, int slots, Gr
   g->n_strips = ns;
   g->tile_w = (nx + 2 * ns - 1) / (2 * ns);
   g->seg_cut = g->seg_last = 0;
-  if (seg_h <= 0) {
-    // as many segments as fit in one wave of `slots` resident CTAs: the step lasts as long as the
-    // busiest SM, so a count just above the slots adds a nearly empty wave.  Segments of a few rows spend
-    // most of their h + 7 iterations on the rows around them, and are still the fastest where the grid has
-    // no more rows to give (601 x 437 with side walls: 18.1 us at 5 rows, 22.4 at 8)
-    const int segs = slots >= ns ? slots / ns : 1;
-    seg_h = (ny + segs - 1) / segs;
-    // A segment that meets a wall row takes longer by about a row (checked iterations, a row that bounces back
-    // cell by cell), and the step waits for it.  Where the wave has segments to spare, the first and the last
-    // are shorter; not below 5 rows, or their neighbours' rows around them would meet the wall too.  2048 x 512:
-    // FP32 34.9 -> 33.0 us, FP16 33.2 -> 30.0.
-    if (ywall && seg_h > 5 && segs > 2) {
-      const int c = std::min((segs * seg_h - ny) / 2, seg_h - 5);
-      if (c > 0) {
-        g->seg_cut = c;
-        g->seg_last = seg_h - c;
-      }
+  int segs = slots >= ns ? slots / ns : 1;
+  // as many segments as fit in one wave of `slots` resident CTAs: the step lasts as long as the
+  // busiest SM, so a count just above the slots adds a nearly empty wave.  Segments of a few rows spend
+  // most of their h + 7 iterations on the rows around them, and are still the fastest where the grid has
+  // no more rows to give (601 x 437 with side walls: 18.1 us at 5 rows, 22.4 at 8)
+  seg_h = seg_h <= 0 ? (ny + segs - 1) / segs : std::min(seg_h, ny);
+  segs = std::max(segs, (ny + seg_h - 1) / seg_h);
+  // A segment that meets a wall row takes longer by about a row (checked iterations, a row that bounces back
+  // cell by cell), and the step waits for it.  Where the wave has segments to spare, the first and the last
+  // are shorter; not below 5 rows, or their neighbours' rows around them would meet the wall too.  2048 x 512:
+  // FP32 34.9 -> 33.0 us, FP16 33.2 -> 30.0.
+  if (ywall && seg_h > 5 && seg_h < ny) {
+    const int c = (int)std::min(((long long)segs * seg_h - ny) / 2, (long long)seg_h - 5);
+    if (c > 0) {
+      g->seg_cut = c;
+      g->seg_last = seg_h - c;
     }
   }
   g->seg_h = seg_h;

@@ -22,7 +22,12 @@
 // Why this form (2048 x 512 and 4096 x 4096, FP32 storage): the step moves 152 B per cell, 6.5 cycles
 // per cell and SM at the measured bandwidth.  With one cell per thread it issued 594-745 warp instructions per
 // 32 cells, 4.6-5.8 cycles per cell at best, and its warps waited 30-48 % of their time on loads that one row of
-// register prefetch could not cover (more warps or L2 prefetches only thrashed L1).
+// register prefetch could not cover (more warps or L2 prefetches only thrashed L1).  This form issues 380 per 32 cells.
+// 4096 x 4096: 527 -> 408 us a step (152 B per cell at 0.92 of the measured copy bandwidth); 2048 x 512 with walls on y:
+// 40.8 -> 33.0, of which 1.5 us pass between two launches, 5.3 in the iterations before a segment's first S3 (1.4 of
+// them for the first row), 1.4 in each of the others.  What bounds an iteration is a warp's own chain of about 760
+// instructions at 4.3 cycles (2 warps per scheduler; issue slots half used, shared-memory pipe 65 %): warps that skip
+// columns beyond the halo, or more rows in flight, change nothing.
 #pragma once
 #include "lbm_device.cuh"
 

@@ -4,7 +4,7 @@
 // owns the device memory (a server that has reserved the whole budget for its own pools, or a
 // solver loop that must not take the implicit device-wide synchronisation of a fresh
 // allocation), can still reduce fields it holds.  It passes the four input fields and the
-// output record; the per-row partial sums live in a fixed file-scope device array instead of
+// output record; the partial sums live in a fixed file-scope device array instead of
 // memory the library would allocate.
 //
 // The array is shared by every call in the process on a given device and keeps the last

@@ -141,7 +141,7 @@ class Server:
         # stretches every member's latency (processor sharing) without adding throughput
         self.max_cells = max_cells
         # a member of at least this many cells steps alone, with the single-simulation kernels
-        # (the small-grid tile kernel up to 512K cells, the row march above), on a stream of its
+        # (the small-grid tile kernel up to 256K cells, the row march above), on a stream of its
         # own; smaller members share the batch.  On the c5 stream, 64K cells and 8 streams served
         # 23.1 GLUPS against 22.0 with a 1M threshold and 4 streams (256 requests).
         self.solo_cells = solo_cells
