@@ -8,6 +8,7 @@
 #include <array>
 #include <map>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "lbm_batch.cuh"
@@ -28,6 +29,7 @@ struct lbm_batch {
   bool dirty = true;                   // descriptors / work list need rebuilding
   SimDesc* d_sims = nullptr;
   int4* d_work = nullptr;
+  unsigned int* d_next = nullptr;      // two tile counters per part
   size_t cap_sims = 0, cap_work = 0;
   int n_work = 0;
   struct Part {                        // tiles of one storage and one form of the mass defect: a launch each
@@ -49,9 +51,9 @@ static int rebuild(lbm_batch* b) {
   std::vector<int> members;
   for (size_t i = 0; i < b->slots.size(); ++i)
     if (b->slots[i]) members.push_back((int)i);
-  // interleave the members' tiles so concurrent CTAs spread over simulations; members of different
-  // storages, and those with the direct mass defect, have launches of their own
-  std::vector<std::vector<int4>> per[N_PARTS];
+  // members of different storages, and those with the direct mass defect, have launches of their own; a launch
+  // takes its tiles in order of falling cost (rows, the h + 7 iterations around them, about one more at a wall)
+  std::vector<std::pair<int, int4>> per[N_PARTS];
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -61,7 +63,7 @@ static int rebuild(lbm_batch* b) {
   auto part_of = [](const lbm_sim* s) { return s->params.storage + (s->params.s_form ? 3 : 0); };
   // Rows per tile.  A launch takes as many rounds as its tiles fill of the device's slots, and a round as many row
   // iterations as its tiles have: the height that makes rounds x (h + 7) least, heights evened out within each member
-  // (48 members of the c4 mix: 2 full rounds instead of 3.5, taken as 4, at a fixed 32 rows).
+  // (48 members of the c4 mix, us a step: 179 at the chosen 53 rows, 189 at 40, 198 at 56).
   int rows[N_PARTS];
   for (int part = 0; part < N_PARTS; ++part) {
     std::vector<std::array<int, 3>> shape;   // strips, rows, own rows per tile
@@ -103,20 +105,19 @@ static int rebuild(lbm_batch* b) {
     d.buf1 = s->buf[1];
     d.cur0 = s->cur;
     sims.push_back(d);
-    std::vector<int4> tl;
     const int nseg = march_segs(g);
-    for (int sg = 0; sg < nseg; ++sg)
-      for (int st = 0; st < g.n_strips; ++st) tl.push_back(make_int4((int)m, st, sg, 0));
-    per[part_of(s)].push_back(std::move(tl));
+    for (int sg = 0; sg < nseg; ++sg) {
+      int ya, yb;
+      seg_rows(g, sg, &ya, &yb);
+      const int cost = yb - ya + (g.bc_y == BC_WALL && (sg == 0 || sg == nseg - 1) ? 1 : 0);
+      for (int st = 0; st < g.n_strips; ++st) per[part_of(s)].push_back({cost, make_int4((int)m, st, sg, 0)});
+    }
   }
   lbm_batch::Part parts[N_PARTS];
   for (int part = 0; part < N_PARTS; ++part) {
     parts[part].first = (int)work.size();
-    size_t most = 0;
-    for (auto& v : per[part]) most = std::max(most, v.size());
-    for (size_t k = 0; k < most; ++k)
-      for (auto& v : per[part])
-        if (k < v.size()) work.push_back(v[k]);
+    std::stable_sort(per[part].begin(), per[part].end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+    for (const auto& v : per[part]) work.push_back(v.second);
     parts[part].count = (int)work.size() - parts[part].first;
     parts[part].grid = std::min(parts[part].count, slots);
   }
@@ -143,6 +144,10 @@ static int rebuild(lbm_batch* b) {
       (e = cudaMemcpyAsync(b->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream)) !=
           cudaSuccess)
     return cuda_fail(e, "batch work upload");
+  if (!b->d_next && (e = cudaMalloc(&b->d_next, 2 * N_PARTS * sizeof(unsigned int))) != cudaSuccess)
+    return cuda_fail(e, "batch tile counters");
+  if ((e = cudaMemsetAsync(b->d_next, 0, 2 * N_PARTS * sizeof(unsigned int), b->stream)) != cudaSuccess)
+    return cuda_fail(e, "batch tile counters");
   // host vectors die here: make the uploads complete first
   if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) return cuda_fail(e, "batch upload sync");
   b->n_work = (int)work.size();
@@ -159,7 +164,7 @@ static cudaError_t launch_batch(lbm_batch* b, int parity, cudaStream_t st) {
   for (int k = 0; k < N_PARTS; ++k) {
     const lbm_batch::Part& p = b->parts[k];
     if (p.count == 0) continue;
-    const cudaError_t e = by_storage[k % 3](b->d_sims, b->d_work + p.first, p.count, p.grid, parity, k >= 3, b->xwall, st);
+    const cudaError_t e = by_storage[k % 3](b->d_sims, b->d_work + p.first, p.count, p.grid, parity, b->d_next + 2 * k, k >= 3, b->xwall, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -302,6 +307,7 @@ int lbm_batch_destroy(lbm_batch* b) {
   drop_graphs(b);
   cudaFree(b->d_sims);
   cudaFree(b->d_work);
+  cudaFree(b->d_next);
   if (b->cap) cudaStreamDestroy(b->cap);
   delete b;
   return LBM_OK;
