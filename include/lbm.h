@@ -231,8 +231,7 @@ LBM_API int lbm_restore(lbm_sim* sim, const void* buf, size_t bytes);
 LBM_API int lbm_set_stream(lbm_sim* sim, void* cuda_stream);
 
 /* Tile shape of the row march: rows per CTA (>= 1).  0 keeps the current value; a new simulation has as
- * many rows per CTA as make one wave of resident CTAs (fewer in the CTAs at walls on y, where the wave has
- * CTAs to spare).  threads (64, 128, 256 or 0) is accepted and has
+ * many rows per CTA as make one wave of resident CTAs.  threads (64, 128, 256 or 0) is accepted and has
  * no effect: every CTA has 128 threads of two columns each.  Results do not depend on the shape. */
 LBM_API int lbm_set_tile(lbm_sim* sim, int threads, int seg_rows);
 

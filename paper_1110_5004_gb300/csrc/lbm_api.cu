@@ -63,30 +63,16 @@ Phys make_phys(const lbm_params& p) {
   return P;
 }
 
-void tile_geometry(int nx, int ny, bool sd, bool ywall, int seg_h, int slots, Grid* g) {
+void tile_geometry(int nx, int ny, bool sd, int seg_h, int slots, Grid* g) {
   const int most = 2 * march_width(sd), ns = (nx + most - 1) / most;
   g->n_strips = ns;
   g->tile_w = (nx + 2 * ns - 1) / (2 * ns);
-  g->seg_cut = g->seg_last = 0;
-  int segs = slots >= ns ? slots / ns : 1;
   // as many segments as fit in one wave of `slots` resident CTAs: the step lasts as long as the
   // busiest SM, so a count just above the slots adds a nearly empty wave.  Segments of a few rows spend
   // most of their h + 7 iterations on the rows around them, and are still the fastest where the grid has
   // no more rows to give (601 x 437 with side walls: 18.1 us at 5 rows, 22.4 at 8)
-  seg_h = seg_h <= 0 ? (ny + segs - 1) / segs : std::min(seg_h, ny);
-  segs = std::max(segs, (ny + seg_h - 1) / seg_h);
-  // A segment that meets a wall row takes longer by about a row (checked iterations, a row that bounces back
-  // cell by cell), and the step waits for it.  Where the wave has segments to spare, the first and the last
-  // are shorter; not below 5 rows, or their neighbours' rows around them would meet the wall too.  2048 x 512:
-  // FP32 34.9 -> 33.0 us, FP16 33.2 -> 30.0.
-  if (ywall && seg_h > 5 && seg_h < ny) {
-    const int c = (int)std::min(((long long)segs * seg_h - ny) / 2, (long long)seg_h - 5);
-    if (c > 0) {
-      g->seg_cut = c;
-      g->seg_last = seg_h - c;
-    }
-  }
-  g->seg_h = seg_h;
+  const int segs = slots >= ns ? slots / ns : 1;
+  g->seg_h = seg_h <= 0 ? (ny + segs - 1) / segs : std::min(seg_h, ny);
 }
 
 Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
@@ -102,7 +88,7 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
   g.pitch = s->pitch;
   g.bc_x = s->params.bc_x;
   g.bc_y = s->params.bc_y;
-  tile_geometry(s->nx, s->ny, s->params.s_form != 0, s->params.bc_y == LBM_WALL, s->seg_h, s->sms * MARCH_CTAS, &g);
+  tile_geometry(s->nx, s->ny, s->params.s_form != 0, s->seg_h, s->sms * MARCH_CTAS, &g);
   g.gave_up = gave_up(s);
   g.spoff = s->params.s_form ? (long long)s->pop_bytes : 0;
   return g;

@@ -52,7 +52,7 @@ static int rebuild(lbm_batch* b) {
   for (size_t i = 0; i < b->slots.size(); ++i)
     if (b->slots[i]) members.push_back((int)i);
   // members of different storages, and those with the direct mass defect, have launches of their own; a launch
-  // takes its tiles in order of falling cost (rows, the h + 7 iterations around them, about one more at a wall)
+  // takes its tiles in order of falling height
   std::vector<std::pair<int, int4>> per[N_PARTS];
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -63,7 +63,7 @@ static int rebuild(lbm_batch* b) {
   auto part_of = [](const lbm_sim* s) { return s->params.storage + (s->params.s_form ? 3 : 0); };
   // Rows per tile.  A launch takes as many rounds as its tiles fill of the device's slots, and a round as many row
   // iterations as its tiles have: the height that makes rounds x (h + 7) least, heights evened out within each member
-  // (48 members of the c4 mix, us a step: 179 at the chosen 53 rows, 189 at 40, 198 at 56).
+  // (48 members of the c4 mix, us a step: 171 at the chosen 53 rows, 193 at 56).
   int rows[N_PARTS];
   for (int part = 0; part < N_PARTS; ++part) {
     std::vector<std::array<int, 3>> shape;   // strips, rows, own rows per tile
@@ -71,7 +71,7 @@ static int rebuild(lbm_batch* b) {
       const lbm_sim* s = b->slots[m];
       if (part_of(s) != part) continue;
       Grid g{};
-      tile_geometry(s->nx, s->ny, s->params.s_form != 0, false, 1, 0, &g);
+      tile_geometry(s->nx, s->ny, s->params.s_form != 0, 1, 0, &g);
       shape.push_back({g.n_strips, s->ny, s->seg_h ? s->seg_h : b->seg_h});
     }
     long long best = -1;
@@ -99,18 +99,16 @@ static int rebuild(lbm_batch* b) {
       const int segs = (s->ny + rows[part_of(s)] - 1) / rows[part_of(s)];
       h = (s->ny + segs - 1) / segs;
     }
-    tile_geometry(s->nx, s->ny, s->params.s_form != 0, false, h, 0, &g);
+    tile_geometry(s->nx, s->ny, s->params.s_form != 0, h, 0, &g);
     d.g = g;
     d.buf0 = s->buf[0];
     d.buf1 = s->buf[1];
     d.cur0 = s->cur;
     sims.push_back(d);
-    const int nseg = march_segs(g);
+    const int nseg = (s->ny + g.seg_h - 1) / g.seg_h;
     for (int sg = 0; sg < nseg; ++sg) {
-      int ya, yb;
-      seg_rows(g, sg, &ya, &yb);
-      const int cost = yb - ya + (g.bc_y == BC_WALL && (sg == 0 || sg == nseg - 1) ? 1 : 0);
-      for (int st = 0; st < g.n_strips; ++st) per[part_of(s)].push_back({cost, make_int4((int)m, st, sg, 0)});
+      const int tile_rows = std::min(g.seg_h, s->ny - sg * g.seg_h);
+      for (int st = 0; st < g.n_strips; ++st) per[part_of(s)].push_back({tile_rows, make_int4((int)m, st, sg, 0)});
     }
   }
   lbm_batch::Part parts[N_PARTS];

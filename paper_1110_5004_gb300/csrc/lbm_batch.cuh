@@ -29,9 +29,9 @@ struct BatchSmem {
 // did not fit 255 registers (1.2-1.9 KB of spills per thread).  XW: some member may have walls on x.
 //
 // A CTA takes its first tile by its index and further ones from a counter, the list being in order of falling
-// cost: tiles differ in height, those at walls cost more, and CTAs that share no SM run faster, so that fixed rounds
+// height: tiles differ in it, and CTAs that share no SM run faster, so that fixed rounds
 // left CTAs idle (us a step, FP32 and BF16: 48 members 184 and 194 -> 179 and 187, 256 members 1036 and 1028 -> 971
-// and 997).  next: two counters; a launch uses the one of its
+// and 997; 171 and 171, 935 and 947 since the march has one row body, which left no spills here).  next: two counters; a launch uses the one of its
 // parity, zero when it starts, and clears the other for the launch that follows it on the stream.
 template <int ST, bool SD, bool XW>
 __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* __restrict__ sims, const int4* __restrict__ work,

@@ -240,22 +240,10 @@ struct Grid {
   int bc_x, bc_y;
   int tile_w;           // columns per lane of a row-march CTA (a CTA covers two lanes)
   int seg_h;            // rows per segment
-  int seg_cut;          // rows by which the first segment is shorter
-  int seg_last;         // rows of the last segment (0: whatever the others leave)
   int n_strips;         // CTAs across the grid
   unsigned int* gave_up; // raised by a wait that ran out (never in a sound run)
   long long spoff;      // s_form 1: byte offset of the [rho, div(rho u)] planes in src/dst (else 0)
 };
-
-// Segments of the row march, and the rows [ya, yb) of one.
-__host__ __device__ __forceinline__ int march_segs(const Grid& g) {
-  return (g.ny - g.seg_last + g.seg_cut + g.seg_h - 1) / g.seg_h + (g.seg_last > 0 ? 1 : 0);
-}
-__host__ __device__ __forceinline__ void seg_rows(const Grid& g, int seg, int* ya, int* yb) {
-  const int body = g.ny - g.seg_last, a = seg * g.seg_h - g.seg_cut, b = a + g.seg_h;
-  *ya = a < 0 ? 0 : (a < body ? a : body);
-  *yb = a >= body ? g.ny : (b < body ? b : body);
-}
 
 // Outputs of the moment pass (row-major); each may be null.  fax, fay: the
 // additional interfacial force F_a = -u s of Eq. 12 (s by the simulation's s_form), evaluated

@@ -64,7 +64,7 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst);
 // Lane width, strip count and segment height of the row march for an nx x ny grid: strips of two lanes of
 // at most march_width(sd) columns, all alike; seg_h = 0 picks the height that puts about one full wave of CTAs
 // (slots = SMs x CTAs per SM) on the device.
-void tile_geometry(int nx, int ny, bool sd, bool ywall, int seg_h, int slots, Grid* g);
+void tile_geometry(int nx, int ny, bool sd, int seg_h, int slots, Grid* g);
 // The small-grid step kernel (lbm_tile2d.cu): s_form 0 and f_form 0.
 bool tile2d_eligible(const lbm_params& p);
 // 384-thread CTAs when the grid's tiles fit one wave of them on `sms` multiprocessors, else 256.

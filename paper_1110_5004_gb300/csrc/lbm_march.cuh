@@ -24,7 +24,7 @@
 // 32 cells, 4.6-5.8 cycles per cell at best, and its warps waited 30-48 % of their time on loads that one row of
 // register prefetch could not cover (more warps or L2 prefetches only thrashed L1).  This form issues 380 per 32 cells.
 // 4096 x 4096: 527 -> 408 us a step (152 B per cell at 0.92 of the measured copy bandwidth); 2048 x 512 with walls on y:
-// 40.8 -> 33.0, of which 1.5 us pass between two launches, 5.3 in the iterations before a segment's first S3 (1.4 of
+// 40.8 -> 32.4, of which 1.5 us pass between two launches, 5.3 in the iterations before a segment's first S3 (1.4 of
 // them for the first row), 1.4 in each of the others.  What bounds an iteration is a warp's own chain of about 760
 // instructions at 4.3 cycles (2 warps per scheduler; issue slots half used, shared-memory pipe 65 %): warps that skip
 // columns beyond the halo, or more rows in flight, change nothing.
@@ -138,76 +138,47 @@ struct OutLanes {
       x[a] = B ? hi : lo;
     }
   }
-  // next to a wall: cell by cell
-  template <bool B, class Out>
-  __device__ __forceinline__ void store_cell(const Out& o) const {
-    float x[Q + Q + 1];
-    lane<B>(x);
-    o.template put<0>(x[0]);
-    o.template put<1>(x[1]);
-    o.template put<2>(x[2]);
-    o.template put<3>(x[3]);
-    o.template put<4>(x[4]);
-    o.template put<5>(x[5]);
-    o.template put<6>(x[6]);
-    o.template put<7>(x[7]);
-    o.template put<8>(x[8]);
-    o.template put<9>(x[9]);
-    o.template put<10>(x[10]);
-    o.template put<11>(x[11]);
-    o.template put<12>(x[12]);
-    o.template put<13>(x[13]);
-    o.template put<14>(x[14]);
-    o.template put<15>(x[15]);
-    o.template put<16>(x[16]);
-    o.template put<17>(x[17]);
-    if constexpr (ST == ST_FP32) o.template put<A_F0LO>(x[A_F0LO]);
-  }
-  // rows: the destination buffer's rows y-1, y, y+1; c: the lane's column; key: its BF16 rounding place.  XW: the column
-  // may lie at the left (wl) or the right (wr) wall; the populations that would cross it go back reversed, to the
-  // column xw beyond the wall (wrapped), row y.
+  // rows: the destination buffer's rows y-1, y, y+1; x: the lane's column; key: its BF16 rounding place.  wb, wt: the row
+  // lies at the bottom or the top wall (uniform); XW: the column may lie at the left (wl) or the right (wr) wall.  The
+  // populations that would cross a wall go back reversed: to row y, column x + e_x (wrapped).  (Storing all
+  // populations of such a cell by tests of their own instead took a row body for the segments at walls on y, cold code
+  // that few CTAs ran: a step after a flush of L2 42 us against 37 on 2048 x 512; and with walls on x 39.5 against 37.6
+  // on 1200 x 900.)
   template <bool B, bool XW>
-  __device__ __forceinline__ void store_lane(char* rm, char* r0, char* rq, const ColB& c, int nblk, unsigned int key, bool on, bool wl,
-                                             bool wr, int xw) const {
+  __device__ __forceinline__ void store_lane(const Grid& gr, char* rm, char* r0, char* rq, int x_, unsigned int key, bool on, bool wl,
+                                             bool wr, bool wb, bool wt) const {
     float x[Q + Q + 1];
     lane<B>(x);
-    if constexpr (XW) {
-      if (on && (wl || wr)) {
-        const ColB cw = col_bytes<ST>(xw);
-        auto back = [&](auto pop) {   // population A of the right wall, its mirror image of the left
-          constexpr int A = decltype(pop)::value, M = opp(A % Q) + (A >= Q ? Q : 0);
-          char* const q = r0 + region_start(ST, region_of(A)) * nblk + (wr ? pop_in_region<ST>(M, cw) : pop_in_region<ST>(A, cw));
-          if constexpr (ST == ST_FP32) *reinterpret_cast<float*>(q) = wr ? x[A] : x[M];
-          else *reinterpret_cast<unsigned short*>(q) = wr ? enc_pop<ST>(x[A], A, key) : enc_pop<ST>(x[M], M, key);
-        };
-        back(std::integral_constant<int, 1>{});
-        back(std::integral_constant<int, 5>{});
-        back(std::integral_constant<int, 8>{});
-        back(std::integral_constant<int, Q + 1>{});
-        back(std::integral_constant<int, Q + 5>{});
-        back(std::integral_constant<int, Q + 8>{});
-      }
-    }
+    const int nblk = gr.nblk;
+    const ColB c = col_bytes<ST>(x_);
     const int right = on && !(XW && wr), left = on && !(XW && wl);
+    const int up = on && !wt, down = on && !wb, up_r = right && !wt, up_l = left && !wt, down_r = right && !wb, down_l = left && !wb;
     const int g = region_start(ST, R_G) * nblk + c.g;
     static_assert(BLK == 32, "offsets below");
     if constexpr (ST == ST_FP32) {
       asm volatile(
-          "{\n\t.reg .pred q, r, l;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %13, 0;\n\tsetp.ne.s32 l, %14, 0;\n\t"
-          "@q st.global.f32 [%1+256], %4;\n\t@r st.global.f32 [%1+640], %5;\n\t@l st.global.f32 [%1+768], %6;\n\t"
+          "{\n\t.reg .pred q, r, l, t, tr, tl, b, br, bl;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %13, 0;\n\tsetp.ne.s32 l, %14, 0;\n\t"
+          "setp.ne.s32 t, %15, 0;\n\tsetp.ne.s32 tr, %16, 0;\n\tsetp.ne.s32 tl, %17, 0;\n\tsetp.ne.s32 b, %18, 0;\n\t"
+          "setp.ne.s32 br, %19, 0;\n\tsetp.ne.s32 bl, %20, 0;\n\t"
+          "@t st.global.f32 [%1+256], %4;\n\t@tr st.global.f32 [%1+640], %5;\n\t@tl st.global.f32 [%1+768], %6;\n\t"
           "@q st.global.f32 [%2], %7;\n\t@r st.global.f32 [%2+128], %8;\n\t@l st.global.f32 [%2+384], %9;\n\t"
-          "@q st.global.f32 [%3+512], %10;\n\t@l st.global.f32 [%3+896], %11;\n\t@r st.global.f32 [%3+1024], %12;\n\t}" ::"r"(
+          "@b st.global.f32 [%3+512], %10;\n\t@bl st.global.f32 [%3+896], %11;\n\t@br st.global.f32 [%3+1024], %12;\n\t}" ::"r"(
               (int)on),
           "l"(rq + g), "l"(r0 + g), "l"(rm + g), "f"(x[Q + 2]), "f"(x[Q + 5]), "f"(x[Q + 6]), "f"(x[Q + 0]), "f"(x[Q + 1]),
-          "f"(x[Q + 3]), "f"(x[Q + 4]), "f"(x[Q + 7]), "f"(x[Q + 8]), "r"(right), "r"(left));
+          "f"(x[Q + 3]), "f"(x[Q + 4]), "f"(x[Q + 7]), "f"(x[Q + 8]), "r"(right), "r"(left), "r"(up), "r"(up_r), "r"(up_l),
+          "r"(down), "r"(down_r), "r"(down_l));
       asm volatile(
-          "{\n\t.reg .pred q, r, l;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %15, 0;\n\tsetp.ne.s32 l, %16, 0;\n\t"
-          "@q st.global.f32 [%1+256], %5;\n\t@r st.global.f32 [%1+640], %6;\n\t@l st.global.f32 [%1+768], %7;\n\t"
+          "{\n\t.reg .pred q, r, l, t, tr, tl, b, br, bl;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %15, 0;\n\tsetp.ne.s32 l, %16, 0;\n\t"
+          "setp.ne.s32 t, %17, 0;\n\tsetp.ne.s32 tr, %18, 0;\n\tsetp.ne.s32 tl, %19, 0;\n\tsetp.ne.s32 b, %20, 0;\n\t"
+          "setp.ne.s32 br, %21, 0;\n\tsetp.ne.s32 bl, %22, 0;\n\t"
+          "@t st.global.f32 [%1+256], %5;\n\t@tr st.global.f32 [%1+640], %6;\n\t@tl st.global.f32 [%1+768], %7;\n\t"
           "@q st.global.f32 [%2], %8;\n\t@r st.global.f32 [%2+128], %9;\n\t@l st.global.f32 [%2+384], %10;\n\t"
-          "@q st.global.f32 [%3+512], %11;\n\t@l st.global.f32 [%3+896], %12;\n\t@r st.global.f32 [%3+1024], %13;\n\t"
+          "@b st.global.f32 [%3+512], %11;\n\t@bl st.global.f32 [%3+896], %12;\n\t@br st.global.f32 [%3+1024], %13;\n\t"
           "@q st.global.f32 [%4], %14;\n\t}" ::"r"((int)on),
           "l"(rq + c.f4), "l"(r0 + c.f4), "l"(rm + c.f4), "l"(r0 + region_start(ST, R_L) * nblk + c.l), "f"(x[2]), "f"(x[5]),
-          "f"(x[6]), "f"(x[0]), "f"(x[1]), "f"(x[3]), "f"(x[4]), "f"(x[7]), "f"(x[8]), "f"(x[A_F0LO]), "r"(right), "r"(left));
+          "f"(x[6]), "f"(x[0]), "f"(x[1]), "f"(x[3]), "f"(x[4]), "f"(x[7]), "f"(x[8]), "f"(x[A_F0LO]), "r"(right), "r"(left), "r"(up), "r"(up_r), "r"(up_l),
+          "r"(down), "r"(down_r), "r"(down_l));
+      if (wl || wr || wb || wt) back<XW>(gr, r0, x_, on, wl, wr, wb, wt, [&](auto a) { return x[decltype(a)::value]; });
     } else {
       unsigned short h[Q + Q];
 #pragma unroll
@@ -222,33 +193,71 @@ struct OutLanes {
         h[Q + Q - 1] = enc_pop<ST>(x[Q + Q - 1], Q + Q - 1, key);
       }
       asm volatile(
-          "{\n\t.reg .pred q, r, l;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %13, 0;\n\tsetp.ne.s32 l, %14, 0;\n\t"
-          "@q st.global.u16 [%1+128], %4;\n\t@r st.global.u16 [%1+320], %5;\n\t@l st.global.u16 [%1+384], %6;\n\t"
+          "{\n\t.reg .pred q, r, l, t, tr, tl, b, br, bl;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %13, 0;\n\tsetp.ne.s32 l, %14, 0;\n\t"
+          "setp.ne.s32 t, %15, 0;\n\tsetp.ne.s32 tr, %16, 0;\n\tsetp.ne.s32 tl, %17, 0;\n\tsetp.ne.s32 b, %18, 0;\n\t"
+          "setp.ne.s32 br, %19, 0;\n\tsetp.ne.s32 bl, %20, 0;\n\t"
+          "@t st.global.u16 [%1+128], %4;\n\t@tr st.global.u16 [%1+320], %5;\n\t@tl st.global.u16 [%1+384], %6;\n\t"
           "@q st.global.u16 [%2], %7;\n\t@r st.global.u16 [%2+64], %8;\n\t@l st.global.u16 [%2+192], %9;\n\t"
-          "@q st.global.u16 [%3+256], %10;\n\t@l st.global.u16 [%3+448], %11;\n\t@r st.global.u16 [%3+512], %12;\n\t}" ::"r"(
+          "@b st.global.u16 [%3+256], %10;\n\t@bl st.global.u16 [%3+448], %11;\n\t@br st.global.u16 [%3+512], %12;\n\t}" ::"r"(
               (int)on),
           "l"(rq + g), "l"(r0 + g), "l"(rm + g), "h"(h[Q + 2]), "h"(h[Q + 5]), "h"(h[Q + 6]), "h"(h[Q + 0]), "h"(h[Q + 1]),
-          "h"(h[Q + 3]), "h"(h[Q + 4]), "h"(h[Q + 7]), "h"(h[Q + 8]), "r"(right), "r"(left));
+          "h"(h[Q + 3]), "h"(h[Q + 4]), "h"(h[Q + 7]), "h"(h[Q + 8]), "r"(right), "r"(left), "r"(up), "r"(up_r), "r"(up_l),
+          "r"(down), "r"(down_r), "r"(down_l));
       asm volatile(
-          "{\n\t.reg .pred q, r, l;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %14, 0;\n\tsetp.ne.s32 l, %15, 0;\n\t"
-          "@q st.global.u16 [%1+192], %5;\n\t@r st.global.u16 [%1+384], %6;\n\t@l st.global.u16 [%1+448], %7;\n\t"
+          "{\n\t.reg .pred q, r, l, t, tr, tl, b, br, bl;\n\tsetp.ne.s32 q, %0, 0;\n\tsetp.ne.s32 r, %14, 0;\n\tsetp.ne.s32 l, %15, 0;\n\t"
+          "setp.ne.s32 t, %16, 0;\n\tsetp.ne.s32 tr, %17, 0;\n\tsetp.ne.s32 tl, %18, 0;\n\tsetp.ne.s32 b, %19, 0;\n\t"
+          "setp.ne.s32 br, %20, 0;\n\tsetp.ne.s32 bl, %21, 0;\n\t"
+          "@t st.global.u16 [%1+192], %5;\n\t@tr st.global.u16 [%1+384], %6;\n\t@tl st.global.u16 [%1+448], %7;\n\t"
           "@r st.global.u16 [%2+128], %8;\n\t@l st.global.u16 [%2+256], %9;\n\t"
-          "@q st.global.u16 [%3+320], %10;\n\t@l st.global.u16 [%3+512], %11;\n\t@r st.global.u16 [%3+576], %12;\n\t"
+          "@b st.global.u16 [%3+320], %10;\n\t@bl st.global.u16 [%3+512], %11;\n\t@br st.global.u16 [%3+576], %12;\n\t"
           "@q st.global.f32 [%4], %13;\n\t}" ::"r"((int)on),
           "l"(rq + c.f2), "l"(r0 + c.f2), "l"(rm + c.f2), "l"(r0 + c.f4), "h"(h[2]), "h"(h[5]), "h"(h[6]), "h"(h[1]), "h"(h[3]),
-          "h"(h[4]), "h"(h[7]), "h"(h[8]), "f"(x[0]), "r"(right), "r"(left));
+          "h"(h[4]), "h"(h[7]), "h"(h[8]), "f"(x[0]), "r"(right), "r"(left), "r"(up), "r"(up_r), "r"(up_l),
+          "r"(down), "r"(down_r), "r"(down_l));
+      if (wl || wr || wb || wt) back<XW>(gr, r0, x_, on, wl, wr, wb, wt, [&](auto a) { return h[decltype(a)::value]; });
+    }
+  }
+
+  // The populations that cross a wall, from value(a).
+  template <bool XW, class F>
+  __device__ __forceinline__ static void back(const Grid& g, char* r0, int x, bool on, bool wl, bool wr, bool wb, bool wt, F value) {
+    const ColB c = col_bytes<ST>(x), cq = col_bytes<ST>(x == g.nx - 1 ? 0 : x + 1), cm = col_bytes<ST>(x == 0 ? g.nx - 1 : x - 1);
+    // population first ? A : opp(A), to the reversed population at column to
+    auto put = [&](auto pop, bool first, const ColB& to) {
+      constexpr int A = decltype(pop)::value, M = opp(A % Q) + (A >= Q ? Q : 0);
+      char* const q = r0 + region_start(ST, region_of(A)) * g.nblk + (first ? pop_in_region<ST>(M, to) : pop_in_region<ST>(A, to));
+      const auto v = first ? value(std::integral_constant<int, A>{}) : value(std::integral_constant<int, M>{});
+      if (on) *reinterpret_cast<std::remove_const_t<decltype(v)>*>(q) = v;
+    };
+    if (wb || wt) {
+      put(std::integral_constant<int, 2>{}, wt, c);
+      put(std::integral_constant<int, 5>{}, wt, wt ? cq : cm);
+      put(std::integral_constant<int, 6>{}, wt, wt ? cm : cq);
+      put(std::integral_constant<int, Q + 2>{}, wt, c);
+      put(std::integral_constant<int, Q + 5>{}, wt, wt ? cq : cm);
+      put(std::integral_constant<int, Q + 6>{}, wt, wt ? cm : cq);
+    }
+    if (XW && (wl || wr)) {
+      const ColB& cw = wr ? cq : cm;
+      put(std::integral_constant<int, 1>{}, wr, cw);
+      put(std::integral_constant<int, 5>{}, wr, cw);
+      put(std::integral_constant<int, 8>{}, wr, cw);
+      put(std::integral_constant<int, Q + 1>{}, wr, cw);
+      put(std::integral_constant<int, Q + 5>{}, wr, cw);
+      put(std::integral_constant<int, Q + 8>{}, wr, cw);
     }
   }
 };
 
-// One row iteration (kinds):
-//   IT_CHECKED  a wall row may be among the rows: every stage tests its row range and fills ghost rows.
-//   IT_FILL     the first iterations of a segment that touches no wall row: no S3 yet, S2 from its
-//               first needed row on.
-//   IT_INNER    no row test and no branch.
+// One row iteration (kinds).  Rows at a wall on y have no kind of their own: their stencils take the row itself for the
+// one beyond it, and their stores turn back what crosses the wall.  (A third, checked body for segments at a wall: 228
+// instead of 208 registers, spills in the batch, and those segments the slowest: 2048 x 512 FP32 35.0 us a step against
+// 32.4, FP16 33.2 against 29.4; 900 x 300 14.6 against 13.1; 48 batched members BF16 187 against 171.)
+//   IT_FILL     the first iterations of a segment: no S3 yet, S2 from its first needed row on.
+//   IT_INNER    all stages.
 // Threads whose column a stage does not need compute it anyway, from whatever the rings hold;
 // only stores to the new state (and, with walls on x, to the rings) are predicated.
-enum { IT_CHECKED = 0, IT_FILL = 1, IT_INNER = 2 };
+enum { IT_FILL = 1, IT_INNER = 2 };
 
 // The stage the next row of f (or gbar) is read from, and the parity of its barrier.
 struct StageAt {
@@ -274,8 +283,8 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
   const int w = g.tile_w;
   const int x0 = strip * 2 * w;
   const int wa = min(w, g.nx - x0), wb = min(w, g.nx - x0 - w);   // columns of each lane (wb may be < 1)
-  int ya, yb;
-  seg_rows(g, seg, &ya, &yb);
+  const int ya = seg * g.seg_h;
+  const int yb = min(ya + g.seg_h, g.ny);
   const int te = min(t, w + 5);                    // threads beyond the halo repeat its last column
   const int xla = x0 - 3 + te, xlb = xla + w;      // logical columns (may lie outside [0, nx))
   const int xpa = wrap1(xla, g.nx), xpb = wrap1(xlb, g.nx);
@@ -357,7 +366,6 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
   constexpr int HI = offsetof(typename S::Row5, hi), LO = offsetof(typename S::Row5, lo);
   constexpr int MU = offsetof(typename S::Row3, mu), PP = offsetof(typename S::Row3, p), UX = offsetof(typename S::Row3, ux),
                 UY = offsetof(typename S::Row3, uy), JX = offsetof(typename S::Row3, j), JY = JX + 8 * NT;
-  auto row_ok = [&](int r) { return !ywall || (r >= 0 && r < g.ny); };
   // The lanes whose column is real store it, and next to a wall on x also its mirror image in the ghost column.
   // Threads away from the walls store both lanes at once.
   const bool plain = !XW || (real_a && real_b && tga < 0 && tgb < 0);
@@ -371,11 +379,11 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     if (tgb >= 0) f[2 * (tgb - t) + 1] = y;
   };
   auto put = [&](int off, V2 v) { *at(off) = v; };
-  // Offsets of the rows south and north of row r.  Beyond a wall they are the row itself, its mirror image.
-  auto south = [&](int r, int s, int c, auto kind) { return decltype(kind)::value == IT_CHECKED && ywall && r == 0 ? c : s; };
-  auto north = [&](int r, int n, int c, auto kind) {
-    return decltype(kind)::value == IT_CHECKED && ywall && r == g.ny - 1 ? c : n;
-  };
+  // Offsets of the rows south and north of row r.  Beyond a wall they are the row itself, its mirror image.  (The rows
+  // beyond it go through the stages too, from the wrapped rows of the grid: no valid row reads what they leave.)
+  const int wall_lo = ywall ? 0 : -8, wall_hi = ywall ? g.ny - 1 : g.ny + 8;
+  auto south = [&](int r, int s, int c) { return r == wall_lo ? c : s; };
+  auto north = [&](int r, int n, int c) { return r == wall_hi ? c : n; };
 
   // ---- population pop of both lanes from a staged region
   auto staged = [&](const unsigned char* reg, auto pop, const ColB& a, const ColB& b) {
@@ -426,13 +434,10 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
 
   auto iter = [&](int a, auto kind) {
     constexpr int KIND = decltype(kind)::value;
-    constexpr bool CK = KIND == IT_CHECKED, IN = KIND == IT_INNER;
+    constexpr bool IN = KIND == IT_INNER;
     const int fs = fat.stage, gs = gat.stage;
     const int r1 = a - 1, r2 = a - 3, r3 = a - 4;   // rows of S1, S2, S3
     const bool s2_runs = IN || a >= ya + 2;
-    const bool do0 = !CK || (row_ok(a) && a <= yb + 2);
-    const bool do1 = !CK || (r1 >= ya - 2 && r1 <= yb + 1 && row_ok(r1));
-    const bool do2 = s2_runs && (!CK || row_ok(r2));
     // ================ phase 1: S0 and S2; all stores to the rings at its end
     mbar_wait(&sm.fbar[fs], fat.parity, g.gave_up);
     if (s2_runs) mbar_wait(&sm.gbar[gs], gat.parity, g.gave_up);
@@ -447,7 +452,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     // ---- S2: u, p at row a-3 (rows a-4 .. a-2 of phi and mu)
     S2Out<V2> o;
     auto stage2 = [&] {
-      const int c3 = q3[0], s3 = south(r2, q3[1], c3, kind), n3 = north(r2, q3[2], c3, kind);
+      const int c3 = q3[0], s3 = south(r2, q3[1], c3), n3 = north(r2, q3[2], c3);
       const V2 *ms = at(s3 + MU), *m0 = at(c3 + MU), *mn = at(n3 + MU);
       const V2 ph = pg3.ph, gphx = pg3.gx, gphy = pg3.gy;
       V2 gmx, gmy;                                 // 12 x the isotropic gradient
@@ -497,15 +502,12 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
         }
       }
     };
-    if (do0) stage0();
-    if (do2) stage2();
-    else if (MODE == MODE_STEP && s2_runs) shift();   // (a row beyond a wall has no record)
+    stage0();
+    if (s2_runs) stage2();
     auto puts1 = [&](auto put_) {
-      if (do0) {
-        put_(q5[0] + HI, hi);
-        put_(q5[0] + LO, lo);
-      }
-      if (do2) {
+      put_(q5[0] + HI, hi);
+      put_(q5[0] + LO, lo);
+      if (s2_runs) {
         put_(q3[0] + PP, o.p);
         if constexpr (MODE == MODE_STEP) {
           put_(q3[0] + UX, o.ux);
@@ -519,7 +521,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     };
     if (!XW || plain) puts1(put);
     else puts1(put_wall);
-    if (MODE == MODE_STEP && do0) {
+    if (MODE == MODE_STEP) {
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         *reinterpret_cast<ulonglong2*>(base + q5[0] + t * 8 + k * NT * 16) = make_ulonglong2(fp[2 * k + 1].v, fp[2 * k + 2].v);
@@ -532,7 +534,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     // ---- S1: mu at row a-1 (rows a-2 .. a of phi)
     V2 mu;
     auto stage1 = [&] {
-      const int c = q5[1], sr = south(r1, q5[2], c, kind), n = north(r1, q5[0], c, kind);
+      const int c = q5[1], sr = south(r1, q5[2], c), n = north(r1, q5[0], c);
       mu = chem_potential(P, at(sr + HI), at(c + HI), at(n + HI), at(sr + LO), at(c + LO), at(n + LO));
       // grad phi only feeds grad rho (density and pressure terms): the high words suffice
       pg2.ph = fadd(*at(c + HI), *at(c + LO));
@@ -540,7 +542,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     };
     // ---- S3: collide and store row a-4 (p, u of rows a-5 .. a-3)
     auto stage3 = [&] {
-      const int c = q3[1], os = south(r3, q3[2], c, kind), on = north(r3, q3[0], c, kind);
+      const int c = q3[1], os = south(r3, q3[2], c), on = north(r3, q3[0], c);
       V2 gpx, gpy;                                 // 12 grad p
       grad12(P, at(os + PP), at(c + PP), at(on + PP), gpx, gpy);
       // phi div(u) of the convective form; computed either way, so that no branch splits the block
@@ -568,33 +570,21 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
       }
       OutLanes<ST> out;
       collide_store<ST, FF>(P, prev, *at(c + PP), gpx, gpy, *at(q5[4] + HI), *at(q5[4] + LO), phiD, f, gprev, out);
-      // a row next to a wall, where populations bounce back, takes the general path
-      const bool wrow = CK && ywall && (r3 == 0 || r3 == g.ny - 1);
       char* const dst = static_cast<char*>(g.dst);
       char* const row0 = dst + (long long)r3 * g.row_bytes;
       char* const rowm = r3 == 0 ? dst + (long long)(g.ny - 1) * g.row_bytes : row0 - g.row_bytes;
       char* const rowq = r3 == g.ny - 1 ? dst : row0 + g.row_bytes;
-      if constexpr (CK) {
-        if (on_a && wrow) out.template store_cell<false>(out_cell<ST, XW, true>(g, xpa, r3));
-        if (on_b && wrow) out.template store_cell<true>(out_cell<ST, XW, true>(g, xpb, r3));
-      }
-      const bool wr_a = xwall && xla == g.nx - 1, wr_b = xwall && xlb == g.nx - 1;
-      out.template store_lane<false, XW>(rowm, row0, rowq, col_bytes<ST>(xpa), g.nblk, hash_key<ST>(xpa, r3, g), on_a && !wrow,
-                                         xwall && xla == 0, wr_a, wr_a ? 0 : g.nx - 1);
-      out.template store_lane<true, XW>(rowm, row0, rowq, col_bytes<ST>(xpb), g.nblk, hash_key<ST>(xpb, r3, g), on_b && !wrow,
-                                        xwall && xlb == 0, wr_b, wr_b ? 0 : g.nx - 1);
+      const bool wb = r3 == wall_lo, wt = r3 == wall_hi;
+      out.template store_lane<false, XW>(g, rowm, row0, rowq, xpa, hash_key<ST>(xpa, r3, g), on_a, xwall && xla == 0,
+                                         xwall && xla == g.nx - 1, wb, wt);
+      out.template store_lane<true, XW>(g, rowm, row0, rowq, xpb, hash_key<ST>(xpb, r3, g), on_b, xwall && xlb == 0,
+                                        xwall && xlb == g.nx - 1, wb, wt);
     };
     pg3 = pg2;
-    if (do1) stage1();
-    if constexpr (MODE == MODE_STEP) {
-      if constexpr (IN) stage3();
-      if constexpr (CK)
-        if (a >= ya + 4) stage3();
-    }
-    if (do1) {
-      if (!XW || plain) put(q3[1] + MU, mu);
-      else put_wall(q3[1] + MU, mu);
-    }
+    stage1();
+    if constexpr (MODE == MODE_STEP && IN) stage3();
+    if (!XW || plain) put(q3[1] + MU, mu);
+    else put_wall(q3[1] + MU, mu);
     {
       const int x5 = q5[RING5 - 1], x3 = q3[RING3 - 1];
 #pragma unroll
@@ -609,20 +599,11 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     __syncthreads();
   };
 
-  using Checked = std::integral_constant<int, IT_CHECKED>;
   using Fill = std::integral_constant<int, IT_FILL>;
   using Inner = std::integral_constant<int, IT_INNER>;
   int a = ya - 3;
-  // S0 meets a wall row only in segments within 4 rows of a wall; a periodic y axis has none
-  if (!ywall || (ya >= 4 && yb + 3 <= g.ny - 2)) {
-    for (; a < ya + 4 && a <= a_end; ++a) iter(a, Fill{});
-    for (; a <= a_end; ++a) iter(a, Inner{});
-  } else {
-    const int a_in0 = max(ya + 4, 5), a_in1 = min(a_end, g.ny - 2);
-    for (; a < a_in0 && a <= a_end; ++a) iter(a, Checked{});
-    for (; a <= a_in1; ++a) iter(a, Inner{});
-    for (; a <= a_end; ++a) iter(a, Checked{});
-  }
+  for (; a < ya + 4 && a <= a_end; ++a) iter(a, Fill{});
+  for (; a <= a_end; ++a) iter(a, Inner{});
 }
 
 }  // namespace lbm

@@ -23,7 +23,7 @@ static cudaError_t launch_march(const Phys2& P, const Grid& g, const MomentOut& 
   static const cudaError_t attr_set = cudaFuncSetAttribute(
       k_march<MODE, ST, SD, FF, XW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MarchSmem<ST, SD>));
   if (attr_set != cudaSuccess) return attr_set;
-  const int tiles = g.n_strips * march_segs(g);
+  const int tiles = g.n_strips * ((g.ny + g.seg_h - 1) / g.seg_h);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(tiles);
   cfg.blockDim = dim3(MARCH_NT);

@@ -102,9 +102,9 @@ def test_march_only_forms_match_oracle(lbm, nx, form):
 @pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny", [(2000, 165), (2000, 198), (2000, 197), (2000, 196), (2000, 190), (2100, 520), (4900, 77),
                                    (40, 3200), (73000, 9)])
-def test_uneven_segments_at_y_walls_equal_even_ones(lbm, nx, ny):
-    """Automatic heights of 5 rows (even segments), 6 and more (shorter ones at the walls, with no, one or many rows to
-    spare), and 20 rows by choice, against 5 rows everywhere: step and moments, bitwise."""
+def test_segment_heights_at_y_walls(lbm, nx, ny):
+    """Automatic heights from one row to the whole grid, with wall rows in any iteration of a segment and of its
+    neighbours, and 20 rows by choice, against 5 rows everywhere: step and moments, bitwise."""
     for st, sform in [(0, 0), (1, 0), (2, 0), (0, 1)]:
         w = workload(nx, ny, (nx + st) & 1, W.WALL, seed=ny + st, s_form=sform)
         out = []
