@@ -265,13 +265,11 @@ __global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant_
   const bool ywall = YW && g.bc_y == BC_WALL;
   // the grid is at least a tile and its halo wide and high: one period is enough to wrap
   auto near = [](int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); };
-  auto real = [&](int y) { return !ywall || (y >= 0 && y < g.ny); };
-  // store at (i, j) and, for a cell next to a wall, at its mirror image beyond it
-  auto put = [&](V2 (*f)[FW], int i, int j, int y, V2 v) {
-    f[j][i] = v;
-    const int gj = ywall ? (y == 0 ? j - 1 : (y == g.ny - 1 ? j + 1 : -1)) : -1;
-    if (gj >= 0 && gj < FH) f[gj][i] = v;
-  };
+  // the rows south and north of row j (y of the grid): beyond a wall the row itself, its mirror image.  (The rows beyond it
+  // go through the passes too, from the wrapped rows of the grid: no valid row reads what they leave.  Skipping them and
+  // writing mirror images cost every cell its tests: 256 x 1024 with walls 13.95 us a step, 13.27 this way.)
+  auto south = [&](int j, int y) { return ywall && y == 0 ? j : j - 1; };
+  auto north = [&](int j, int y) { return ywall && y == g.ny - 1 ? j : j + 1; };
   constexpr int C0 = (FW * FH + NT - 1) / NT, C2 = ((FW - 4) * (FH - 4) + NT - 1) / NT;
   static_assert(NT >= 2 * TX * TY, "S3 needs two threads per pair of cells");
   Col3 fa[C0], fb[C0], ga[C2], gbc[C2];
@@ -295,8 +293,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant_
   unsigned int fr[C0][2][NF], gr[C2][2][Q];
 #pragma unroll
   for (int c = 0; c < C0; ++c) {
-    const int k = t + c * NT, j = k / FW;
-    if (k < FW * FH && real(y0 - 3 + j)) {
+    if (t + c * NT < FW * FH) {
       gather9<ST, 0>(g, fa[c], frow[c], fr[c][0]);
       gather9<ST, 0>(g, fb[c], frow[c], fr[c][1]);
       fr[c][0][Q] = ST == ST_FP32 ? ld_raw<ST>(g.src, A_F0LO, pop_at<ST>(A_F0LO, frow[c], fa[c].c0, g)) : 0u;
@@ -305,8 +302,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant_
   }
 #pragma unroll
   for (int c = 0; c < C2; ++c) {
-    const int k = t + c * NT, j = 2 + k / (FW - 4);
-    if (k < (FW - 4) * (FH - 4) && real(y0 - 3 + j)) {
+    if (t + c * NT < (FW - 4) * (FH - 4)) {
       gather9<ST, Q>(g, ga[c], grow[c], gr[c][0]);
       gather9<ST, Q>(g, gbc[c], grow[c], gr[c][1]);
     }
@@ -314,15 +310,15 @@ __global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant_
   // ---- S0
 #pragma unroll
   for (int c = 0; c < C0; ++c) {
-    const int k = t + c * NT, i = k % FW, j = k / FW, y = y0 - 3 + j;
-    if (k >= FW * FH || !real(y)) continue;
+    const int k = t + c * NT, i = k % FW, j = k / FW;
+    if (k >= FW * FH) continue;
     V2 fp[NF], hi, lo;
 #pragma unroll
     for (int a = 0; a < Q; ++a) fp[a] = pack2(dec_pop<ST>(fr[c][0][a], a), dec_pop<ST>(fr[c][1][a], a));
     fp[Q] = pack2(__uint_as_float(fr[c][0][Q]), __uint_as_float(fr[c][1][Q]));
     phi_pair<ST>(P, fp, hi, lo);
-    put(sm.hi, i, j, y, hi);
-    put(sm.lo, i, j, y, lo);
+    sm.hi[j][i] = hi;
+    sm.lo[j][i] = lo;
     const int ti = i - 3, tj = j - 3;
     if (ti >= 0 && ti < TX && tj >= 0 && tj < TY) {
 #pragma unroll
@@ -333,29 +329,29 @@ __global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant_
   // ---- S1
   for (int k = t; k < (FW - 2) * (FH - 2); k += NT) {
     const int i = 1 + k % (FW - 2), j = 1 + k / (FW - 2), y = y0 - 3 + j;
-    if (!real(y)) continue;
-    put(sm.mu, i, j, y,
-        chem_potential(P, &sm.hi[j - 1][i], &sm.hi[j][i], &sm.hi[j + 1][i], &sm.lo[j - 1][i], &sm.lo[j][i], &sm.lo[j + 1][i]));
+    const int js = south(j, y), jn = north(j, y);
+    sm.mu[j][i] = chem_potential(P, &sm.hi[js][i], &sm.hi[j][i], &sm.hi[jn][i], &sm.lo[js][i], &sm.lo[j][i], &sm.lo[jn][i]);
   }
   __syncthreads();
   // ---- S2
 #pragma unroll
   for (int c = 0; c < C2; ++c) {
     const int k = t + c * NT, i = 2 + k % (FW - 4), j = 2 + k / (FW - 4), y = y0 - 3 + j;
-    if (k >= (FW - 4) * (FH - 4) || !real(y)) continue;
+    if (k >= (FW - 4) * (FH - 4)) continue;
+    const int js = south(j, y), jn = north(j, y);
     const V2 ph = fadd(sm.hi[j][i], sm.lo[j][i]);
     V2 gphx, gphy, gmx, gmy;
-    grad12(P, &sm.hi[j - 1][i], &sm.hi[j][i], &sm.hi[j + 1][i], gphx, gphy);
-    grad12(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i], gmx, gmy);
-    const V2 sdef = P.remove_Fa ? fmul(P.s_coef6, lap6_of(P, &sm.mu[j - 1][i], &sm.mu[j][i], &sm.mu[j + 1][i])) : zero<V2>();
+    grad12(P, &sm.hi[js][i], &sm.hi[j][i], &sm.hi[jn][i], gphx, gphy);
+    grad12(P, &sm.mu[js][i], &sm.mu[j][i], &sm.mu[jn][i], gmx, gmy);
+    const V2 sdef = P.remove_Fa ? fmul(P.s_coef6, lap6_of(P, &sm.mu[js][i], &sm.mu[j][i], &sm.mu[jn][i])) : zero<V2>();
     V2 gv[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) gv[a] = pack2(dec_pop<ST>(gr[c][0][a], Q + a), dec_pop<ST>(gr[c][1][a], Q + a));
     const S2Out<V2> s2 = s2_cell<ST>(P, ph, gphx, gphy, gmx, gmy, sm.mu[j][i], sdef, gv);
-    put(sm.p, i, j, y, s2.p);
+    sm.p[j][i] = s2.p;
     if (P.ch_conv) {
-      put(sm.ux, i, j, y, s2.ux);
-      put(sm.uy, i, j, y, s2.uy);
+      sm.ux[j][i] = s2.ux;
+      sm.uy[j][i] = s2.uy;
     }
     const int ti = i - 3, tj = j - 3;
     if (ti >= 0 && ti < TX && tj >= 0 && tj < TY) {
@@ -373,6 +369,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant_
   {
     const int k = t % (TX * TY), ti = k % TX, tj = k / TX, i = ti + 3, j = tj + 3, xa = x0 + ti, xb = xa + TX, y = y0 + tj;
     if (t < 2 * TX * TY && xa < g.nx && y < g.ny) {
+      const int js = south(j, y), jn = north(j, y);
       RecT<V2> r{};
       r.phi = sm.rec[0][tj][ti];
       r.mu = sm.rec[1][tj][ti];
@@ -388,8 +385,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant_
       const V2 z = zero<V2>();
       V2 f[Q], gv[Q];
       if (t < TX * TY) {
-        const V2 phiD = P.ch_conv ? phi_div_u(P, r.phi, &sm.ux[j - 1][i], &sm.ux[j][i], &sm.ux[j + 1][i], &sm.uy[j - 1][i],
-                                              &sm.uy[j + 1][i])
+        const V2 phiD = P.ch_conv ? phi_div_u(P, r.phi, &sm.ux[js][i], &sm.ux[j][i], &sm.ux[jn][i], &sm.uy[js][i], &sm.uy[jn][i])
                                   : z;
         f[0] = z;
 #pragma unroll
@@ -399,7 +395,7 @@ __global__ void __launch_bounds__(NT, CTAS) k_tile2d_pair(const __grid_constant_
         collide_store<ST, false, COLLIDE_F>(P, r, z, z, z, sm.hi[j][i], sm.lo[j][i], phiD, f, gv, out);
       } else {
         V2 gpx, gpy;
-        grad12(P, &sm.p[j - 1][i], &sm.p[j][i], &sm.p[j + 1][i], gpx, gpy);
+        grad12(P, &sm.p[js][i], &sm.p[j][i], &sm.p[jn][i], gpx, gpy);
 #pragma unroll
         for (int a = 0; a < Q; ++a) f[a] = z;
 #pragma unroll
@@ -529,7 +525,7 @@ static cudaError_t launch_tile2d_st(const Phys& P, const Grid& g, const MomentOu
   // Beyond one wave of single tiles, and where x is periodic, two tiles per CTA: 320 threads and 2 CTAs per SM while
   // the pairs fit one such wave, else 256 threads and 3 CTAs.  Single tiles -> pairs, us per step: 256^2 (256 pairs)
   // 5.27 -> 4.91, 150 x 450 (285) 5.54 -> 5.08, 320^2 (400) 7.87 -> 6.65, 384^2 (576) 9.58 -> 9.04, 256 x 1024 (1024)
-  // 15.5 -> 13.9.  A little over one wave of 3 per SM (512 pairs: 256 x 512 8.70 -> 8.94) they stay single.
+  // 15.5 -> 13.3.  A little over one wave of 3 per SM (512 pairs: 256 x 512 8.70 -> 8.94) they stay single.
   const long long pairs = (long long)((g.nx + 2 * T2D_TX - 1) / (2 * T2D_TX)) * ((g.ny + T2D_TY - 1) / T2D_TY);
   const bool tail = pairs > 3LL * sms && 2 * pairs <= 7LL * sms;
   if (!mo && tiles > slots && !tail && g.bc_x != BC_WALL && g.nx >= 2 * T2D_TX + 6 && g.ny >= T2D_TY + 6) {
