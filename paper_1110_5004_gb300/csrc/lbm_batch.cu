@@ -29,7 +29,7 @@ struct lbm_batch {
   bool dirty = true;                   // descriptors / work list need rebuilding
   SimDesc* d_sims = nullptr;
   int4* d_work = nullptr;
-  unsigned int* d_next = nullptr;      // two tile counters per part
+  unsigned int* d_next = nullptr;      // a tile counter per part
   size_t cap_sims = 0, cap_work = 0;
   int n_work = 0;
   struct Part {                        // tiles of one storage and one form of the mass defect: a launch each
@@ -142,9 +142,9 @@ static int rebuild(lbm_batch* b) {
       (e = cudaMemcpyAsync(b->d_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream)) !=
           cudaSuccess)
     return cuda_fail(e, "batch work upload");
-  if (!b->d_next && (e = cudaMalloc(&b->d_next, 2 * N_PARTS * sizeof(unsigned int))) != cudaSuccess)
+  if (!b->d_next && (e = cudaMalloc(&b->d_next, N_PARTS * sizeof(unsigned int))) != cudaSuccess)
     return cuda_fail(e, "batch tile counters");
-  if ((e = cudaMemsetAsync(b->d_next, 0, 2 * N_PARTS * sizeof(unsigned int), b->stream)) != cudaSuccess)
+  if ((e = cudaMemsetAsync(b->d_next, 0, N_PARTS * sizeof(unsigned int), b->stream)) != cudaSuccess)
     return cuda_fail(e, "batch tile counters");
   // host vectors die here: make the uploads complete first
   if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) return cuda_fail(e, "batch upload sync");
@@ -162,7 +162,7 @@ static cudaError_t launch_batch(lbm_batch* b, int parity, cudaStream_t st) {
   for (int k = 0; k < N_PARTS; ++k) {
     const lbm_batch::Part& p = b->parts[k];
     if (p.count == 0) continue;
-    const cudaError_t e = by_storage[k % 3](b->d_sims, b->d_work + p.first, p.count, p.grid, parity, b->d_next + 2 * k, k >= 3, b->xwall, st);
+    const cudaError_t e = by_storage[k % 3](b->d_sims, b->d_work + p.first, p.count, p.grid, parity, b->d_next + k, k >= 3, b->xwall, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -29,10 +29,10 @@ struct BatchSmem {
 // did not fit 255 registers (1.2-1.9 KB of spills per thread).  XW: some member may have walls on x.
 //
 // A CTA takes its first tile by its index and further ones from a counter, the list being in order of falling
-// height: tiles differ in it, and CTAs that share no SM run faster, so that fixed rounds
-// left CTAs idle (us a step, FP32 and BF16: 48 members 184 and 194 -> 179 and 187, 256 members 1036 and 1028 -> 971
-// and 997; 171 and 171, 935 and 947 since the march has one row body, which left no spills here).  next: two counters; a launch uses the one of its
-// parity, zero when it starts, and clears the other for the launch that follows it on the stream.
+// height: tiles differ in it, and CTAs that share no SM run faster, so that fixed rounds left CTAs idle (us a
+// step, FP32 and BF16: 48 members 184 and 194 -> 179 and 187, 256 members 1036 and 1028 -> 971 and 997; since the march
+// has one row body, which left no spills here, 171 and 171, 935 and 947).  next: the counter, zero before and
+// after a launch.
 template <int ST, bool SD, bool XW>
 __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* __restrict__ sims, const int4* __restrict__ work,
                                                                 int n_work, int parity, unsigned int* __restrict__ next) {
@@ -40,10 +40,12 @@ __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* _
   BatchSmem<ST, SD>& sm = *reinterpret_cast<BatchSmem<ST, SD>*>(smem_raw);
   march_init(sm.m);
   StageAt fat, gat;
-  if (blockIdx.x == 0 && threadIdx.x == 0) next[(parity & 1) ^ 1] = 0u;
   for (int w = blockIdx.x; w < n_work;) {
     unsigned int taken = 0;
-    if (threadIdx.x == 0) taken = atomicAdd(next + (parity & 1), 1u);
+    if (threadIdx.x == 0) {
+      taken = atomicAdd(next, 1u);
+      if (taken == n_work - 1u) *next = 0u;   // one addition per tile: this was the last
+    }
     const int4 it = work[w];
     const SimDesc& d = sims[it.x];
     const unsigned int* from = reinterpret_cast<const unsigned int*>(&d.P);

@@ -390,3 +390,31 @@ def test_steps_captured_in_a_graph_equal_eager(lbm, nx, ny, kernel):
     ref.step(2)
     got, want = s.moments(), ref.moments()
     assert all(np.array_equal(got[k], want[k]) for k in FIELDS)
+
+
+@pytest.mark.gpu
+def test_batch_steps_captured_in_a_graph_equal_eager(lbm):
+    """Direct batch launches (fewer steps than the batch's own graph) recorded and replayed between eager ones: every
+    launch finds its tile counter at zero.  More tiles than one wave, so that the counter hands some out."""
+    import torch
+    ws = [workload(250 + 3 * i, 190 + i, 0, W.WALL, seed=i) for i in range(40)]
+    stream = torch.cuda.Stream()
+    batch = lbm.Batch(stream=stream)
+    batch.set_tile(0, 20)
+    sims = [lbm.Sim.from_workload(w) for w in ws]
+    slots = [batch.add(s) for s in sims]
+    batch.step(2)                                     # builds the work list
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        batch.step(2)
+    with torch.cuda.stream(stream):
+        for _ in range(3):
+            graph.replay()
+    batch.step(4)
+    for w, s, slot in zip(ws, sims, slots):
+        batch.remove(slot)
+        alone = lbm.Sim.from_workload(w, kernel=lbm.LBM_KERNEL_ROWS)
+        alone.step(2 + 3 * 2 + 4)
+        got, want = s.moments(), alone.moments()
+        assert all(np.array_equal(got[k], want[k]) for k in FIELDS)
