@@ -575,15 +575,15 @@ constexpr uint32_t CKPT_VERSION = 2;
 
 size_t payload_bytes(const lbm_sim* s) { return s->buf_bytes; }
 
-// The current state between its buffer (class by class) and a checkpoint's payload
-// (blocks of 32 cells, then the s_form planes).  A device payload that is 16-byte aligned is read or
-// written by the reordering kernel itself; otherwise the populations pass through the field work
-// planes, as many at a time as those hold (no allocation: a server evicts when memory is short).
+// The current state between its buffer and a checkpoint's payload (blocks of 32 cells, then the s_form planes).  A
+// payload on a 16-byte boundary of memory that this device addresses is read or written by the reordering kernel
+// itself; otherwise (host memory, another device's) the populations pass through the field work planes, as many at
+// a time as those hold (no allocation: a server evicts when memory is short).
 cudaError_t move_payload(lbm_sim* s, char* payload, bool to_payload, bool dev) {
   char* state = static_cast<char*>(s->buf[s->cur]);
   const long long units = (long long)(s->pop_bytes / 16);
   cudaError_t e = cudaSuccess;
-  if (dev && reinterpret_cast<uintptr_t>(payload) % 16 == 0) {
+  if (reinterpret_cast<uintptr_t>(payload) % 16 == 0 && addressable(payload)) {
     e = launch_reorder(s, state, payload, 0, units, to_payload, s->stream);
   } else {
     const long long room = (long long)((size_t)N_FIELDS * s->plane * sizeof(float) / 16);
