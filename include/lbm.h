@@ -250,13 +250,17 @@ LBM_API int lbm_set_kernel(lbm_sim* sim, int kernel);
  * cells of it (the farthest a step reads) have finished the previous step; the result is bitwise
  * that of LBM_KERNEL_TILES.  n = 1 runs the tile kernel.
  *
- * lbm_set_wait_limit: every such wait gives up after timeout_ns nanoseconds (default 1e9, > 0);
- *   the launch then ends early and leaves the state undefined, later resident launches do
- *   nothing, and the next lbm_step_status or lbm_diagnostics returns LBM_ERR_TIMEOUT (which
- *   re-arms the waits; lbm_init_fields or lbm_restore then gives a defined state again).
- *   hold_tile >= 0 is a test hook: that tile (row-major 16 x 8 tiles) never announces a finished
- *   step, so the waits of its neighbours run out; -1 (default) disables it.
- * lbm_step_status: synchronises the simulation's stream; LBM_ERR_TIMEOUT if a resident launch
+ * lbm_set_wait_limit: every such wait, and every wait of the row march (alone or in a batch) for its
+ *   rows, gives up after timeout_ns nanoseconds (default 1e9, > 0); the launch then ends early and
+ *   leaves the state undefined, later resident launches do nothing, and the next lbm_step_status or
+ *   lbm_diagnostics returns LBM_ERR_TIMEOUT (which re-arms the waits; lbm_init_fields or lbm_restore
+ *   then gives a defined state again).  For the row march lbm_moments, lbm_moments_packed,
+ *   lbm_interfacial_force and lbm_checkpoint return it too.
+ *   hold_tile >= 0 is a test hook: that tile (resident: row-major 16 x 8 tiles) never announces a
+ *   finished step, so the waits of its neighbours run out; in steps of the row march the CTA of that
+ *   index never gets its rows.  -1 (default) disables it.  A batch takes both values when the
+ *   simulation joins.
+ * lbm_step_status: synchronises the simulation's stream; LBM_ERR_TIMEOUT if a launch
  *   gave up since the status was last read, else LBM_OK.
  * Errors: LBM_ERR_INVALID_ARG for a NULL sim or timeout_ns <= 0; LBM_ERR_CUDA. */
 LBM_API int lbm_set_wait_limit(lbm_sim* sim, long long timeout_ns, int hold_tile);

@@ -131,13 +131,13 @@ class Sim:
         return _lib.check_value(lib().lbm_active_kernel(self._h))
 
     def set_wait_limit(self, timeout_ns, hold_tile=-1):
-        """lbm_set_wait_limit: bound of the resident kernel's waits; hold_tile >= 0 makes that
-        tile never announce a finished step (the test of the bound)."""
+        """lbm_set_wait_limit: bound of the waits of the resident kernel and of the row march; hold_tile >= 0
+        makes that tile never announce a finished step, or never get its rows (the test of the bound)."""
         _lib.check(lib().lbm_set_wait_limit(self._h, int(timeout_ns), int(hold_tile)))
 
     def step_status(self):
-        """lbm_step_status: LBM_OK (0), or LBM_ERR_TIMEOUT if a resident launch gave up since the
-        last read (returned, not raised)."""
+        """lbm_step_status: LBM_OK (0), or LBM_ERR_TIMEOUT if a launch gave up since the last read
+        (returned, not raised)."""
         return int(lib().lbm_step_status(self._h))
 
     def set_stream(self, stream):

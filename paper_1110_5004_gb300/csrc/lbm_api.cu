@@ -89,7 +89,8 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
   g.bc_x = s->params.bc_x;
   g.bc_y = s->params.bc_y;
   tile_geometry(s->nx, s->ny, s->params.s_form != 0, s->seg_h, s->sms * MARCH_CTAS, &g);
-  g.gave_up = gave_up(s);
+  const long long tries = s->wait_ns / WAIT_TRY_NS + 2;
+  g.wait = WaitLimit{gave_up(s), s->slot ? &s->slot->gave_up : nullptr, (int)std::min(tries, 1LL << 30), -1};
   g.spoff = s->params.s_form ? (long long)s->pop_bytes : 0;
   return g;
 }
@@ -139,26 +140,29 @@ static int check_params(int nx, int ny, const lbm_params* p) {
   return LBM_OK;
 }
 
-// Page-locked diagnostics records, so that the kernel writes a simulation's record to the host and no copy follows.
-// One block for the process, allocated with the first simulation (allocating page-locked memory orders the
-// streams of the device, so it is not done again); a simulation that finds no free slot copies its record.
+// Page-locked records, so that kernels write a simulation's diagnostics and its give-up word to the host and no copy
+// follows.  One block for the process, allocated with the first simulation (allocating page-locked memory orders the
+// streams of the device, so it is not done again); a simulation that finds no free record copies.
 namespace {
 class RecordPool {
  public:
-  lbm_diag* take() {
+  HostRecord* take() {
     std::lock_guard<std::mutex> lock(mu_);
     if (!tried_) {
       tried_ = true;
       void* p = nullptr;
-      if (cudaHostAlloc(&p, SLOTS * sizeof(lbm_diag), cudaHostAllocPortable) == cudaSuccess) {
-        for (int k = SLOTS - 1; k >= 0; --k) free_[n_++] = static_cast<lbm_diag*>(p) + k;
+      if (cudaHostAlloc(&p, SLOTS * sizeof(HostRecord), cudaHostAllocPortable) == cudaSuccess) {
+        for (int k = SLOTS - 1; k >= 0; --k) free_[n_++] = static_cast<HostRecord*>(p) + k;
       } else {
         cudaGetLastError();
       }
     }
-    return n_ > 0 ? free_[--n_] : nullptr;
+    if (n_ == 0) return nullptr;
+    HostRecord* r = free_[--n_];
+    r->gave_up = 0u;
+    return r;
   }
-  void give(lbm_diag* d) {
+  void give(HostRecord* d) {
     std::lock_guard<std::mutex> lock(mu_);
     free_[n_++] = d;
   }
@@ -168,7 +172,7 @@ class RecordPool {
   std::mutex mu_;
   bool tried_ = false;
   int n_ = 0;
-  lbm_diag* free_[SLOTS];
+  HostRecord* free_[SLOTS];
 };
 RecordPool g_records;
 }  // namespace
@@ -377,23 +381,43 @@ int lbm_init_fields_packed(lbm_sim* s, const float* fields) {
   return LBM_OK;
 }
 
-// Status of the resident launches since the last read (synchronising the stream when one ran;
-// `sync` forces the synchronisation).  A launch that gave up returns LBM_ERR_TIMEOUT and re-arms
-// the waits (flags and status zeroed).
-static int read_resident_status(lbm_sim* s, bool sync) {
-  cudaError_t e = cudaSuccess;
-  if (!s->res_used) {
-    if (sync && (e = cudaStreamSynchronize(s->stream)) != cudaSuccess) return cuda_fail(e, "stream synchronise");
-    return LBM_OK;
-  }
+// Zero the row march's give-up words, on a stream that has been synchronised.
+static cudaError_t clear_gave_up(lbm_sim* s) {
+  if (s->slot) *static_cast<volatile unsigned int*>(&s->slot->gave_up) = 0u;
+  return cudaMemsetAsync(gave_up(s), 0, sizeof(unsigned int), s->stream);
+}
+
+// Behind a synchronisation of the stream: LBM_ERR_TIMEOUT if a wait of the row march ran out since the state was set or
+// this was last read.  Costs a look at page-locked memory (a copy for a simulation without a record).
+static int march_status(lbm_sim* s) {
   unsigned int st = 0;
-  e = cudaMemcpyAsync(&st, s->res_mem + resident_tiles(s->nx, s->ny), sizeof st, cudaMemcpyDeviceToHost, s->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "status copy");
-  s->res_used = false;
+  cudaError_t e = cudaSuccess;
+  if (s->slot) {
+    st = *static_cast<volatile unsigned int*>(&s->slot->gave_up);
+  } else {
+    e = cudaMemcpyAsync(&st, gave_up(s), sizeof st, cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "status copy");
+  }
   if (st == 0) return LBM_OK;
+  if ((e = clear_gave_up(s)) != cudaSuccess) return cuda_fail(e, "status reset");
+  set_error("a wait of the row march ran out (%lld ns); the state is undefined", s->wait_ns);
+  return LBM_ERR_TIMEOUT;
+}
+
+// Status of the launches since the last read; synchronises the stream.  A launch that gave up returns LBM_ERR_TIMEOUT
+// and re-arms the waits (flags and status zeroed).
+static int read_status(lbm_sim* s) {
+  unsigned int st = 0;
+  cudaError_t e = cudaSuccess;
+  if (s->res_used)
+    e = cudaMemcpyAsync(&st, s->res_mem + resident_tiles(s->nx, s->ny), sizeof st, cudaMemcpyDeviceToHost, s->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "status");
+  s->res_used = false;
+  if (st == 0) return march_status(s);
   if ((e = resident_reset(s)) != cudaSuccess) return cuda_fail(e, "status reset");
-  set_error("a wait of the resident step kernel ran out (%lld ns); the state is undefined", s->res_timeout_ns);
+  set_error("a wait of the resident step kernel ran out (%lld ns); the state is undefined", s->wait_ns);
   return LBM_ERR_TIMEOUT;
 }
 
@@ -413,6 +437,7 @@ int lbm_step(lbm_sim* s, int n) {
   const bool tiles = uses_tile2d(s);
   for (int i = 0; i < n; ++i) {
     Grid g = make_grid(s, s->buf[s->cur], s->buf[s->cur ^ 1]);
+    g.wait.hold = s->hold;
     cudaError_t e = tiles ? launch_tile2d(s->phys, g, nullptr, s->sms, s->stream) : launch_step(s->phys2, g, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "lbm_step launch");
     s->cur ^= 1;
@@ -451,7 +476,7 @@ static int copy_out(lbm_sim* s, float* const* outs, int n, const char* what) {
     if (e != cudaSuccess) return cuda_fail(e, what);
   }
   cudaError_t e = cudaStreamSynchronize(s->stream);
-  return e == cudaSuccess ? LBM_OK : cuda_fail(e, what);
+  return e == cudaSuccess ? march_status(s) : cuda_fail(e, what);
 }
 
 // Outputs of the moment pass.  Where it can address all of a call's outputs it writes them in place; otherwise all go
@@ -503,7 +528,7 @@ int lbm_moments_packed(lbm_sim* s, float* fields) {
     if (e != cudaSuccess) return cuda_fail(e, "lbm_moments_packed copy");
   }
   e = cudaStreamSynchronize(s->stream);
-  return e == cudaSuccess ? LBM_OK : cuda_fail(e, "lbm_moments_packed sync");
+  return e == cudaSuccess ? march_status(s) : cuda_fail(e, "lbm_moments_packed sync");
 }
 
 int lbm_interfacial_force(lbm_sim* s, float* fa_x, float* fa_y) {
@@ -535,8 +560,8 @@ int lbm_diagnostics(lbm_sim* s, lbm_diag* out) {
                         s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "diagnostics copy");
   }
-  if ((rc = read_resident_status(s, true)) != LBM_OK) return rc;
-  *out = s->slot ? *s->slot : s->h_diag;
+  if ((rc = read_status(s)) != LBM_OK) return rc;
+  *out = s->slot ? s->slot->diag : s->h_diag;
   if (!out->finite) {
     set_error("simulation diverged (non-finite state) at step %lld", out->step);
     return LBM_ERR_DIVERGED;
@@ -637,7 +662,7 @@ int lbm_checkpoint(lbm_sim* s, void* buf, size_t bytes) {
   if (e == cudaSuccess)
     e = move_payload(s, static_cast<char*>(buf) + sizeof(h), true, dev);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);   // h lives on this stack frame
-  return e == cudaSuccess ? LBM_OK : cuda_fail(e, "lbm_checkpoint copy");
+  return e == cudaSuccess ? march_status(s) : cuda_fail(e, "lbm_checkpoint copy");
 }
 
 int lbm_restore(lbm_sim* s, const void* buf, size_t bytes) {
@@ -659,6 +684,7 @@ int lbm_restore(lbm_sim* s, const void* buf, size_t bytes) {
   e = move_payload(s, const_cast<char*>(static_cast<const char*>(buf)) + sizeof(h), false, dev);
   if (e == cudaSuccess) e = rearm_resident(s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  if (e == cudaSuccess) e = clear_gave_up(s);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_restore copy");
   s->steps = h.steps;
   return LBM_OK;
@@ -695,14 +721,14 @@ int lbm_set_kernel(lbm_sim* s, int kernel) {
 
 int lbm_set_wait_limit(lbm_sim* s, long long timeout_ns, int hold_tile) {
   if (!s || timeout_ns <= 0) return set_error("invalid sim or timeout"), LBM_ERR_INVALID_ARG;
-  s->res_timeout_ns = timeout_ns;
-  s->res_hold = hold_tile < 0 ? -1 : hold_tile;
+  s->wait_ns = timeout_ns;
+  s->hold = hold_tile < 0 ? -1 : hold_tile;
   return LBM_OK;
 }
 
 int lbm_step_status(lbm_sim* s) {
   if (!s) return set_error("sim is NULL"), LBM_ERR_INVALID_ARG;
-  return read_resident_status(s, true);
+  return read_status(s);
 }
 
 int lbm_active_kernel(const lbm_sim* s) {

@@ -100,6 +100,7 @@ static int rebuild(lbm_batch* b) {
       h = (s->ny + segs - 1) / segs;
     }
     tile_geometry(s->nx, s->ny, s->params.s_form != 0, h, 0, &g);
+    g.wait.hold = s->hold;
     d.g = g;
     d.buf0 = s->buf[0];
     d.buf1 = s->buf[1];

@@ -58,7 +58,12 @@ __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* _
     if (threadIdx.x == 0) sm.next = (int)(gridDim.x + taken);
     __syncthreads();
     w = __shfl_sync(0xffffffffu, sm.next, 0);   // (uniform to the compiler, which keeps addresses in uniform registers)
-    march<MODE_STEP, ST, SD, false, XW, false>(sm.P, g, MomentOut{}, it.y, it.z, sm.m, fat, gat);
+    if (sm.m.quit != 0u) {  // a wait ran out in an earlier tile (of any thread: behind its last barrier): not done
+      if (threadIdx.x == 0) d.g.wait.raise();
+      __syncthreads();      // sm.next is read above and written for the next tile
+      continue;
+    }
+    march<MODE_STEP, ST, SD, false, XW, false>(sm.P, g, &d.g.wait, MomentOut{}, it.y, it.z, sm.m, fat, gat);
   }
 }
 

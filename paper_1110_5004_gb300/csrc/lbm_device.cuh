@@ -229,6 +229,19 @@ __host__ __device__ constexpr int pop_off(int st, int a) {
                   : (st == ST_FP32 ? a * BLK * 4 : (a == 0 ? 0 : BLK * 4 + (a - 1) * BLK * 2));
 }
 
+// The waits of the row march for its copies.  They end with the copies; the limit keeps a fault elsewhere from turning
+// into a hang.  A launch whose wait runs out raises both words.
+struct WaitLimit {
+  unsigned int* word;   // on the device, kept until the next state (k_init_pop, lbm_restore) or until it is read
+  unsigned int* host;   // the same in page-locked memory, which the host reads without a copy; or null
+  int tries;            // of a wait
+  int hold;             // test hook: this tile's rows are never copied (-1: none)
+  __device__ __forceinline__ void raise() const {
+    *static_cast<volatile unsigned int*>(word) = 1u;
+    if (host) *static_cast<volatile unsigned int*>(host) = 1u;
+  }
+};
+
 struct Grid {
   const void* src;      // post-collision state at t-1 (read)
   void* dst;            // post-collision state at t (write)
@@ -241,8 +254,8 @@ struct Grid {
   int tile_w;           // columns per lane of a row-march CTA (a CTA covers two lanes)
   int seg_h;            // rows per segment
   int n_strips;         // CTAs across the grid
-  unsigned int* gave_up; // raised by a wait that ran out (never in a sound run)
   long long spoff;      // s_form 1: byte offset of the [rho, div(rho u)] planes in src/dst (else 0)
+  WaitLimit wait;
 };
 
 // Outputs of the moment pass (row-major); each may be null.  fax, fay: the

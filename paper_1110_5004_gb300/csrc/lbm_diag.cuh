@@ -35,7 +35,6 @@ struct DiagIn {
   double* part;                     // 12 partials per block
   double* out;                      // lbm_diag record
   unsigned int* done;               // blocks finished; zero before and after a launch
-  const unsigned int* gave_up;      // or null
   long long step;
 };
 
@@ -228,7 +227,7 @@ static __global__ void __launch_bounds__(DIAG_T) k_diag(const __grid_constant__ 
     o.max_u = total[6];
     o.p_liquid = quot[4];
     o.p_gas = quot[5];
-    o.finite = isfinite(o.sum_phi) && isfinite(o.max_u) && (!d.gave_up || *d.gave_up == 0u);
+    o.finite = isfinite(o.sum_phi) && isfinite(o.max_u);
     o.pad = 0;
     *reinterpret_cast<lbm_diag*>(d.out) = o;
     *d.done = 0u;

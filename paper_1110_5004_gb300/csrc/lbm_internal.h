@@ -9,6 +9,15 @@
 #include "lbm.h"  // include/ is on the include path
 #include "lbm_device.cuh"
 
+namespace lbm {
+constexpr long long WAIT_TRY_NS = 1300;   // what a try of a row march's wait takes (measured: 26 ms for 20 003)
+// Page-locked words of a simulation that its kernels write: the host reads them without a copy.
+struct HostRecord {
+  lbm_diag diag;
+  unsigned int gave_up;
+};
+}  // namespace lbm
+
 struct lbm_sim {
   int nx = 0, ny = 0, pitch = 0;
   long long plane = 0;      // elements per plane
@@ -23,7 +32,7 @@ struct lbm_sim {
   float* fields = nullptr;             // 6 planes: phi, rho, ux, uy, p, mu (moments and init)
   double* red = nullptr;               // reduction scratch: ny rows x 12 partials + final record
   lbm_diag h_diag{};                   // host copy of the final record, for a simulation without a slot
-  lbm_diag* slot = nullptr;            // page-locked record the diagnostics kernel writes itself
+  lbm::HostRecord* slot = nullptr;     // or null (more simulations than records)
   cudaEvent_t uploaded = nullptr;      // recorded after lbm_init_fields' host-to-device copies
   long long steps = 0;
   long long launches = 0;
@@ -34,8 +43,8 @@ struct lbm_sim {
   // table in one stream-ordered allocation made at first use
   unsigned int* res_mem = nullptr;
   unsigned int res_base = 0;           // flag value of every tile between launches
-  long long res_timeout_ns = 1000000000LL;
-  int res_hold = -1;                   // test hook: this tile never announces a finished step
+  long long wait_ns = 1000000000LL;    // limit of a wait, of the resident kernel and of the row march
+  int hold = -1;                       // test hook: this tile never announces a finished step, or gets its rows
   bool res_used = false;               // a resident launch ran since the status was last read
   lbm_batch* batch = nullptr;
 };
@@ -52,8 +61,8 @@ struct Range {
 
 constexpr int N_FIELDS = 6;
 constexpr int DIAG_PARTIALS = 12;
-// Words in the spare doubles behind the diagnostics record: raised by a wait that ran out; blocks of a
-// diagnostics launch that have finished.
+// Words in the spare doubles behind the diagnostics record: raised by a wait of the row march that ran out
+// (WaitLimit::word); blocks of a diagnostics launch that have finished.
 inline unsigned int* gave_up(const lbm_sim* s) { return reinterpret_cast<unsigned int*>(s->red + (size_t)s->ny * DIAG_PARTIALS + 14); }
 inline unsigned int* diag_done(const lbm_sim* s) { return gave_up(s) + 1; }
 

@@ -24,7 +24,10 @@ cudaError_t launch_step(const Phys2& P, const Grid& g, cudaStream_t st) {
 template <int ST>
 __global__ void k_init_pop(Phys P, Grid g, InitIn in) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x == 0 && blockIdx.y == 0) *g.gave_up = 0u;         // a new state
+  if (x == 0 && blockIdx.y == 0 && *g.wait.word != 0u) {   // a new state
+    *g.wait.word = 0u;
+    if (g.wait.host) *static_cast<volatile unsigned int*>(g.wait.host) = 0u;
+  }
   if (x >= g.nx) return;
   const Col3 col = col3<ST>(x, g.nx);
   // neighbours: beyond a wall the mirrored row or column (zero gradient)
@@ -221,10 +224,9 @@ cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u
 
 cudaError_t launch_diag(const lbm_sim* s, cudaStream_t st) {
   const float* f = s->fields;
-  double* record = s->slot ? reinterpret_cast<double*>(s->slot) : s->red + (long long)s->ny * DIAG_PARTIALS;
-  DiagIn d = diag_in(f, f + 2 * s->plane, f + 3 * s->plane, f + 4 * s->plane, s->nx, s->ny, s->pitch, s->phys.phi_star, s->red,
+  double* record = s->slot ? reinterpret_cast<double*>(&s->slot->diag) : s->red + (long long)s->ny * DIAG_PARTIALS;
+  const DiagIn d = diag_in(f, f + 2 * s->plane, f + 3 * s->plane, f + 4 * s->plane, s->nx, s->ny, s->pitch, s->phys.phi_star, s->red,
                      record, diag_done(s), s->steps);
-  d.gave_up = gave_up(s);
   return launch_diag_rows(d, st);
 }
 

@@ -63,9 +63,10 @@ struct MarchSmem {
     V2 mu[MARCH_NT], p[MARCH_NT], ux[MARCH_NT], uy[MARCH_NT];
     V2 j[SD ? 2 : 0][MARCH_NT];           // rho u (direct mass defect)
   };
-  // barriers first: at the same place for every storage, since a batch CTA changes storage between tiles
   alignas(128) unsigned long long fbar[STAGES];
   unsigned long long gbar[STAGES];
+  unsigned int quit;                      // a wait of this CTA ran out
+  int2 left[2];                           // where its producers of f and of gbar then stopped (StageAt)
   alignas(128) Stage stage[STAGES];
   Row5 r5[RING5];
   Row3 r3[RING3];
@@ -84,21 +85,14 @@ __device__ __forceinline__ void bulk_load(unsigned int dst, const void* src, int
                "l"(src), "r"(bytes), "r"(smem_u32(b))
                : "memory");
 }
-// Wait for the phase `parity` of a barrier.  The copies it counts always complete; the bound only
-// keeps a fault elsewhere from turning into a hang: the launch then goes on with what is in shared
-// memory and raises `gave_up`, which the diagnostics report as a diverged state.
-constexpr int WAIT_TRIES = 1 << 20;
-__device__ __forceinline__ void mbar_wait(unsigned long long* b, int parity, unsigned int* gave_up) {
-  const unsigned int addr = smem_u32(b);
-  for (int n = 0; n < WAIT_TRIES; ++n) {
-    unsigned int done;
-    asm volatile("{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-                 : "=r"(done)
-                 : "r"(addr), "r"(parity)
-                 : "memory");
-    if (done) return;
-  }
-  *gave_up = 1u;
+// True once the phase `parity` of a barrier has completed (after a short wait in the instruction itself).
+__device__ __forceinline__ bool mbar_try(unsigned long long* b, int parity) {
+  unsigned int done;
+  asm volatile("{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(done)
+               : "r"(smem_u32(b)), "r"(parity)
+               : "memory");
+  return done != 0;
 }
 
 // Before the first tile of a CTA.
@@ -109,6 +103,7 @@ __device__ __forceinline__ void march_init(MarchSmem<ST, SD>& sm) {
       mbar_init(&sm.fbar[k]);
       mbar_init(&sm.gbar[k]);
     }
+    sm.quit = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -275,9 +270,11 @@ struct StageAt {
 // FP32 storage only).  XW: the x axis may have walls.  K: the scheme constants (Phys2, in the constant bank
 // or in shared memory).
 // PDL: the launch is a programmatic dependent of the previous one and waits for it here, once its addresses are formed.
+// limit: of its waits (in the constant bank or in global memory).  When one runs out the tile is left undone, sm.quit is set,
+// and the CTA must not march again.
 template <int MODE, int ST, bool SD, bool FF, bool XW, bool PDL, class K>
-__device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut& mo, int strip, int seg, MarchSmem<ST, SD>& sm,
-                                      StageAt& fat, StageAt& gat) {
+__device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit* limit, const MomentOut& mo, int strip, int seg,
+                                      MarchSmem<ST, SD>& sm, StageAt& fat, StageAt& gat) {
   constexpr int NT = MARCH_NT;
   const int t = threadIdx.x;
   const int w = g.tile_w;
@@ -328,14 +325,15 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     bulk_load(smem_u32(dst), row + b0 * blk, run1 * blk, bar);
     if (run2 > 0) bulk_load(smem_u32(dst) + run1 * blk, row, run2 * blk, bar);
   };
+  int role = t;                            // 0, 32: producer; -1 once a wait of this thread has run out
   // rows fr of f into stage fs and gr of gbar into stage gs
   auto produce = [&](bool do_f, int fr, int fs, bool do_g, int gr, int gs) {
-    if (t == 0 && do_f) {
+    if (role == 0 && do_f) {
       mbar_expect(&sm.fbar[fs], (run1 + run2) * (region_block(ST, R_F) + region_block(ST, R_L)));
       load_piece(sm.stage[fs].f, fr, R_F, &sm.fbar[fs]);
       if constexpr (region_block(ST, R_L) > 0) load_piece(sm.stage[fs].l, fr, R_L, &sm.fbar[fs]);
     }
-    if (t == 32 && do_g) {
+    if (role == 32 && do_g) {
       mbar_expect(&sm.gbar[gs], (run1 + run2) * region_block(ST, R_G));
       load_piece(sm.stage[gs].g, gr, R_G, &sm.gbar[gs]);
     }
@@ -349,8 +347,9 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
+  const bool held = MODE == MODE_STEP && g.wait.hold == seg * g.n_strips + strip;
   for (int k = 0; k < STAGES; ++k)
-    produce(true, ya - 3 + k, fat.ahead(k), ya - 1 + k <= a_end - 3, ya - 1 + k, gat.ahead(k));
+    produce(!held, ya - 3 + k, fat.ahead(k), !held && ya - 1 + k <= a_end - 3, ya - 1 + k, gat.ahead(k));
 
   // ---- rings: byte offsets of this thread's place in the rows a-k (mod 5) and a-k (mod 3) of iteration a.  The
   // rows of mu (read a-4 .. a-2, then a-1 written) and of p, u (a-3 written, then a-5 .. a-3 read) share
@@ -432,6 +431,21 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     for (int k = 0; k < Q; ++k) gprev[k] = gcur[k];
   };
 
+  // Wait for a staged row, a counted number of tries.  Past that the thread waits no more and copies no more, and what is
+  // left of the tile runs through on what the rings hold, so that the iterations need no test of their own.  (With one
+  // and a way out of the loop, or with a clock in the wait: 2048 x 512 FP16 5-7 % slower, 601 x 437 with x walls 6-10 %.)
+  int tries = limit->tries;
+  auto wait_row = [&](unsigned long long* b, int parity) {
+    for (int n = 0; n < tries; ++n)
+      if (mbar_try(b, parity)) return;
+    if (role == 0) sm.left[0] = make_int2(fat.stage, fat.parity);
+    if (role == 32) sm.left[1] = make_int2(gat.stage, gat.parity);
+    tries = 1;
+    role = -1;
+    sm.quit = 1u;
+    limit->raise();
+  };
+
   auto iter = [&](int a, auto kind) {
     constexpr int KIND = decltype(kind)::value;
     constexpr bool IN = KIND == IT_INNER;
@@ -439,8 +453,8 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
     const int r1 = a - 1, r2 = a - 3, r3 = a - 4;   // rows of S1, S2, S3
     const bool s2_runs = IN || a >= ya + 2;
     // ================ phase 1: S0 and S2; all stores to the rings at its end
-    mbar_wait(&sm.fbar[fs], fat.parity, g.gave_up);
-    if (s2_runs) mbar_wait(&sm.gbar[gs], gat.parity, g.gave_up);
+    wait_row(&sm.fbar[fs], fat.parity);
+    if (s2_runs) wait_row(&sm.gbar[gs], gat.parity);
     // ---- S0: phi at row a (as an unevaluated pair hi + lo)
     V2 fp[NF], hi, lo;
     auto stage0 = [&] {
@@ -604,6 +618,20 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const MomentOut
   int a = ya - 3;
   for (; a < ya + 4 && a <= a_end; ++a) iter(a, Fill{});
   for (; a <= a_end; ++a) iter(a, Inner{});
+  // A tile that was given up: copies in flight write to this CTA's shared memory, so their producer waits for them, as
+  // long again.
+  if (sm.quit != 0u) {
+    if (role != t && (t == 0 || t == 32)) {
+      unsigned long long* const bar = t == 0 ? sm.fbar : sm.gbar;
+      StageAt at;
+      at.stage = sm.left[t != 0].x;
+      at.parity = sm.left[t != 0].y;
+      int n = 0;
+      for (int k = 0; k < STAGES; ++k, at.next())
+        while (n < limit->tries && !mbar_try(bar + at.stage, at.parity)) ++n;
+    }
+    __syncthreads();
+  }
 }
 
 }  // namespace lbm

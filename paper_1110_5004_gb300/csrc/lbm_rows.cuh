@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_march(const __grid_con
   MarchSmem<ST, SD>& sm = *reinterpret_cast<MarchSmem<ST, SD>*>(smem_raw);
   march_init(sm);
   StageAt fat, gat;
-  march<MODE, ST, SD, FF, XW, true>(P, g, mo, blockIdx.x % g.n_strips, blockIdx.x / g.n_strips, sm, fat, gat);
+  march<MODE, ST, SD, FF, XW, true>(P, g, &g.wait, mo, blockIdx.x % g.n_strips, blockIdx.x / g.n_strips, sm, fat, gat);
 }
 
 template <int MODE, int ST, bool SD, bool FF, bool XW>

@@ -689,8 +689,8 @@ static cudaError_t launch_resident_st(lbm_sim* s, const Grid& g, int n) {
   R.base = s->res_base;
   R.nsteps = n;
   R.ntiles = nt;
-  R.timeout_ns = s->res_timeout_ns;
-  R.hold_tile = s->res_hold;
+  R.timeout_ns = s->wait_ns;
+  R.hold_tile = s->hold;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nt < slots ? nt : slots);
   cfg.blockDim = dim3(T2D_NT);
