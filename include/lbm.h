@@ -232,7 +232,8 @@ LBM_API int lbm_set_stream(lbm_sim* sim, void* cuda_stream);
 
 /* Tile shape of the row march: rows per CTA (>= 1).  0 keeps the current value; a new simulation has as
  * many rows per CTA as make one wave of resident CTAs.  threads (64, 128, 256 or 0) is accepted and has
- * no effect: every CTA has 128 threads of two columns each.  Results do not depend on the shape. */
+ * no effect: the grid's width decides (128, 64 or 32 threads of two columns each).  Results do not depend on the
+ * shape. */
 LBM_API int lbm_set_tile(lbm_sim* sim, int threads, int seg_rows);
 
 /* Step kernel of the simulation (no counterpart in the paper; both kernels compute every cell

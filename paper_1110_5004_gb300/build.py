@@ -14,6 +14,7 @@ ROOT = os.path.dirname(HERE)
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblbm.so")
 SOURCES = ["lbm_rows_fp32.cu", "lbm_rows_fp16.cu", "lbm_rows_bf16.cu", "lbm_rows_moments.cu",
+           "lbm_narrow_fp32.cu", "lbm_narrow_fp16.cu", "lbm_narrow_bf16.cu", "lbm_narrow_moments.cu",
            "lbm_kernels.cu", "lbm_tile2d.cu", "lbm_batch.cu", "lbm_batch_fp32.cu", "lbm_batch_fp16.cu", "lbm_batch_bf16.cu",
            "lbm_api.cu", "lbm_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

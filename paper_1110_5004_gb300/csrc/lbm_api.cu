@@ -63,16 +63,45 @@ Phys make_phys(const lbm_params& p) {
   return P;
 }
 
-void tile_geometry(int nx, int ny, bool sd, int seg_h, int slots, Grid* g) {
-  const int most = 2 * march_width(sd), ns = (nx + most - 1) / most;
-  g->n_strips = ns;
-  g->tile_w = (nx + 2 * ns - 1) / (2 * ns);
-  // as many segments as fit in one wave of `slots` resident CTAs: the step lasts as long as the
+MarchShape march_shape_of(int nx, int storage, bool sd, int nt) {
+  const int most = 2 * (nt - 6), slots = march_slots(nt, storage, sd);
+  for (int strips = (nx + most - 1) / most;; ++strips) {
+    const int width = (nx + 2 * strips - 1) / (2 * strips);
+    if (nt < MARCH_NT && width < 16 && strips > 1) return MarchShape{nt, 0, 0};   // more halo than strip
+    int blocks = 0;
+    for (int k = 0; k < strips; ++k) {
+      const StagedRun r = staged_run(nx, k * 2 * width, width);
+      blocks = std::max(blocks, r.run1 + r.run2);
+    }
+    if (blocks <= slots) return MarchShape{nt, strips, width};
+  }
+}
+
+// An SM works on the columns of 2 strips of 128-thread CTAs at a time, or of 4 of 64-thread ones, or of 8: fewer threads
+// where that is more columns by a seventh, else the wider strip with its smaller share of halo.  That is up to 116
+// columns (whole rows) and 245 to 270 (three strips of 90 instead of two) for 64, up to 52 for 32.  us a step, 128
+// threads -> fewer, FP32 and FP16: 32 x 65536 279 -> 82 and 294 -> 80, 64 x 32768 145 -> 79 and 155 -> 76, 100 x 20000
+// 93 -> 69 and 99 -> 51, 250 x 8000 79 -> 65 and 82 -> 60.
+MarchShape march_shape(int nx, int storage, bool sd) {
+  MarchShape best = march_shape_of(nx, storage, sd, MARCH_NT);
+  for (int nt = MARCH_NT / 2; nt >= 32; nt /= 2) {
+    if (nx > 4 * MARCH_NT) break;                  // three strips of 128 threads and more leave nothing to gain
+    const MarchShape m = march_shape_of(nx, storage, sd, nt);
+    if (m.strips > 0 && 6LL * march_ctas(nt) * best.strips > 7LL * march_ctas(best.nt) * m.strips) best = m;
+  }
+  return best;
+}
+
+void tile_geometry(const MarchShape& m, int seg_h, int sms, Grid* g) {
+  g->march_nt = m.nt;
+  g->n_strips = m.strips;
+  g->tile_w = m.width;
+  // as many segments as fit in one wave of resident CTAs: the step lasts as long as the
   // busiest SM, so a count just above the slots adds a nearly empty wave.  Segments of a few rows spend
   // most of their h + 7 iterations on the rows around them, and are still the fastest where the grid has
   // no more rows to give (601 x 437 with side walls: 18.1 us at 5 rows, 22.4 at 8)
-  const int segs = slots >= ns ? slots / ns : 1;
-  g->seg_h = seg_h <= 0 ? (ny + segs - 1) / segs : std::min(seg_h, ny);
+  const int slots = sms * march_ctas(m.nt), segs = slots >= m.strips ? slots / m.strips : 1;
+  g->seg_h = seg_h <= 0 ? (g->ny + segs - 1) / segs : std::min(seg_h, g->ny);
 }
 
 Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
@@ -88,7 +117,7 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
   g.pitch = s->pitch;
   g.bc_x = s->params.bc_x;
   g.bc_y = s->params.bc_y;
-  tile_geometry(s->nx, s->ny, s->params.s_form != 0, s->seg_h, s->sms * MARCH_CTAS, &g);
+  tile_geometry(s->shape, s->seg_h, s->sms, &g);
   const long long tries = s->wait_ns / WAIT_TRY_NS + 2;
   g.wait = WaitLimit{gave_up(s), s->slot ? &s->slot->gave_up : nullptr, (int)std::min(tries, 1LL << 30), -1};
   g.spoff = s->params.s_form ? (long long)s->pop_bytes : 0;
@@ -222,6 +251,7 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
   s->phys = make_phys(*params);
   s->phys2 = widen(s->phys);
   s->stream = (cudaStream_t)cuda_stream;
+  s->shape = march_shape(nx, params->storage, params->s_form != 0);
   const size_t pop_bytes = (size_t)state_bytes_per_cell(params->storage) * s->plane;
   s->pop_bytes = pop_bytes;
   s->buf_bytes = pop_bytes + (params->s_form ? 2 * sizeof(float) * (size_t)s->plane : 0);

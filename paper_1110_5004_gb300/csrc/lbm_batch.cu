@@ -33,7 +33,7 @@ struct lbm_batch {
   size_t cap_sims = 0, cap_work = 0;
   int n_work = 0;
   struct Part {                        // tiles of one storage and one form of the mass defect: a launch each
-    int first = 0, count = 0, grid = 0;
+    int first = 0, count = 0, grid = 0, nt = 0;
   } parts[N_PARTS];
   int flip = 0;                        // parity offset of every member since the last rebuild
   bool xwall = true;                   // some member has walls on x (the general kernel form)
@@ -59,33 +59,48 @@ static int rebuild(lbm_batch* b) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->xwall = false;
   for (int m : members) b->xwall = b->xwall || b->slots[m]->params.bc_x == LBM_WALL;
-  const int slots = sms * MARCH_CTAS;
   auto part_of = [](const lbm_sim* s) { return s->params.storage + (s->params.s_form ? 3 : 0); };
   // Rows per tile.  A launch takes as many rounds as its tiles fill of the device's slots, and a round as many row
   // iterations as its tiles have: the height that makes rounds x (h + 7) least, heights evened out within each member
   // (48 members of the c4 mix, us a step: 171 at the chosen 53 rows, 193 at 56).
-  int rows[N_PARTS];
+  // CTAs of 64 or 32 threads where they save a seventh of that: an iteration takes as long, four or eight CTAs share an
+  // SM, and narrow members leave fewer of their threads idle (us a step, FP32: 256 members of
+  // 64 x 64 98.5 -> 54.9, 64 of 256 x 256 173.6 -> 138.1, 100 of 33 x 200 101.5 -> 39.3; mixes of 64 to 512 columns stay).
+  int rows[N_PARTS], threads[N_PARTS];
   for (int part = 0; part < N_PARTS; ++part) {
-    std::vector<std::array<int, 3>> shape;   // strips, rows, own rows per tile
-    for (int m : members) {
-      const lbm_sim* s = b->slots[m];
-      if (part_of(s) != part) continue;
-      Grid g{};
-      tile_geometry(s->nx, s->ny, s->params.s_form != 0, 1, 0, &g);
-      shape.push_back({g.n_strips, s->ny, s->seg_h ? s->seg_h : b->seg_h});
-    }
     long long best = -1;
     rows[part] = 32;
-    for (int h = 4; h <= 512 && !shape.empty(); h += h < 64 ? 1 : h / 16) {
-      long long tiles = 0;
-      for (const auto& q : shape) {
-        const int hh = q[2] ? q[2] : h;
-        tiles += (long long)q[0] * ((q[1] + hh - 1) / hh);
+    threads[part] = MARCH_NT;
+    for (int nt = MARCH_NT; nt >= 32; nt /= 2) {
+      std::vector<std::array<int, 3>> shape;   // strips, rows, own rows per tile
+      bool fits = true;
+      for (int m : members) {
+        const lbm_sim* s = b->slots[m];
+        if (part_of(s) != part) continue;
+        const MarchShape q = march_shape_of(s->nx, s->params.storage, s->params.s_form != 0, nt);
+        fits = fits && q.strips > 0;
+        shape.push_back({q.strips, s->ny, s->seg_h ? s->seg_h : b->seg_h});
       }
-      const long long cost = (tiles + slots - 1) / slots * (h + 7);
-      if (best < 0 || cost < best) {
-        best = cost;
-        rows[part] = h;
+      if (!fits || shape.empty()) continue;
+      const long long slots = (long long)sms * march_ctas(nt);
+      long long least = -1;
+      int least_h = 32;
+      for (int h = 4; h <= 512; h += h < 64 ? 1 : h / 16) {
+        long long tiles = 0;
+        for (const auto& q : shape) {
+          const int hh = q[2] ? q[2] : h;
+          tiles += (long long)q[0] * ((q[1] + hh - 1) / hh);
+        }
+        const long long cost = (tiles + slots - 1) / slots * (h + 7);
+        if (least < 0 || cost < least) {
+          least = cost;
+          least_h = h;
+        }
+      }
+      if (best < 0 || 7 * least < 6 * best) {
+        best = least;
+        rows[part] = least_h;
+        threads[part] = nt;
       }
     }
   }
@@ -94,12 +109,13 @@ static int rebuild(lbm_batch* b) {
     SimDesc d{};
     d.P = s->phys2;
     Grid g = make_grid(s, nullptr, nullptr);
+    const int part = part_of(s);
     int h = s->seg_h ? s->seg_h : b->seg_h;
     if (!h) {
-      const int segs = (s->ny + rows[part_of(s)] - 1) / rows[part_of(s)];
+      const int segs = (s->ny + rows[part] - 1) / rows[part];
       h = (s->ny + segs - 1) / segs;
     }
-    tile_geometry(s->nx, s->ny, s->params.s_form != 0, h, 0, &g);
+    tile_geometry(march_shape_of(s->nx, s->params.storage, s->params.s_form != 0, threads[part]), h, sms, &g);
     g.wait.hold = s->hold;
     d.g = g;
     d.buf0 = s->buf[0];
@@ -109,7 +125,7 @@ static int rebuild(lbm_batch* b) {
     const int nseg = (s->ny + g.seg_h - 1) / g.seg_h;
     for (int sg = 0; sg < nseg; ++sg) {
       const int tile_rows = std::min(g.seg_h, s->ny - sg * g.seg_h);
-      for (int st = 0; st < g.n_strips; ++st) per[part_of(s)].push_back({tile_rows, make_int4((int)m, st, sg, 0)});
+      for (int st = 0; st < g.n_strips; ++st) per[part].push_back({tile_rows, make_int4((int)m, st, sg, 0)});
     }
   }
   lbm_batch::Part parts[N_PARTS];
@@ -118,7 +134,8 @@ static int rebuild(lbm_batch* b) {
     std::stable_sort(per[part].begin(), per[part].end(), [](const auto& a, const auto& b) { return a.first > b.first; });
     for (const auto& v : per[part]) work.push_back(v.second);
     parts[part].count = (int)work.size() - parts[part].first;
-    parts[part].grid = std::min(parts[part].count, slots);
+    parts[part].nt = threads[part];
+    parts[part].grid = std::min(parts[part].count, sms * march_ctas(threads[part]));
   }
   cudaError_t e;
   if (sims.size() > b->cap_sims) {
@@ -163,7 +180,8 @@ static cudaError_t launch_batch(lbm_batch* b, int parity, cudaStream_t st) {
   for (int k = 0; k < N_PARTS; ++k) {
     const lbm_batch::Part& p = b->parts[k];
     if (p.count == 0) continue;
-    const cudaError_t e = by_storage[k % 3](b->d_sims, b->d_work + p.first, p.count, p.grid, parity, b->d_next + k, k >= 3, b->xwall, st);
+    const BatchPart q{b->d_sims, b->d_work + p.first, p.count, p.grid, parity, p.nt, b->d_next + k, k >= 3, b->xwall};
+    const cudaError_t e = by_storage[k % 3](q, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -18,9 +18,9 @@ static_assert(sizeof(Phys2) % 4 == 0, "copied in words");
 
 // The row march's shared memory and the constants of the tile's member, from which its packed
 // instructions read them (a kernel parameter cannot differ between CTAs).
-template <int ST, bool SD>
+template <int ST, bool SD, int NT>
 struct BatchSmem {
-  MarchSmem<ST, SD> m;
+  MarchSmem<ST, SD, NT> m;
   Phys2 P;
   int next;               // the tile after this one
 };
@@ -33,11 +33,11 @@ struct BatchSmem {
 // step, FP32 and BF16: 48 members 184 and 194 -> 179 and 187, 256 members 1036 and 1028 -> 971 and 997; since the march
 // has one row body, which left no spills here, 171 and 171, 935 and 947).  next: the counter, zero before and
 // after a launch.
-template <int ST, bool SD, bool XW>
-__global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* __restrict__ sims, const int4* __restrict__ work,
+template <int ST, bool SD, bool XW, int NT>
+__global__ void __launch_bounds__(NT, march_ctas(NT)) k_batch(const SimDesc* __restrict__ sims, const int4* __restrict__ work,
                                                                 int n_work, int parity, unsigned int* __restrict__ next) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  BatchSmem<ST, SD>& sm = *reinterpret_cast<BatchSmem<ST, SD>*>(smem_raw);
+  BatchSmem<ST, SD, NT>& sm = *reinterpret_cast<BatchSmem<ST, SD, NT>*>(smem_raw);
   march_init(sm.m);
   StageAt fat, gat;
   for (int w = blockIdx.x; w < n_work;) {
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* _
     const SimDesc& d = sims[it.x];
     const unsigned int* from = reinterpret_cast<const unsigned int*>(&d.P);
     unsigned int* to = reinterpret_cast<unsigned int*>(&sm.P);
-    for (int k = threadIdx.x; k < (int)(sizeof(Phys2) / 4); k += MARCH_NT) to[k] = from[k];
+    for (int k = threadIdx.x; k < (int)(sizeof(Phys2) / 4); k += NT) to[k] = from[k];
     Grid g = d.g;
     const bool odd = ((d.cur0 + parity) & 1) != 0;
     g.src = odd ? d.buf1 : d.buf0;
@@ -63,32 +63,44 @@ __global__ void __launch_bounds__(MARCH_NT, MARCH_CTAS) k_batch(const SimDesc* _
       __syncthreads();      // sm.next is read above and written for the next tile
       continue;
     }
-    march<MODE_STEP, ST, SD, false, XW, false>(sm.P, g, &d.g.wait, MomentOut{}, it.y, it.z, sm.m, fat, gat);
+    march<MODE_STEP, ST, SD, false, XW, false, NT>(sm.P, g, &d.g.wait, MomentOut{}, it.y, it.z, sm.m, fat, gat);
   }
 }
 
-template <int ST, bool SD, bool XW>
-static cudaError_t launch_batch_t(const SimDesc* sims, const int4* work, int n, int grid, int parity, unsigned int* next, cudaStream_t st) {
+// The tiles work[0, n) of one storage and one form of the mass defect; nt: threads per CTA.
+struct BatchPart {
+  const SimDesc* sims;
+  const int4* work;
+  int n, grid, parity, nt;
+  unsigned int* next;
+  bool sd, xw;
+};
+
+template <int ST, bool SD, bool XW, int NT>
+static cudaError_t launch_batch_t(const BatchPart& p, cudaStream_t st) {
   // set once, thread-safely (one GPU per process)
   static const cudaError_t attr_set =
-      cudaFuncSetAttribute(k_batch<ST, SD, XW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BatchSmem<ST, SD>));
+      cudaFuncSetAttribute(k_batch<ST, SD, XW, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BatchSmem<ST, SD, NT>));
   if (attr_set != cudaSuccess) return attr_set;
-  k_batch<ST, SD, XW><<<grid, MARCH_NT, sizeof(BatchSmem<ST, SD>), st>>>(sims, work, n, parity, next);
+  k_batch<ST, SD, XW, NT><<<p.grid, NT, sizeof(BatchSmem<ST, SD, NT>), st>>>(p.sims, p.work, p.n, p.parity, p.next);
   return cudaGetLastError();
 }
 
-// The tiles work[0, n) of members of one storage and one form of the mass defect.
+template <int ST, int NT>
+static cudaError_t launch_batch_nt(const BatchPart& p, cudaStream_t st) {
+  if (p.sd) return launch_batch_t<ST, true, true, NT>(p, st);
+  return p.xw ? launch_batch_t<ST, false, true, NT>(p, st) : launch_batch_t<ST, false, false, NT>(p, st);
+}
+
 template <int ST>
-static cudaError_t launch_batch_st(const SimDesc* sims, const int4* work, int n, int grid, int parity, unsigned int* next, bool sd,
-                                   bool xw, cudaStream_t st) {
-  if (sd) return launch_batch_t<ST, true, true>(sims, work, n, grid, parity, next, st);
-  return xw ? launch_batch_t<ST, false, true>(sims, work, n, grid, parity, next, st)
-            : launch_batch_t<ST, false, false>(sims, work, n, grid, parity, next, st);
+static cudaError_t launch_batch_st(const BatchPart& p, cudaStream_t st) {
+  if (p.nt == MARCH_NT) return launch_batch_nt<ST, MARCH_NT>(p, st);
+  return p.nt == 64 ? launch_batch_nt<ST, 64>(p, st) : launch_batch_nt<ST, 32>(p, st);
 }
 
 // (in the storages' translation units)
-cudaError_t launch_batch_fp32(const SimDesc*, const int4*, int n, int grid, int parity, unsigned int* next, bool sd, bool xw, cudaStream_t st);
-cudaError_t launch_batch_fp16(const SimDesc*, const int4*, int n, int grid, int parity, unsigned int* next, bool sd, bool xw, cudaStream_t st);
-cudaError_t launch_batch_bf16(const SimDesc*, const int4*, int n, int grid, int parity, unsigned int* next, bool sd, bool xw, cudaStream_t st);
+cudaError_t launch_batch_fp32(const BatchPart& p, cudaStream_t st);
+cudaError_t launch_batch_fp16(const BatchPart& p, cudaStream_t st);
+cudaError_t launch_batch_bf16(const BatchPart& p, cudaStream_t st);
 
 }  // namespace lbm

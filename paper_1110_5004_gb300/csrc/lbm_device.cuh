@@ -251,6 +251,7 @@ struct Grid {
   int storage;          // ST_FP32 / ST_FP16 / ST_BF16
   int nx, ny, pitch;
   int bc_x, bc_y;
+  int march_nt;         // threads of a row-march CTA
   int tile_w;           // columns per lane of a row-march CTA (a CTA covers two lanes)
   int seg_h;            // rows per segment
   int n_strips;         // CTAs across the grid

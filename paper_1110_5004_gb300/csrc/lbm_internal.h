@@ -18,6 +18,13 @@ struct HostRecord {
 };
 }  // namespace lbm
 
+namespace lbm {
+// Threads per CTA of the row march, strips across the grid and columns per lane.
+struct MarchShape {
+  int nt = 0, strips = 0, width = 0;
+};
+}  // namespace lbm
+
 struct lbm_sim {
   int nx = 0, ny = 0, pitch = 0;
   long long plane = 0;      // elements per plane
@@ -37,6 +44,7 @@ struct lbm_sim {
   long long steps = 0;
   long long launches = 0;
   int kernel = LBM_KERNEL_AUTO;        // step kernel choice (lbm_set_kernel)
+  lbm::MarchShape shape;               // of the row march
   int seg_h = 0;                       // rows per CTA (0: one wave of resident CTAs)
   int sms = 0;                         // multiprocessors of the device
   // resident tile kernel (lbm_tile2d.cu): per-tile step flags, the status word and the reach
@@ -70,10 +78,13 @@ void set_error(const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);
 Phys make_phys(const lbm_params& p);
 Grid make_grid(const lbm_sim* s, const void* src, void* dst);
-// Lane width, strip count and segment height of the row march for an nx x ny grid: strips of two lanes of
-// at most march_width(sd) columns, all alike; seg_h = 0 picks the height that puts about one full wave of CTAs
-// (slots = SMs x CTAs per SM) on the device.
-void tile_geometry(int nx, int ny, bool sd, int seg_h, int slots, Grid* g);
+// The fewest strips of two lanes, all alike, in which CTAs of nt threads can march nx columns; strips = 0: none.
+MarchShape march_shape_of(int nx, int storage, bool sd, int nt);
+// The best of the thread counts.
+MarchShape march_shape(int nx, int storage, bool sd);
+// The row march's part of a grid; seg_h = 0 picks the segment height that puts about one full wave of CTAs on `sms`
+// multiprocessors.
+void tile_geometry(const MarchShape& m, int seg_h, int sms, Grid* g);
 // The small-grid step kernel (lbm_tile2d.cu): s_form 0 and f_form 0.
 bool tile2d_eligible(const lbm_params& p);
 // 384-thread CTAs when the grid's tiles fit one wave of them on `sms` multiprocessors, else 256.
@@ -97,7 +108,11 @@ cudaError_t launch_step(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_step_fp32(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_step_fp16(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_step_bf16(const Phys2& P, const Grid& g, cudaStream_t st);
+cudaError_t launch_narrow_fp32(const Phys2& P, const Grid& g, cudaStream_t st);   // 64 and 32 threads
+cudaError_t launch_narrow_fp16(const Phys2& P, const Grid& g, cudaStream_t st);
+cudaError_t launch_narrow_bf16(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_moments(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st);
+cudaError_t launch_moments_narrow(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st);
 cudaError_t launch_init(const lbm_sim* s, const InitIn& in, cudaStream_t st);
 // 16-byte units [u0, u1) of the checkpoint's population order between a state buffer and `lin`.
 cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u0, long long u1, bool out, cudaStream_t st);

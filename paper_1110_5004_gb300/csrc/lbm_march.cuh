@@ -3,7 +3,7 @@
 //
 // A CTA marches up a strip of columns and a segment of rows [ya, yb).  Each thread owns two columns, one
 // in each half ("lane") of the strip: thread t has the columns x0 - 3 + t and x0 + w - 3 + t, w columns per
-// lane plus a 3-column halo on each side.  Every value is a V2, the pair of the two lanes, so one
+// lane plus a 3-column halo on each side (march_shape in lbm_api.cu has the choice of threads and strips).  Every value is a V2, the pair of the two lanes, so one
 // packed instruction, one 64-bit shared-memory access and one address serve two cells.
 //
 // Row iteration a runs four stages in two phases, a barrier after each:
@@ -35,33 +35,41 @@ namespace lbm {
 
 enum { MODE_STEP = 0, MODE_MOMENTS = 1 };
 
-constexpr int MARCH_NT = 128;             // threads per CTA
-constexpr int MARCH_CTAS = 2;             // CTAs per SM (shared memory; 8 warps of up to 255 registers)
-// Blocks of a staged row, and the most columns per lane for them: 2 w + 8 columns, up to 31 cells lost at
-// the first block and 31 at the last block of a wrapped row.  The direct mass defect (s_form 1) takes a block less,
-// so that its additional rings fit.
-__host__ __device__ constexpr int march_slots(bool sd) { return sd ? 9 : 10; }
-__host__ __device__ constexpr int march_width(bool sd) {
-  const int w = (march_slots(sd) * BLK - 2 * (BLK - 1) - 8) / 2;
-  return w < MARCH_NT - 6 ? w : MARCH_NT - 6;
+// Threads per CTA (NT): 128, 64 or 32, and 2, 4 or 8 such CTAs per SM (shared memory; 8 warps of up to 255 registers).
+constexpr int MARCH_NT = 128;
+__host__ __device__ constexpr int march_ctas(int nt) { return 256 / nt; }
+// Blocks of a staged row.  128 threads: what any strip of 2 x 122 columns can touch (s_form 1: one less, so that its
+// additional rings fit).  64: as many as let four CTAs share an SM.  32: whole rows of up to 52 columns only.
+__host__ __device__ constexpr int march_slots(int nt, int st, bool sd) {
+  return nt == 128 ? (sd ? 9 : 10) : (nt == 32 ? 2 : (st == ST_FP32 ? (sd ? 4 : 5) : 6));
+}
+// The blocks of columns that a strip of w columns per lane at x0 stages: [b0, b0 + run1) and, where it wraps, [0, run2).
+struct StagedRun {
+  int b0, run1, run2;
+};
+__host__ __device__ __forceinline__ StagedRun staged_run(int nx, int x0, int w) {
+  const int nbx = (nx + BLK - 1) / BLK;
+  if (nx < 2 * w + 8) return StagedRun{0, nbx, 0};
+  const int xs = wrap1(x0 - 4, nx), xe = wrap1(x0 + 2 * w + 3, nx), b0 = xs / BLK;
+  return xs <= xe ? StagedRun{b0, xe / BLK - b0 + 1, 0} : StagedRun{b0, nbx - b0, xe / BLK + 1};
 }
 constexpr int STAGES = 2;                 // rows of f and of gbar in shared memory or in flight
 constexpr int RING5 = 5;                  // rows a-4 .. a of phi and of the f populations awaiting S3
 constexpr int RING3 = 3;                  // rows of mu, p, u
 
-template <int ST, bool SD>
+template <int ST, bool SD, int NT>
 struct MarchSmem {
-  static constexpr int NSLOT = march_slots(SD);
+  static constexpr int NSLOT = march_slots(NT, ST, SD);
   struct Stage {                          // 16-byte aligned pieces
     unsigned char f[NSLOT * region_block(ST, R_F)], l[NSLOT * region_block(ST, R_L)], g[NSLOT * region_block(ST, R_G)];
   };
   struct Row5 {
-    ulonglong2 f[4][MARCH_NT];            // f_1..f_8 of both lanes, own column
-    V2 hi[MARCH_NT], lo[MARCH_NT];
+    ulonglong2 f[4][NT];                  // f_1..f_8 of both lanes, own column
+    V2 hi[NT], lo[NT];
   };
   struct Row3 {
-    V2 mu[MARCH_NT], p[MARCH_NT], ux[MARCH_NT], uy[MARCH_NT];
-    V2 j[SD ? 2 : 0][MARCH_NT];           // rho u (direct mass defect)
+    V2 mu[NT], p[NT], ux[NT], uy[NT];
+    V2 j[SD ? 2 : 0][NT];                 // rho u (direct mass defect)
   };
   alignas(128) unsigned long long fbar[STAGES];
   unsigned long long gbar[STAGES];
@@ -96,8 +104,8 @@ __device__ __forceinline__ bool mbar_try(unsigned long long* b, int parity) {
 }
 
 // Before the first tile of a CTA.
-template <int ST, bool SD>
-__device__ __forceinline__ void march_init(MarchSmem<ST, SD>& sm) {
+template <int ST, bool SD, int NT>
+__device__ __forceinline__ void march_init(MarchSmem<ST, SD, NT>& sm) {
   if (threadIdx.x == 0) {
     for (int k = 0; k < STAGES; ++k) {
       mbar_init(&sm.fbar[k]);
@@ -272,10 +280,10 @@ struct StageAt {
 // PDL: the launch is a programmatic dependent of the previous one and waits for it here, once its addresses are formed.
 // limit: of its waits (in the constant bank or in global memory).  When one runs out the tile is left undone, sm.quit is set,
 // and the CTA must not march again.
-template <int MODE, int ST, bool SD, bool FF, bool XW, bool PDL, class K>
+template <int MODE, int ST, bool SD, bool FF, bool XW, bool PDL, int NT, class K>
 __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit* limit, const MomentOut& mo, int strip, int seg,
-                                      MarchSmem<ST, SD>& sm, StageAt& fat, StageAt& gat) {
-  constexpr int NT = MARCH_NT;
+                                      MarchSmem<ST, SD, NT>& sm, StageAt& fat, StageAt& gat) {
+  constexpr int GT = NT > 32 ? 32 : 16;            // the thread that copies gbar (thread 0 copies f)
   const int t = threadIdx.x;
   const int w = g.tile_w;
   const int x0 = strip * 2 * w;
@@ -288,19 +296,9 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
   const bool on_a = t >= 3 && t < wa + 3, on_b = t >= 3 && t < wb + 3;
   const bool ywall = g.bc_y == BC_WALL;
 
-  // ---- staged columns: blocks [b0, b0 + run1) and, for a strip that wraps, [0, run2)
-  const int nbx = (g.nx + BLK - 1) / BLK;
-  int b0 = 0, run1 = nbx, run2 = 0;
-  if (g.nx >= 2 * w + 8) {
-    const int xs = wrap1(x0 - 4, g.nx), xe = wrap1(x0 + 2 * w + 3, g.nx);
-    b0 = xs / BLK;
-    if (xs <= xe) {
-      run1 = xe / BLK - b0 + 1;
-    } else {
-      run1 = nbx - b0;
-      run2 = xe / BLK + 1;
-    }
-  }
+  // ---- staged columns
+  const StagedRun run = staged_run(g.nx, x0, w);
+  const int b0 = run.b0, run1 = run.run1, run2 = run.run2;
   auto staged_col = [&](int xp) {
     const int blk = xp / BLK;
     return col_bytes<ST>(blk >= b0 ? blk - b0 : run1 + blk, xp & (BLK - 1));
@@ -318,14 +316,14 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
   };
   const int tga = ghost_of(xla), tgb = ghost_of(xlb);
 
-  // ---- producer: one thread copies the rows of f, one of another warp those of gbar
+  // ---- producer: one thread copies the rows of f, another (of another warp, if there is one) those of gbar
   auto load_piece = [&](unsigned char* dst, int r, int region, unsigned long long* bar) {
     const int blk = region_block(ST, region);
     const char* row = static_cast<const char*>(g.src) + (long long)wrap1(r, g.ny) * g.row_bytes + region_start(ST, region) * g.nblk;
     bulk_load(smem_u32(dst), row + b0 * blk, run1 * blk, bar);
     if (run2 > 0) bulk_load(smem_u32(dst) + run1 * blk, row, run2 * blk, bar);
   };
-  int role = t;                            // 0, 32: producer; -1 once a wait of this thread has run out
+  int role = t;                            // 0, GT: producer; -1 once a wait of this thread has run out
   // rows fr of f into stage fs and gr of gbar into stage gs
   auto produce = [&](bool do_f, int fr, int fs, bool do_g, int gr, int gs) {
     if (role == 0 && do_f) {
@@ -333,7 +331,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
       load_piece(sm.stage[fs].f, fr, R_F, &sm.fbar[fs]);
       if constexpr (region_block(ST, R_L) > 0) load_piece(sm.stage[fs].l, fr, R_L, &sm.fbar[fs]);
     }
-    if (role == 32 && do_g) {
+    if (role == GT && do_g) {
       mbar_expect(&sm.gbar[gs], (run1 + run2) * region_block(ST, R_G));
       load_piece(sm.stage[gs].g, gr, R_G, &sm.gbar[gs]);
     }
@@ -354,7 +352,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
   // ---- rings: byte offsets of this thread's place in the rows a-k (mod 5) and a-k (mod 3) of iteration a.  The
   // rows of mu (read a-4 .. a-2, then a-1 written) and of p, u (a-3 written, then a-5 .. a-3 read) share
   // the second set.
-  using S = MarchSmem<ST, SD>;
+  using S = MarchSmem<ST, SD, NT>;
   char* const base = reinterpret_cast<char*>(&sm);
   int q5[RING5], q3[RING3];
 #pragma unroll
@@ -443,7 +441,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
     for (int n = 0; n < tries; ++n)
       if (mbar_try(b, parity)) return;
     if (role == 0) sm.left[0] = make_int2(fat.stage, fat.parity);
-    if (role == 32) sm.left[1] = make_int2(gat.stage, gat.parity);
+    if (role == GT) sm.left[1] = make_int2(gat.stage, gat.parity);
     tries = 1;
     role = -1;
     sm.quit = 1u;
@@ -625,7 +623,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
   // A tile that was given up: copies in flight write to this CTA's shared memory, so their producer waits for them, as
   // long again.
   if (sm.quit != 0u) {
-    if (role != t && (t == 0 || t == 32)) {
+    if (role != t && (t == 0 || t == GT)) {
       unsigned long long* const bar = t == 0 ? sm.fbar : sm.gbar;
       StageAt at;
       at.stage = sm.left[t != 0].x;

@@ -4,7 +4,7 @@
 namespace lbm {
 
 cudaError_t launch_step_bf16(const Phys2& P, const Grid& g, cudaStream_t st) {
-  return launch_rows_st<MODE_STEP, ST_BF16>(P, g, MomentOut{}, st);
+  return g.march_nt == MARCH_NT ? launch_rows_nt<MODE_STEP, ST_BF16, MARCH_NT>(P, g, MomentOut{}, st) : launch_narrow_bf16(P, g, st);
 }
 
 }  // namespace lbm

@@ -11,7 +11,7 @@ typedef struct { unsigned x, y, z; } dim3_t;
 typedef struct { int type, device; void *devicePointer, *hostPointer; long reserved[8]; } attributes_t;
 
 /* Memory: address ranges with a type (cudaMemoryType: 0 unregistered, 1 host, 2 device, 3 managed) and a device. */
-static struct { char *p; size_t n; int type, device; } ranges[4096];
+static struct { char *p; size_t n; int type, device; } ranges[1 << 17];
 static int n_ranges;
 API void fake_range(void* p, size_t n, int type, int device) {
   ranges[n_ranges].p = p;
@@ -40,15 +40,18 @@ static int allocate(void** p, size_t n, int type) {
 API int cudaMalloc(void** p, size_t n) { return allocate(p, n, 2); }
 API int cudaMallocAsync(void** p, size_t n, void* st) { return allocate(p, n, 2); }
 API int cudaHostAlloc(void** p, size_t n, unsigned flags) { return allocate(p, n, 1); }
-API int cudaFree(void* p) { return 0; }
-API int cudaFreeAsync(void* p, void* st) { return 0; }
+API int cudaFree(void* p) {
+  free(p);
+  return 0;
+}
+API int cudaFreeAsync(void* p, void* st) { return cudaFree(p); }
 
 /* Copies and launches, in the order in which they were queued. */
 struct event { char what[64]; void *a, *b; long long n; };
 static struct event events[65536];
 static int n_events;
 static void record(const char* what, const void* a, const void* b, long long n) {
-  struct event* e = &events[n_events++];
+  struct event* e = &events[n_events++ & 65535];
   snprintf(e->what, sizeof e->what, "%s", what);
   e->a = (void*)a;
   e->b = (void*)b;
@@ -74,7 +77,8 @@ API int cudaMemsetAsync(void* d, int v, size_t n, void* st) {
   return 0;
 }
 
-/* Kernels: the name that was registered with the host stub; a, b: the first two parameters' first words. */
+/* Kernels: the name that was registered with the host stub; a, b: the first two parameters' first words; n: blocks x 1024 +
+ * threads. */
 static struct { const void* stub; char name[256]; } kernels[1024];
 static int n_kernels;
 API void __cudaRegisterFunction(void** h, const char* stub, char* dev, const char* name, int lim, void* a, void* b, void* c, void* d,
@@ -82,7 +86,7 @@ API void __cudaRegisterFunction(void** h, const char* stub, char* dev, const cha
   kernels[n_kernels].stub = stub;
   snprintf(kernels[n_kernels++].name, sizeof kernels[0].name, "%s", name);
 }
-static int launch(const void* stub, void** args) {
+static int launch(const void* stub, void** args, const dim3_t* g) {
   for (int i = 0; i < n_kernels; ++i)
     if (kernels[i].stub == stub) {
       const char* k = strstr(kernels[i].name, "k_");
@@ -90,7 +94,7 @@ static int launch(const void* stub, void** args) {
       size_t n = 0;
       while (k && n < sizeof plain - 1 && (k[n] == '_' || (k[n] >= 'a' && k[n] <= 'z') || (k[n] >= '0' && k[n] <= '9'))) ++n;
       snprintf(plain, sizeof plain, "%.*s", (int)n, k ? k : "");
-      record(plain, *(void**)args[0], *(void**)args[1], 0);
+      record(plain, *(void**)args[0], *(void**)args[1], g[0].x * 1024LL + g[1].x);
       return 0;
     }
   return 98;
@@ -114,8 +118,11 @@ API int __cudaGetKernel(const void** k, const void* stub) {
   *k = stub;
   return 0;
 }
-API int __cudaLaunchKernel(const void* k, dim3_t g, dim3_t b, void** args, size_t smem, void* st) { return launch(k, args); }
-API int cudaLaunchKernelExC(const void* cfg, const void* stub, void** args) { return launch(stub, args); }
+API int __cudaLaunchKernel(const void* k, dim3_t g, dim3_t b, void** args, size_t smem, void* st) {
+  const dim3_t gb[2] = {g, b};
+  return launch(k, args, gb);
+}
+API int cudaLaunchKernelExC(const void* cfg, const void* stub, void** args) { return launch(stub, args, cfg); }
 static void* module;
 API void** __cudaRegisterFatBinary(void* bin) { return &module; }
 API void __cudaRegisterFatBinaryEnd(void** h) {}

@@ -22,9 +22,9 @@ def fake(tmp_path_factory):
     return so
 
 
-def run(fake, function, *args):
-    """`function` of this file in a process of its own, on the fake runtime."""
-    code = "import sys; sys.path[:0] = [%r, %r]; import test_host_runtime as t; t.%s(*%r)" % (ROOT, HERE, function, args)
+def run(fake, function, *args, module="test_host_runtime"):
+    """`function` of a test module in a process of its own, on the fake runtime."""
+    code = "import sys; sys.path[:0] = [%r, %r]; import %s as t; t.%s(*%r)" % (ROOT, HERE, module, function, args)
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, env=dict(os.environ, LD_PRELOAD=fake))
     assert r.returncode == 0, r.stdout + r.stderr
 

@@ -1,0 +1,147 @@
+"""CTAs of 64 and 32 threads of the row march (narrow strips): the rule that picks them, and their states against the tile
+kernel, against 128-thread CTAs and against the FP64 oracle."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+from test_host_runtime import fake, library, run, simulation   # noqa: F401 (fixture)
+
+TOL = 1e-5                     # of the FP64 oracle, FP32 storage
+# blocks of 32 columns that a staged row has room for
+SLOTS = {128: {(0, 0): 10, (0, 1): 9, (1, 0): 10, (1, 1): 9}, 64: {(0, 0): 5, (0, 1): 4, (1, 0): 6, (1, 1): 6},
+         32: {(0, 0): 2, (0, 1): 2, (1, 0): 2, (1, 1): 2}}
+FIELDS = ("phi", "rho", "ux", "uy", "p")
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1110_5004_gb300 import build
+    build.build()
+    import paper_1110_5004_gb300 as m
+    return m
+
+
+def launched_shapes(widths, storage, s_form):
+    lbm, f, events = library()
+    seen = {}
+    for nx in widths:
+        s = simulation(lbm, nx, 9, storage, s_form)
+        s.set_kernel(lbm.LBM_KERNEL_ROWS)
+        s.set_tile(0, 9)                                    # one segment: as many CTAs as strips
+        f.fake_clear()
+        s.step(1)
+        (e,) = events()
+        assert e.what == b"k_march"
+        threads, strips = e.n % 1024, e.n // 1024
+        w = -(-nx // (2 * strips))
+        assert w <= threads - 6, (nx, threads, strips)
+        blocks = -(-nx // 32)
+        for k in range(strips):
+            need = blocks
+            if nx >= 2 * w + 8:
+                lo, hi = (2 * w * k - 4) % nx // 32, (2 * w * k + 2 * w + 3) % nx // 32
+                wraps = (2 * w * k - 4) % nx > (2 * w * k + 2 * w + 3) % nx
+                need = blocks - lo + hi + 1 if wraps else hi - lo + 1
+            assert need <= SLOTS[threads][min(storage, 1), s_form], (nx, threads, strips, k, need)
+        seen.setdefault(threads, []).append(nx)
+        s.close()
+    assert {32, 64, 128} <= set(seen)
+    assert max(seen[32]) <= 52 and 52 in seen[32] and 116 in seen[64] and 128 in seen[128] and 244 in seen[128]
+
+
+@pytest.mark.parametrize("storage,s_form", [(0, 0), (0, 1), (1, 0), (2, 1)])
+def test_every_strip_fits_its_cta(fake, storage, s_form):   # noqa: F811
+    """Columns within the threads and staged blocks within the shared memory of the CTA that is launched, for every width
+    to 1200 and some beyond."""
+    run(fake, "launched_shapes", list(range(3, 1201)) + [2047, 2048, 4096, 14521, 73000], storage, s_form, module="test_march_narrow")
+
+
+def workload(nx, ny, bcx, bcy, seed, rf=1, **phys):
+    w = W.random_small(nx, ny, seed=seed, bc_x=bcx, bc_y=bcy, gravity=1e-5 if bcy == W.WALL else 0.0, remove_Fa=rf)
+    return dataclasses.replace(w, phys=dataclasses.replace(w.phys, **phys))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx", [3, 4, 9, 26, 32, 51, 52, 53, 64, 77, 96, 115, 116, 117, 245, 250, 256, 267, 270, 271])
+def test_narrow_strips_equal_tiles_bitwise(lbm, nx):
+    """Both sides of each change of the thread count: step and moments, each wall combination and storage, segments of one
+    row to the whole grid."""
+    for k, (bcx, bcy, ny, st) in enumerate([(0, 0, 5, 0), (1, 1, 9, 0), (0, 1, 12, 1), (1, 0, 16, 2), (0, 0, 7, 2),
+                                            (1, 1, 21, 1), (0, 1, 33, 0)]):
+        if nx < 4 and bcx:
+            continue
+        w = workload(nx, ny, bcx, bcy, seed=nx + k, rf=k & 1, ch_conservative=k == 2, fs_form=k % 3 == 0)
+        want = lbm.Sim.from_workload(w, storage=st, kernel=lbm.LBM_KERNEL_TILES)
+        want.step(8)
+        want = want.checkpoint()
+        for rows in (1, 4, 0):
+            s = lbm.Sim.from_workload(w, storage=st, kernel=lbm.LBM_KERNEL_ROWS)
+            s.set_tile(0, rows)
+            s.step(8)
+            assert np.array_equal(s.checkpoint(), want), (k, rows)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [(30, 9000), (52, 6000), (100, 3000), (250, 1100), (268, 1009)])
+def test_narrow_moments_equal_a_copy_of_the_state(lbm, nx, ny):
+    """The march's moment pass (more than 2^18 cells): a periodic box of five equal parts, one above the other, has the
+    tile kernel's fields of one part in each."""
+    part, reps = workload(nx, ny // 5, 0, 0, seed=nx), 5
+    assert part.nx * part.ny * reps > 1 << 18 >= part.nx * part.ny
+    tile = lambda a: np.ascontiguousarray(np.tile(np.asarray(a, np.float32), (reps, 1)))
+    whole = dataclasses.replace(part, ny=part.ny * reps, phi0=tile(part.phi0), ux0=tile(part.ux0), uy0=tile(part.uy0), p0=tile(part.p0))
+    for st in (0, 1):                                   # (BF16 rounding depends on the row)
+        a = lbm.Sim.from_workload(part, storage=st, kernel=lbm.LBM_KERNEL_TILES)
+        b = lbm.Sim.from_workload(whole, storage=st, kernel=lbm.LBM_KERNEL_ROWS)
+        a.step(4)
+        b.step(4)
+        got, want = b.moments(), a.moments()
+        assert all(np.array_equal(got[k], np.tile(want[k], (reps, 1))) for k in FIELDS), st
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("form", ["s_form", "f_form"])
+@pytest.mark.parametrize("nx", [26, 52, 60, 116, 117, 250])
+def test_march_only_forms_of_narrow_grids_match_oracle(lbm, nx, form):
+    for bcx, bcy in [(W.PERIODIC, W.WALL), (W.WALL, W.PERIODIC)]:
+        w = workload(nx, 13, bcx, bcy, seed=nx, **{form: 1})
+        ref = oracle.run(w, steps=10).moments()
+        states = []
+        for rows in (0, 1, 5):
+            s = lbm.Sim.from_workload(w)
+            s.set_tile(0, rows)
+            s.step(10)
+            states.append(s.checkpoint())
+        assert all(np.array_equal(c, states[0]) for c in states)
+        got = s.moments()
+        u_den = max(np.abs(ref["ux"]).max(), np.abs(ref["uy"]).max(), w.phys.sigma / (w.phys.rho_A * w.phys.nu_A))
+        for k in FIELDS:
+            den = u_den if k in ("ux", "uy") else np.abs(ref[k]).max()
+            assert np.abs(got[k] - ref[k]).max() <= TOL * den, (k, bcx, bcy)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("widest,wide_too", [(52, False), (116, False), (116, True)])
+def test_batches_of_narrow_members_equal_alone(lbm, storage, widest, wide_too):
+    """Batches whose members are all narrow take 32 or 64 threads, with one wide member 128: each member's state is the one
+    it has alone, in both forms of the mass defect."""
+    ws = [workload(9 + (37 * i) % (widest - 8), 300 + (53 * i) % 260, i & 1, (i >> 1) & 1, seed=i, rf=1, s_form=(i >> 2) & 1)
+          for i in range(70)]
+    if wide_too:
+        ws += [workload(1500, 1500, 0, 1, seed=99), workload(1500, 1500, 0, 1, seed=98, s_form=1)]
+    batch = lbm.Batch()
+    sims = [lbm.Sim.from_workload(w, storage=storage) for w in ws]
+    slots = [batch.add(s) for s in sims]
+    batch.step(5)
+    for s, w, slot in zip(sims, ws, slots):
+        batch.remove(slot)
+        alone = lbm.Sim.from_workload(w, storage=storage, kernel=lbm.LBM_KERNEL_ROWS)
+        alone.step(5)
+        assert np.array_equal(s.checkpoint(), alone.checkpoint()), w.nx
