@@ -77,17 +77,27 @@ MarchShape march_shape_of(int nx, int storage, bool sd, int nt) {
   }
 }
 
-// An SM works on the columns of 2 strips of 128-thread CTAs at a time, or of 4 of 64-thread ones, or of 8: fewer threads
-// where that is more columns by a seventh, else the wider strip with its smaller share of halo.  That is up to 116
-// columns (whole rows) and 245 to 270 (three strips of 90 instead of two) for 64, up to 52 for 32.  us a step, 128
-// threads -> fewer, FP32 and FP16: 32 x 65536 279 -> 82 and 294 -> 80, 64 x 32768 145 -> 79 and 155 -> 76, 100 x 20000
-// 93 -> 69 and 99 -> 51, 250 x 8000 79 -> 65 and 82 -> 60.
-MarchShape march_shape(int nx, int storage, bool sd) {
+// Rows of a segment: as many segments as fit in one wave of resident CTAs.  The step lasts as long as the
+// busiest SM, so a count just above the slots adds a nearly empty wave.  Segments of a few rows spend
+// most of their h + 7 iterations on the rows around them, and are still the fastest where the grid has
+// no more rows to give (601 x 437 with side walls: 18.1 us at 5 rows, 22.4 at 8)
+static int wave_rows(const MarchShape& m, int ny, int sms) {
+  const int slots = sms * march_ctas(m.nt), segs = slots >= m.strips ? slots / m.strips : 1;
+  return (ny + segs - 1) / segs;
+}
+
+// An SM works on the columns of 2 strips of 128-thread CTAs at a time, or of 4 of 64-thread ones, or of 8; a row
+// iteration takes as long.  So fewer threads where they shorten a segment's h + 7 iterations by a seventh, else the wider
+// strip with its smaller share of halo.  On long grids that is up to 116 columns (whole rows) and 245 to 270 (three
+// strips of 90 instead of two) for 64, up to 52 for 32.  us a step, 128 threads -> fewer, FP32 and FP16: 32 x 65536
+// 279 -> 82 and 294 -> 80, 64 x 32768 145 -> 79 and 155 -> 76, 100 x 20000 93 -> 69 and 99 -> 51, 250 x 8000 79 -> 65 and
+// 82 -> 60; 16 x 16, one row a segment either way, 6.6 -> 7.2.
+MarchShape march_shape(int nx, int ny, int storage, bool sd, int sms) {
   MarchShape best = march_shape_of(nx, storage, sd, MARCH_NT);
   for (int nt = MARCH_NT / 2; nt >= 32; nt /= 2) {
     if (nx > 4 * MARCH_NT) break;                  // three strips of 128 threads and more leave nothing to gain
     const MarchShape m = march_shape_of(nx, storage, sd, nt);
-    if (m.strips > 0 && 6LL * march_ctas(nt) * best.strips > 7LL * march_ctas(best.nt) * m.strips) best = m;
+    if (m.strips > 0 && 7LL * (wave_rows(m, ny, sms) + 7) < 6LL * (wave_rows(best, ny, sms) + 7)) best = m;
   }
   return best;
 }
@@ -96,12 +106,7 @@ void tile_geometry(const MarchShape& m, int seg_h, int sms, Grid* g) {
   g->march_nt = m.nt;
   g->n_strips = m.strips;
   g->tile_w = m.width;
-  // as many segments as fit in one wave of resident CTAs: the step lasts as long as the
-  // busiest SM, so a count just above the slots adds a nearly empty wave.  Segments of a few rows spend
-  // most of their h + 7 iterations on the rows around them, and are still the fastest where the grid has
-  // no more rows to give (601 x 437 with side walls: 18.1 us at 5 rows, 22.4 at 8)
-  const int slots = sms * march_ctas(m.nt), segs = slots >= m.strips ? slots / m.strips : 1;
-  g->seg_h = seg_h <= 0 ? (g->ny + segs - 1) / segs : std::min(seg_h, g->ny);
+  g->seg_h = seg_h <= 0 ? wave_rows(m, g->ny, sms) : std::min(seg_h, g->ny);
 }
 
 Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
@@ -251,7 +256,6 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
   s->phys = make_phys(*params);
   s->phys2 = widen(s->phys);
   s->stream = (cudaStream_t)cuda_stream;
-  s->shape = march_shape(nx, params->storage, params->s_form != 0);
   const size_t pop_bytes = (size_t)state_bytes_per_cell(params->storage) * s->plane;
   s->pop_bytes = pop_bytes;
   s->buf_bytes = pop_bytes + (params->s_form ? 2 * sizeof(float) * (size_t)s->plane : 0);
@@ -263,6 +267,7 @@ int lbm_create(int nx, int ny, const lbm_params* params, void* cuda_stream, lbm_
     delete s;
     return rc;
   }
+  s->shape = march_shape(nx, ny, params->storage, params->s_form != 0, s->sms);
   const size_t field_bytes = (size_t)N_FIELDS * s->plane * sizeof(float);
   const size_t red_bytes = ((size_t)ny * DIAG_PARTIALS + 16) * sizeof(double);
   // Stream-ordered allocations from the device's memory pool, on the simulation's stream: unlike
@@ -411,9 +416,13 @@ int lbm_init_fields_packed(lbm_sim* s, const float* fields) {
   return LBM_OK;
 }
 
-// Zero the row march's give-up words, on a stream that has been synchronised.
+// Zero the row march's give-up words, on a stream that has been synchronised (both or neither are raised).
 static cudaError_t clear_gave_up(lbm_sim* s) {
-  if (s->slot) *static_cast<volatile unsigned int*>(&s->slot->gave_up) = 0u;
+  if (s->slot) {
+    volatile unsigned int& host = s->slot->gave_up;
+    if (host == 0u) return cudaSuccess;
+    host = 0u;
+  }
   return cudaMemsetAsync(gave_up(s), 0, sizeof(unsigned int), s->stream);
 }
 

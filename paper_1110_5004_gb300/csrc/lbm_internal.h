@@ -81,7 +81,7 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst);
 // The fewest strips of two lanes, all alike, in which CTAs of nt threads can march nx columns; strips = 0: none.
 MarchShape march_shape_of(int nx, int storage, bool sd, int nt);
 // The best of the thread counts.
-MarchShape march_shape(int nx, int storage, bool sd);
+MarchShape march_shape(int nx, int ny, int storage, bool sd, int sms);
 // The row march's part of a grid; seg_h = 0 picks the segment height that puts about one full wave of CTAs on `sms`
 // multiprocessors.
 void tile_geometry(const MarchShape& m, int seg_h, int sms, Grid* g);

@@ -24,10 +24,9 @@ cudaError_t launch_step(const Phys2& P, const Grid& g, cudaStream_t st) {
 template <int ST>
 __global__ void k_init_pop(Phys P, Grid g, InitIn in) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x == 0 && blockIdx.y == 0 && *g.wait.word != 0u) {   // a new state
-    *g.wait.word = 0u;
-    if (g.wait.host) *static_cast<volatile unsigned int*>(g.wait.host) = 0u;
-  }
+  // a new state: the old one's give-up words are cleared, at the end, where the look at one has arrived
+  const bool first = x == 0 && blockIdx.y == 0;
+  const unsigned int stale = first ? *static_cast<volatile unsigned int*>(g.wait.word) : 0u;
   if (x >= g.nx) return;
   const Col3 col = col3<ST>(x, g.nx);
   // neighbours: beyond a wall the mirrored row or column (zero gradient)
@@ -101,6 +100,10 @@ __global__ void k_init_pop(Phys P, Grid g, InitIn in) {
     } else {
       put(std::integral_constant<int, 0>{}, hi + lo);
     }
+  }
+  if (first && stale != 0u) {
+    *g.wait.word = 0u;
+    if (g.wait.host) *static_cast<volatile unsigned int*>(g.wait.host) = 0u;
   }
 }
 
