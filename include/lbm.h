@@ -216,7 +216,8 @@ LBM_API long long lbm_step_count(const lbm_sim* sim);
  * lbm_checkpoint: writes it to `buf` (host or device memory, at least checkpoint_bytes long,
  *   caller-owned); synchronous.  A batch member must be removed from its batch first.
  *   A checkpoint holds every population at the cell it leaves; simulations keep them in another
- *   order, so both calls convert (through the simulation's own work planes, without allocating).
+ *   order, so both calls convert, without allocating: in place for memory of the simulation's device,
+ *   else through the state buffer that the next step overwrites.
  * lbm_restore: replaces the state of `sim` (same nx, ny and storage; its parameters and stream
  *   are its own) by the checkpoint in `buf`, including the step count; synchronous.
  * Errors: LBM_ERR_INVALID_ARG for NULL arguments, a short buffer, a batch member, a bad header

@@ -640,30 +640,23 @@ constexpr uint32_t CKPT_VERSION = 2;
 size_t payload_bytes(const lbm_sim* s) { return s->buf_bytes; }
 
 // The current state between its buffer and a checkpoint's payload (blocks of 32 cells, then the s_form planes).  A
-// payload on a 16-byte boundary of memory that this device addresses is read or written by the reordering kernel
-// itself; otherwise (host memory, another device's) the populations pass through the field work planes, as many at
-// a time as those hold (no allocation: a server evicts when memory is short).
+// payload in memory that this device addresses is read or written by the reordering kernel itself; otherwise (host
+// memory, another device's) the populations pass through the other buffer of the pair, which the next step overwrites
+// (no allocation: a server evicts when memory is short).
 cudaError_t move_payload(lbm_sim* s, char* payload, bool to_payload, bool dev) {
   char* state = static_cast<char*>(s->buf[s->cur]);
-  const long long units = (long long)(s->pop_bytes / 16);
   cudaError_t e = cudaSuccess;
-  if (reinterpret_cast<uintptr_t>(payload) % 16 == 0 && addressable(payload)) {
-    e = launch_reorder(s, state, payload, 0, units, to_payload, s->stream);
+  if (addressable(payload)) {
+    e = launch_reorder(s, state, payload, to_payload, s->stream);
   } else {
-    const long long room = (long long)((size_t)N_FIELDS * s->plane * sizeof(float) / 16);
-    for (long long u0 = 0; u0 < units && e == cudaSuccess; u0 += room) {
-      const long long u1 = u0 + room < units ? u0 + room : units;
-      char* part = payload + u0 * 16;
-      if (to_payload) {
-        e = launch_reorder(s, state, s->fields, u0, u1, true, s->stream);
-        if (e == cudaSuccess)
-          e = cudaMemcpyAsync(part, s->fields, (size_t)(u1 - u0) * 16,
-                              dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s->stream);
-      } else {
-        e = cudaMemcpyAsync(s->fields, part, (size_t)(u1 - u0) * 16,
-                            dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s->stream);
-        if (e == cudaSuccess) e = launch_reorder(s, state, s->fields, u0, u1, false, s->stream);
-      }
+    void* lin = s->buf[s->cur ^ 1];
+    if (to_payload) {
+      e = launch_reorder(s, state, lin, true, s->stream);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(payload, lin, s->pop_bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s->stream);
+    } else {
+      e = cudaMemcpyAsync(lin, payload, s->pop_bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s->stream);
+      if (e == cudaSuccess) e = launch_reorder(s, state, lin, false, s->stream);
     }
   }
   const size_t rest = s->buf_bytes - s->pop_bytes;
@@ -696,11 +689,11 @@ int lbm_checkpoint(lbm_sim* s, void* buf, size_t bytes) {
   h.steps = s->steps;
   h.payload = payload_bytes(s);
   const bool dev = is_device_ptr(buf);
-  const cudaMemcpyKind kh = dev ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost;
-  cudaError_t e = cudaMemcpyAsync(buf, &h, sizeof(h), kh, s->stream);
+  cudaError_t e = dev ? cudaMemcpyAsync(buf, &h, sizeof(h), cudaMemcpyHostToDevice, s->stream) : cudaSuccess;
   if (e == cudaSuccess)
     e = move_payload(s, static_cast<char*>(buf) + sizeof(h), true, dev);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);   // h lives on this stack frame
+  if (e == cudaSuccess && !dev) memcpy(buf, &h, sizeof(h));     // (behind the stream's earlier work on buf)
   return e == cudaSuccess ? march_status(s) : cuda_fail(e, "lbm_checkpoint copy");
 }
 
@@ -711,8 +704,9 @@ int lbm_restore(lbm_sim* s, const void* buf, size_t bytes) {
   if (bytes < sizeof(CkptHeader)) return set_error("checkpoint shorter than its header"), LBM_ERR_INVALID_ARG;
   const bool dev = is_device_ptr(buf);
   CkptHeader h{};
-  cudaError_t e = cudaMemcpyAsync(&h, buf, sizeof(h), dev ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost, s->stream);
+  cudaError_t e = dev ? cudaMemcpyAsync(&h, buf, sizeof(h), cudaMemcpyDeviceToHost, s->stream) : cudaSuccess;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  if (e == cudaSuccess && !dev) memcpy(&h, buf, sizeof(h));
   if (e != cudaSuccess) return cuda_fail(e, "lbm_restore header");
   if (h.magic != CKPT_MAGIC || h.version != CKPT_VERSION) return set_error("not a checkpoint (bad magic or version)"), LBM_ERR_INVALID_ARG;
   if (h.nx != s->nx || h.ny != s->ny || h.pitch != s->pitch || h.storage != s->params.storage ||

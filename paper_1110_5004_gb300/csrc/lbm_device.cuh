@@ -425,8 +425,9 @@ struct OutCell {
   int nblk;
   bool wl, wr, wb, wt;  // x-1, x+1, y-1, y+1 lie beyond a wall
   unsigned int key;     // the cell's place for BF16 rounding
+  // byte offset of the place of population A
   template <int A>
-  __device__ __forceinline__ void put(float v) const {
+  __device__ __forceinline__ int at() const {
     constexpr int ex = A == A_F0LO ? 0 : cx(A % Q), ey = A == A_F0LO ? 0 : cy(A % Q);
     int off = (ey > 0 ? rq : (ey < 0 ? rm : r0)) + region_start(ST, region_of(A)) * nblk + pop_in_region<ST>(A, c.c0);
     if constexpr (ex != 0 || ey != 0) {
@@ -434,7 +435,11 @@ struct OutCell {
       const bool hit = (XW && ((ex > 0 && wr) || (ex < 0 && wl))) || (YW && ((ey > 0 && wt) || (ey < 0 && wb)));
       if (hit) off = r0 + region_start(ST, region_of(A)) * nblk + pop_in_region<ST>(B, ex > 0 ? c.cq : (ex < 0 ? c.cm : c.c0));
     }
-    char* p = dst + off;
+    return off;
+  }
+  template <int A>
+  __device__ __forceinline__ void put(float v) const {
+    char* p = dst + at<A>();
     if (pop_bytes(ST, A) == 4) *reinterpret_cast<float*>(p) = v;
     else *reinterpret_cast<unsigned short*>(p) = enc_pop<ST>(v, A, key);
   }

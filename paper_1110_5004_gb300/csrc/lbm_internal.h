@@ -114,8 +114,8 @@ cudaError_t launch_narrow_bf16(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_moments(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st);
 cudaError_t launch_moments_narrow(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st);
 cudaError_t launch_init(const lbm_sim* s, const InitIn& in, cudaStream_t st);
-// 16-byte units [u0, u1) of the checkpoint's population order between a state buffer and `lin`.
-cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u0, long long u1, bool out, cudaStream_t st);
+// The populations between a state buffer and `lin` (4-byte aligned), which has a checkpoint's order.
+cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, bool out, cudaStream_t st);
 cudaError_t launch_diag(const lbm_sim* s, cudaStream_t st);  // from fields -> red -> final record
 
 }  // namespace lbm

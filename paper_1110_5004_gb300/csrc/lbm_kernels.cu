@@ -2,6 +2,8 @@
 // FP64 diagnostics, with their launchers.
 #include <math.h>
 
+#include <utility>
+
 #include "lbm_diag.cuh"
 #include "lbm_internal.h"
 
@@ -151,76 +153,83 @@ cudaError_t launch_init(const lbm_sim* s, const InitIn& in, cudaStream_t st) {
 // ------------------------------------------------------------------ checkpoint order
 // A checkpoint holds the post-collision populations at their source cells, a row in blocks of 32 cells with
 // every population of the block's cells in turn (FP32: f_0..f_8, gbar_0..gbar_8, f_0lo, 128 bytes each;
-// 16-bit: the FP32 rest population, then 17 of 64 bytes).  `lin` holds its 16-byte units [u0, u1), each
-// some consecutive cells of one population; pad columns keep their place.
+// 16-bit: the FP32 rest population, then 17 of 64 bytes).  Pad columns hold zeros.
+//
+// A lane moves a cell, or takes two neighbours of 16-bit storage out, whose halves share the checkpoint's words: the
+// accesses of a population are 32 neighbouring columns or pairs on both sides, and all populations of a lane are in flight
+// together.  4096 x 4096 out / in, us: FP32 392 / 401, 16-bit 258 / 256 (one cell a lane out: 271; two in: 302-335); a copy
+// is 405 and 220.  With 16-byte units of the checkpoint, 4 or 8 cells of one population, it was 1003 / 1005 and 1180 / 1150.
+template <int... A, class F>
+__device__ __forceinline__ void each_pop(std::integer_sequence<int, A...>, F f) {
+  (f(std::integral_constant<int, A>{}), ...);
+}
+constexpr int reorder_cells(int st, bool out) { return st != ST_FP32 && out ? 2 : 1; }
 template <int ST, bool OUT>
-__global__ void k_reorder(char* __restrict__ state, int4* __restrict__ lin, long long u0, long long u1, Grid g) {
-  constexpr int UNITS = 2 * (int)state_bytes_per_cell(ST);   // per 32-cell block
-  const unsigned int nb = g.pitch / 32;
-  const long long step = (long long)gridDim.x * blockDim.x;
-  for (long long u = u0 + (long long)blockIdx.x * blockDim.x + threadIdx.x; u < u1; u += step) {
-    const unsigned int b = (unsigned int)(u / UNITS);
-    const int k = (int)(u - (long long)b * UNITS);
-    const int y = (int)(b / nb), xb = (int)(b - (unsigned int)y * nb) * 32;
-    int a = k / 8, x0 = xb + (k - a * 8) * 4, n = 4;
-    if (ST != ST_FP32) {
-      if (k < 8) {
-        a = 0;
-        x0 = xb + k * 4;
+__global__ void __launch_bounds__(256) k_reorder(char* __restrict__ state, char* __restrict__ lin, Grid g) {
+  constexpr auto pops = std::make_integer_sequence<int, ST == ST_FP32 ? 19 : 18>{};
+  constexpr int BYTES = 32 * (int)state_bytes_per_cell(ST);   // of a block
+  constexpr int PER = reorder_cells(ST, OUT);                 // of a lane
+  const int groups = (g.nblk + PER - 1) / PER;                // of a row: what a warp moves
+  const long long n = (long long)g.ny * groups, warps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += warps) {
+    const int y = (int)(k / groups), x = (int)(k - (long long)y * groups) * 32 * PER + (threadIdx.x & 31) * PER;
+    if (x >= g.pitch) continue;
+    char* const part = lin + ((long long)y * g.nblk + (x >> 5)) * BYTES;
+    const int at = x & 31;
+    const bool in0 = x < g.nx, in1 = x + 1 < g.nx;
+    const OutCell<ST> c0 = out_cell<ST>(g, in0 ? x : g.nx - 1, y), c1 = out_cell<ST>(g, in1 ? x + 1 : g.nx - 1, y);
+    auto word = [](char* p) -> unsigned int& { return *reinterpret_cast<unsigned int*>(p); };
+    auto half = [](char* p) -> unsigned short& { return *reinterpret_cast<unsigned short*>(p); };
+    unsigned int v[19];                                       // (16-bit storage: [18] the second rest population)
+    each_pop(pops, [&](auto pop) {
+      constexpr int A = decltype(pop)::value;
+      if constexpr (ST == ST_FP32) {
+        v[A] = OUT ? (in0 ? word(state + c0.template at<A>()) : 0u) : word(part + A * 128 + at * 4);
+      } else if constexpr (A == 0) {
+        v[0] = OUT ? (in0 ? word(state + c0.template at<0>()) : 0u) : word(part + at * 4);
+        if (OUT) v[18] = in1 ? word(state + c1.template at<0>()) : 0u;
+      } else if constexpr (OUT) {
+        const unsigned int lo = in0 ? half(state + c0.template at<A>()) : 0u, hi = in1 ? half(state + c1.template at<A>()) : 0u;
+        v[A] = lo | hi << 16;
       } else {
-        a = 1 + (k - 8) / 4;
-        x0 = xb + (k - 8 - (a - 1) * 4) * 8;
-        n = 8;
+        v[A] = half(part + 128 + (A - 1) * 64 + at * 2);
       }
-    }
-    const int d = a == A_F0LO ? 0 : a % Q;
-    union {
-      int4 v;
-      unsigned int w[4];
-      unsigned short h[8];
-    } unit;
-    unit.v = OUT ? make_int4(0, 0, 0, 0) : lin[u - u0];
-    for (int i = 0; i < n; ++i) {
-      const int x = x0 + i;
-      int to = a, row = y, col = x;
-      if (x < g.nx && d > 0) {
-        const int tx = x + cx(d), ty = y + cy(d);
-        const bool hit = (g.bc_x == BC_WALL && (tx < 0 || tx >= g.nx)) || (g.bc_y == BC_WALL && (ty < 0 || ty >= g.ny));
-        if (hit) {
-          to = opp(d) + (a >= Q ? Q : 0);
-          col = wrap1(tx, g.nx);
+    });
+    each_pop(pops, [&](auto pop) {
+      constexpr int A = decltype(pop)::value;
+      if constexpr (OUT) {
+        if constexpr (ST == ST_FP32) {
+          word(part + A * 128 + at * 4) = v[A];
+        } else if constexpr (A == 0) {
+          word(part + at * 4) = v[0];
+          word(part + at * 4 + 4) = v[18];
         } else {
-          row = wrap1(ty, g.ny);
+          word(part + 128 + (A - 1) * 64 + at * 2) = v[A];
         }
-      }
-      char* p = state + (long long)row * g.row_bytes + pop_at<ST>(to, 0, col_bytes<ST>(col), g);
-      if (n == 4) {
-        if (OUT) unit.w[i] = *reinterpret_cast<unsigned int*>(p);
-        else *reinterpret_cast<unsigned int*>(p) = unit.w[i];
+      } else if constexpr (pop_bytes(ST, A) == 4) {
+        if (in0) word(state + c0.template at<A>()) = v[A];
       } else {
-        if (OUT) unit.h[i] = *reinterpret_cast<unsigned short*>(p);
-        else *reinterpret_cast<unsigned short*>(p) = unit.h[i];
+        if (in0) half(state + c0.template at<A>()) = (unsigned short)v[A];
       }
-    }
-    if (OUT) lin[u - u0] = unit.v;
+    });
   }
 }
 
 template <int ST>
-static cudaError_t launch_reorder_st(const lbm_sim* s, void* state, void* lin, long long u0, long long u1, bool out,
-                                     cudaStream_t st) {
+static cudaError_t launch_reorder_st(const lbm_sim* s, void* state, void* lin, bool out, cudaStream_t st) {
   const Grid g = make_grid(s, nullptr, nullptr);
-  const long long want = (u1 - u0 + 255) / 256;
-  const int grid = (int)(want < 16LL * s->sms ? want : 16LL * s->sms);
-  if (out) k_reorder<ST, true><<<grid, 256, 0, st>>>(static_cast<char*>(state), static_cast<int4*>(lin), u0, u1, g);
-  else k_reorder<ST, false><<<grid, 256, 0, st>>>(static_cast<char*>(state), static_cast<int4*>(lin), u0, u1, g);
+  const int per = reorder_cells(ST, out);
+  const long long want = ((long long)g.ny * ((g.nblk + per - 1) / per) + 7) / 8;
+  const int grid = (int)(want < 64LL * s->sms ? want : 64LL * s->sms);
+  if (out) k_reorder<ST, true><<<grid, 256, 0, st>>>(static_cast<char*>(state), static_cast<char*>(lin), g);
+  else k_reorder<ST, false><<<grid, 256, 0, st>>>(static_cast<char*>(state), static_cast<char*>(lin), g);
   return cudaGetLastError();
 }
 
-cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long u0, long long u1, bool out, cudaStream_t st) {
+cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, bool out, cudaStream_t st) {
   // the two 16-bit storages are laid out alike
-  return s->params.storage == LBM_FP32 ? launch_reorder_st<ST_FP32>(s, state, lin, u0, u1, out, st)
-                                       : launch_reorder_st<ST_FP16>(s, state, lin, u0, u1, out, st);
+  return s->params.storage == LBM_FP32 ? launch_reorder_st<ST_FP32>(s, state, lin, out, st)
+                                       : launch_reorder_st<ST_FP16>(s, state, lin, out, st);
 }
 
 // ------------------------------------------------------------------ FP64 diagnostics

@@ -58,7 +58,7 @@ def checkpoint_memory(storage, s_form, mtype, device, offset):
     buf = raw[at:at + n]
     f.fake_range(buf.ctypes.data, n, mtype, device)
     lo, hi = buf.ctypes.data, buf.ctypes.data + n
-    in_place = (mtype == 3 or (mtype == 2 and device == 0)) and (lo + 64) % 16 == 0
+    in_place = (mtype == 3 or (mtype == 2 and device == 0)) and lo % 4 == 0
     for move in (s.checkpoint, s.restore):
         f.fake_clear()
         move(buf)
@@ -71,13 +71,15 @@ def checkpoint_memory(storage, s_form, mtype, device, offset):
         size = [e.n for e in ev if e.what == b"copy"]
         copied = sum(k for a, k in zip(ends, size) if lo <= a < hi)
         populations = 96 * 29 * (76 if storage == 0 else 38)
-        assert copied == (n - populations if in_place else n)
+        on_device = mtype in (2, 3)
+        assert copied == n - (populations if in_place else 0) - (0 if on_device else 64)   # (host: the header directly)
+    assert bytes(buf[:4]) == b"LBMC"
 
 
 @pytest.mark.parametrize("storage,s_form", [(0, 0), (1, 0), (0, 1)])
 @pytest.mark.parametrize("mtype,device,offset", [
-    (2, 0, 0), (2, 0, 8), (3, 0, 0),      # this device's memory, on a 16-byte boundary and off it; managed memory
-    (2, 1, 0), (2, 1, 16), (2, 1, 8),     # another device's
+    (2, 0, 0), (2, 0, 4), (2, 0, 1), (3, 0, 0),   # this device's memory, on a word's boundary and off it; managed memory
+    (2, 1, 0), (2, 1, 16), (2, 1, 1),     # another device's
     (1, 0, 0), (0, -2, 0)])               # page-locked and pageable host memory
 def test_checkpoint_kernel_gets_only_memory_it_can_address(fake, storage, s_form, mtype, device, offset):
     run(fake, "checkpoint_memory", storage, s_form, mtype, device, offset)
