@@ -88,12 +88,25 @@ __device__ __forceinline__ double diag_tree(const double* v, int lane) {
   return s;
 }
 
+struct DiagSmem {
+  double sh[7][DIAG_T];                     // phi, c x, c u_x, c u_y, |u|^2, p in the liquid, p in the gas
+  double row_c[DIAG_ROWS][DIAG_T];
+  double chord[DIAG_ROWS], total[DIAG_PARTIALS];
+  double quot[6];
+  int count[2][DIAG_T / 32];
+  bool last;
+};
+
 static __global__ void __launch_bounds__(DIAG_T) k_diag(const __grid_constant__ DiagIn d) {
-  __shared__ double sh[7][DIAG_T];          // phi, c x, c u_x, c u_y, |u|^2, p in the liquid, p in the gas
-  __shared__ double row_c[DIAG_ROWS][DIAG_T];
-  __shared__ double chord[DIAG_ROWS], total[DIAG_PARTIALS];
-  __shared__ int count[2][DIAG_T / 32];
-  __shared__ bool last;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  DiagSmem& sm = *reinterpret_cast<DiagSmem*>(smem_raw);
+  auto& sh = sm.sh;
+  auto& row_c = sm.row_c;
+  auto& chord = sm.chord;
+  auto& total = sm.total;
+  auto& quot = sm.quot;
+  auto& count = sm.count;
+  bool& last = sm.last;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int y0 = blockIdx.x * d.rows, rows = min(d.rows, d.ny - y0);
   // launched as a programmatic dependent of the moment pass
@@ -208,7 +221,6 @@ static __global__ void __launch_bounds__(DIAG_T) k_diag(const __grid_constant__ 
   }
   __syncthreads();
   // the six quotients by six threads: FP64 divisions are long
-  __shared__ double quot[6];
   if (t < 6) {
     const int num = t < 4 ? 2 + t : (t == 4 ? 7 : 9), den = t < 4 ? 1 : (t == 4 ? 8 : 10);
     quot[t] = total[den] > 0 ? total[num] / total[den] : 0.0;
@@ -234,11 +246,19 @@ static __global__ void __launch_bounds__(DIAG_T) k_diag(const __grid_constant__ 
   }
 }
 
-// dependent: launched behind a moment pass on the same stream, which it waits for.
-inline cudaError_t launch_diag_rows(const DiagIn& d, cudaStream_t st) {
+// Launched behind a moment pass on the same stream, which it waits for.  Its blocks are placed while that pass still
+// runs, wherever an SM has room: each asks for so much shared memory that no SM takes more than its share.  (They
+// piled up on the first SMs that had room, FP64-bound; us a call with the moment pass: 4096 x 152 108 -> 55, 16384 x 64
+// 169 -> 111, 74176 x 8 865 -> 322, 1000 x 701 85 -> 74.)
+static cudaError_t launch_diag_rows(const DiagIn& d, int sms, cudaStream_t st) {
+  static const cudaError_t attr_set =   // once, thread-safely (one GPU per process)
+      cudaFuncSetAttribute(k_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_for_cap((int)sizeof(DiagSmem), 1));
+  if (attr_set != cudaSuccess) return attr_set;
+  const int blocks = (d.ny + d.rows - 1) / d.rows;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((d.ny + d.rows - 1) / d.rows);
+  cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(DIAG_T);
+  cfg.dynamicSmemBytes = smem_for_cap((int)sizeof(DiagSmem), (blocks + sms - 1) / sms);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -93,6 +93,9 @@ cudaError_t launch_tile2d(const Phys& P, const Grid& g, const MomentOut* mo, int
 // Grids of at most this many cells take the tile kernel for their moments (one call, kernel and host: 128^2
 // 18.5 us against 21.1 for the row march, 256 x 1024 27.6 against 29.1; 700^2 49.4 against 42.9).
 constexpr long long SMALL_GRID_MOMENTS = 1 << 18;
+// Shared memory to ask for so that at most `cap` CTAs fit on an SM, at least `need` (`need` where the device's limits
+// cannot be read).
+int smem_for_cap(int need, int cap);
 // Grids of at most this many cells run the small-grid kernel by default (measured faster up to
 // 2^18 cells, slower from 2^19 on, with and without x walls).
 constexpr long long SMALL_GRID_CELLS = 1 << 18;

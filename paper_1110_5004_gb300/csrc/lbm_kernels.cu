@@ -239,7 +239,7 @@ cudaError_t launch_diag(const lbm_sim* s, cudaStream_t st) {
   double* record = s->slot ? reinterpret_cast<double*>(&s->slot->diag) : s->red + (long long)s->ny * DIAG_PARTIALS;
   const DiagIn d = diag_in(f, f + 2 * s->plane, f + 3 * s->plane, f + 4 * s->plane, s->nx, s->ny, s->pitch, s->phys.phi_star, s->red,
                      record, diag_done(s), s->steps);
-  return launch_diag_rows(d, st);
+  return launch_diag_rows(d, s->sms, st);
 }
 
 }  // namespace lbm

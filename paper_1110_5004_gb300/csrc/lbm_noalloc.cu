@@ -91,6 +91,9 @@ extern "C" int lbm_diagnostics_fields_noalloc(const float* phi, const float* ux,
       return set_error("lbm_diagnostics_fields_noalloc: a host out cannot be filled on a capturing stream; "
                        "pass a device out"), LBM_ERR_INVALID_ARG;
   }
+  int sms = 0;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return cuda_fail(e, "lbm_diagnostics_fields_noalloc: device query");
   double* scratch = nullptr;
   int rc = noalloc_scratch(&scratch);
   if (rc) return rc;
@@ -99,7 +102,7 @@ extern "C" int lbm_diagnostics_fields_noalloc(const float* phi, const float* ux,
   unsigned int* done = reinterpret_cast<unsigned int*>(record + 15);
   if ((e = cudaMemsetAsync(done, 0, sizeof(unsigned int), st)) != cudaSuccess)
     return cuda_fail(e, "lbm_diagnostics_fields_noalloc: block count");
-  e = launch_diag_rows(diag_in(phi, ux, uy, p, nx, ny, nx, phi_star, scratch, record, done, step), st);
+  e = launch_diag_rows(diag_in(phi, ux, uy, p, nx, ny, nx, phi_star, scratch, record, done, step), sms, st);
   if (e != cudaSuccess) return cuda_fail(e, "lbm_diagnostics_fields_noalloc: kernel");
   e = cudaMemcpyAsync(out, record, sizeof(lbm_diag), host_out ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess && host_out) e = cudaStreamSynchronize(st);

@@ -413,10 +413,9 @@ __global__ void __launch_bounds__(NT) k_tile2d_moments(Phys P, Grid g, int tiles
   tile2d_step<ST, TX, TY, NT, false, XW, YW, true>(P, g, tiles_x, blockIdx.x, *reinterpret_cast<Smem2D<TX, TY>*>(smem_raw), mo);
 }
 
-// Shared memory to ask for so that at most `cap` CTAs fit on an SM (at least `need`): a grid of
-// few tiles then spreads evenly over the SMs instead of piling several CTAs onto some while
-// others idle.  0 when the device attributes cannot be read.
-static int smem_for_cap(int need, int cap) {
+// A grid of few tiles then spreads evenly over the SMs instead of piling several CTAs onto some while
+// others idle.
+int smem_for_cap(int need, int cap) {
   struct Attrs {
     int per_sm = 0, reserved = 0, optin = 0;
   };

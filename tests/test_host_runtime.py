@@ -30,7 +30,7 @@ def run(fake, function, *args, module="test_host_runtime"):
 
 
 class Event(ctypes.Structure):
-    _fields_ = [("what", ctypes.c_char * 64), ("a", ctypes.c_void_p), ("b", ctypes.c_void_p), ("n", ctypes.c_longlong)]
+    _fields_ = [("what", ctypes.c_char * 64), ("a", ctypes.c_void_p), ("b", ctypes.c_void_p), ("n", ctypes.c_longlong), ("smem", ctypes.c_longlong)]
 
 
 def library():
@@ -83,3 +83,22 @@ def checkpoint_memory(storage, s_form, mtype, device, offset):
     (1, 0, 0), (0, -2, 0)])               # page-locked and pageable host memory
 def test_checkpoint_kernel_gets_only_memory_it_can_address(fake, storage, s_form, mtype, device, offset):
     run(fake, "checkpoint_memory", storage, s_form, mtype, device, offset)
+
+
+def diagnostics_share():
+    lbm, f, events = library()
+    for ny in (8, 100, 152, 153, 304, 305, 500, 608, 609, 3000):
+        s = simulation(lbm, 33, ny)
+        f.fake_clear()
+        s.diagnostics()
+        (e,) = [e for e in events() if e.what == b"k_diag"]
+        blocks = e.n // 1024
+        share = -(-blocks // 152)
+        assert blocks <= ny and share * (e.smem + 1024) <= 233472, (ny, blocks, e.smem)
+        assert (share + 1) * (e.smem + 1024) > 233472, (ny, blocks, e.smem)
+        s.close()
+
+
+def test_diagnostics_blocks_spread_over_the_device(fake):
+    """The diagnostics' blocks are placed while the moment pass still runs: no SM has room for more than its share."""
+    run(fake, "diagnostics_share")
