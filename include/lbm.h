@@ -217,7 +217,7 @@ LBM_API long long lbm_step_count(const lbm_sim* sim);
  *   caller-owned); synchronous.  A batch member must be removed from its batch first.
  *   A checkpoint holds every population at the cell it leaves; simulations keep them in another
  *   order, so both calls convert, without allocating: in place for memory of the simulation's device,
- *   else through the state buffer that the next step overwrites.
+ *   else through the simulation's own work planes.
  * lbm_restore: replaces the state of `sim` (same nx, ny and storage; its parameters and stream
  *   are its own) by the checkpoint in `buf`, including the step count; synchronous.
  * Errors: LBM_ERR_INVALID_ARG for NULL arguments, a short buffer, a batch member, a bad header

@@ -641,22 +641,28 @@ size_t payload_bytes(const lbm_sim* s) { return s->buf_bytes; }
 
 // The current state between its buffer and a checkpoint's payload (blocks of 32 cells, then the s_form planes).  A
 // payload in memory that this device addresses is read or written by the reordering kernel itself; otherwise (host
-// memory, another device's) the populations pass through the other buffer of the pair, which the next step overwrites
-// (no allocation: a server evicts when memory is short).
+// memory, another device's) the populations pass through the field work planes and the diagnostics' partials behind
+// them, as many at a time as those hold (no allocation: a server evicts when memory is short; and not through the other
+// state buffer, whose pad columns would not keep what they hold).
 cudaError_t move_payload(lbm_sim* s, char* payload, bool to_payload, bool dev) {
   char* state = static_cast<char*>(s->buf[s->cur]);
+  const long long groups = reorder_groups(s, to_payload);
   cudaError_t e = cudaSuccess;
   if (addressable(payload)) {
-    e = launch_reorder(s, state, payload, to_payload, s->stream);
+    e = launch_reorder(s, state, payload, 0, groups, to_payload, s->stream);
   } else {
-    void* lin = s->buf[s->cur ^ 1];
-    if (to_payload) {
-      e = launch_reorder(s, state, lin, true, s->stream);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(payload, lin, s->pop_bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s->stream);
-    } else {
-      e = cudaMemcpyAsync(lin, payload, s->pop_bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s->stream);
-      if (e == cudaSuccess) e = launch_reorder(s, state, lin, false, s->stream);
+    const cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : (to_payload ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice);
+    const long long room = reorder_fit(s, to_payload, N_FIELDS * (size_t)s->plane * sizeof(float) + (size_t)s->ny * DIAG_PARTIALS * sizeof(double));
+    for (long long k = 0; k < groups && e == cudaSuccess; k += room) {
+      const long long end = std::min(groups, k + room), at = reorder_offset(s, to_payload, k);
+      const size_t n = (size_t)((end < groups ? reorder_offset(s, to_payload, end) : (long long)s->pop_bytes) - at);
+      if (to_payload) {
+        e = launch_reorder(s, state, s->fields, k, end, true, s->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(payload + at, s->fields, n, kind, s->stream);
+      } else {
+        e = cudaMemcpyAsync(s->fields, payload + at, n, kind, s->stream);
+        if (e == cudaSuccess) e = launch_reorder(s, state, s->fields, k, end, false, s->stream);
+      }
     }
   }
   const size_t rest = s->buf_bytes - s->pop_bytes;

@@ -117,8 +117,13 @@ cudaError_t launch_narrow_bf16(const Phys2& P, const Grid& g, cudaStream_t st);
 cudaError_t launch_moments(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st);
 cudaError_t launch_moments_narrow(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st);
 cudaError_t launch_init(const lbm_sim* s, const InitIn& in, cudaStream_t st);
-// The populations between a state buffer and `lin` (4-byte aligned), which has a checkpoint's order.
-cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, bool out, cudaStream_t st);
+// Groups of blocks in which populations move between a state buffer and a checkpoint's order: how many the grid has, at
+// what byte of the order a group starts, how many fit into `bytes` (at least one into a simulation's work planes and
+// partials), and the move of [k0, k1), `lin` (4-byte aligned) being the place of group k0.
+long long reorder_groups(const lbm_sim* s, bool out);
+long long reorder_offset(const lbm_sim* s, bool out, long long k);
+long long reorder_fit(const lbm_sim* s, bool out, size_t bytes);
+cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long k0, long long k1, bool out, cudaStream_t st);
 cudaError_t launch_diag(const lbm_sim* s, cudaStream_t st);  // from fields -> red -> final record
 
 }  // namespace lbm

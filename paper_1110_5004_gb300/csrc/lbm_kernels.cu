@@ -153,7 +153,7 @@ cudaError_t launch_init(const lbm_sim* s, const InitIn& in, cudaStream_t st) {
 // ------------------------------------------------------------------ checkpoint order
 // A checkpoint holds the post-collision populations at their source cells, a row in blocks of 32 cells with
 // every population of the block's cells in turn (FP32: f_0..f_8, gbar_0..gbar_8, f_0lo, 128 bytes each;
-// 16-bit: the FP32 rest population, then 17 of 64 bytes).  Pad columns hold zeros.
+// 16-bit: the FP32 rest population, then 17 of 64 bytes).  Pad columns keep their place.
 //
 // A lane moves a cell, or takes two neighbours of 16-bit storage out, whose halves share the checkpoint's words: the
 // accesses of a population are 32 neighbouring columns or pairs on both sides, and all populations of a lane are in flight
@@ -164,32 +164,39 @@ __device__ __forceinline__ void each_pop(std::integer_sequence<int, A...>, F f) 
   (f(std::integral_constant<int, A>{}), ...);
 }
 constexpr int reorder_cells(int st, bool out) { return st != ST_FP32 && out ? 2 : 1; }
+// Groups [k0, k1) of the grid, each the `PER` blocks (fewer at a row's end) that a warp moves; lin: where group 0 would lie.
 template <int ST, bool OUT>
-__global__ void __launch_bounds__(256) k_reorder(char* __restrict__ state, char* __restrict__ lin, Grid g) {
+__global__ void __launch_bounds__(256) k_reorder(char* __restrict__ state, char* __restrict__ lin, Grid g, long long k0, long long k1) {
   constexpr auto pops = std::make_integer_sequence<int, ST == ST_FP32 ? 19 : 18>{};
   constexpr int BYTES = 32 * (int)state_bytes_per_cell(ST);   // of a block
   constexpr int PER = reorder_cells(ST, OUT);                 // of a lane
-  const int groups = (g.nblk + PER - 1) / PER;                // of a row: what a warp moves
-  const long long n = (long long)g.ny * groups, warps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += warps) {
+  const int groups = (g.nblk + PER - 1) / PER;                // of a row
+  const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long k = k0 + (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5); k < k1; k += warps) {
     const int y = (int)(k / groups), x = (int)(k - (long long)y * groups) * 32 * PER + (threadIdx.x & 31) * PER;
     if (x >= g.pitch) continue;
     char* const part = lin + ((long long)y * g.nblk + (x >> 5)) * BYTES;
     const int at = x & 31;
-    const bool in0 = x < g.nx, in1 = x + 1 < g.nx;
-    const OutCell<ST> c0 = out_cell<ST>(g, in0 ? x : g.nx - 1, y), c1 = out_cell<ST>(g, in1 ? x + 1 : g.nx - 1, y);
+    auto cell = [&](int xx) {
+      OutCell<ST> c = out_cell<ST>(g, xx < g.nx ? xx : 0, y);
+      if (xx >= g.nx) {                                       // a pad column: its own place
+        c.rm = c.rq = c.r0;
+        c.c.c0 = col_bytes<ST>(xx);
+        c.wl = c.wr = c.wb = c.wt = false;
+      }
+      return c;
+    };
+    const OutCell<ST> c0 = cell(x), c1 = cell(x + PER - 1);
     auto word = [](char* p) -> unsigned int& { return *reinterpret_cast<unsigned int*>(p); };
     auto half = [](char* p) -> unsigned short& { return *reinterpret_cast<unsigned short*>(p); };
     unsigned int v[19];                                       // (16-bit storage: [18] the second rest population)
     each_pop(pops, [&](auto pop) {
       constexpr int A = decltype(pop)::value;
-      if constexpr (ST == ST_FP32) {
-        v[A] = OUT ? (in0 ? word(state + c0.template at<A>()) : 0u) : word(part + A * 128 + at * 4);
-      } else if constexpr (A == 0) {
-        v[0] = OUT ? (in0 ? word(state + c0.template at<0>()) : 0u) : word(part + at * 4);
-        if (OUT) v[18] = in1 ? word(state + c1.template at<0>()) : 0u;
+      if constexpr (pop_bytes(ST, A) == 4) {
+        v[A] = OUT ? word(state + c0.template at<A>()) : word(part + A * 128 + at * 4);
+        if constexpr (PER == 2) v[18] = word(state + c1.template at<A>());
       } else if constexpr (OUT) {
-        const unsigned int lo = in0 ? half(state + c0.template at<A>()) : 0u, hi = in1 ? half(state + c1.template at<A>()) : 0u;
+        const unsigned int lo = half(state + c0.template at<A>()), hi = half(state + c1.template at<A>());
         v[A] = lo | hi << 16;
       } else {
         v[A] = half(part + 128 + (A - 1) * 64 + at * 2);
@@ -197,39 +204,46 @@ __global__ void __launch_bounds__(256) k_reorder(char* __restrict__ state, char*
     });
     each_pop(pops, [&](auto pop) {
       constexpr int A = decltype(pop)::value;
-      if constexpr (OUT) {
-        if constexpr (ST == ST_FP32) {
-          word(part + A * 128 + at * 4) = v[A];
-        } else if constexpr (A == 0) {
-          word(part + at * 4) = v[0];
-          word(part + at * 4 + 4) = v[18];
-        } else {
-          word(part + 128 + (A - 1) * 64 + at * 2) = v[A];
-        }
-      } else if constexpr (pop_bytes(ST, A) == 4) {
-        if (in0) word(state + c0.template at<A>()) = v[A];
+      if constexpr (pop_bytes(ST, A) == 4) {
+        word(OUT ? part + A * 128 + at * 4 : state + c0.template at<A>()) = v[A];
+        if constexpr (PER == 2) word(part + at * 4 + 4) = v[18];
+      } else if constexpr (OUT) {
+        word(part + 128 + (A - 1) * 64 + at * 2) = v[A];
       } else {
-        if (in0) half(state + c0.template at<A>()) = (unsigned short)v[A];
+        half(state + c0.template at<A>()) = (unsigned short)v[A];
       }
     });
   }
 }
 
 template <int ST>
-static cudaError_t launch_reorder_st(const lbm_sim* s, void* state, void* lin, bool out, cudaStream_t st) {
+static cudaError_t launch_reorder_st(const lbm_sim* s, void* state, char* lin, long long k0, long long k1, bool out, cudaStream_t st) {
   const Grid g = make_grid(s, nullptr, nullptr);
-  const int per = reorder_cells(ST, out);
-  const long long want = ((long long)g.ny * ((g.nblk + per - 1) / per) + 7) / 8;
+  const long long want = (k1 - k0 + 7) / 8;
   const int grid = (int)(want < 64LL * s->sms ? want : 64LL * s->sms);
-  if (out) k_reorder<ST, true><<<grid, 256, 0, st>>>(static_cast<char*>(state), static_cast<char*>(lin), g);
-  else k_reorder<ST, false><<<grid, 256, 0, st>>>(static_cast<char*>(state), static_cast<char*>(lin), g);
+  char* const first = lin - reorder_offset(s, out, k0);
+  if (out) k_reorder<ST, true><<<grid, 256, 0, st>>>(static_cast<char*>(state), first, g, k0, k1);
+  else k_reorder<ST, false><<<grid, 256, 0, st>>>(static_cast<char*>(state), first, g, k0, k1);
   return cudaGetLastError();
 }
 
-cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, bool out, cudaStream_t st) {
+static long long reorder_row(const lbm_sim* s, bool out) {
+  const int per = reorder_cells(s->params.storage, out);
+  return (s->pitch / BLK + per - 1) / per;
+}
+long long reorder_groups(const lbm_sim* s, bool out) { return s->ny * reorder_row(s, out); }
+long long reorder_offset(const lbm_sim* s, bool out, long long k) {
+  const long long row = reorder_row(s, out), per = reorder_cells(s->params.storage, out);
+  return ((k / row) * (s->pitch / BLK) + (k % row) * per) * BLK * state_bytes_per_cell(s->params.storage);
+}
+long long reorder_fit(const lbm_sim* s, bool out, size_t bytes) {
+  return (long long)bytes / (reorder_cells(s->params.storage, out) * BLK * state_bytes_per_cell(s->params.storage));
+}
+
+cudaError_t launch_reorder(const lbm_sim* s, void* state, void* lin, long long k0, long long k1, bool out, cudaStream_t st) {
   // the two 16-bit storages are laid out alike
-  return s->params.storage == LBM_FP32 ? launch_reorder_st<ST_FP32>(s, state, lin, out, st)
-                                       : launch_reorder_st<ST_FP16>(s, state, lin, out, st);
+  return s->params.storage == LBM_FP32 ? launch_reorder_st<ST_FP32>(s, state, static_cast<char*>(lin), k0, k1, out, st)
+                                       : launch_reorder_st<ST_FP16>(s, state, static_cast<char*>(lin), k0, k1, out, st);
 }
 
 // ------------------------------------------------------------------ FP64 diagnostics
