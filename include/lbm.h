@@ -236,6 +236,8 @@ LBM_API int lbm_set_stream(lbm_sim* sim, void* cuda_stream);
  * no effect: the grid's width decides (128, 64 or 32 threads of two columns each).  Results do not depend on the
  * shape. */
 LBM_API int lbm_set_tile(lbm_sim* sim, int threads, int seg_rows);
+/* Back to the rows per CTA of a new simulation. */
+LBM_API int lbm_set_tile_auto(lbm_sim* sim);
 
 /* Step kernel of the simulation (no counterpart in the paper; both kernels compute every cell
  * bitwise alike): LBM_KERNEL_AUTO (default), LBM_KERNEL_ROWS, LBM_KERNEL_TILES or
@@ -326,6 +328,8 @@ LBM_API int lbm_batch_step(lbm_batch* b, int k);
 /* Rows per tile of the batch kernel for members that did not set their own (>= 1; 0 keeps the current
  * value); threads as in lbm_set_tile.  Takes effect at the next step. */
 LBM_API int lbm_batch_set_tile(lbm_batch* b, int threads, int seg_rows);
+/* Back to the rows per tile that the library chooses for the members. */
+LBM_API int lbm_batch_set_tile_auto(lbm_batch* b);
 /* Members, device bytes in use. */
 LBM_API int lbm_batch_size(const lbm_batch* b);
 LBM_API size_t lbm_batch_bytes(const lbm_batch* b);

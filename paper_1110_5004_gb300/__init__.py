@@ -17,8 +17,11 @@ from ._lib import (LBM_BF16_DEV, LBM_ERR_BUDGET, LBM_ERR_DIVERGED, LBM_FP16_DEV,
 
 __all__ = ["Sim", "Batch", "LBMError", "params_from_physical", "lbm_params", "LBM_FP32",
            "LBM_FP16_DEV", "LBM_BF16_DEV", "LBM_PERIODIC", "LBM_WALL", "LBM_ERR_DIVERGED",
-           "LBM_ERR_BUDGET", "LBM_KERNEL_AUTO", "LBM_KERNEL_ROWS", "LBM_KERNEL_TILES", "LBM_KERNEL_RESIDENT",
+           "LBM_ERR_BUDGET", "AUTO_ROWS", "LBM_KERNEL_AUTO", "LBM_KERNEL_ROWS", "LBM_KERNEL_TILES", "LBM_KERNEL_RESIDENT",
            "device_bytes"]
+
+
+AUTO_ROWS = "auto"   # set_tile's seg_rows: the library's own choice
 
 
 def lib():
@@ -116,8 +119,12 @@ class Sim:
             pass
 
     def set_tile(self, threads=0, seg_rows=0):
-        """Tile of the row march: rows per CTA (0 keeps the current value; a simulation starts with
-        as many as fill one wave of resident CTAs).  `threads` (64, 128, 256 or 0) has no effect."""
+        """Tile of the row march: rows per CTA (0 keeps the current value; AUTO_ROWS goes back to what a
+        simulation starts with, as many as fill one wave of resident CTAs).  `threads` (64, 128, 256 or 0)
+        has no effect."""
+        if seg_rows == AUTO_ROWS:
+            _lib.check(lib().lbm_set_tile_auto(self._h))
+            seg_rows = 0
         _lib.check(lib().lbm_set_tile(self._h, int(threads), int(seg_rows)))
 
     def set_kernel(self, kernel):
@@ -252,7 +259,10 @@ class Batch:
 
     def set_tile(self, threads=0, seg_rows=0):
         """Rows per tile of the batch kernel for members without their own; 0 keeps the current
-        value.  `threads` as in Sim.set_tile."""
+        value, AUTO_ROWS leaves them to the library again.  `threads` as in Sim.set_tile."""
+        if seg_rows == AUTO_ROWS:
+            _lib.check(lib().lbm_batch_set_tile_auto(self._h))
+            seg_rows = 0
         _lib.check(lib().lbm_batch_set_tile(self._h, int(threads), int(seg_rows)))
 
     @property

@@ -26,7 +26,7 @@ EXPORTS = (
     "lbm_batch_add", "lbm_batch_remove", "lbm_batch_step", "lbm_batch_size", "lbm_batch_bytes",
     "lbm_batch_destroy", "lbm_diagnostics_fields_noalloc", "lbm_batch_set_tile", "lbm_checkpoint_bytes",
     "lbm_checkpoint", "lbm_restore", "lbm_sim_device_bytes", "lbm_init_fields_packed", "lbm_moments_packed",
-    "lbm_set_kernel", "lbm_set_wait_limit", "lbm_step_status", "lbm_active_kernel",
+    "lbm_set_kernel", "lbm_set_wait_limit", "lbm_step_status", "lbm_active_kernel", "lbm_set_tile_auto", "lbm_batch_set_tile_auto",
 )
 
 
@@ -84,6 +84,7 @@ def load(path: str = LIB_PATH):
         "lbm_restore": (ip, [vp, vp, ctypes.c_size_t]),
         "lbm_set_stream": (ip, [vp, vp]),
         "lbm_set_tile": (ip, [vp, ip, ip]),
+        "lbm_set_tile_auto": (ip, [vp]),
         "lbm_set_kernel": (ip, [vp, ip]),
         "lbm_set_wait_limit": (ip, [vp, ctypes.c_longlong, ip]),
         "lbm_step_status": (ip, [vp]),
@@ -96,6 +97,7 @@ def load(path: str = LIB_PATH):
         "lbm_batch_remove": (ip, [vp, ip]),
         "lbm_batch_step": (ip, [vp, ip]),
         "lbm_batch_set_tile": (ip, [vp, ip, ip]),
+        "lbm_batch_set_tile_auto": (ip, [vp]),
         "lbm_batch_size": (ip, [vp]),
         "lbm_batch_bytes": (ctypes.c_size_t, [vp]),
         "lbm_batch_destroy": (ip, [vp]),

@@ -747,6 +747,12 @@ int lbm_set_tile(lbm_sim* s, int threads, int seg_rows) {
   return LBM_OK;
 }
 
+int lbm_set_tile_auto(lbm_sim* s) {
+  if (!s) return set_error("sim is NULL"), LBM_ERR_INVALID_ARG;
+  s->seg_h = 0;
+  return LBM_OK;
+}
+
 int lbm_set_kernel(lbm_sim* s, int kernel) {
   if (!s) return set_error("sim is NULL"), LBM_ERR_INVALID_ARG;
   if (kernel != LBM_KERNEL_AUTO && kernel != LBM_KERNEL_ROWS && kernel != LBM_KERNEL_TILES &&

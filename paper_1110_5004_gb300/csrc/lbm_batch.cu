@@ -307,6 +307,13 @@ int lbm_batch_set_tile(lbm_batch* b, int threads, int seg_rows) {
   return LBM_OK;
 }
 
+int lbm_batch_set_tile_auto(lbm_batch* b) {
+  if (!b) return set_error("batch is NULL"), LBM_ERR_INVALID_ARG;
+  b->seg_h = 0;
+  b->dirty = true;
+  return LBM_OK;
+}
+
 int lbm_batch_size(const lbm_batch* b) {
   if (!b) return 0;
   int n = 0;
