@@ -524,9 +524,11 @@ static cudaError_t launch_tile2d_st(const Phys& P, const Grid& g, const MomentOu
   // Beyond one wave of single tiles, and where x is periodic, two tiles per CTA: 320 threads and 2 CTAs per SM while
   // the pairs fit one such wave, else 256 threads and 3 CTAs.  Single tiles -> pairs, us per step: 256^2 (256 pairs)
   // 5.27 -> 4.91, 150 x 450 (285) 5.54 -> 5.08, 320^2 (400) 7.87 -> 6.65, 384^2 (576) 9.58 -> 9.04, 256 x 1024 (1024)
-  // 15.5 -> 13.3.  A little over one wave of 3 per SM (512 pairs: 256 x 512 8.70 -> 8.94) they stay single.
+  // 15.5 -> 13.3.  A little over one wave of 3 per SM they stay single where y is periodic (456 to 532 pairs, single against
+  // pairs: 256 x 512 FP32 8.00 / 8.10, FP16 7.94 / 8.40, BF16 8.00 / 8.62, 13 more grids alike; 536 pairs 8.12 / 8.12; with walls on y
+  // 8.73 / 8.42, 8.76 / 8.49, 8.83 / 8.88).
   const long long pairs = (long long)((g.nx + 2 * T2D_TX - 1) / (2 * T2D_TX)) * ((g.ny + T2D_TY - 1) / T2D_TY);
-  const bool tail = pairs > 3LL * sms && 2 * pairs <= 7LL * sms;
+  const bool tail = g.bc_y != BC_WALL && pairs > 3LL * sms && 2 * pairs <= 7LL * sms;
   if (!mo && tiles > slots && !tail && g.bc_x != BC_WALL && g.nx >= 2 * T2D_TX + 6 && g.ny >= T2D_TY + 6) {
     const Phys2 P2 = widen(P);
     const bool yw = g.bc_y == BC_WALL;
