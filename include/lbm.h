@@ -303,9 +303,9 @@ LBM_API const char* lbm_last_error(void);
  *                   LBM_ERR_INVALID_ARG, and a device out must be passed.
  * The reduction is the one lbm_diagnostics performs (same partials, order and result).  The
  * first call on a device looks up the array's device address with that device current; make
- * that first call before any stream capture.  All calls share the array: nothing in it has to
- * start at zero (every partial read is written first by the same call), but two calls whose
- * kernels overlap on the GPU race on it. */
+ * that first call before any stream capture.  All calls share the array: each writes what it
+ * reads first, but two calls whose kernels overlap on the GPU race on it, and the record of either may then
+ * be a mixture, or an earlier call's. */
 LBM_API int lbm_diagnostics_fields_noalloc(const float* phi, const float* ux, const float* uy, const float* p,
                                            int nx, int ny, double phi_star, long long step, void* cuda_stream,
                                            lbm_diag* out);

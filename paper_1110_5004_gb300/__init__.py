@@ -154,8 +154,8 @@ class Sim:
         _lib.check(lib().lbm_init_fields(self._h, _ptr(phi0), _ptr(ux0), _ptr(uy0), _ptr(p0)))
 
     def init_fields_packed(self, fields):
-        """lbm_init_fields_packed: phi0, ux0, uy0, p0 in one (4, ny, nx) float32 block (host
-        array or device tensor), copied in one transfer."""
+        """lbm_init_fields_packed: phi0, ux0, uy0, p0 in one (4, ny, nx) float32 block: a host array, copied
+        in one transfer, or a device tensor, read in place."""
         _lib.check(lib().lbm_init_fields_packed(self._h, _ptr(fields)))
 
     def moments_packed(self, out=None):

@@ -72,8 +72,8 @@ __device__ __forceinline__ void unpack2(V2 p, float& a, float& b) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p.v));
 }
 
-// Every floating-point operation of the step is an explicit round-to-nearest instruction, so no
-// multiply-add contraction is left to the compiler: a cell's arithmetic is the same in every
+// Every floating-point operation of the step is an explicit round-to-nearest instruction, and a product that an addition
+// takes is a scalar one (fmul_add), so that no multiply-add is contracted: a cell's arithmetic is the same in every
 // kernel, alone or in a batch.
 __device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b); }
@@ -89,6 +89,7 @@ __device__ __forceinline__ V2 fsub(V2 a, V2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
   return r;
 }
+// (not where an addition takes the product: fmul_add)
 __device__ __forceinline__ V2 fmul(V2 a, V2 b) {
   V2 r;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
@@ -278,8 +279,6 @@ __host__ __device__ __forceinline__ int wrap(int i, int n) {
   i %= n;
   return i < 0 ? i + n : i;
 }
-// Mirror about a wall half a cell outside the edge: -1 -> 0, -2 -> 1, n -> n-1.
-__device__ __forceinline__ int mirror(int i, int n) { return i < 0 ? -1 - i : (i >= n ? 2 * n - 1 - i : i); }
 
 // Wrap an index that lies within one period of [0, n) (the general case takes a modulo).
 __host__ __device__ __forceinline__ int wrap1(int i, int n) {

@@ -477,7 +477,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
       if constexpr (SD) sdef = fadd(fsub(density(P, ph), pack2(sp_ra, sp_rb)), pack2(sp_da, sp_db));
       else sdef = fmul(P.s_coef6, lap6_of(P, ms, m0, mn));
       asm("" : "+l"(sdef.v));                      // computed either way: no branch around the stencil
-      const V2 s_all = sdef;                       // F_a is reported whether or not the scheme removes it
+      [[maybe_unused]] const V2 s_all = sdef;      // F_a is reported whether or not the scheme removes it
       sdef.v = P.remove_Fa ? sdef.v : 0ull;
       V2 gb[Q];
       pull9(G0{}, sm.stage[gs].g, gb);

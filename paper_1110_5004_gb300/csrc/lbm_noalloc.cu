@@ -8,9 +8,10 @@
 // memory the library would allocate.
 //
 // The array is shared by every call in the process on a given device and keeps the last
-// call's contents.  Every partial a call reads is written earlier by the same call, so nothing
-// has to start at zero; two calls whose kernels overlap on the GPU (different streams, no
-// ordering between them) race on it and must not be issued.
+// call's contents.  Every partial a call reads is written earlier by the same call, and the count of
+// finished blocks is cleared by it; two calls whose kernels overlap on the GPU (different streams, no
+// ordering between them) race on both and must not be issued: the record of either may be a mixture, or
+// an earlier call's.
 #include <math.h>
 #include <mutex>
 

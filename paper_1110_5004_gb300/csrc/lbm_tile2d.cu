@@ -1,7 +1,7 @@
 // Small-grid form of the fused step: one CTA computes a TX x TY tile of cells in four passes over
 // shared memory instead of marching a strip of rows.
 //
-// On a small grid the row march is latency-bound: a segment of h rows takes h + 8 dependent row
+// On a small grid the row march is latency-bound: a segment of h rows takes h + 7 dependent row
 // iterations, each waiting on the last, however few rows it has.  Here a step is one round of
 // population loads (all issued at once) and four short passes separated by three barriers:
 //   S0  phi on the tile plus a 3-cell halo          (pull of f, bounce-back at walls)
@@ -11,8 +11,8 @@
 // S0 keeps the pulled f of the tile's own cells and S2 their pulled gbar for S3, which splits
 // each cell's collision between two threads (f and gbar).
 // Every per-cell operation is the shared stage function the row march uses (lbm_device.cuh), with
-// the same neighbour values: cells next to a wall also write their value into the mirrored ghost
-// position, as in the row march, so the state is bitwise the one the row march computes.
+// the same neighbour values, so the state is bitwise the one the row march computes: beyond a wall the cell's own
+// value, its mirror image, which single tiles write into a ghost position and pairs of tiles read in its place.
 // Scope: s by Eq. 5 (s_form 0) and the mu-term order-parameter equilibrium (f_form 0), any storage
 // and boundaries; other configurations run the row march.
 #include <vector>
@@ -231,7 +231,8 @@ __global__ void __launch_bounds__(NT) k_tile2d(Phys P, Grid g, int tiles_x) {
 }
 
 // ---- Two tiles per CTA, side by side in x, each value the pair of the two tiles' cells (V2): the same four passes
-// with packed arithmetic and one shared-memory access for both.  For a periodic x axis.
+// with packed arithmetic and one shared-memory access for both.  For a periodic x axis.  76-96 registers; three CTAs of 256
+// threads leave 80, of which BF16 with walls on y spills 12 bytes a thread.
 template <int TX, int TY>
 struct SmemPair {
   static constexpr int FW = TX + 6, FH = TY + 6;
