@@ -123,8 +123,9 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
   g.bc_x = s->params.bc_x;
   g.bc_y = s->params.bc_y;
   tile_geometry(s->shape, s->seg_h, s->sms, &g);
-  const long long tries = s->wait_ns / WAIT_TRY_NS + 2;
-  g.wait = WaitLimit{gave_up(s), s->slot ? &s->slot->gave_up : nullptr, (int)std::min(tries, 1LL << 30), -1};
+  g.wait_tries = (int)std::min(s->wait_ns / WAIT_TRY_NS + 2, 1LL << 30);
+  g.wait_hold = -1;
+  g.give_up = GiveUp{gave_up(s), s->slot ? &s->slot->gave_up : nullptr};
   g.spoff = s->params.s_form ? (long long)s->pop_bytes : 0;
   return g;
 }
@@ -476,7 +477,7 @@ int lbm_step(lbm_sim* s, int n) {
   const bool tiles = uses_tile2d(s);
   for (int i = 0; i < n; ++i) {
     Grid g = make_grid(s, s->buf[s->cur], s->buf[s->cur ^ 1]);
-    g.wait.hold = s->hold;
+    g.wait_hold = s->hold;
     cudaError_t e = tiles ? launch_tile2d(s->phys, g, nullptr, s->sms, s->stream) : launch_step(s->phys2, g, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "lbm_step launch");
     s->cur ^= 1;

@@ -116,7 +116,7 @@ static int rebuild(lbm_batch* b) {
       h = (s->ny + segs - 1) / segs;
     }
     tile_geometry(march_shape_of(s->nx, s->params.storage, s->params.s_form != 0, threads[part]), h, sms, &g);
-    g.wait.hold = s->hold;
+    g.wait_hold = s->hold;
     d.g = g;
     d.buf0 = s->buf[0];
     d.buf1 = s->buf[1];

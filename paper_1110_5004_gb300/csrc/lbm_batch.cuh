@@ -59,11 +59,11 @@ __global__ void __launch_bounds__(NT, march_ctas(NT)) k_batch(const SimDesc* __r
     __syncthreads();
     w = __shfl_sync(0xffffffffu, sm.next, 0);   // (uniform to the compiler, which keeps addresses in uniform registers)
     if (sm.m.quit != 0u) {  // a wait ran out in an earlier tile (of any thread: behind its last barrier): not done
-      if (threadIdx.x == 0) d.g.wait.raise();
+      if (threadIdx.x == 0) d.g.give_up.raise();
       __syncthreads();      // sm.next is read above and written for the next tile
       continue;
     }
-    march<MODE_STEP, ST, SD, false, XW, false, NT>(sm.P, g, &d.g.wait, MomentOut{}, it.y, it.z, sm.m, fat, gat);
+    march<MODE_STEP, ST, SD, false, XW, false, NT>(sm.P, g, &d.g.give_up, MomentOut{}, it.y, it.z, sm.m, fat, gat);
   }
 }
 

@@ -232,11 +232,9 @@ __host__ __device__ constexpr int pop_off(int st, int a) {
 
 // The waits of the row march for its copies.  They end with the copies; the limit keeps a fault elsewhere from turning
 // into a hang.  A launch whose wait runs out raises both words.
-struct WaitLimit {
+struct GiveUp {
   unsigned int* word;   // on the device, kept until the next state (k_init_pop, lbm_restore) or until it is read
   unsigned int* host;   // the same in page-locked memory, which the host reads without a copy; or null
-  int tries;            // of a wait
-  int hold;             // test hook: this tile's rows are never copied (-1: none)
   __device__ __forceinline__ void raise() const {
     *static_cast<volatile unsigned int*>(word) = 1u;
     if (host) *static_cast<volatile unsigned int*>(host) = 1u;
@@ -256,8 +254,10 @@ struct Grid {
   int tile_w;           // columns per lane of a row-march CTA (a CTA covers two lanes)
   int seg_h;            // rows per segment
   int n_strips;         // CTAs across the grid
+  int wait_tries;       // limit of a wait of the row march
+  int wait_hold;        // test hook: this tile's rows are never copied (-1: none)
   long long spoff;      // s_form 1: byte offset of the [rho, div(rho u)] planes in src/dst (else 0)
-  WaitLimit wait;
+  GiveUp give_up;
 };
 
 // Outputs of the moment pass (row-major); each may be null.  fax, fay: the

@@ -70,7 +70,7 @@ struct Range {
 constexpr int N_FIELDS = 6;
 constexpr int DIAG_PARTIALS = 12;
 // Words in the spare doubles behind the diagnostics record: raised by a wait of the row march that ran out
-// (WaitLimit::word); blocks of a diagnostics launch that have finished.
+// (GiveUp::word); blocks of a diagnostics launch that have finished.
 inline unsigned int* gave_up(const lbm_sim* s) { return reinterpret_cast<unsigned int*>(s->red + (size_t)s->ny * DIAG_PARTIALS + 14); }
 inline unsigned int* diag_done(const lbm_sim* s) { return gave_up(s) + 1; }
 

@@ -28,7 +28,7 @@ __global__ void k_init_pop(Phys P, Grid g, InitIn in) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   // a new state: the old one's give-up words are cleared, at the end, where the look at one has arrived
   const bool first = x == 0 && blockIdx.y == 0;
-  const unsigned int stale = first ? *static_cast<volatile unsigned int*>(g.wait.word) : 0u;
+  const unsigned int stale = first ? *static_cast<volatile unsigned int*>(g.give_up.word) : 0u;
   if (x >= g.nx) return;
   const Col3 col = col3<ST>(x, g.nx);
   // neighbours: beyond a wall the mirrored row or column (zero gradient)
@@ -104,8 +104,8 @@ __global__ void k_init_pop(Phys P, Grid g, InitIn in) {
     }
   }
   if (first && stale != 0u) {
-    *g.wait.word = 0u;
-    if (g.wait.host) *static_cast<volatile unsigned int*>(g.wait.host) = 0u;
+    *g.give_up.word = 0u;
+    if (g.give_up.host) *static_cast<volatile unsigned int*>(g.give_up.host) = 0u;
   }
 }
 

@@ -278,10 +278,10 @@ struct StageAt {
 // FP32 storage only).  XW: the x axis may have walls.  K: the scheme constants (Phys2, in the constant bank
 // or in shared memory).
 // PDL: the launch is a programmatic dependent of the previous one and waits for it here, once its addresses are formed.
-// limit: of its waits (in the constant bank or in global memory).  When one runs out the tile is left undone, sm.quit is set,
-// and the CTA must not march again.
+// give_up: in the constant bank or in global memory, read when a wait runs out: the tile is then left undone, sm.quit is
+// set, and the CTA must not march again.
 template <int MODE, int ST, bool SD, bool FF, bool XW, bool PDL, int NT, class K>
-__device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit* limit, const MomentOut& mo, int strip, int seg,
+__device__ __forceinline__ void march(const K& P, const Grid& g, const GiveUp* give_up, const MomentOut& mo, int strip, int seg,
                                       MarchSmem<ST, SD, NT>& sm, StageAt& fat, StageAt& gat) {
   constexpr int GT = NT > 32 ? 32 : 16;            // the thread that copies gbar (thread 0 copies f)
   const int t = threadIdx.x;
@@ -345,7 +345,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
-  const bool held = MODE == MODE_STEP && g.wait.hold == seg * g.n_strips + strip;
+  const bool held = MODE == MODE_STEP && g.wait_hold == seg * g.n_strips + strip;
   for (int k = 0; k < STAGES; ++k)
     produce(!held, ya - 3 + k, fat.ahead(k), !held && ya - 1 + k <= a_end - 3, ya - 1 + k, gat.ahead(k));
 
@@ -436,7 +436,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
   // Wait for a staged row, a counted number of tries.  Past that the thread waits no more and copies no more, and what is
   // left of the tile runs through on what the rings hold, so that the iterations need no test of their own.  (With one
   // and a way out of the loop, or with a clock in the wait: 2048 x 512 FP16 5-7 % slower, 601 x 437 with x walls 6-10 %.)
-  int tries = limit->tries;
+  int tries = g.wait_tries;
   auto wait_row = [&](unsigned long long* b, int parity) {
     for (int n = 0; n < tries; ++n)
       if (mbar_try(b, parity)) return;
@@ -445,7 +445,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
     tries = 1;
     role = -1;
     sm.quit = 1u;
-    limit->raise();
+    give_up->raise();
   };
 
   auto iter = [&](int a, auto kind) {
@@ -630,7 +630,7 @@ __device__ __forceinline__ void march(const K& P, const Grid& g, const WaitLimit
       at.parity = sm.left[t != 0].y;
       int n = 0;
       for (int k = 0; k < STAGES; ++k, at.next())
-        while (n < limit->tries && !mbar_try(bar + at.stage, at.parity)) ++n;
+        while (n < g.wait_tries && !mbar_try(bar + at.stage, at.parity)) ++n;
     }
     __syncthreads();
   }

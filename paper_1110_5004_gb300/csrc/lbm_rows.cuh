@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(NT, march_ctas(NT)) k_march(const __grid_const
   MarchSmem<ST, SD, NT>& sm = *reinterpret_cast<MarchSmem<ST, SD, NT>*>(smem_raw);
   march_init(sm);
   StageAt fat, gat;
-  march<MODE, ST, SD, FF, XW, true, NT>(P, g, &g.wait, mo, blockIdx.x % g.n_strips, blockIdx.x / g.n_strips, sm, fat, gat);
+  march<MODE, ST, SD, FF, XW, true, NT>(P, g, &g.give_up, mo, blockIdx.x % g.n_strips, blockIdx.x / g.n_strips, sm, fat, gat);
 }
 
 template <int MODE, int ST, bool SD, bool FF, bool XW, int NT>
