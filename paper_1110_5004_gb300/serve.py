@@ -142,8 +142,8 @@ class Server:
         self.max_cells = max_cells
         # a member of at least this many cells steps alone, with the single-simulation kernels
         # (the small-grid tile kernel up to 256K cells, the row march above), on a stream of its
-        # own; smaller members share the batch.  On the c5 stream, 64K cells and 8 streams served
-        # 23.1 GLUPS against 22.0 with a 1M threshold and 4 streams (256 requests).
+        # own; smaller members share the batch.  On the c5 stream (256 requests, steps x 0.2) thresholds of
+        # 64K to 1M cells serve alike, 31-34 GLUPS, within what runs of one setting differ.
         self.solo_cells = solo_cells
         self.solo_bytes = 0
         self._solo_key = 0
