@@ -64,16 +64,17 @@ Phys make_phys(const lbm_params& p) {
 }
 
 MarchShape march_shape_of(int nx, int storage, bool sd, int nt) {
-  const int most = 2 * (nt - 6), slots = march_slots(nt, storage, sd);
-  for (int strips = (nx + most - 1) / most;; ++strips) {
-    const int width = (nx + 2 * strips - 1) / (2 * strips);
+  const int slots = march_slots(nt, storage, sd);
+  for (int most = nt - 6;;) {
+    const int strips = (nx + 2 * most - 1) / (2 * most), width = (nx + 2 * strips - 1) / (2 * strips);
     if (nt < MARCH_NT && width < 16 && strips > 1) return MarchShape{nt, 0, 0};   // more halo than strip
-    int blocks = 0;
-    for (int k = 0; k < strips; ++k) {
+    bool fits = true;
+    for (int k = 0; k < strips && fits; ++k) {
       const StagedRun r = staged_run(nx, k * 2 * width, width);
-      blocks = std::max(blocks, r.run1 + r.run2);
+      fits = r.run1 + r.run2 <= slots;
     }
-    if (blocks <= slots) return MarchShape{nt, strips, width};
+    if (fits) return MarchShape{nt, strips, width};
+    most = width - 1;                              // (more strips of the same width stage the same columns)
   }
 }
 

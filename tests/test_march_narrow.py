@@ -153,3 +153,20 @@ def test_batches_of_narrow_members_equal_alone(lbm, storage, widest, wide_too):
         alone = lbm.Sim.from_workload(w, storage=storage, kernel=lbm.LBM_KERNEL_ROWS)
         alone.step(5)
         assert np.array_equal(s.checkpoint(), alone.checkpoint()), w.nx
+
+
+def wide_members():
+    import time
+    lbm, f, events = library()
+    sims = [simulation(lbm, nx, ny) for nx, ny in ((3000000, 3), (52, 600))]
+    batch = lbm.Batch()
+    for s in sims:
+        batch.add(s)
+    t0 = time.perf_counter()
+    batch.step(1)
+    assert time.perf_counter() - t0 < 2.0
+
+
+def test_strips_of_very_wide_members_are_chosen_quickly(fake):   # noqa: F811
+    """A batch tries each thread count for each member: by width, not strip by strip (9 s for this one)."""
+    run(fake, "wide_members", module="test_march_narrow")
