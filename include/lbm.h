@@ -255,7 +255,8 @@ LBM_API int lbm_set_kernel(lbm_sim* sim, int kernel);
  * that of LBM_KERNEL_TILES.  n = 1 runs the tile kernel.
  *
  * lbm_set_wait_limit: every such wait, and every wait of the row march (alone or in a batch) for its
- *   rows, gives up after timeout_ns nanoseconds (default 1e9, > 0); the launch then ends early and
+ *   rows, gives up after timeout_ns nanoseconds (default 1e9, > 0; the row march's after 1 ms at
+ *   least, and within about a third of it); the launch then ends early and
  *   leaves the state undefined, later resident launches do nothing, and the next lbm_step_status or
  *   lbm_diagnostics returns LBM_ERR_TIMEOUT (which re-arms the waits; lbm_init_fields or lbm_restore
  *   then gives a defined state again).  For the row march lbm_moments, lbm_moments_packed,

@@ -124,7 +124,7 @@ Grid make_grid(const lbm_sim* s, const void* src, void* dst) {
   g.bc_x = s->params.bc_x;
   g.bc_y = s->params.bc_y;
   tile_geometry(s->shape, s->seg_h, s->sms, &g);
-  g.wait_tries = (int)std::min(s->wait_ns / WAIT_TRY_NS + 2, 1LL << 30);
+  g.wait_tries = (int)std::min(std::max(s->wait_ns, WAIT_LEAST_NS) / WAIT_TRY_NS + 1, 1LL << 30);
   g.wait_hold = -1;
   g.give_up = GiveUp{gave_up(s), s->slot ? &s->slot->gave_up : nullptr};
   g.spoff = s->params.s_form ? (long long)s->pop_bytes : 0;

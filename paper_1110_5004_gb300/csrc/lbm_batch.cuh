@@ -78,6 +78,7 @@ struct BatchPart {
 
 template <int ST, bool SD, bool XW, int NT>
 static cudaError_t launch_batch_t(const BatchPart& p, cudaStream_t st) {
+  static_assert((sizeof(BatchSmem<ST, SD, NT>) + 1024) * march_ctas(NT) <= 233472, "the CTAs of an SM fit its shared memory");
   // set once, thread-safely (one GPU per process)
   static const cudaError_t attr_set =
       cudaFuncSetAttribute(k_batch<ST, SD, XW, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BatchSmem<ST, SD, NT>));

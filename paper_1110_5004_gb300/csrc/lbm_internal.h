@@ -11,6 +11,7 @@
 
 namespace lbm {
 constexpr long long WAIT_TRY_NS = 1300;   // what a try of a row march's wait takes (measured: 26 ms for 20 003)
+constexpr long long WAIT_LEAST_NS = 1000000;   // its least limit: longer than copies take on a busy device
 // Page-locked words of a simulation that its kernels write: the host reads them without a copy.
 struct HostRecord {
   lbm_diag diag;

@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(NT, march_ctas(NT)) k_march(const __grid_const
 
 template <int MODE, int ST, bool SD, bool FF, bool XW, int NT>
 static cudaError_t launch_march(const Phys2& P, const Grid& g, const MomentOut& mo, cudaStream_t st) {
+  static_assert((sizeof(MarchSmem<ST, SD, NT>) + 1024) * march_ctas(NT) <= 233472, "the CTAs of an SM fit its shared memory");
   // set once, thread-safely (host threads may step simulations concurrently; one GPU per process)
   static const cudaError_t attr_set = cudaFuncSetAttribute(
       k_march<MODE, ST, SD, FF, XW, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MarchSmem<ST, SD, NT>));

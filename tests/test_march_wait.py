@@ -101,3 +101,18 @@ def test_a_batch_goes_on_after_a_wait_that_ran_out(lbm):
         alone.step(18)
         batch.remove(slot)
         assert np.array_equal(s.checkpoint(), alone.checkpoint())
+
+
+@pytest.mark.gpu
+def test_a_short_limit_of_the_resident_kernel_leaves_the_march_its_own(lbm):
+    """A limit of a nanosecond, as a resident simulation may set, is no reason for the march to give up sound rows."""
+    w = workload(2100, 300)
+    a = lbm.Sim.from_workload(w, kernel=lbm.LBM_KERNEL_ROWS)
+    b = lbm.Sim.from_workload(w, kernel=lbm.LBM_KERNEL_ROWS)
+    a.set_wait_limit(1)
+    for _ in range(5):
+        a.step(20)
+        b.step(20)
+        assert a.step_status() == 0
+    assert np.array_equal(a.checkpoint(), b.checkpoint())
+    assert np.array_equal(a.moments()["phi"], b.moments()["phi"])
